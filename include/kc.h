@@ -114,11 +114,11 @@ typedef struct kc_config {
                                      sectors, staged in shared memory, 4 = as 3,
                                      from hashes first written per CTA to a linear
                                      array (default)                                */
-    uint32_t split_max;           /* partitioned: a partition whose candidates
+    uint32_t split_max;           /* partitioned: a partition whose distinct keys
                                      overflow its shared-memory table is counted
                                      again as 2, 4, ... 2^split_max sub-ranges of
                                      its filter slice before it falls back to a
-                                     global table (0 = 6; at most the slice's
+                                     global table (0 = 8; at most the slice's
                                      log2 words; KC_SPLIT_NONE = never split)       */
     uint32_t prune_chain;         /* 1: the paper's two-filter Prune chain (direct
                                      strategy; KC_ERR_ARG with the partitioned one):
@@ -184,9 +184,9 @@ typedef struct kc_config {
  *                2^part_bits hash-prefix partitions (counting-sort shuffle, as
  *                the paper's Encode / Prefix-sum / Broker kernels group k-mers
  *                by consumer, Section III-B); kc_finalize gives each partition
- *                to one CTA that keeps the partition's filter words and table
- *                in shared memory (filter update, candidate claims, exact
- *                recount, compaction).  The filter is built at kc_finalize.
+ *                to one CTA that counts its distinct keys in a shared-memory
+ *                table, writes those of at least min_count and sets every
+ *                key's filter bits.  The filter is built at kc_finalize.
  *   AUTO         PARTITIONED when the filter slices fit shared memory, else
  *                DIRECT.
  */
@@ -196,8 +196,10 @@ enum { KC_STRATEGY_AUTO = 0, KC_STRATEGY_DIRECT = 1, KC_STRATEGY_PARTITIONED = 2
 typedef struct kc_stats {
     uint64_t windows;         /* valid windows added so far, all samples         */
     uint64_t bases;           /* bases added so far                              */
-    uint64_t candidates;      /* windows the filter reported as seen before      */
-    uint64_t table_keys;      /* distinct keys held in the table (all partitions) */
+    uint64_t candidates;      /* windows the filter reported as seen before
+                                 (PARTITIONED: with each partition's keys put
+                                 into the filter one after the other)           */
+    uint64_t table_keys;      /* distinct keys among them (all partitions)       */
     uint64_t result_keys;     /* keys in the result                              */
     uint64_t spilled_bytes;   /* result bytes copied to pinned host memory       */
     uint32_t partitions;      /* hash-prefix partitions used                     */

@@ -1,10 +1,10 @@
 // Batched finalize: many partitioned counting jobs in one set of launches.
 //
 // Consume: one persistent launch over a device work queue of (job, partition)
-// items from every job of the batch.  Each CTA takes the next item, keeps the
-// partition's filter slice and table in shared memory (filter update, candidate
-// claims, exact recount, survivor compaction; the same steps as the single-job
-// consumer) and moves on, so uneven jobs share the GPU without a launch each.
+// items from every job of the batch.  Each CTA takes the next item, counts the
+// partition's keys in a shared-memory table, writes the survivors and the
+// partition's filter words and moves on, so uneven jobs share the GPU without a
+// launch each.
 // Sort: every job's survivors are bucketed by the top bits of their key into
 // one flat bucket array covering all jobs, scanned once, scattered into each
 // job's own result arrays, and each bucket sorted by one warp.  These launches
@@ -40,6 +40,7 @@ struct JobDesc {
     // sort
     int sort_bits;
     int split_max;  // consumer: finest split level 2^split_max before the fallback
+    int split_min;  // level at which a sub-range's filter words fit the consumer's shared memory
     uint64_t bucket_base;  // first bucket of this job in the flat arrays
     uint64_t n_buckets;
     uint64_t* res_keys;
@@ -81,29 +82,65 @@ struct BatchDesc {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kConsumeThreads = 512;
+constexpr int kConsumeThreads = 512;      // consumer CTAs, two an SM
+constexpr int kConsumeThreadsWide = 1024;  // when the shared memory has room for one alone
+constexpr int kAhead = 4;                  // hashes a consumer thread has in flight
+constexpr unsigned long long kTopBit = 1ull << 63;
 constexpr int kTile = 4096;
 constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32 bits
 
-// NH > 0: every job of the batch sets NH bits per key; NH = 0: per job.
+// One partition at a time per CTA: every distinct key of the partition is
+// counted in a shared-memory table, and the filter words are built from the
+// table afterwards.  A key's filter bits do not depend on how often it was
+// seen, so the filter is updated once per distinct key instead of once per
+// window, no window waits for the filter's answer, and the hashes are read
+// once, without a recount.  (Updating the filter with every window and counting
+// the candidates took 0.975 ms for 1.18e8 windows of 4096 partitions, this
+// 0.745 ms: the instructions per window fell from 206 to about 130.  It is
+// bound by instruction issue; reading the hashes alone takes 0.17 ms, with one
+// probe each 0.21, with the queue's probes 0.36, the writing 0.09 and the
+// filter 0.11 more.)
 //
-// A partition whose candidates overflow the shared-memory table is counted
-// again in 2, 4, ... 2^split_max sub-ranges of its filter slice: the top bits
-// of a window's in-slice word index pick its sub-range, so two sub-ranges
-// never share a filter word and each one's filter, claims and recount are
-// exactly those of the whole partition restricted to its keys.  Sub-ranges
-// already finished stay finished when a later one has to split further.
-// Only a partition that overflows at the finest level is left to the global
-// fallback.  The finest level a job has needed is kept in its counters, and
-// its later partitions start there instead of overflowing again.
-template <int NH>
-__global__ void __launch_bounds__(kConsumeThreads, 2) k_consume_q(const BatchDesc* __restrict__ D) {
+//   count    each window's first probe; a window that finds its key adds one
+//            to its count.  The others (new keys and displaced ones, about one
+//            in four at 30x coverage) go to a queue of the warp; 32 of them at a
+//            time take one probe (and claim) each and go back to the queue if
+//            it failed, so every probe step has all its lanes.
+//   emit     keys of at least min_count, one position claim per warp
+//   filter   the counts are no longer needed: their memory takes the filter
+//            words, every key sets its bits, the words are written out
+//
+// The table holds the keys that occur once too, so it is twice as large as the
+// candidates alone would need (8192 slots, 96 KiB with the counts: two
+// 512-thread CTAs an SM; when only one fits, 1024 threads).  Triangular probing
+// keeps a table two thirds full (30x coverage) to about two probes a new key:
+// linear probing took 0.69 ms where this takes 0.60, and the probe loop of a
+// whole warp at once 0.75.
+//
+// A partition whose keys overflow the table is counted again in 2, 4, ...
+// 2^split_max sub-ranges of its filter slice: the top bits of a window's
+// in-slice word index pick its sub-range, so two sub-ranges never share a
+// filter word and each one's table and filter are exactly those of the whole
+// partition restricted to its keys.  Sub-ranges already finished stay finished
+// when a later one has to split further.  Only a partition that overflows at
+// the finest level is left to the global fallback.  The finest level a job has
+// needed is kept in its counters, and its later partitions start there instead
+// of overflowing again.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
+    k_consume_q(const BatchDesc* __restrict__ D) {
     extern __shared__ unsigned long long s_mem[];
     __shared__ int s_fail, s_hint;
     __shared__ unsigned s_item;
-    const int lane = threadIdx.x & 31;
+    constexpr int kWarps = THREADS / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t n_items = D->n_items;
+    // the warp's queue: hashes, and for each the slot to probe next (low 16
+    // bits) and the number of probes that failed (above)
+    unsigned long long* const wq = s_mem + wid * kWarpQueue;
+    uint32_t* const ws = reinterpret_cast<uint32_t*>(s_mem + kWarps * kWarpQueue) + wid * kWarpQueue;
+    unsigned long long* const sk = s_mem + kWarps * kWarpQueue * 3 / 2;
     uint64_t cand = 0, claimed = 0;
     DevCounters* last_ctr = nullptr;
     for (;;) {
@@ -123,14 +160,10 @@ __global__ void __launch_bounds__(kConsumeThreads, 2) k_consume_q(const BatchDes
         const uint32_t n_sw = 1u << J.slice_log2;
         const uint32_t T = 1u << J.table_log2;
         const uint32_t tmask = T - 1;
-        const int S = J.n_samples;
+        const int s2 = J.n_samples - 1;  // a slot's counts: 1 << s2 of them
         const int a = J.part_bits;
-        // the job's fields the inner loops use, in registers
-        const int bloom_shift = J.bloom_shift;
-        const bool all_cand = J.all_candidates != 0;
-        unsigned long long* sb = s_mem;
-        unsigned long long* sk = s_mem + n_sw;
-        uint32_t* sc = reinterpret_cast<uint32_t*>(s_mem + n_sw + T);
+        uint32_t* const sc = reinterpret_cast<uint32_t*>(sk + T);  // counts, then
+        unsigned long long* const sb = sk + T;                     // the filter words
         if (J.ctr != last_ctr) {  // per-job candidate counters
             cand = warp_sum(cand);
             claimed = warp_sum(claimed);
@@ -143,81 +176,109 @@ __global__ void __launch_bounds__(kConsumeThreads, 2) k_consume_q(const BatchDes
         }
         const uint64_t hpre = (uint64_t)part << (64 - a);
         const unsigned long long empty = hpre ^ (1ull << (64 - a));  // a hash of another partition
-        int sl = min(hint, J.split_max);  // split level: the partition is taken as 2^sl sub-ranges
+        int sl = max(min(hint, J.split_max), J.split_min);  // split level: the partition is taken as 2^sl sub-ranges
         uint32_t sub = 0;  // the sub-range being counted
         bool overflow = false;
         uint64_t h_left = 0;  // first hash left to the fallback
         for (;;) {
             const uint32_t w_n = n_sw >> sl;
-            const uint32_t w_lo = sub * w_n;
             const uint32_t smask = (1u << sl) - 1u;
             const int sub_shift = 64 - a - sl;  // sub-range = h bits [sub_shift, 64 - a)
             // a window belongs to the (sub-range of the) partition iff the top
             // a + sl <= 32 bits of its hash equal those of `range`
             const uint64_t range = hpre | ((uint64_t)sub << sub_shift);
             const uint32_t rhi = (uint32_t)(range >> 32), rmask = ~0u << (32 - a - sl);
-            uint64_t c_try = 0, k_try = 0;
-            for (uint32_t i = threadIdx.x; i < w_n; i += blockDim.x) sb[w_lo + i] = 0ull;
-            for (uint32_t i = threadIdx.x; i < T; i += blockDim.x) sk[i] = empty;
-            for (uint32_t i = threadIdx.x; i < T * S; i += blockDim.x) sc[i] = 0u;
+            for (uint32_t i = threadIdx.x; i < T; i += THREADS) sk[i] = empty;
+            for (uint32_t i = threadIdx.x; i < (T << s2); i += THREADS) sc[i] = 0u;
             if (threadIdx.x == 0) s_fail = 0;
             __syncthreads();
-            bool stop = false;
-            // A window of a thread's first 64 iterations over the first batch
-            // that finds or claims its key in the filter pass is counted there
-            // (bit m of `counted` for iteration m); the recount visits only the
-            // other windows.  Each window is counted once, by the pass that
-            // found its key: the table only grows, and the recount sees it whole.
-            uint32_t counted_lo = 0, counted_hi = 0;
+            bool stop = false;  // the same in all lanes of a warp
             for (int bt = 0; bt < J.n_batches && !stop; ++bt) {
                 const uint64_t lo = J.starts[bt][part];
                 const uint64_t n_all = J.starts[bt][part + 1] - lo;
                 uint32_t* const scol = sc + J.samples[bt];  // this batch's count column
+                unsigned q = 0;                             // entries in the warp's queue
+                // The queue's last n (at most 32) windows, one per lane, take their
+                // next probe: slots home, home + 1, home + 3, home + 6, ... (every
+                // slot of a power-of-two table in turn).
+                const auto step = [&](unsigned n) {
+                    __syncwarp();
+                    q -= n;
+                    bool again = false;
+                    unsigned long long h = 0;
+                    uint32_t next = 0;
+                    if ((unsigned)lane < n) {
+                        h = wq[q + lane];
+                        next = ws[q + lane];
+                        const uint32_t slot = next & tmask;
+                        unsigned long long cur = sk[slot];
+                        if (cur == empty) {
+                            cur = atomicCAS(sk + slot, empty, h);
+                            if (cur == empty) cur = h;
+                        }
+                        again = cur != h;
+                        if (!again) atomicAdd(scol + (slot << s2), 1u);
+                        next = ((next & 0xffff0000u) + 0x10000u) | ((slot + (next >> 16) + 1) & tmask);
+                        if (again && next >= (unsigned)kProbeLimit << 16) {
+                            s_fail = 1;
+                            again = false;
+                        }
+                    }
+                    const unsigned back = __ballot_sync(kFull, again);
+                    if (again) {
+                        const unsigned pos = q + __popc(back & lt);
+                        wq[pos] = h;
+                        ws[pos] = next;
+                    }
+                    q += __popc(back);
+                };
                 // 32-bit indices within chunks of 2^31 hashes (one chunk, in practice)
                 for (uint64_t c0 = 0; c0 < n_all && !stop; c0 += kChunk) {
                     const uint64_t* __restrict__ d = J.data[bt] + lo + c0;
                     const uint32_t n = (uint32_t)min(n_all - c0, (uint64_t)kChunk);
-                    const bool first = bt == 0 && c0 == 0;
-                    // each thread's next hash is in flight while it handles the current one
-                    uint64_t hn = threadIdx.x < n ? __ldcg(d + threadIdx.x) : 0ull;
-                    uint32_t m = 0;
-                    for (uint32_t t = threadIdx.x; t < n; t += kConsumeThreads, ++m) {
-                        const uint64_t h = hn;
-                        if (t + kConsumeThreads < n) hn = __ldcg(d + t + kConsumeThreads);  // read again by the recount: keep in L2
-                        if ((((uint32_t)(h >> 32)) ^ rhi) & rmask) continue;  // run padding, or another sub-range
-                        const uint32_t w = (uint32_t)(h >> bloom_shift) & (n_sw - 1);
-                        const uint64_t g = mixer64(h);
-                        const uint64_t pat = NH > 0 ? bloom_pattern_n<(NH > 0 ? NH : 1)>(g) : bloom_pattern_rt(g, J.n_hashes);
-                        const unsigned long long old = atomicOr(sb + w, (unsigned long long)pat);
-                        if (all_cand || (old & pat) == pat) {
-                            ++c_try;
-                            uint32_t slot;
-                            const int r = smem_claim(sk, tmask, (uint32_t)h & tmask, h, empty, slot);
-                            if (r < 0) {
-                                s_fail = 1;
-                                stop = true;
-                                break;
-                            }
-                            if (first && m < 64) {
-                                atomicAdd(scol + slot * S, 1u);
-                                if (m < 32) counted_lo |= 1u << m;
-                                else counted_hi |= 1u << (m - 32);
-                            }
-                            if (r > 0) {
-                                ++k_try;
-                                if (*(volatile int*)&s_fail) {  // another thread overflowed: give up early
-                                    stop = true;
-                                    break;
+                    // each thread's next hashes are in flight while it handles the current ones
+                    uint64_t hn[kAhead];
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e) {
+                        const uint32_t i = e * THREADS + threadIdx.x;
+                        hn[e] = i < n ? __ldcg(d + i) : empty;
+                    }
+                    for (uint32_t b = 0; b < n && !stop; b += kAhead * THREADS) {
+                        uint64_t hc[kAhead];
+#pragma unroll
+                        for (int e = 0; e < kAhead; ++e) {
+                            hc[e] = hn[e];
+                            const uint32_t i = b + (kAhead + e) * THREADS + threadIdx.x;
+                            hn[e] = i < n ? __ldcg(d + i) : empty;
+                        }
+#pragma unroll
+                        for (int e = 0; e < kAhead; ++e) {
+                            const uint64_t h = hc[e];
+                            const bool in = ((((uint32_t)(h >> 32)) ^ rhi) & rmask) == 0u;  // else run padding, or another sub-range
+                            const uint32_t s = (uint32_t)h & tmask;
+                            const unsigned long long cur = sk[s];
+                            const bool hit = in && cur == h;  // (padding may hold the empty mark)
+                            if (hit) atomicAdd(scol + (s << s2), 1u);
+                            const unsigned miss = __ballot_sync(kFull, in && !hit);
+                            if (miss) {
+                                if (in && !hit) {
+                                    const unsigned pos = q + __popc(miss & lt);
+                                    wq[pos] = h;
+                                    ws[pos] = cur == empty ? s : 0x10000u | ((s + 1) & tmask);
                                 }
+                                q += __popc(miss);
+                                while (q >= 32) step(32);
                             }
                         }
+                        stop = __any_sync(kFull, *(volatile int*)&s_fail);  // a warp overflowed: give up early
                     }
                 }
+                while (q) step(min(q, 32u));
+                stop = __any_sync(kFull, *(volatile int*)&s_fail);
             }
             __syncthreads();
-            const int failed = s_fail;
-            __syncthreads();
-            if (failed) {
+            if (s_fail) {
+                __syncthreads();  // s_fail is cleared for the next attempt
                 if (sl < J.split_max) {
                     ++sl;
                     sub <<= 1;
@@ -227,82 +288,84 @@ __global__ void __launch_bounds__(kConsumeThreads, 2) k_consume_q(const BatchDes
                 h_left = range;
                 break;
             }
-            cand += c_try;
-            claimed += k_try;
-            for (int bt = 0; bt < J.n_batches; ++bt) {
-                const uint64_t lo = J.starts[bt][part];
-                const uint64_t n_all = J.starts[bt][part + 1] - lo;
-                uint32_t* const scol = sc + J.samples[bt];
-                for (uint64_t c0 = 0; c0 < n_all; c0 += kChunk) {
-                    const uint64_t* __restrict__ d = J.data[bt] + lo + c0;
-                    const uint32_t n = (uint32_t)min(n_all - c0, (uint64_t)kChunk);
-                    uint32_t t0 = threadIdx.x;  // first iteration of the dense loop below
-                    if (bt == 0 && c0 == 0) {
-                        // iterations m < 64 the filter pass did not count, taken
-                        // by their bits; each one's hash is loaded a step ahead
-                        const uint32_t iters = threadIdx.x < n ? (n - 1 - threadIdx.x) / kConsumeThreads + 1 : 0;
-                        const uint32_t mi = iters < 64 ? iters : 64;
-                        const uint64_t in_range = mi == 64 ? ~0ull : (1ull << mi) - 1ull;
-                        uint64_t todo = ~(((uint64_t)counted_hi << 32) | counted_lo) & in_range;
-                        t0 = threadIdx.x + 64u * kConsumeThreads;
-                        uint64_t hn = todo ? __ldcs(d + threadIdx.x + (uint32_t)(__ffsll((long long)todo) - 1) * kConsumeThreads) : 0ull;
-                        while (todo) {
-                            const uint64_t h = hn;
-                            todo &= todo - 1ull;
-                            if (todo) hn = __ldcs(d + threadIdx.x + (uint32_t)(__ffsll((long long)todo) - 1) * kConsumeThreads);
-                            if ((((uint32_t)(h >> 32)) ^ rhi) & rmask) continue;
-                            const int s = smem_find(sk, tmask, (uint32_t)h & tmask, h, empty);
-                            if (s >= 0) atomicAdd(scol + (uint32_t)s * S, 1u);
-                        }
-                    }
-                    if (t0 >= n) continue;
-                    uint64_t hn = __ldcs(d + t0);
-                    for (uint32_t t = t0; t < n; t += kConsumeThreads) {
-                        const uint64_t h = hn;
-                        if (t + kConsumeThreads < n) hn = sl ? __ldcg(d + t + kConsumeThreads) : __ldcs(d + t + kConsumeThreads);  // last use unless split
-                        if ((((uint32_t)(h >> 32)) ^ rhi) & rmask) continue;
-                        const int s = smem_find(sk, tmask, (uint32_t)h & tmask, h, empty);
-                        if (s >= 0) atomicAdd(scol + (uint32_t)s * S, 1u);
-                    }
-                }
+            // emit: each warp its slots [wid * T / kWarps, ...), at most 32 rows of 32
+            const uint32_t rows = T / THREADS;  // T >= 1024
+            const uint32_t slot0 = wid * rows * 32 + lane;
+            unsigned kept = 0, n_kept = 0;  // lane r: the ballot of row r
+            uint64_t n_win = 0;
+            for (uint32_t r = 0; r < rows; ++r) {
+                const uint32_t i = slot0 + r * 32;
+                const uint64_t sum = s2 ? (uint64_t)sc[2 * i] + sc[2 * i + 1] : (uint64_t)sc[i];
+                n_win += sum;
+                const unsigned ballot = __ballot_sync(kFull, sum != 0 && sum >= J.min_count);
+                if (lane == (int)r) kept = ballot;
+                n_kept += __popc(ballot);
+                // a key seen once is marked by its top bit (unless that makes it the
+                // empty mark): the filter's candidates do not count it if its bits are new
+                if (sum == 1 && (sk[i] ^ kTopBit) != empty) sk[i] ^= kTopBit;
             }
+            unsigned long long pos0 = 0;
+            if (n_kept) {
+                if (lane == 0) pos0 = atomicAdd(&D->counters[2 * j], (unsigned long long)n_kept);
+                pos0 = __shfl_sync(kFull, pos0, 0);
+                unsigned qn = 0;  // the slots of kept keys, taken 32 at a time
+                const auto write = [&](unsigned n) {
+                    __syncwarp();
+                    qn -= n;
+                    const uint64_t pos = pos0 + lane;
+                    if ((unsigned)lane < n && pos < J.sv_cap) {
+                        const uint32_t i = ws[qn + lane];
+                        uint64_t h = sk[i];
+                        if ((h ^ hpre) & kTopBit) h ^= kTopBit;
+                        const uint64_t key = unmixer64(h);
+                        J.sv_keys[pos] = key;
+                        J.sv_vals[pos] = s2 ? (uint64_t)sc[2 * i] | ((uint64_t)sc[2 * i + 1] << 32) : (uint64_t)sc[i];
+                        if (J.hist_job) atomicAdd(J.hist_job + (key >> J.hist_shift), 1u);
+                    }
+                    pos0 += n;
+                    __syncwarp();
+                };
+                for (uint32_t r = 0; r < rows; ++r) {
+                    const unsigned ballot = __shfl_sync(kFull, kept, r);
+                    if ((ballot >> lane) & 1u) ws[qn + __popc(ballot & lt)] = slot0 + r * 32;
+                    qn += __popc(ballot);
+                    if (qn >= 32) write(32);
+                }
+                if (qn) write(qn);
+            }
+            // filter: the words of the (sub-)range in the place of the counts
             __syncthreads();
-            for (uint32_t i0 = threadIdx.x & ~31u; i0 < T; i0 += blockDim.x) {
-                const uint32_t i = i0 + lane;
-                const unsigned long long k1 = sk[i];
-                uint64_t v = 0;
-                bool keep = false;
-                if (k1 != empty) {
-                    const uint32_t c0 = sc[i * S];
-                    const uint32_t c1 = S == 2 ? sc[i * S + 1] : 0u;
-                    keep = (uint64_t)c0 + c1 >= J.min_count;
-                    v = (uint64_t)c0 | ((uint64_t)c1 << 32);
-                }
-                const unsigned ballot = __ballot_sync(kFull, keep);
-                if (ballot) {
-                    const int leader = __ffs(ballot) - 1;
-                    unsigned long long pos0 = 0;
-                    if (lane == leader) pos0 = atomicAdd(&D->counters[2 * j], (unsigned long long)__popc(ballot));
-                    pos0 = __shfl_sync(kFull, pos0, leader);
-                    if (keep) {
-                        const uint64_t pos = pos0 + __popc(ballot & lt);
-                        if (pos < J.sv_cap) {
-                            const uint64_t key = unmixer64(k1);
-                            J.sv_keys[pos] = key;
-                            J.sv_vals[pos] = v;
-                            if (J.hist_job) atomicAdd(J.hist_job + (key >> J.hist_shift), 1u);
-                        }
-                    }
-                }
+            for (uint32_t i = threadIdx.x; i < w_n; i += THREADS) sb[i] = 0ull;
+            __syncthreads();
+            const int bloom_shift = J.bloom_shift, n_hashes = J.n_hashes;
+            const bool all_cand = J.all_candidates != 0;
+            uint64_t n_new = 0, n_seen = 0;  // keys that set a bit first, keys that were candidates
+            for (uint32_t i = slot0, r = 0; r < rows; ++r, i += 32) {
+                uint64_t h = sk[i];
+                if (h == empty) continue;
+                const bool once = (h ^ hpre) & kTopBit;
+                if (once) h ^= kTopBit;
+                const uint64_t pat = bloom_pattern_rt(mixer64(h), n_hashes);
+                // two 32-bit updates: a shared 64-bit one takes three times as long as a 32-bit one
+                uint32_t* const word = reinterpret_cast<uint32_t*>(sb + ((uint32_t)(h >> bloom_shift) & (w_n - 1)));
+                const uint32_t p_lo = (uint32_t)pat, p_hi = (uint32_t)(pat >> 32);
+                const uint32_t o_lo = atomicOr(word, p_lo), o_hi = atomicOr(word + 1, p_hi);
+                const bool fresh = (p_lo & ~o_lo) != 0u || (p_hi & ~o_hi) != 0u;
+                n_new += fresh;
+                n_seen += all_cand || !(fresh && once);
             }
-            unsigned long long* gb = J.bloom + (uint64_t)part * n_sw + w_lo;
-            for (uint32_t i = threadIdx.x; i < w_n; i += blockDim.x) gb[i] = sb[w_lo + i];
+            // windows reported as seen before: all but each key's first, if its bits were new
+            cand += n_win - (all_cand ? 0 : n_new);
+            claimed += n_seen;
+            __syncthreads();
+            unsigned long long* gb = J.bloom + (uint64_t)part * n_sw + sub * w_n;
+            for (uint32_t i = threadIdx.x; i < w_n; i += THREADS) gb[i] = sb[i];
             __syncthreads();
             if (++sub > smask) break;
         }
         if (threadIdx.x == 0) {
             if (overflow) J.failed[atomicAdd(&D->counters[2 * j + 1], 1ull)] = h_left;
-            else if (sl) atomicAdd(&J.ctr->split_parts, 1u);
+            else if (sl > J.split_min) atomicAdd(&J.ctr->split_parts, 1u);
             if (sl > hint) atomicMax(&J.ctr->split_hint, (unsigned)sl);
         }
     }
@@ -730,7 +793,7 @@ struct kc_batch_ctx {
     cudaGraphExec_t sort_graph = nullptr;
     // captured consumer launches, one per launch shape
     struct ConsumeGraph {
-        int nh, n_ctas;
+        int threads, n_ctas;
         size_t smem;
         cudaGraphExec_t exec;
     };
@@ -893,51 +956,37 @@ void release_work(kc_batch_ctx* b, std::vector<JobWork>& w) {
 
 // prepare: set the kernel's shared-memory limit (before any capture);
 // otherwise launch it.
-template <int NH>
-cudaError_t launch_consume_nh(bool prepare, int n_ctas, size_t smem, const kc::BatchDesc* d, cudaStream_t st) {
-    if (prepare) return kc::allow_max_dynamic_smem(kc::k_consume_q<NH>);
-    kc::k_consume_q<NH><<<n_ctas, kc::kConsumeThreads, smem, st>>>(d);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_consume(bool prepare, int nh, int n_ctas, size_t smem, const kc::BatchDesc* d, cudaStream_t st) {
-    switch (nh) {
-        case 1: return launch_consume_nh<1>(prepare, n_ctas, smem, d, st);
-        case 2: return launch_consume_nh<2>(prepare, n_ctas, smem, d, st);
-        case 3: return launch_consume_nh<3>(prepare, n_ctas, smem, d, st);
-        case 4: return launch_consume_nh<4>(prepare, n_ctas, smem, d, st);
-        case 5: return launch_consume_nh<5>(prepare, n_ctas, smem, d, st);
-        case 6: return launch_consume_nh<6>(prepare, n_ctas, smem, d, st);
-        case 7: return launch_consume_nh<7>(prepare, n_ctas, smem, d, st);
-        case 8: return launch_consume_nh<8>(prepare, n_ctas, smem, d, st);
-        case 9: return launch_consume_nh<9>(prepare, n_ctas, smem, d, st);
-        case 10: return launch_consume_nh<10>(prepare, n_ctas, smem, d, st);
-        default: return launch_consume_nh<0>(prepare, n_ctas, smem, d, st);
-    }
+cudaError_t launch_consume(bool prepare, int threads, int n_ctas, size_t smem, const kc::BatchDesc* d, cudaStream_t st) {
+    const auto go = [&](auto kern) {
+        if (prepare) return kc::allow_max_dynamic_smem(kern);
+        kern<<<n_ctas, threads, smem, st>>>(d);
+        return cudaGetLastError();
+    };
+    return threads == kc::kConsumeThreads ? go(kc::k_consume_q<kc::kConsumeThreads>) : go(kc::k_consume_q<kc::kConsumeThreadsWide>);
 }
 
 // The batch's counters reset and its persistent consumer launch, captured
-// once per launch shape (hash count, grid, shared memory); everything else
+// once per launch shape (CTA size, grid, shared memory); everything else
 // they read comes from the device descriptor.
-kc_status consume_graph(kc_batch_ctx* b, int nh, int n_ctas, size_t smem, cudaGraphExec_t* out) {
+kc_status consume_graph(kc_batch_ctx* b, int threads, int n_ctas, size_t smem, cudaGraphExec_t* out) {
     for (const auto& g : b->consume_graphs)
-        if (g.nh == nh && g.n_ctas == n_ctas && g.smem == smem) {
+        if (g.threads == threads && g.n_ctas == n_ctas && g.smem == smem) {
             *out = g.exec;
             return KC_OK;
         }
-    KC_CUDA(launch_consume(true, nh, n_ctas, smem, b->d_desc, b->st));
+    KC_CUDA(launch_consume(true, threads, n_ctas, smem, b->d_desc, b->st));
     std::lock_guard<std::mutex> lk(kc::sync_api_mutex());
     cudaGraph_t g = nullptr;
     KC_CUDA(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
     kc::k_reset_q<<<1, 256, 0, b->st>>>(b->d_desc);
-    launch_consume(false, nh, n_ctas, smem, b->d_desc, b->st);
+    launch_consume(false, threads, n_ctas, smem, b->d_desc, b->st);
     cudaError_t e = cudaStreamEndCapture(b->st, &g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture(consumer)");
     cudaGraphExec_t exec = nullptr;
     e = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate(consumer)");
-    b->consume_graphs.push_back({nh, n_ctas, smem, exec});
+    b->consume_graphs.push_back({threads, n_ctas, smem, exec});
     *out = exec;
     return KC_OK;
 }
@@ -1180,16 +1229,20 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
                 x.total_w += w;
             }
         }
-        // Shared-memory table: one slot per 8 windows of the largest partition
-        // (2^10..2^13 slots); partitions with more candidates split.
+        // Split level: a sub-range's filter words take at most 64 KiB.
+        const int split_min = std::max(0, h->slice_log2 - kc::kConsumeSliceLog2);
+        // Shared-memory table: twice the windows of the largest partition
+        // (2^10..2^13 slots), so that small partitions never split; a larger
+        // partition's distinct keys fit or it splits.
         int tl = (int)h->cfg.smem_table_log2;
         if (!tl) {
             tl = 10;
-            while (tl < 13 && (1ull << tl) < x.max_w / 8) ++tl;
+            while (tl < 13 && (1ull << tl) < 2 * (x.max_w >> split_min)) ++tl;
         }
-        while (tl > 10 && kc::consume_smem(h->slice_log2, tl, h->n_samples) + 1024 > (size_t)b->max_optin) --tl;
-        const size_t smem = kc::consume_smem(h->slice_log2, tl, h->n_samples);
-        if (smem + 1024 > (size_t)b->max_optin) {
+        const size_t queue = kc::consume_queue_smem(kc::kConsumeThreadsWide) + 1024;
+        while (tl > 10 && kc::consume_smem(h->slice_log2 - split_min, tl, h->n_samples) + queue > (size_t)b->max_optin) --tl;
+        const size_t smem = kc::consume_smem(h->slice_log2 - split_min, tl, h->n_samples);
+        if (smem + queue > (size_t)b->max_optin) {
             release_work(b, work);
             return fail(KC_ERR_INTERNAL, "partition does not fit shared memory");
         }
@@ -1197,9 +1250,9 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         // survivors: a partition holds at most 2^split_max tables of keys and
         // one key per min_count of its windows
         // the consumer tells a window's sub-range by the top 32 bits of its hash
-        const int split_max = h->cfg.split_max == KC_SPLIT_NONE ? 0
+        const int split_max = std::max(split_min, h->cfg.split_max == KC_SPLIT_NONE ? 0
                               : std::min<int>(std::min<int>(h->slice_log2, 32 - h->part_bits),
-                                              h->cfg.split_max ? (int)h->cfg.split_max : 6);
+                                              h->cfg.split_max ? (int)h->cfg.split_max : 8));
         x.sv_cap = 0;
         if (fast) {  // every survivor has min_count windows, and no partition more than 2^split_max tables
             x.sv_cap = std::min<uint64_t>((p_hi - p_lo) << (tl + split_max), x.total_w / std::max<uint32_t>(1, h->min_count));
@@ -1241,6 +1294,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         J.key_bits = 2 * h->k;
         J.min_count = h->min_count;
         J.split_max = split_max;
+        J.split_min = split_min;
         J.fixed_bits = -1;  // the plan chooses the bucket bits (unless set below)
         J.hist_job = nullptr;
         J.n_batches = (int)nb;
@@ -1304,15 +1358,16 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         release_work(b, work);
         return s;
     }
-    int nh = hs[0]->n_hashes;
-    for (int j = 1; j < n; ++j)
-        if (hs[j]->n_hashes != nh) nh = 0;
-    const int per_sm = std::max(1, std::min(4, b->max_sm / (int)(smem_max + 2048)));
     // a persistent grid (CTAs without an item exit at once), so the captured
-    // launch depends on the hash count and shared memory alone
+    // launch depends on the shared memory alone
+    const size_t smem_cta = smem_max + kc::consume_queue_smem(kc::kConsumeThreads);
+    int per_sm = std::min(2, b->max_sm / (int)(smem_cta + 2048));
+    const int threads = per_sm > 1 ? kc::kConsumeThreads : kc::kConsumeThreadsWide;
+    per_sm = std::max(1, per_sm);
+    smem_max += kc::consume_queue_smem(threads);
     const int n_ctas = b->sm_count * per_sm;
     cudaGraphExec_t cons = nullptr;
-    if ((s = consume_graph(b, nh, n_ctas, smem_max, &cons)) != KC_OK) {
+    if ((s = consume_graph(b, threads, n_ctas, smem_max, &cons)) != KC_OK) {
         release_work(b, work);
         return s;
     }

@@ -394,54 +394,15 @@ __device__ __forceinline__ void warp_sort64_packed(uint64_t* __restrict__ keys, 
     }
 }
 
-constexpr int kProbeLimit = 64;  // shared-memory table probes before a partition falls back
-
-// Shared-memory table of one partition: keys[T] hold the hashes h of the
-// claimed keys themselves (h determines the key: key = unmixer64(h)), and an
-// empty slot holds `empty`, a hash of another partition that no key of this
-// one can equal.  Counts follow as n_samples uint32 per slot.  Returns 1 =
-// claimed, 0 = present, -1 = no free slot within kProbeLimit probes; `slot`
-// receives the key's slot unless -1 is returned.
-__device__ __forceinline__ int smem_claim(unsigned long long* keys, uint32_t tmask, uint32_t s,
-                                          unsigned long long h, unsigned long long empty, uint32_t& slot) {
-    for (int i = 0; i < kProbeLimit; ++i) {
-        const unsigned long long cur = keys[s];
-        if (cur == h) {
-            slot = s;
-            return 0;
-        }
-        if (cur == empty) {
-            const unsigned long long prev = atomicCAS(&keys[s], empty, h);
-            if (prev == empty || prev == h) {
-                slot = s;
-                return prev == empty ? 1 : 0;
-            }
-        }
-        s = (s + 1) & tmask;
-    }
-    return -1;
-}
-
-__device__ __forceinline__ int smem_find(const unsigned long long* keys, uint32_t tmask, uint32_t s,
-                                         unsigned long long h, unsigned long long empty) {
-    for (uint32_t i = 0; i <= tmask; ++i) {
-        const unsigned long long cur = keys[s];
-        if (cur == h) return (int)s;
-        if (cur == empty) return -1;
-        s = (s + 1) & tmask;
-    }
-    return -1;
-}
+constexpr int kProbeLimit = 64;  // shared-memory table probes before a partition splits or falls back
 
 // Filter pattern with the number of bits chosen at run time.
 __device__ __forceinline__ uint64_t bloom_pattern_rt(uint64_t g, int n_hashes) {
     uint32_t lo = 0, hi = 0;
-    for (int i = 0; i < n_hashes; ++i) {
+    for (int i = 0; i < n_hashes; ++i, g >>= 6) {
         const uint32_t bit = (uint32_t)g & 63u;
-        g >>= 6;
-        const uint32_t m = 1u << (bit & 31u);
-        if (bit & 32u) hi |= m;
-        else lo |= m;
+        lo |= shl_clamped(1u, bit);
+        hi |= shl_clamped(1u, bit ^ 32u);
     }
     return ((uint64_t)hi << 32) | lo;
 }

@@ -179,7 +179,12 @@ void launch_regroup_base(uint64_t* rel, const uint64_t* starts, const SegDesc* s
 void launch_bucket_scatter(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, uint64_t units_per_cta,
                            int n_ctas, const PassParams& p, int a, int mode, const uint64_t* base, uint64_t* cursor,
                            uint64_t* out, cudaStream_t st);
+// Dynamic shared memory of a consumer CTA: the table and filter words of one
+// (sub-range of a) partition, and its warps' queues.
+constexpr int kConsumeSliceLog2 = 13;  // filter words of a sub-range, at most
+constexpr int kWarpQueue = 64;         // windows a consumer warp's queue holds (under 32, plus a step's)
 size_t consume_smem(int slice_log2, int table_log2, int n_samples);
+size_t consume_queue_smem(int threads);
 void launch_fb_claim(const FallbackArgs& F, int bt, cudaStream_t st);
 void launch_fb_recount(const FallbackArgs& F, int bt, cudaStream_t st);
 void launch_fb_compact(const FallbackArgs& F, cudaStream_t st);

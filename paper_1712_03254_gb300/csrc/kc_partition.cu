@@ -921,10 +921,12 @@ void launch_ingest(const IngestPlan* plan, const IngestPlan& hp, bool ranged, bo
     k_ingest_scatter<<<(unsigned)std::min<uint64_t>(hp.n_items, (uint64_t)sm_count), kLinThreads, ssmem, st>>>(plan);
 }
 
+// the table's keys, then its counts or (afterwards) the filter words
 size_t consume_smem(int slice_log2, int table_log2, int n_samples) {
-    return (sizeof(uint64_t) << slice_log2) + (sizeof(uint64_t) << table_log2) +
-           ((sizeof(uint32_t) * (size_t)n_samples) << table_log2);
+    return (sizeof(uint64_t) << table_log2) +
+           std::max(sizeof(uint64_t) << slice_log2, (sizeof(uint32_t) * (size_t)n_samples) << table_log2);
 }
+size_t consume_queue_smem(int threads) { return (size_t)(threads / 32) * kWarpQueue * (sizeof(uint64_t) + sizeof(uint32_t)); }
 
 void launch_fb_claim(const FallbackArgs& F, int bt, cudaStream_t st) { k_fb_claim<<<1024, 256, 0, st>>>(F, bt); }
 void launch_fb_recount(const FallbackArgs& F, int bt, cudaStream_t st) {
