@@ -67,6 +67,11 @@ __host__ __device__ __forceinline__ uint32_t stage_depth(int a) {
     return d < 4u ? 4u : d;
 }
 
+// Entries from one bucket's stage to the next: two more than its depth, so
+// that the threads that flush neighbouring buckets read other banks (with 4
+// entries a bucket, the rows lie 32 bytes apart and need no padding).
+__host__ __device__ __forceinline__ uint32_t stage_row(uint32_t depth) { return depth == 4u ? 4u : depth + 2u; }
+
 // kCountPerCta: per-CTA histogram of the windows' buckets in shared memory,
 // written out CTA-major.  kScatterRegion: the same windows again; each CTA
 // owns one run per bucket (exact offsets from the counts) and stores each h
@@ -340,7 +345,8 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
     __shared__ unsigned s_front[2], s_back[2];  // entries at the front / back of each retry list
     const uint32_t P = 1u << a2;
     const uint32_t D = stage_depth(a2);  // entries staged per bucket, a multiple of 4
-    uint32_t* fill = reinterpret_cast<uint32_t*>(s_stage + (size_t)D * P);
+    const uint32_t R = stage_row(D);
+    uint32_t* fill = reinterpret_cast<uint32_t*>(s_stage + (size_t)R * P);
     uint64_t* cursor = reinterpret_cast<uint64_t*>(fill + P);  // next output position of each run
     uint64_t* retry = cursor + P;                              // two lists of kRetryCap hashes
     const uint64_t* my_base = base;
@@ -353,7 +359,6 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
     const uint32_t group = (uint32_t)pieces[0].group;
     // a1 + a2 <= 20: bucket and group are bits of h's high word
     const int shift = 32 - a1 - a2, gshift = 32 - a1;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     int par = 0;  // retry list read this round
     for (int pc = 0; pc < n_pieces; ++pc)
     for (uint64_t c0 = 0; c0 < pieces[(size_t)pc * stride].len; c0 += kPieceMax) {
@@ -386,7 +391,7 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                 const uint64_t h = rin[i < n_front ? i : kRetryCap - 1 - (i - n_front)];
                 const uint32_t b = ((uint32_t)(h >> 32) >> shift) & (P - 1);
                 const uint32_t pos = atomicAdd(&fill[b], 1u);
-                if (pos < D) s_stage[(size_t)b * D + pos] = h;
+                if (pos < D) s_stage[(size_t)b * R + pos] = h;
                 else rout[atomicAdd(&s_front[par ^ 1], 1u)] = h;  // at most n_in of these
             }
             // Warp-uniform: a warp takes its next rows only when none of its lanes
@@ -417,7 +422,7 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                     const uint32_t b = ((uint32_t)(h >> 32) >> shift) & (P - 1);
                     const uint32_t pos = atomicAdd(&fill[b], 1u);
                     if (pos < D) {
-                        s_stage[(size_t)b * D + pos] = h;
+                        s_stage[(size_t)b * R + pos] = h;
                         pend &= ~(1u << e);
                     } else {
                         // the back of the other list, leaving the n_in entries the
@@ -447,17 +452,28 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                     }
                 }
             } else {
-                // deep stages (few buckets): a warp per bucket writes its whole
-                // sectors, then keeps the 0..3 entries left over at the front
-                for (uint32_t b = wid; b < P; b += nwarps) {
+                // deep stages (few buckets): a group of threads per bucket (one
+                // thread from 1024 buckets on, a warp at 32 and below) writes its
+                // whole sectors, then keeps the 0..3 entries left over at the
+                // front.  A warp for each bucket in turn left most lanes without
+                // a sector to write: 1.2e8 hashes into 2048 buckets 4.03 -> 0.82
+                // ms, 1024 2.49 -> 0.83, 512 1.50 -> 0.67, 256 0.92 -> 0.51, 64
+                // 0.50 -> 0.50 ms.
+                const uint32_t lg = min(5u, 10u - min(10u, (uint32_t)a2));
+                const uint32_t sub = threadIdx.x & ((1u << lg) - 1u);
+                for (uint32_t b = threadIdx.x >> lg; b < P; b += blockDim.x >> lg) {
                     const uint32_t f = min(fill[b], D);
                     const uint32_t whole = f & ~3u;
-                    unsigned long long* st = s_stage + (size_t)b * D;
+                    unsigned long long* st = s_stage + (size_t)b * R;
                     uint64_t* dst = out + cursor[b];
-                    for (uint32_t i = lane * 2; i < whole; i += 64)
-                        *reinterpret_cast<ulonglong2*>(dst + i) = *reinterpret_cast<const ulonglong2*>(st + i);
-                    __syncwarp();
-                    if (lane == 0) {
+                    for (uint32_t i = sub * 4; i < whole; i += 4u << lg) {
+                        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(st + i);
+                        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(st + i + 2);
+                        *reinterpret_cast<ulonglong2*>(dst + i) = x;
+                        *reinterpret_cast<ulonglong2*>(dst + i + 2) = y;
+                    }
+                    __syncwarp();  // the lanes of a warp take the same number of buckets
+                    if (sub == 0) {
                         for (uint32_t i = whole; i < f; ++i) st[i - whole] = st[i];
                         cursor[b] += whole;
                         fill[b] = f - whole;  // hashes beyond D went to the retry list
@@ -473,10 +489,10 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
         const uint32_t f = min(fill[b], D);
         const uint32_t whole = f & ~3u;
         uint64_t* dst = out + cursor[b];
-        for (uint32_t i = 0; i < whole; ++i) dst[i] = s_stage[(size_t)b * D + i];
+        for (uint32_t i = 0; i < whole; ++i) dst[i] = s_stage[(size_t)b * R + i];
         if (f > whole) {
             const uint64_t pad = pad_hash((group << a2) | b, a1 + a2);
-            for (uint32_t i = whole; i < whole + 4; ++i) dst[i] = i < f ? (uint64_t)s_stage[(size_t)b * D + i] : pad;
+            for (uint32_t i = whole; i < whole + 4; ++i) dst[i] = i < f ? (uint64_t)s_stage[(size_t)b * R + i] : pad;
         }
     }
 }
@@ -832,7 +848,7 @@ void launch_extract_count(const uint64_t* pw, const uint64_t* vw, uint64_t n_uni
 
 // stage, fill count and 64-bit output cursor per bucket, then the two retry lists
 size_t staged_seg_smem(int a) {
-    return (((size_t)stage_depth(a) * sizeof(uint64_t) + sizeof(uint32_t) + sizeof(uint64_t)) << a) +
+    return (((size_t)stage_row(stage_depth(a)) * sizeof(uint64_t) + sizeof(uint32_t) + sizeof(uint64_t)) << a) +
            2 * kRetryCap * sizeof(uint64_t);
 }
 
@@ -895,7 +911,13 @@ void launch_bucket_scatter(const uint64_t* pw, const uint64_t* vw, uint64_t n_un
     }
 }
 
-size_t ingest_scatter_smem(int max_a) { return staged_seg_smem(max_a); }
+// every job of a batch has bucket bits up to max_a (2048 buckets take more
+// than 4096: deep stages have padded rows)
+size_t ingest_scatter_smem(int max_a) {
+    size_t m = 0;
+    for (int a = 1; a <= max_a; ++a) m = std::max(m, staged_seg_smem(a));
+    return m;
+}
 
 void launch_ingest(const IngestPlan* plan, const IngestPlan& hp, bool ranged, bool all_k31, int sm_count,
                    cudaStream_t st) {
