@@ -93,7 +93,8 @@ typedef struct kc_config {
                                      least 8 words) when the first kc_add_reads
                                      after create / reset brings more than 32768
                                      windows (bases - reads * (k - 1)) per
-                                     partition                                  */
+                                     partition; from 2^18 windows on, more than
+                                     8192 (slices of at least 256 words)        */
     uint64_t table_slots;         /* direct: open-addressing slots (power of two)
                                      of the global table                            */
     uint32_t spill;               /* partitioned: kc_finalize takes 64 groups of
