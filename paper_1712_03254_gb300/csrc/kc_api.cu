@@ -598,7 +598,7 @@ uint64_t room_bytes(kc_handle h) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
-        return ~0ull;  // unknown: do not defer
+        return ~0ull - 1;  // unknown: do not defer for want of room
     }
     uint64_t cached = 0;
     cudaMemPool_t pool;
@@ -616,9 +616,11 @@ uint64_t room_bytes(kc_handle h) {
 
 // Device bytes bucket_batch needs for a batch of n_local bases: the linear
 // hashes and the grouped hashes (8 bytes per window each, at most one window
-// per base), and the run padding of up to 3 per (CTA, partition).
+// per base), and the run padding of up to 3 per (CTA, partition).  More grouped
+// hashes than the scatter's cursors can address (2^34) never fit.
 uint64_t bucket_bytes(kc_handle h, uint64_t n_local) {
     const int max_ctas = h->grid.sm_count * (h->cfg.ctas_per_sm ? (int)h->cfg.ctas_per_sm : 1);
+    if (n_local + 3ull * (uint64_t)max_ctas * (1ull << h->l1_bits) > kMaxGroupedHashes) return ~0ull;
     return 16 * n_local + 24ull * (uint64_t)max_ctas * (1ull << h->l1_bits) +
            (uint64_t)max_ctas * (1ull << h->l1_bits) * 12;
 }

@@ -56,6 +56,8 @@ constexpr uint64_t kWindowsPerPartition = 32768;
 constexpr uint64_t kWindowsPerFinePartition = 8192;
 constexpr uint64_t kFinePartitionJob = 1ull << 18;
 constexpr int kFineSliceLog2 = 8;
+// grouped hashes of one batch the scatter can address (32-bit sector cursors)
+constexpr uint64_t kMaxGroupedHashes = (1ull << 34) - (1ull << 26);
 
 // Host reads copied in chunks by kc_add_reads: chunk c covers units
 // [u[c], u[c + 1]); its packed words (and the next unit's first word) and

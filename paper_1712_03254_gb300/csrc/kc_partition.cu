@@ -53,6 +53,12 @@ __device__ __forceinline__ void st_u64_l2_hint(uint64_t* p, uint64_t v, uint64_t
     asm volatile("st.global.L2::cache_hint.b64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
 }
 
+// One 32-byte store (p 32-byte aligned; sm_100 on): a sector in one request
+// instead of two.
+__device__ __forceinline__ void st_sector(uint64_t* p, const ulonglong2& x, const ulonglong2& y) {
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(x.x), "l"(x.y), "l"(y.x), "l"(y.y) : "memory");
+}
+
 enum BucketMode { kCountPerCta = 0, kScatterCursor = 1, kScatterRegion = 2, kScatterStaged = 3 };
 
 // Filler for the unused tail of a padded run: a hash whose partition prefix
@@ -316,12 +322,17 @@ __global__ void __launch_bounds__(kExtractThreads) k_extract_count(const uint64_
 }
 
 constexpr int kLinThreads = 1024;
-constexpr int kLinPerThread = 4;
+constexpr int kLinPerThread = 5;
 constexpr uint32_t kRetryCap = 2048;  // hashes one retry list holds
 constexpr uint32_t kPieceMax = 1u << 31;  // hashes a scatter loop indexes with 32 bits
 
+// Bound by the shared-memory staging and the stores' requests: without its
+// stores a round takes two thirds of the time.  1.2e8 hashes into 4096 buckets
+// take 0.69 ms (2.7 TB/s read and written); 0.76 with two 16-byte stores a
+// sector, four hashes a thread placed one after the other and 64-bit cursors.
+//
 // Staged scatter of hashes already in memory.  CTA c moves segment c
-// (seg[c] = {offset into src, length, group}) into its padded runs, 4 hashes
+// (seg[c] = {offset into src, length, group}) into its padded runs, 5 hashes
 // per thread per round; full 4-entry stages leave as aligned 32-byte sectors.
 // A hash goes to bucket (h >> (64 - a1 - a2)) & (2^a2 - 1); with a1 > 0 the
 // segment belongs to level-1 group `group`, hashes of another group (the
@@ -347,12 +358,12 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
     const uint32_t D = stage_depth(a2);  // entries staged per bucket, a multiple of 4
     const uint32_t R = stage_row(D);
     uint32_t* fill = reinterpret_cast<uint32_t*>(s_stage + (size_t)R * P);
-    uint64_t* cursor = reinterpret_cast<uint64_t*>(fill + P);  // next output position of each run
-    uint64_t* retry = cursor + P;                              // two lists of kRetryCap hashes
+    uint32_t* cursor = fill + P;  // next output sector of each run (positions are multiples of 4, below 2^34)
+    uint64_t* retry = reinterpret_cast<uint64_t*>(cursor + P);                              // two lists of kRetryCap hashes
     const uint64_t* my_base = base;
     for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
         fill[i] = 0;
-        cursor[i] = __ldg(my_base + i);
+        cursor[i] = (uint32_t)(__ldg(my_base + i) >> 2);
     }
     if (threadIdx.x == 0) s_front[0] = s_back[0] = s_front[1] = s_back[1] = 0;
     __syncthreads();
@@ -386,14 +397,6 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
             const unsigned n_in = n_front + n_back;
             const uint64_t* rin = retry + (size_t)par * kRetryCap;
             uint64_t* rout = retry + (size_t)(par ^ 1) * kRetryCap;
-            // the retry list first: a failure goes to the front of the other list
-            for (unsigned i = threadIdx.x; i < n_in; i += blockDim.x) {
-                const uint64_t h = rin[i < n_front ? i : kRetryCap - 1 - (i - n_front)];
-                const uint32_t b = ((uint32_t)(h >> 32) >> shift) & (P - 1);
-                const uint32_t pos = atomicAdd(&fill[b], 1u);
-                if (pos < D) s_stage[(size_t)b * R + pos] = h;
-                else rout[atomicAdd(&s_front[par ^ 1], 1u)] = h;  // at most n_in of these
-            }
             // Warp-uniform: a warp takes its next rows only when none of its lanes
             // still holds a pending hash, so every load stays coalesced.
             if (__all_sync(kFull, pend == 0)) {
@@ -415,21 +418,35 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                     next += blockDim.x;
                 }
             }
+            // all places first, so that their atomics are in flight together
+            uint32_t pos[kLinPerThread];
+#pragma unroll
+            for (int e = 0; e < kLinPerThread; ++e)
+                if (pend & (1u << e)) pos[e] = atomicAdd(&fill[((uint32_t)(ph[e] >> 32) >> shift) & (P - 1)], 1u);
 #pragma unroll
             for (int e = 0; e < kLinPerThread; ++e) {
-                if (pend & (1u << e)) {
-                    const uint64_t h = ph[e];
-                    const uint32_t b = ((uint32_t)(h >> 32) >> shift) & (P - 1);
-                    const uint32_t pos = atomicAdd(&fill[b], 1u);
-                    if (pos < D) {
-                        s_stage[(size_t)b * R + pos] = h;
-                        pend &= ~(1u << e);
-                    } else {
+                if ((pend & (1u << e)) && pos[e] < D) {
+                    s_stage[(size_t)(((uint32_t)(ph[e] >> 32) >> shift) & (P - 1)) * R + pos[e]] = ph[e];
+                    pend &= ~(1u << e);
+                }
+            }
+            // the retry list: a failure goes to the front of the other list
+            for (unsigned i = threadIdx.x; i < n_in; i += blockDim.x) {
+                const uint64_t h = rin[i < n_front ? i : kRetryCap - 1 - (i - n_front)];
+                const uint32_t b = ((uint32_t)(h >> 32) >> shift) & (P - 1);
+                const uint32_t pos = atomicAdd(&fill[b], 1u);
+                if (pos < D) s_stage[(size_t)b * R + pos] = h;
+                else rout[atomicAdd(&s_front[par ^ 1], 1u)] = h;  // at most n_in of these
+            }
+            if (pend) {
+#pragma unroll
+                for (int e = 0; e < kLinPerThread; ++e) {
+                    if (pend & (1u << e)) {
                         // the back of the other list, leaving the n_in entries the
                         // front may take; past that the hash stays and retries
                         const unsigned k = atomicAdd(&s_back[par ^ 1], 1u);
                         if (k < kRetryCap - n_in) {
-                            rout[kRetryCap - 1 - k] = h;
+                            rout[kRetryCap - 1 - k] = ph[e];
                             pend &= ~(1u << e);
                         } else {
                             atomicSub(&s_back[par ^ 1], 1u);
@@ -444,10 +461,9 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                 for (uint32_t b = threadIdx.x; b < P; b += blockDim.x) {
                     if (fill[b] >= 4) {
                         const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(s_stage + (size_t)b * 4);
-                        ulonglong2* dst = reinterpret_cast<ulonglong2*>(out + cursor[b]);
-                        dst[0] = sp[0];
-                        dst[1] = sp[1];
-                        cursor[b] += 4;
+                        const uint32_t c = cursor[b];
+                        st_sector(out + ((uint64_t)c << 2), sp[0], sp[1]);
+                        cursor[b] = c + 1;
                         fill[b] = 0;
                     }
                 }
@@ -456,26 +472,25 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                 // thread from 1024 buckets on, a warp at 32 and below) writes its
                 // whole sectors, then keeps the 0..3 entries left over at the
                 // front.  A warp for each bucket in turn left most lanes without
-                // a sector to write: 1.2e8 hashes into 2048 buckets 4.03 -> 0.82
-                // ms, 1024 2.49 -> 0.83, 512 1.50 -> 0.67, 256 0.92 -> 0.51, 64
-                // 0.50 -> 0.50 ms.
+                // a sector to write: 1.2e8 hashes into 2048 buckets 4.03 -> 0.69
+                // ms, 1024 2.49 -> 0.55, 512 1.50 -> 0.51, 256 0.92 -> 0.46, 64
+                // 0.50 -> 0.46 ms (with st_sector).
                 const uint32_t lg = min(5u, 10u - min(10u, (uint32_t)a2));
                 const uint32_t sub = threadIdx.x & ((1u << lg) - 1u);
                 for (uint32_t b = threadIdx.x >> lg; b < P; b += blockDim.x >> lg) {
                     const uint32_t f = min(fill[b], D);
                     const uint32_t whole = f & ~3u;
                     unsigned long long* st = s_stage + (size_t)b * R;
-                    uint64_t* dst = out + cursor[b];
+                    uint64_t* dst = out + ((uint64_t)cursor[b] << 2);
                     for (uint32_t i = sub * 4; i < whole; i += 4u << lg) {
                         const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(st + i);
                         const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(st + i + 2);
-                        *reinterpret_cast<ulonglong2*>(dst + i) = x;
-                        *reinterpret_cast<ulonglong2*>(dst + i + 2) = y;
+                        st_sector(dst + i, x, y);
                     }
                     __syncwarp();  // the lanes of a warp take the same number of buckets
                     if (sub == 0) {
                         for (uint32_t i = whole; i < f; ++i) st[i - whole] = st[i];
-                        cursor[b] += whole;
+                        cursor[b] += whole >> 2;
                         fill[b] = f - whole;  // hashes beyond D went to the retry list
                     }
                     __syncwarp();
@@ -488,7 +503,7 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
     for (uint32_t b = threadIdx.x; b < P; b += blockDim.x) {
         const uint32_t f = min(fill[b], D);
         const uint32_t whole = f & ~3u;
-        uint64_t* dst = out + cursor[b];
+        uint64_t* dst = out + ((uint64_t)cursor[b] << 2);
         for (uint32_t i = 0; i < whole; ++i) dst[i] = s_stage[(size_t)b * R + i];
         if (f > whole) {
             const uint64_t pad = pad_hash((group << a2) | b, a1 + a2);
@@ -846,9 +861,9 @@ void launch_extract_count(const uint64_t* pw, const uint64_t* vw, uint64_t n_uni
         extract_count_k<true>(pw, vw, n_units, units_per_cta, n_ctas, p, a, counts, cur, seg, lin, ctr, st, accumulate);
 }
 
-// stage, fill count and 64-bit output cursor per bucket, then the two retry lists
+// stage, fill count and output cursor (in sectors) per bucket, then the two retry lists
 size_t staged_seg_smem(int a) {
-    return (((size_t)stage_row(stage_depth(a)) * sizeof(uint64_t) + sizeof(uint32_t) + sizeof(uint64_t)) << a) +
+    return (((size_t)stage_row(stage_depth(a)) * sizeof(uint64_t) + 2 * sizeof(uint32_t)) << a) +
            2 * kRetryCap * sizeof(uint64_t);
 }
 

@@ -1,0 +1,140 @@
+"""Partition consumer and staged scatter where they can go wrong: bucket counts
+on both sides of every flush rule, jobs of different bucket counts in one
+launch, tables from one key to overfull, keys that share a home slot.  Results
+and filters are integers and must equal the oracle's (or numpy's) exactly."""
+import numpy as np
+import pytest
+
+import synth
+import paper_1712_03254_gb300 as kc
+
+pytestmark = pytest.mark.gpu
+
+M1, M2, GOLD = np.uint64(0xBF58476D1CE4E5B9), np.uint64(0x94D049BB133111EB), np.uint64(0x9E3779B97F4A7C15)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kc.lib()
+
+
+def _same(c, o):
+    keys, counts = c.dump()
+    ok, oc = o.result()
+    assert np.array_equal(keys, ok)
+    assert np.array_equal(counts, oc)
+    assert np.array_equal(c.export_bloom(), o.bloom())
+
+
+@pytest.mark.parametrize("part_bits", [1, 2, 3, 4, 5, 6, 7, 9, 10, 11, 12])
+def test_bucket_counts(oracle_mod, part_bits):
+    """Every group size of the scatter's flush (a warp, half a warp, ..., one
+    thread per bucket) and both stage depths' row strides."""
+    w = synth.tiny(scale=0.3)
+    w.bloom_bits = 1 << 20
+    o = oracle_mod.count(w)
+    c = kc.KmerCounter(w.k, 1, w.bloom_bits, w.n_hashes, w.min_count, strategy="partitioned", part_bits=part_bits)
+    c.add_readset(0, w.samples[0])
+    c.finalize()
+    _same(c, o)
+    st = c.stats()
+    assert st["result_keys"] <= st["table_keys"] <= st["candidates"] <= st["windows"] == o.windows
+    c.close()
+
+
+def test_batch_of_different_bucket_counts(oracle_mod):
+    """One batched ingest over jobs of 1024, 2048 and 4096 buckets: each item's
+    stages fit the launch's shared memory (2048 buckets take the most)."""
+    counters, oracles = [], []
+    for i, pb in enumerate((12, 11, 10, 3, 12)):
+        g = synth.genome(900 + i, 60_000)
+        rs = synth.reads(900 + i, g, 6_000, 60, 160, 0.01, 0.001)
+        w = synth.Workload(f"job{i}", [rs], (31, 25)[i % 2], 1 << 20, 4, 2)
+        c = kc.KmerCounter(w.k, 1, w.bloom_bits, 4, 2, strategy="partitioned", part_bits=pb, batched_ingest=True)
+        c.add_readset(0, rs)
+        counters.append(c)
+        oracles.append(oracle_mod.count(w))
+    b = kc.KcBatch()
+    b.ingest(counters)
+    b.finalize(counters)
+    for c, o in zip(counters, oracles):
+        _same(c, o)
+
+
+def _mixer(x):
+    with np.errstate(over="ignore"):
+        z = x + GOLD
+        z = (z ^ (z >> np.uint64(30))) * M1
+        z = (z ^ (z >> np.uint64(27))) * M2
+        return z ^ (z >> np.uint64(31))
+
+
+def _canonical_31mers(rng, n):
+    """n distinct canonical 31-mers as (codes uint8[n, 31], keys uint64[n])."""
+    codes = rng.integers(0, 4, (n, 31), dtype=np.uint8)
+    fwd = np.zeros(n, np.uint64)
+    rev = np.zeros(n, np.uint64)
+    for i in range(31):
+        fwd = (fwd << np.uint64(2)) | codes[:, i].astype(np.uint64)
+        rev |= (np.uint64(3) - codes[:, i].astype(np.uint64)) << np.uint64(2 * i)
+    keys, at = np.unique(np.minimum(fwd, rev), return_index=True)
+    return codes[at], keys
+
+
+def _count(codes, keys, repeats, samples, min_count, **kw):
+    """Key i occurs repeats[s][i] times in sample s; the counter's result against them."""
+    c = kc.KmerCounter(31, samples, 1 << 20, 4, min_count, strategy="partitioned", **kw)
+    for s in range(samples):
+        rows = np.repeat(np.arange(len(keys)), repeats[s])
+        np.random.default_rng(5 + s).shuffle(rows)
+        ascii = np.frombuffer(b"ACGT", np.uint8)[codes[rows]].reshape(-1)
+        c.add_readset(s, synth.ReadSet(ascii, np.arange(len(rows) + 1, dtype=np.uint64) * np.uint64(31)))
+    c.finalize()
+    got_k, got_c = c.dump()
+    total = np.sum(repeats[:samples], axis=0)
+    keep = total >= min_count
+    assert np.array_equal(got_k, keys[keep])
+    assert np.array_equal(got_c, np.stack([repeats[s][keep] for s in range(samples)], 1).astype(np.uint32))
+    st = c.stats()
+    c.close()
+    return st
+
+
+@pytest.mark.parametrize("samples,min_count", [(1, 1), (1, 2), (2, 2), (2, 3)])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 700, 1000, 1024, 1025, 2100])
+def test_table_from_one_key_to_overfull(n, samples, min_count):
+    """n distinct keys in one partition of a 1024-slot table: rows, queue and
+    emission at their edges, then a table that fills up and splits."""
+    rng = np.random.default_rng(n)
+    codes, keys = _canonical_31mers(rng, 3 * n + 64)
+    own = (_mixer(keys) >> np.uint64(63)) == 0  # partition 0 of two
+    codes, keys = codes[own][:n], keys[own][:n]
+    assert len(keys) == n
+    repeats = [rng.integers(0, 4, n) for _ in range(2)]
+    repeats[0][:: max(1, n // 3)] += 40  # some keys far above the others
+    st = _count(codes, keys, repeats, samples, min_count, part_bits=1, smem_table_log2=10)
+    assert st["fallback_partitions"] == 0
+    distinct = np.count_nonzero(np.sum(repeats[:samples], axis=0))
+    if distinct <= 800:  # at most 0.78 full: 64 probes fail with probability under 800 * 0.78^64 = 1e-4
+        assert st["split_partitions"] == 0
+    if distinct > 1024:
+        assert st["split_partitions"] == 1
+
+
+@pytest.mark.parametrize("n_same", [2, 33, 64, 65, 90])
+def test_keys_of_one_home_slot(n_same):
+    """Keys whose hashes end in the same bits as the table's last slot: the probes
+    wrap round, and past the probe limit the partition splits."""
+    rng = np.random.default_rng(n_same)
+    codes, keys = _canonical_31mers(rng, 400_000)
+    h = _mixer(keys)
+    own = ((h >> np.uint64(63)) == 0) & ((h & np.uint64(1023)) == 1023)
+    codes, keys = codes[own][:n_same], keys[own][:n_same]
+    assert len(keys) == n_same
+    repeats = [rng.integers(1, 5, n_same), rng.integers(1, 5, n_same)]
+    st = _count(codes, keys, repeats, 2, 2, part_bits=1, smem_table_log2=10)
+    assert st["fallback_partitions"] == 0
+    assert (st["split_partitions"] > 0) == (n_same > 64)
