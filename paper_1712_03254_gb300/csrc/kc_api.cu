@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <mutex>
 #include <memory>
@@ -141,12 +142,77 @@ kc_status check_open(kc_handle h) {
     return KC_OK;
 }
 
+// Bytes all handles of the process keep idle.
+std::atomic<size_t> g_idle_bytes{0};
+
+size_t idle_limit(kc_handle h) {
+    static std::atomic<size_t> cached[64];
+    const int dev = h->device >= 0 && h->device < 64 ? h->device : 0;
+    size_t v = cached[dev].load(std::memory_order_relaxed);
+    if (!v) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+        v = std::max<size_t>(1, total_b / kIdleShare);
+        cached[dev].store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
+void free_idle(kc_handle h) {
+    for (const IdleBlock& b : h->idle) cudaFreeAsync(b.p, h->stream);
+    g_idle_bytes -= h->idle_bytes;
+    h->idle.clear();
+    h->idle_bytes = 0;
+}
+
+cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
+    *bytes = std::max<size_t>(*bytes, 16);
+    size_t best = h->idle.size();
+    for (size_t i = 0; i < h->idle.size(); ++i) {
+        const size_t have = h->idle[i].bytes;
+        if (have >= *bytes && have / 4 <= *bytes && (best == h->idle.size() || have < h->idle[best].bytes)) best = i;
+    }
+    if (best < h->idle.size()) {
+        *p = h->idle[best].p;
+        *bytes = h->idle[best].bytes;
+        h->idle_bytes -= *bytes;
+        g_idle_bytes -= *bytes;
+        h->idle.erase(h->idle.begin() + best);
+        return cudaSuccess;
+    }
+    cudaError_t e = cudaMallocAsync(p, *bytes, st);
+    if (e == cudaErrorMemoryAllocation && !h->idle.empty()) {
+        cudaGetLastError();
+        free_idle(h);
+        cudaStreamSynchronize(h->stream);
+        e = cudaMallocAsync(p, *bytes, st);
+    }
+    return e;
+}
+
+void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st) {
+    if (!p) return;
+    if (h->reused && !h->cfg.device_budget && bytes >= kIdleMinBytes && h->idle.size() < kMaxIdleBlocks &&
+        g_idle_bytes.load() + bytes <= idle_limit(h)) {
+        h->idle.push_back({p, bytes});
+        h->idle_bytes += bytes;
+        g_idle_bytes += bytes;
+        return;
+    }
+    cudaFreeAsync(p, st);
+}
+
+void leave_hashes(kc_handle h, Batch& b) {
+    leave_block(h, b.hdata, b.hash_bytes, h->stream);
+    if (b.hstarts) cudaFreeAsync(b.hstarts, h->stream);
+    b.hdata = b.hstarts = nullptr;
+    b.hash_bytes = 0;
+}
+
 void free_batches(kc_handle h) {
     for (auto& b : h->batches) {
         if (b.pw) cudaFreeAsync(b.pw, h->stream);
-        if (b.vw) cudaFreeAsync(b.vw, h->stream);
-        if (b.hdata) cudaFreeAsync(b.hdata, h->stream);
-        if (b.hstarts) cudaFreeAsync(b.hstarts, h->stream);
+        leave_hashes(h, b);
     }
     h->batches.clear();
 }
@@ -302,26 +368,30 @@ kc_status regroup_batch(kc_handle h, Batch& b, cudaStream_t st) {
     vlo[P1] = (uint32_t)segs.size();
     const uint64_t nv = std::max<size_t>(1, segs.size());
     if (segs.empty()) segs.push_back(kc::SegDesc{0, 0, 0, 0});
-    uint32_t *counts = nullptr, *total = nullptr, *dvlo = nullptr;
-    uint64_t *rel = nullptr, *starts = nullptr, *cursor = nullptr, *out = nullptr;
-    kc::SegDesc* dsegs = nullptr;
+    // the new hashes and their starts; one block for everything else
     const uint64_t cap = total_in + 3 * nv * P2;
+    const size_t scratch_bytes = nv * P2 * 12 + P * 12 + nv * sizeof(kc::SegDesc) + (P1 + 1) * 4 + 64;
+    uint64_t *out = nullptr, *starts = nullptr;
+    void* scratch = nullptr;
+    size_t out_bytes = std::max<uint64_t>(1, cap) * 8;
     cudaError_t e;
     auto bail = [&](cudaError_t err) {
-        for (void* q : {(void*)counts, (void*)total, (void*)dvlo, (void*)rel, (void*)starts, (void*)cursor,
-                        (void*)out, (void*)dsegs})
-            if (q) cudaFreeAsync(q, st);
+        if (out) cudaFreeAsync(out, st);
+        if (starts) cudaFreeAsync(starts, st);
+        if (scratch) cudaFreeAsync(scratch, st);
         return cuda_fail(err, "cudaMallocAsync(second partitioning level)");
     };
-    if ((e = cudaMallocAsync(&counts, nv * P2 * 4, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&rel, nv * P2 * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&total, P * 4, st)) != cudaSuccess ||
+    if ((e = take_block(h, reinterpret_cast<void**>(&out), &out_bytes, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&starts, (P + 1) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&cursor, P * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&out, std::max<uint64_t>(1, cap) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&dsegs, nv * sizeof(kc::SegDesc), st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&dvlo, (P1 + 1) * 4, st)) != cudaSuccess)
+        (e = cudaMallocAsync(&scratch, scratch_bytes, st)) != cudaSuccess)
         return bail(e);
+    char* q = static_cast<char*>(scratch);
+    kc::SegDesc* dsegs = reinterpret_cast<kc::SegDesc*>(q);
+    uint64_t* rel = reinterpret_cast<uint64_t*>(q += nv * sizeof(kc::SegDesc));
+    uint64_t* cursor = reinterpret_cast<uint64_t*>(q += nv * P2 * 8);
+    uint32_t* counts = reinterpret_cast<uint32_t*>(q += P * 8);
+    uint32_t* total = reinterpret_cast<uint32_t*>(q += nv * P2 * 4);
+    uint32_t* dvlo = reinterpret_cast<uint32_t*>(q += P * 4);
     KC_CUDA(cudaMemcpyAsync(dsegs, segs.data(), nv * sizeof(kc::SegDesc), cudaMemcpyHostToDevice, st));
     KC_CUDA(cudaMemcpyAsync(dvlo, vlo.data(), (P1 + 1) * 4, cudaMemcpyHostToDevice, st));
     kc::launch_count_seg(b.hdata, dsegs, (int)nv, a1, a2, counts, st);
@@ -331,11 +401,15 @@ kc_status regroup_batch(kc_handle h, Batch& b, cudaStream_t st) {
     kc::launch_scatter_staged_seg(b.hdata, dsegs, (int)nv, 1, a1, a2, rel, out, st);
     h->launches += 5;
     KC_LAUNCHED("second-level bucketing launches");
-    for (void* q : {(void*)counts, (void*)total, (void*)dvlo, (void*)rel, (void*)cursor, (void*)dsegs})
-        cudaFreeAsync(q, st);
-    cudaFreeAsync(b.hdata, st);
-    cudaFreeAsync(b.hstarts, st);
+    cudaFreeAsync(scratch, st);
+    if (st == h->stream) {
+        leave_hashes(h, b);
+    } else {
+        cudaFreeAsync(b.hdata, st);
+        cudaFreeAsync(b.hstarts, st);
+    }
     b.hdata = out;
+    b.hash_bytes = out_bytes;
     b.hstarts = starts;
     b.hcap = cap;
     return KC_OK;
@@ -375,36 +449,36 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
     // CTAs take a share of every chunk (segment c = its pieces in all chunks)
     const int n_ctas = (int)((b.n_units + upc - 1) / upc);
     const int n_pieces = chunks ? chunks->n : 1;
-    uint32_t *counts = nullptr, *total = nullptr;
-    uint64_t *rel = nullptr, *cursor = nullptr, *lin = nullptr, *g_cursor = nullptr;
-    kc::SegDesc* seg = nullptr;
     // at most one window per base, plus run padding of up to 3 per (CTA, partition)
     b.hcap = n_local + (mode >= 3 ? 3ull * (uint64_t)n_ctas * P : 0ull);
+    // one scratch block: the linear hashes, run bases, cursors, segments, the
+    // output cursor, histogram rows and totals
+    const uint64_t cells = (uint64_t)n_ctas * P, n_lin = mode == 4 ? std::max<uint64_t>(1, n_local) : 0;
+    const uint64_t n_seg = mode == 4 ? (uint64_t)n_ctas * n_pieces : 0;
+    size_t scratch_bytes = n_lin * 8 + cells * 12 + P * 12 + n_seg * sizeof(kc::SegDesc) + 64;
+    void* scratch = nullptr;
     cudaError_t e = cudaSuccess;
     auto bail = [&](cudaError_t err) {
-        if (counts) cudaFreeAsync(counts, st);
-        if (rel) cudaFreeAsync(rel, st);
-        if (total) cudaFreeAsync(total, st);
-        if (cursor) cudaFreeAsync(cursor, st);
-        if (lin) cudaFreeAsync(lin, st);
-        if (seg) cudaFreeAsync(seg, st);
-        if (g_cursor) cudaFreeAsync(g_cursor, st);
+        if (scratch) cudaFreeAsync(scratch, st);
         if (b.hstarts) cudaFreeAsync(b.hstarts, st);
         if (b.hdata) cudaFreeAsync(b.hdata, st);
         b.hstarts = b.hdata = nullptr;
+        b.hash_bytes = 0;
         return cuda_fail(err, "cudaMallocAsync(partition buckets)");
     };
-    if ((e = cudaMallocAsync(&counts, (size_t)n_ctas * P * 4, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&rel, (size_t)n_ctas * P * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&total, P * 4, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&cursor, P * 8, st)) != cudaSuccess ||
+    b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
+    if ((e = take_block(h, &scratch, &scratch_bytes, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
-        (!exact && (e = cudaMallocAsync(&b.hdata, std::max<uint64_t>(1, b.hcap) * 8, st)) != cudaSuccess))
+        (!exact && (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess))
         return bail(e);
-    if (mode == 4 && ((e = cudaMallocAsync(&lin, std::max<uint64_t>(1, n_local) * 8, st)) != cudaSuccess ||
-                      (e = cudaMallocAsync(&seg, (size_t)n_ctas * n_pieces * sizeof(kc::SegDesc), st)) != cudaSuccess ||
-                      (e = cudaMallocAsync(&g_cursor, 8, st)) != cudaSuccess))
-        return bail(e);
+    char* q = static_cast<char*>(scratch);
+    kc::SegDesc* seg = reinterpret_cast<kc::SegDesc*>(q);
+    uint64_t* lin = reinterpret_cast<uint64_t*>(q += n_seg * sizeof(kc::SegDesc));
+    uint64_t* rel = reinterpret_cast<uint64_t*>(q += n_lin * 8);
+    uint64_t* cursor = reinterpret_cast<uint64_t*>(q += cells * 8);
+    uint64_t* g_cursor = reinterpret_cast<uint64_t*>(q += P * 8);
+    uint32_t* counts = reinterpret_cast<uint32_t*>(q += 8);
+    uint32_t* total = reinterpret_cast<uint32_t*>(q += cells * 4);
     if (mode == 4 && chunks) {
         KC_CUDA(cudaMemsetAsync(g_cursor, 0, 8, st));
         for (int c = 0; c < chunks->n; ++c) {
@@ -430,19 +504,14 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
         KC_CUDA(cudaMemcpyAsync(&need, b.hstarts + P, 8, cudaMemcpyDeviceToHost, st));
         KC_CUDA(cudaStreamSynchronize(st));
         b.hcap = need;
-        if ((e = cudaMallocAsync(&b.hdata, std::max<uint64_t>(1, need) * 8, st)) != cudaSuccess) return bail(e);
+        b.hash_bytes = std::max<uint64_t>(1, need) * 8;
+        if ((e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess) return bail(e);
     }
     if (mode != 1) kc::launch_bucket_base(rel, b.hstarts, n_ctas, a, st);
     if (mode == 4) kc::launch_scatter_staged_seg(lin, seg, n_ctas, n_pieces, 0, a, rel, b.hdata, st);
     else kc::launch_bucket_scatter(b.pw, b.vw, b.n_units, upc, n_ctas, p, a, mode, rel, cursor, b.hdata, st);
     h->launches += mode != 1 ? 5 : 4;
-    cudaFreeAsync(counts, st);
-    cudaFreeAsync(rel, st);
-    cudaFreeAsync(total, st);
-    cudaFreeAsync(cursor, st);
-    if (lin) cudaFreeAsync(lin, st);
-    if (seg) cudaFreeAsync(seg, st);
-    if (g_cursor) cudaFreeAsync(g_cursor, st);
+    leave_block(h, scratch, scratch_bytes, st);  // every caller's st is the handle's stream
     if (h->l1_bits != h->part_bits) return regroup_batch(h, b, st);
     return KC_OK;
 }
@@ -473,6 +542,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
     std::vector<kc::IngestBatch> ib(refs.size());
     std::vector<uint32_t> item_batch;
     std::vector<void*> scratch(refs.size(), nullptr);
+    std::vector<size_t> scratch_bytes(refs.size(), 0);
     kc::IngestPlan plan{};
     bool ranged = false, all_k31 = true;
     auto bail = [&](cudaError_t e) {
@@ -482,6 +552,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
             if (b.hdata) cudaFreeAsync(b.hdata, st);
             if (b.hstarts) cudaFreeAsync(b.hstarts, st);
             b.hdata = b.hstarts = nullptr;
+            b.hash_bytes = 0;
         }
         return cuda_fail(e, "cudaMallocAsync(batched ingest)");
     };
@@ -509,9 +580,9 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         item_batch.insert(item_batch.end(), B.n_items, (uint32_t)i);
         // scratch: counts, relative bases, segments, totals, cursor, linear hashes
         const uint64_t cells = (uint64_t)B.n_items * P;
-        const uint64_t bytes = cells * 4 + cells * 8 + B.n_items * sizeof(kc::SegDesc) + P * 4 + 8 + b.n_local * 8 + 64;
+        scratch_bytes[i] = cells * 4 + cells * 8 + B.n_items * sizeof(kc::SegDesc) + P * 4 + 8 + b.n_local * 8 + 64;
         cudaError_t e;
-        if ((e = cudaMallocAsync(&scratch[i], bytes, st)) != cudaSuccess) return bail(e);
+        if ((e = take_block(h, &scratch[i], &scratch_bytes[i], st)) != cudaSuccess) return bail(e);
         char* q = static_cast<char*>(scratch[i]);
         B.rel = reinterpret_cast<uint64_t*>(q);
         q += cells * 8;
@@ -525,8 +596,9 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         q += cells * 4;
         B.total = reinterpret_cast<uint32_t*>(q);
         b.hcap = b.n_local + 3 * cells;
+        b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
         if ((e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&b.hdata, std::max<uint64_t>(1, b.hcap) * 8, st)) != cudaSuccess)
+            (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess)
             return bail(e);
         B.starts = b.hstarts;
         B.out = b.hdata;
@@ -556,11 +628,14 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
     KC_LAUNCHED("batched ingest launches");
     if (timed) phase_end(hs[0], kPass1, t0, st);
     cudaFreeAsync(blk, st);
+    // (two grouping levels: the second one's blocks are taken on st before that)
+    bool keep = true;
+    for (const Ref& r : refs) keep = keep && r.h->l1_bits == r.h->part_bits;
     for (size_t i = 0; i < refs.size(); ++i) {
-        cudaFreeAsync(scratch[i], st);
+        if (keep) leave_block(refs[i].h, scratch[i], scratch_bytes[i], st);  // the handle's stream will wait for st
+        else cudaFreeAsync(scratch[i], st);
         Batch& b = refs[i].h->batches[refs[i].t];
         cudaFreeAsync(b.pw, st);  // the hashes replace the reads
-        cudaFreeAsync(b.vw, st);
         b.pw = b.vw = nullptr;
         b.pending = false;
     }
@@ -580,7 +655,7 @@ uint64_t bucket_bytes(kc_handle h, uint64_t n_local);
 // Device bytes the handle holds now: filter, table and counters, resident
 // batches (reads and grouped hashes) and its result.
 uint64_t held_bytes(kc_handle h) {
-    uint64_t bytes = h->fixed_bytes + h->res_cap * 16;
+    uint64_t bytes = h->fixed_bytes + h->res_cap * 16;  // idle blocks are there to be taken
     for (const auto& b : h->batches) {
         if (b.pw) bytes += (2 * b.n_units + 2) * 8 + b.n_units * 8;
         if (b.hdata) bytes += b.hcap * 8 + ((1ull << h->part_bits) + 1) * 8;
@@ -610,9 +685,13 @@ uint64_t room_bytes(kc_handle h) {
         else
             cudaGetLastError();
     }
-    const uint64_t avail = (uint64_t)free_b + cached, margin = 1ull << 30;
+    const uint64_t avail = (uint64_t)free_b + cached + h->idle_bytes, margin = 1ull << 30;
     return avail > margin ? avail - margin : 0;
 }
+
+bool small_need(kc_handle h, uint64_t bytes) { return bytes <= kSmallNeed && !h->cfg.device_budget && !h->owner; }
+
+bool fits_device(kc_handle h, uint64_t bytes) { return small_need(h, bytes) || bytes <= room_bytes(h); }
 
 // Device bytes bucket_batch needs for a batch of n_local bases: the linear
 // hashes and the grouped hashes (8 bytes per window each, at most one window
@@ -986,14 +1065,13 @@ kc_status kc_create_ex(int k, int n_samples, uint64_t bloom_bits, int n_hashes, 
     }
     const size_t bloom_bytes = bloom_bits / 8, table_bytes = slots * sizeof(kc::Slot);
     // stream-ordered pool allocations: no device-wide synchronisation
-    if ((e = cudaMallocAsync(&h->bloom, bloom_bytes, h->stream)) != cudaSuccess)
+    if ((e = cudaMallocAsync(&h->bloom, bloom_bytes + sizeof(kc::DevCounters), h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(filter)"));
+    h->ctr = reinterpret_cast<kc::DevCounters*>(reinterpret_cast<char*>(h->bloom) + bloom_bytes);  // behind the filter
     if (table_bytes && (e = cudaMallocAsync(&h->table, table_bytes, h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(table)"));
     if (c.prune_chain && (e = cudaMallocAsync(&h->bloom2, bloom_bytes, h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(second filter)"));
-    if ((e = cudaMallocAsync(&h->ctr, sizeof(kc::DevCounters), h->stream)) != cudaSuccess)
-        return bail(cuda_fail(e, "cudaMallocAsync(counters)"));
     h->fixed_bytes = bloom_bytes * (c.prune_chain ? 2 : 1) + table_bytes + sizeof(kc::DevCounters);
     kc_status s = kc_reset(h);
     if (s != KC_OK) return bail(s);
@@ -1003,6 +1081,7 @@ kc_status kc_create_ex(int k, int n_samples, uint64_t bloom_bits, int n_hashes, 
 
 kc_status kc_reset(kc_handle h) {
     if (!h) return fail(KC_ERR_ARG, "null handle");
+    h->reused = h->reused || !h->batches.empty();
     free_batches(h);
     h->n_result = 0;  // the result arrays stay allocated for the next job (finalize reuses them)
     free_selection(h);
@@ -1040,7 +1119,9 @@ kc_status kc_reset(kc_handle h) {
 void kc_destroy(kc_handle h) {
     if (!h) return;
     if (h->stream) {
+        h->reused = false;
         free_batches(h);
+        free_idle(h);
         free_result(h);
         free_selection(h);
         free_stems(h);
@@ -1050,7 +1131,6 @@ void kc_destroy(kc_handle h) {
         if (h->bloom) cudaFreeAsync(h->bloom, h->stream);
         if (h->bloom2) cudaFreeAsync(h->bloom2, h->stream);
         if (h->table) cudaFreeAsync(h->table, h->stream);
-        if (h->ctr) cudaFreeAsync(h->ctr, h->stream);
         if (h->chk_ctr) cudaFreeAsync(h->chk_ctr, h->copy_stream);
     }
     for (const auto& m : h->marks) {
@@ -1083,14 +1163,14 @@ cudaError_t pinned_words(kc_handle h) {
 }
 
 // kc_add_reads of host reads in n_chunks chunks (the read store b.pw / b.vw
-// and the scratch nm, bd, doff are allocated on the copy stream; all are
+// and the scratch nm, bd, doff, in temp, are allocated on the copy stream; all are
 // freed here, the grouped hashes replacing the reads).  On the copy stream: the offsets,
 // their check (read starts marked into bd, error bits into chk_ctr), then
 // each chunk's packed and N-mask words.  On the handle's stream, after the
 // check: per chunk its valid-window bits and extraction, then the grouping.
 kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* packed_reads, const uint64_t* offsets,
                             const uint64_t* n_mask, uint64_t n_reads, uint64_t b0, uint64_t b1, int n_chunks,
-                            uint64_t* nm, uint64_t* bd, uint64_t* doff) {
+                            uint64_t* nm, uint64_t* bd, uint64_t* doff, void* temp) {
     cudaStream_t st = h->stream, cs = h->copy_stream;
     const uint64_t B = (b0 / 64) * 64;
     const uint64_t n_local = b1 - B;
@@ -1098,7 +1178,7 @@ kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* p
     const uint64_t n_pwords_src = (n_local + 31) / 32;
     const uint64_t n_pwords = 2 * n_units + 2;
     auto release = [&]() {
-        for (void* q : {(void*)b.pw, (void*)b.vw, (void*)nm, (void*)bd, (void*)doff}) cudaFreeAsync(q, cs);
+        for (void* q : {(void*)b.pw, temp}) cudaFreeAsync(q, cs);
         b.pw = b.vw = nullptr;
     };
     cudaError_t e = cudaSuccess;
@@ -1157,13 +1237,13 @@ kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* p
     phase_end(h, kPass1, t0);
     if (s != KC_OK) {
         KC_CUDA(cudaStreamSynchronize(cs));
-        for (void* q : {(void*)nm, (void*)bd, (void*)doff, (void*)b.pw, (void*)b.vw}) cudaFreeAsync(q, st);
+        for (void* q : {temp, (void*)b.pw}) cudaFreeAsync(q, st);
         b.pw = b.vw = nullptr;
         return s;
     }
     h->launches += 4;
     KC_LAUNCHED("ingest launches");
-    for (void* q : {(void*)nm, (void*)bd, (void*)doff, (void*)b.pw, (void*)b.vw}) cudaFreeAsync(q, st);
+    for (void* q : {temp, (void*)b.pw}) cudaFreeAsync(q, st);
     b.pw = b.vw = nullptr;  // the hashes replace the reads: nothing rescans them
     KC_CUDA(cudaEventSynchronize(h->ev_chunk[n_chunks - 1]));  // caller may reuse its arrays
     return KC_OK;
@@ -1225,7 +1305,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     // the handle.
     const int n_chunks = (int)std::min<uint64_t>(kMaxChunks, n_units / kChunkUnits);
     const bool chunked = !data_dev && !mask_dev && n_chunks >= 2 && h->strategy != KC_STRATEGY_DIRECT &&
-                         !h->cfg.batched_ingest && scatter_mode_of(h) == 4 && bucket_bytes(h, n_local) <= room_bytes(h);
+                         !h->cfg.batched_ingest && scatter_mode_of(h) == 4 && fits_device(h, bucket_bytes(h, n_local));
     // The N mask and offsets serve this call's kernels only: device ones are
     // read where they are (in stream order), host ones copied.  The packed
     // words are always copied: the store is padded for the kernels' loads and
@@ -1233,20 +1313,20 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     const bool own_nm = chunked || !is_local_device_ptr(n_mask, h->device);
     const bool own_off = chunked || !is_local_device_ptr(offsets, h->device);
     cudaError_t e;
-    if ((e = cudaMallocAsync(&b.pw, n_pwords * 8, cs)) != cudaSuccess ||
-        (e = cudaMallocAsync(&b.vw, n_units * 8, cs)) != cudaSuccess ||
-        (own_nm && (e = cudaMallocAsync(&nm, n_units * 8, cs)) != cudaSuccess) ||
-        (e = cudaMallocAsync(&bd, n_units * 8, cs)) != cudaSuccess ||
-        (own_off && (e = cudaMallocAsync(&doff, (n_reads + 1) * 8, cs)) != cudaSuccess)) {
-        cudaFreeAsync(b.pw, cs);
-        cudaFreeAsync(b.vw, cs);
-        cudaFreeAsync(nm, cs);
-        cudaFreeAsync(bd, cs);
-        cudaFreeAsync(doff, cs);
+    // the read store (packed words, valid-window bits) and, for this call, the
+    // read-start bits and the copies of the N mask and offsets
+    void* temp = nullptr;
+    if ((e = cudaMallocAsync(&b.pw, (n_pwords + n_units) * 8, cs)) != cudaSuccess ||
+        (e = cudaMallocAsync(&temp, (n_units + (own_nm ? n_units : 0) + (own_off ? n_reads + 1 : 0)) * 8, cs)) != cudaSuccess) {
+        if (b.pw) cudaFreeAsync(b.pw, cs);
         return cuda_fail(e, "cudaMallocAsync(read store)");
     }
+    b.vw = b.pw + n_pwords;
+    bd = static_cast<uint64_t*>(temp);
+    if (own_nm) nm = bd + n_units;
+    if (own_off) doff = bd + (own_nm ? 2 : 1) * n_units;
     if (chunked) {
-        s = add_reads_chunked(h, b, sample, packed_reads, offsets, n_mask, n_reads, b0, b1, n_chunks, nm, bd, doff);
+        s = add_reads_chunked(h, b, sample, packed_reads, offsets, n_mask, n_reads, b0, b1, n_chunks, nm, bd, doff, temp);
         if (s != KC_OK) return s;
         h->batches.push_back(b);
         h->bases += b1 - b0;
@@ -1264,7 +1344,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
         for (uint64_t r = 0; r < n_reads && !decreasing; ++r) decreasing = offsets[r + 1] < offsets[r];
         if (decreasing) {
             KC_CUDA(cudaStreamSynchronize(cs));
-            for (void* q : {(void*)b.pw, (void*)b.vw, (void*)nm, (void*)bd, (void*)doff}) cudaFreeAsync(q, cs);
+            for (void* q : {(void*)b.pw, temp}) cudaFreeAsync(q, cs);
             return fail(KC_ERR_ARG, "read offsets decrease");
         }
     }
@@ -1284,7 +1364,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
         else
             kc::launch_pass1(b.pw, b.vw, n_units, h->params(sample), h->bloom, h->table, h->ctr, h->grid, st);
         h->launches += 3;
-    } else if (bucket_bytes(h, n_local) > room_bytes(h)) {
+    } else if (!fits_device(h, bucket_bytes(h, n_local))) {
         // the window hashes would not fit the device budget: keep the packed
         // reads (about 3 bits per base), extracted again at kc_finalize one
         // hash range at a time
@@ -1295,8 +1375,15 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
         b.n_local = n_local;
     } else {
         s = bucket_batch(h, b, n_local, st, h->params(sample), false);
+        if (s == KC_ERR_OOM_DEVICE && small_need(h, bucket_bytes(h, n_local))) {
+            cudaGetLastError();
+            leave_hashes(h, b);  // no room after all: kept as reads
+            b.deferred = true;
+            ++h->deferred;
+            s = KC_OK;
+        }
         if (s != KC_OK) {
-            for (void* q : {(void*)nm, (void*)bd, (void*)doff, (void*)b.pw, (void*)b.vw}) cudaFreeAsync(q, st);
+            for (void* q : {temp, (void*)b.pw}) cudaFreeAsync(q, st);
             if (any_host) cudaEventSynchronize(h->ev_copy);  // the caller's arrays are no longer read
             return s;
         }
@@ -1304,13 +1391,10 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     }
     phase_end(h, kPass1, t0);
     KC_LAUNCHED("ingest launches");
-    cudaFreeAsync(nm, st);
-    cudaFreeAsync(bd, st);
-    cudaFreeAsync(doff, st);
+    cudaFreeAsync(temp, st);
     if (h->strategy != KC_STRATEGY_DIRECT && !b.deferred && !b.pending) {
         // the hashes replace the reads: nothing rescans them
         cudaFreeAsync(b.pw, st);
-        cudaFreeAsync(b.vw, st);
         b.pw = b.vw = nullptr;
     }
     h->batches.push_back(b);
@@ -1448,7 +1532,7 @@ kc_status kc_stats_get(kc_handle h, kc_stats* out) {
         if (b.pw) bytes += (2 * b.n_units + 2) * 8 + b.n_units * 8;
         if (b.hdata) bytes += b.hcap * 8 + ((1ull << h->part_bits) + 1) * 8;
     }
-    out->device_bytes = bytes;
+    out->device_bytes = bytes + h->idle_bytes;
     out->launches = h->launches;
     out->ms_ingest = h->ms[kIngest];
     out->ms_pass1 = h->ms[kPass1];

@@ -935,19 +935,19 @@ struct JobWork {
     kc_handle h;
     std::vector<uint64_t> hs;  // partition starts of every batch
     uint64_t total_w = 0, max_w = 0;
+    // survivors: keys, then values, in one block of the handle's (take_block)
     uint64_t* sv_keys = nullptr;
     uint64_t* sv_vals = nullptr;
     uint64_t sv_cap = 0;
-    uint64_t* failed = nullptr;
+    size_t sv_bytes = 0;
+    uint64_t* failed = nullptr;  // failed partitions, then the batches' pointers (meta)
     void* meta = nullptr;
 };
 
 void release_work(kc_batch_ctx* b, std::vector<JobWork>& w) {
     for (auto& x : w) {
         if (x.sv_keys) cudaFreeAsync(x.sv_keys, b->st);
-        if (x.sv_vals) cudaFreeAsync(x.sv_vals, b->st);
         if (x.failed) cudaFreeAsync(x.failed, b->st);
-        if (x.meta) cudaFreeAsync(x.meta, b->st);
         x.sv_keys = x.sv_vals = nullptr;
         x.failed = nullptr;
         x.meta = nullptr;
@@ -1027,21 +1027,18 @@ kc_status run_fallbacks(kc_batch_ctx* b, JobWork& x, uint32_t j, uint32_t n_fail
     for (uint64_t hl : fl) extra += windows_of((uint32_t)(hl >> (64 - a)));
     const uint64_t need = n_sv + extra;
     if (need > x.sv_cap) {
-        uint64_t *nk = nullptr, *nv = nullptr;
-        cudaError_t e;
-        if ((e = cudaMallocAsync(&nk, need * 8, b->st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&nv, need * 8, b->st)) != cudaSuccess) {
-            if (nk) cudaFreeAsync(nk, b->st);
-            return cuda_fail(e, "cudaMallocAsync(fallback survivors)");
-        }
+        uint64_t* nk = nullptr;
+        cudaError_t e = cudaMallocAsync(&nk, need * 16, b->st);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(fallback survivors)");
+        uint64_t* nv = nk + need;
         const uint64_t have = std::min<uint64_t>(n_sv, x.sv_cap);
         KC_CUDA(cudaMemcpyAsync(nk, x.sv_keys, have * 8, cudaMemcpyDeviceToDevice, b->st));
         KC_CUDA(cudaMemcpyAsync(nv, x.sv_vals, have * 8, cudaMemcpyDeviceToDevice, b->st));
         cudaFreeAsync(x.sv_keys, b->st);
-        cudaFreeAsync(x.sv_vals, b->st);
         x.sv_keys = nk;
         x.sv_vals = nv;
         x.sv_cap = need;
+        x.sv_bytes = need * 16;
     }
     const uint64_t n_sw = 1ull << h->slice_log2;
     for (uint64_t hl : fl) {
@@ -1266,13 +1263,16 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         x.sv_cap = std::max<uint64_t>(1, x.sv_cap);
         const size_t meta_bytes = std::max<size_t>(16, nb * 20);
         cudaError_t e;
-        if ((e = cudaMallocAsync(&x.sv_keys, x.sv_cap * 8, st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&x.sv_vals, x.sv_cap * 8, st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&x.failed, P * 8, st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&x.meta, meta_bytes, st)) != cudaSuccess) {
+        // (the survivors' block is first used by the consumer, after the
+        // handle's stream; the other one is written at once)
+        x.sv_bytes = x.sv_cap * 16;
+        if ((e = take_block(h, reinterpret_cast<void**>(&x.sv_keys), &x.sv_bytes, st)) != cudaSuccess ||
+            (e = cudaMallocAsync(&x.failed, P * 8 + meta_bytes, st)) != cudaSuccess) {
             release_work(b, work);
             return cuda_fail(e, "cudaMallocAsync(batch consumer)");
         }
+        x.sv_vals = x.sv_keys + x.sv_cap;
+        x.meta = x.failed + P;
         std::vector<unsigned char> hm(meta_bytes, 0);
         for (size_t t = 0; t < nb; ++t) {
             const uint64_t dp = (uint64_t)(uintptr_t)h->batches[t].hdata;
@@ -1520,8 +1520,12 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         KC_LAUNCHED("batched global sort launches");
     }
     if (t0) phase_end(hs[0], kSort, t0, st);
-    release_work(b, work);
     KC_CUDA(cudaStreamSynchronize(st));
+    for (JobWork& x : work) {  // nothing uses them any more
+        leave_block(x.h, x.sv_keys, x.sv_bytes, st);
+        x.sv_keys = x.sv_vals = nullptr;
+    }
+    release_work(b, work);
     for (int j = 0; j < n; ++j) {
         kc_handle h = hs[j];
         h->host_ctr.survivors = h->n_result;
@@ -1670,8 +1674,7 @@ kc_status finalize_grouped(kc_batch_ctx* b, kc_handle h) {
         }
         for (Batch& pc : pieces)
             if (pc.deferred) {
-                if (pc.hdata) cudaFreeAsync(pc.hdata, st);
-                if (pc.hstarts) cudaFreeAsync(pc.hstarts, st);
+                leave_hashes(h, pc);
             }
         h->batches = kept;
     }
@@ -1720,7 +1723,14 @@ kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
         // survivors and sorted result, 16 bytes each per key, at most one
         // key per min_count windows (and per base): spill when they would
         // not fit
-        if (32 * (h->bases / std::max<uint32_t>(1, h->min_count)) > room_bytes(h)) return finalize_spilled(b, h);
+        const uint64_t need = 32 * (h->bases / std::max<uint32_t>(1, h->min_count));
+        if (!fits_device(h, need)) return finalize_spilled(b, h);
+        kc_status s = finalize_core(b, hs, n, 0, 0xffffffffu, true);
+        if (s != KC_ERR_OOM_DEVICE || !small_need(h, need)) return s;
+        cudaGetLastError();  // no room after all: counted again, group by group
+        KC_CUDA(cudaMemsetAsync(&h->ctr->candidates, 0, 2 * sizeof(unsigned long long), b->st));  // and claimed
+        KC_CUDA(cudaMemsetAsync(&h->ctr->split_parts, 0, sizeof(unsigned), b->st));
+        return finalize_spilled(b, h);
     }
     if (!hs || n <= 1) return finalize_core(b, hs, n, 0, 0xffffffffu, true);
     // handles whose reads passed the device budget are finalized alone, in

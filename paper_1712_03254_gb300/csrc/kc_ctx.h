@@ -27,12 +27,13 @@ struct Batch {
     int sample = 0;
     // direct strategy: the resident reads, rescanned by the recount
     uint64_t* pw = nullptr;  // packed words, 2 * n_units + 2
-    uint64_t* vw = nullptr;  // valid-window-start words, n_units
+    uint64_t* vw = nullptr;  // valid-window-start words, n_units (in pw's block)
     uint64_t n_units = 0;
     // partitioned strategy: window hashes grouped by partition
     uint64_t* hdata = nullptr;    // capacity: one per base of the batch
     uint64_t* hstarts = nullptr;  // partition starts, 2^part_bits + 1
     uint64_t hcap = 0;
+    size_t hash_bytes = 0;  // size of hdata's block
     // partitioned, over the device budget: the reads are kept (pw, vw) and
     // extracted again at kc_finalize, one hash range at a time
     bool deferred = false;
@@ -88,6 +89,27 @@ struct SpillRun {
 
 // Pinned host memory the spilled runs are placed in; kept across kc_reset so
 // a repeated out-of-core job does not pin memory again.
+// Device blocks a handle keeps for its next job (idle between their uses): the
+// grouped hashes and the scratch of the grouping and the finalize, a few bytes
+// per base each.  Taking blocks of this size from the stream-ordered pool for
+// every job cost 0.35 ms each when several handles took turns (the pool maps
+// their memory anew).  A handle keeps blocks from its second job on
+// (kc_reset), unless it has a device budget, and all handles together at most
+// kIdleShare of the device's memory; kc_destroy gives them back, and so does a
+// failed allocation of the handle.  A block is taken for work ordered after
+// the handle's stream and left when the handle's stream is ordered after its
+// last use.
+struct IdleBlock {
+    void* p = nullptr;
+    size_t bytes = 0;
+};
+constexpr size_t kMaxIdleBlocks = 12;
+constexpr size_t kIdleShare = 8;
+constexpr size_t kIdleMinBytes = 1ull << 20;  // smaller blocks come from the pool at once
+// Needs up to this are allocated without asking for the free memory first
+// (cudaMemGetInfo takes 16 us); if that fails, they are handled as not fitting.
+constexpr uint64_t kSmallNeed = 64ull << 20;  // (below any batch copied in chunks)
+
 struct PinnedChunk {
     uint64_t* p = nullptr;
     uint64_t words = 0, used = 0;
@@ -152,6 +174,11 @@ struct kc_ctx {
     uint64_t* res_vals = nullptr;
     uint64_t n_result = 0;
     uint64_t res_cap = 0;
+
+    // blocks kept for the next job (IdleBlock); reused: a job has been reset
+    std::vector<kcapi::IdleBlock> idle;
+    size_t idle_bytes = 0;
+    bool reused = false;
 
     kc::DevCounters host_ctr{};
     kcapi::State state = kcapi::State::Open;
@@ -238,6 +265,16 @@ void phase_collect(kc_handle h);
 kc_status read_counters(kc_handle h);
 kc_status device_errors(kc_handle h);
 void free_result(kc_handle h);
+// A device block of at least *bytes for work on stream st, which is ordered
+// after the handle's stream: an idle block of the handle (*bytes becomes its
+// size) or one from the pool.
+cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st);
+// Give a block back, last used on stream st, which the handle's stream is (or
+// will be, before its next work) ordered after: kept idle, or to the pool.
+void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st);
+// The batch's grouped hashes and their starts, last used on the handle's stream.
+void leave_hashes(kc_handle h, Batch& b);
+void free_idle(kc_handle h);
 void release_spill(kc_handle h);
 void free_spill_chunks(kc_handle h);
 uint64_t* spill_alloc(kc_handle h, uint64_t words);  // nullptr when pinning fails
@@ -260,6 +297,9 @@ uint64_t held_bytes(kc_handle h);
 // handles on stream st, ordered after each handle's stream by the caller.
 kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count);
 uint64_t room_bytes(kc_handle h);
+// Whether the handle may allocate `bytes` (a small need: try it and see).
+bool fits_device(kc_handle h, uint64_t bytes);
+bool small_need(kc_handle h, uint64_t bytes);
 // Sort n (key, value) pairs (keys below 2^key_bits) from tk/tv into out_k/out_v;
 // ctr->survivors holds n on the device; synchronises the stream.
 kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64_t n, int key_bits,

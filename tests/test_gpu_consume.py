@@ -138,3 +138,33 @@ def test_keys_of_one_home_slot(n_same):
     st = _count(codes, keys, repeats, 2, 2, part_bits=1, smem_table_log2=10)
     assert st["fallback_partitions"] == 0
     assert (st["split_partitions"] > 0) == (n_same > 64)
+
+
+def test_blocks_kept_between_jobs(oracle_mod):
+    """Two handles in turn, each reset between jobs of very different sizes, one
+    and two kc_add_reads calls, host and device reads: blocks kept for the next
+    job never carry anything over."""
+    import torch
+
+    g = synth.genome(71, 200_000)
+    sets = [synth.reads(71 + n, g, n, 80, 180, 0.01, 0.001) for n in (20_000, 1_500, 30_000, 200, 24_000)]
+    oracles = {}
+    for k in (31, 25):
+        for i, rs in enumerate(sets):
+            oracles[k, i] = oracle_mod.count(synth.Workload("job", [rs], k, 1 << 22, 4, 2))
+    handles = {k: kc.KmerCounter(k, 1, 1 << 22, 4, 2, strategy="partitioned") for k in (31, 25)}
+    for i, rs in enumerate(sets):
+        for k, c in handles.items():
+            c.reset()
+            parts = [rs] if i % 2 == 0 else [rs.slice(0, rs.n_reads // 2), rs.slice(rs.n_reads // 2, rs.n_reads)]
+            for p in parts:
+                packed, mask = kc.pack_ascii(p.ascii)
+                arrays = [packed, np.ascontiguousarray(p.offsets, dtype=np.uint64), mask]
+                if k == 25:
+                    arrays = [torch.from_numpy(a.view(np.int64)).cuda() for a in arrays]
+                    torch.cuda.synchronize()
+                c.add_reads(0, *arrays)
+            c.finalize()
+            _same(c, oracles[k, i])
+    for c in handles.values():
+        c.close()
