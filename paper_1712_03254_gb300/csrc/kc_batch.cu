@@ -126,7 +126,10 @@ constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32
 // the finest level is left to the global fallback.  The finest level a job has
 // needed is kept in its counters, and its later partitions start there instead
 // of overflowing again.
-template <int THREADS>
+//
+// ONE: every job of the batch has one sample (a slot's counts at a constant
+// place).
+template <int THREADS, bool ONE>
 __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
     k_consume_q(const BatchDesc* __restrict__ D) {
     extern __shared__ unsigned long long s_mem[];
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
         const uint32_t n_sw = 1u << J.slice_log2;
         const uint32_t T = 1u << J.table_log2;
         const uint32_t tmask = T - 1;
-        const int s2 = J.n_samples - 1;  // a slot's counts: 1 << s2 of them
+        const int s2 = ONE ? 0 : J.n_samples - 1;  // a slot's counts: 1 << s2 of them
         const int a = J.part_bits;
         uint32_t* const sc = reinterpret_cast<uint32_t*>(sk + T);  // counts, then
         unsigned long long* const sb = sk + T;                     // the filter words
@@ -196,7 +199,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             for (int bt = 0; bt < J.n_batches && !stop; ++bt) {
                 const uint64_t lo = J.starts[bt][part];
                 const uint64_t n_all = J.starts[bt][part + 1] - lo;
-                uint32_t* const scol = sc + J.samples[bt];  // this batch's count column
+                uint32_t* const scol = ONE ? sc : sc + J.samples[bt];  // this batch's count column
                 unsigned q = 0;                             // entries in the warp's queue
                 // The queue's last n (at most 32) windows, one per lane, take their
                 // next probe: slots home, home + 1, home + 3, home + 6, ... (every
@@ -293,11 +296,12 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             const uint32_t slot0 = wid * rows * 32 + lane;
             unsigned kept = 0, n_kept = 0;  // lane r: the ballot of row r
             uint64_t n_win = 0;
+            const uint32_t min_count = J.min_count;
             for (uint32_t r = 0; r < rows; ++r) {
                 const uint32_t i = slot0 + r * 32;
                 const uint64_t sum = s2 ? (uint64_t)sc[2 * i] + sc[2 * i + 1] : (uint64_t)sc[i];
                 n_win += sum;
-                const unsigned ballot = __ballot_sync(kFull, sum != 0 && sum >= J.min_count);
+                const unsigned ballot = __ballot_sync(kFull, sum != 0 && sum >= min_count);
                 if (lane == (int)r) kept = ballot;
                 n_kept += __popc(ballot);
                 // a key seen once is marked by its top bit (unless that makes it the
@@ -308,19 +312,24 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             if (n_kept) {
                 if (lane == 0) pos0 = atomicAdd(&D->counters[2 * j], (unsigned long long)n_kept);
                 pos0 = __shfl_sync(kFull, pos0, 0);
+                uint64_t* const sv_keys = J.sv_keys;
+                uint64_t* const sv_vals = J.sv_vals;
+                uint32_t* const hist = J.hist_job;
+                const uint64_t sv_cap = J.sv_cap;
+                const int hist_shift = J.hist_shift;
                 unsigned qn = 0;  // the slots of kept keys, taken 32 at a time
                 const auto write = [&](unsigned n) {
                     __syncwarp();
                     qn -= n;
                     const uint64_t pos = pos0 + lane;
-                    if ((unsigned)lane < n && pos < J.sv_cap) {
+                    if ((unsigned)lane < n && pos < sv_cap) {
                         const uint32_t i = ws[qn + lane];
                         uint64_t h = sk[i];
                         if ((h ^ hpre) & kTopBit) h ^= kTopBit;
                         const uint64_t key = unmixer64(h);
-                        J.sv_keys[pos] = key;
-                        J.sv_vals[pos] = s2 ? (uint64_t)sc[2 * i] | ((uint64_t)sc[2 * i + 1] << 32) : (uint64_t)sc[i];
-                        if (J.hist_job) atomicAdd(J.hist_job + (key >> J.hist_shift), 1u);
+                        sv_keys[pos] = key;
+                        sv_vals[pos] = s2 ? (uint64_t)sc[2 * i] | ((uint64_t)sc[2 * i + 1] << 32) : (uint64_t)sc[i];
+                        if (hist) atomicAdd(hist + (key >> hist_shift), 1u);
                     }
                     pos0 += n;
                     __syncwarp();
@@ -340,20 +349,34 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             const int bloom_shift = J.bloom_shift, n_hashes = J.n_hashes;
             const bool all_cand = J.all_candidates != 0;
             uint64_t n_new = 0, n_seen = 0;  // keys that set a bit first, keys that were candidates
-            for (uint32_t i = slot0, r = 0; r < rows; ++r, i += 32) {
-                uint64_t h = sk[i];
-                if (h == empty) continue;
-                const bool once = (h ^ hpre) & kTopBit;
-                if (once) h ^= kTopBit;
-                const uint64_t pat = bloom_pattern_rt(mixer64(h), n_hashes);
-                // two 32-bit updates: a shared 64-bit one takes three times as long as a 32-bit one
-                uint32_t* const word = reinterpret_cast<uint32_t*>(sb + ((uint32_t)(h >> bloom_shift) & (w_n - 1)));
-                const uint32_t p_lo = (uint32_t)pat, p_hi = (uint32_t)(pat >> 32);
-                const uint32_t o_lo = atomicOr(word, p_lo), o_hi = atomicOr(word + 1, p_hi);
-                const bool fresh = (p_lo & ~o_lo) != 0u || (p_hi & ~o_hi) != 0u;
-                n_new += fresh;
-                n_seen += all_cand || !(fresh && once);
+            unsigned qn = 0;  // the warp's keys, taken 32 at a time (the table's rows are up to three quarters empty)
+            const auto set_bits = [&](unsigned n) {
+                __syncwarp();
+                qn -= n;
+                if ((unsigned)lane < n) {
+                    uint64_t h = wq[qn + lane];
+                    const bool once = (h ^ hpre) & kTopBit;
+                    if (once) h ^= kTopBit;
+                    const uint64_t g = mixer64(h);
+                    const uint64_t pat = n_hashes == 4 ? bloom_pattern_n<4>(g) : bloom_pattern_rt(g, n_hashes);  // (4: every configuration's)
+                    // two 32-bit updates: a shared 64-bit one takes three times as long as a 32-bit one
+                    uint32_t* const word = reinterpret_cast<uint32_t*>(sb + ((uint32_t)(h >> bloom_shift) & (w_n - 1)));
+                    const uint32_t p_lo = (uint32_t)pat, p_hi = (uint32_t)(pat >> 32);
+                    const uint32_t o_lo = atomicOr(word, p_lo), o_hi = atomicOr(word + 1, p_hi);
+                    const bool fresh = (p_lo & ~o_lo) != 0u || (p_hi & ~o_hi) != 0u;
+                    n_new += fresh;
+                    n_seen += all_cand || !(fresh && once);
+                }
+                __syncwarp();
+            };
+            for (uint32_t r = 0; r < rows; ++r) {
+                const uint64_t h = sk[slot0 + r * 32];
+                const unsigned used = __ballot_sync(kFull, h != empty);
+                if (h != empty) wq[qn + __popc(used & lt)] = h;
+                qn += __popc(used);
+                if (qn >= 32) set_bits(32);
             }
+            if (qn) set_bits(qn);
             // windows reported as seen before: all but each key's first, if its bits were new
             cand += n_win - (all_cand ? 0 : n_new);
             claimed += n_seen;
@@ -793,6 +816,7 @@ struct kc_batch_ctx {
     cudaGraphExec_t sort_graph = nullptr;
     // captured consumer launches, one per launch shape
     struct ConsumeGraph {
+        bool one;  // one sample in every job
         int threads, n_ctas;
         size_t smem;
         cudaGraphExec_t exec;
@@ -956,37 +980,39 @@ void release_work(kc_batch_ctx* b, std::vector<JobWork>& w) {
 
 // prepare: set the kernel's shared-memory limit (before any capture);
 // otherwise launch it.
-cudaError_t launch_consume(bool prepare, int threads, int n_ctas, size_t smem, const kc::BatchDesc* d, cudaStream_t st) {
+cudaError_t launch_consume(bool prepare, bool one, int threads, int n_ctas, size_t smem, const kc::BatchDesc* d, cudaStream_t st) {
     const auto go = [&](auto kern) {
         if (prepare) return kc::allow_max_dynamic_smem(kern);
         kern<<<n_ctas, threads, smem, st>>>(d);
         return cudaGetLastError();
     };
-    return threads == kc::kConsumeThreads ? go(kc::k_consume_q<kc::kConsumeThreads>) : go(kc::k_consume_q<kc::kConsumeThreadsWide>);
+    if (threads == kc::kConsumeThreads)
+        return one ? go(kc::k_consume_q<kc::kConsumeThreads, true>) : go(kc::k_consume_q<kc::kConsumeThreads, false>);
+    return one ? go(kc::k_consume_q<kc::kConsumeThreadsWide, true>) : go(kc::k_consume_q<kc::kConsumeThreadsWide, false>);
 }
 
 // The batch's counters reset and its persistent consumer launch, captured
-// once per launch shape (CTA size, grid, shared memory); everything else
+// once per launch shape (samples, CTA size, grid, shared memory); everything else
 // they read comes from the device descriptor.
-kc_status consume_graph(kc_batch_ctx* b, int threads, int n_ctas, size_t smem, cudaGraphExec_t* out) {
+kc_status consume_graph(kc_batch_ctx* b, bool one, int threads, int n_ctas, size_t smem, cudaGraphExec_t* out) {
     for (const auto& g : b->consume_graphs)
-        if (g.threads == threads && g.n_ctas == n_ctas && g.smem == smem) {
+        if (g.one == one && g.threads == threads && g.n_ctas == n_ctas && g.smem == smem) {
             *out = g.exec;
             return KC_OK;
         }
-    KC_CUDA(launch_consume(true, threads, n_ctas, smem, b->d_desc, b->st));
+    KC_CUDA(launch_consume(true, one, threads, n_ctas, smem, b->d_desc, b->st));
     std::lock_guard<std::mutex> lk(kc::sync_api_mutex());
     cudaGraph_t g = nullptr;
     KC_CUDA(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
     kc::k_reset_q<<<1, 256, 0, b->st>>>(b->d_desc);
-    launch_consume(false, threads, n_ctas, smem, b->d_desc, b->st);
+    launch_consume(false, one, threads, n_ctas, smem, b->d_desc, b->st);
     cudaError_t e = cudaStreamEndCapture(b->st, &g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture(consumer)");
     cudaGraphExec_t exec = nullptr;
     e = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate(consumer)");
-    b->consume_graphs.push_back({threads, n_ctas, smem, exec});
+    b->consume_graphs.push_back({one, threads, n_ctas, smem, exec});
     *out = exec;
     return KC_OK;
 }
@@ -1358,8 +1384,10 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         release_work(b, work);
         return s;
     }
+    bool one_sample = true;
+    for (int j = 0; j < n; ++j) one_sample = one_sample && hs[j]->n_samples == 1;
     // a persistent grid (CTAs without an item exit at once), so the captured
-    // launch depends on the shared memory alone
+    // launch depends on the samples and the shared memory alone
     const size_t smem_cta = smem_max + kc::consume_queue_smem(kc::kConsumeThreads);
     int per_sm = std::min(2, b->max_sm / (int)(smem_cta + 2048));
     const int threads = per_sm > 1 ? kc::kConsumeThreads : kc::kConsumeThreadsWide;
@@ -1367,7 +1395,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     smem_max += kc::consume_queue_smem(threads);
     const int n_ctas = b->sm_count * per_sm;
     cudaGraphExec_t cons = nullptr;
-    if ((s = consume_graph(b, threads, n_ctas, smem_max, &cons)) != KC_OK) {
+    if ((s = consume_graph(b, one_sample, threads, n_ctas, smem_max, &cons)) != KC_OK) {
         release_work(b, work);
         return s;
     }
