@@ -1255,12 +1255,16 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         // Split level: a sub-range's filter words take at most 64 KiB.
         const int split_min = std::max(0, h->slice_log2 - kc::kConsumeSliceLog2);
         // Shared-memory table: twice the windows of the largest partition
-        // (2^10..2^13 slots), so that small partitions never split; a larger
-        // partition's distinct keys fit or it splits.
+        // (2^10..2^13 slots, or 2^14), so that small partitions never split; a
+        // larger partition's distinct keys fit or it splits.
         int tl = (int)h->cfg.smem_table_log2;
         if (!tl) {
             tl = 10;
             while (tl < 13 && (1ull << tl) < 2 * (x.max_w >> split_min)) ++tl;
+            // one-sample partitions beyond what 8192 slots take at 30x coverage
+            // (one distinct key in six windows): 16384 slots and one wide CTA an
+            // SM, instead of two passes (43,700 windows: 1.48 -> 1.21 ms)
+            if (h->n_samples == 1 && (x.max_w >> split_min) > 40960) tl = 14;
         }
         const size_t queue = kc::consume_queue_smem(kc::kConsumeThreadsWide) + 1024;
         while (tl > 10 && kc::consume_smem(h->slice_log2 - split_min, tl, h->n_samples) + queue > (size_t)b->max_optin) --tl;
