@@ -39,6 +39,7 @@ struct JobDesc {
     DevCounters* ctr;
     // sort
     int sort_bits;
+    int even;  // buckets of equal shares of the canonical keys' distribution (key_bucket)
     int split_max;  // consumer: finest split level 2^split_max before the fallback
     int split_min;  // level at which a sub-range's filter words fit the consumer's shared memory
     uint64_t bucket_base;  // first bucket of this job in the flat arrays
@@ -49,9 +50,8 @@ struct JobDesc {
     uint64_t flat_base;  // this job's first survivor in the batch's survivors, in job order (set by the plan)
     // survivors histogrammed by the consumer itself (the sort's bucket bits
     // fixed before it runs): fixed_bits >= 0, hist_job = the job's first
-    // bucket counter, hist_shift = key_bits - fixed_bits; else fixed_bits = -1
+    // bucket counter; else fixed_bits = -1
     int fixed_bits;
-    int hist_shift;
     uint32_t* hist_job;
 };
 
@@ -72,7 +72,6 @@ struct BatchDesc {
     uint64_t buckets_cap;  // room of hist / starts / cursor
     int all_packable;      // set by the plan: every job's small buckets sort packed (k_warp_sort_q)
     uint64_t n_flat;       // set by the plan: survivors of all jobs
-    int hist_early;        // the consumer has histogrammed the survivors: the sort does not
     // the survivors scattered into their buckets, (key, value) side by side in
     // the flat bucket order of all jobs; the bucket sorts write the results
     ulonglong2* pairs;
@@ -316,7 +315,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                 uint64_t* const sv_vals = J.sv_vals;
                 uint32_t* const hist = J.hist_job;
                 const uint64_t sv_cap = J.sv_cap;
-                const int hist_shift = J.hist_shift;
+                const int key_bits = J.key_bits, hist_bits = J.fixed_bits;
+                const bool even = even_buckets(key_bits, hist_bits);
                 unsigned qn = 0;  // the slots of kept keys, taken 32 at a time
                 const auto write = [&](unsigned n) {
                     __syncwarp();
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                         const uint64_t key = unmixer64(h);
                         sv_keys[pos] = key;
                         sv_vals[pos] = s2 ? (uint64_t)sc[2 * i] | ((uint64_t)sc[2 * i + 1] << 32) : (uint64_t)sc[i];
-                        if (hist) atomicAdd(hist + (key >> hist_shift), 1u);
+                        if (hist) atomicAdd(hist + key_bucket(key, key_bits, hist_bits, even), 1u);
                     }
                     pos0 += n;
                     __syncwarp();
@@ -440,7 +440,8 @@ __global__ void k_plan_q(BatchDesc* __restrict__ D) {
         J.bucket_base = total;
         J.n_buckets = 1ull << bits;
         total += J.n_buckets;
-        if (J.key_bits - bits > 58) packable = 0;
+        J.even = even_buckets(J.key_bits, bits) ? 1 : 0;
+        if (!J.even && J.key_bits - bits > 57) packable = 0;
     }
     D->all_packable = packable;
     // short result arrays: no bucket and no survivor is sorted at all (a
@@ -456,7 +457,6 @@ __global__ void k_plan_q(BatchDesc* __restrict__ D) {
 }
 
 __global__ void k_zero_hist_q(const BatchDesc* __restrict__ D) {
-    if (D->hist_early) return;  // counted by the consumer
     const uint64_t n = D->n_buckets;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) D->hist[i] = 0u;
@@ -481,10 +481,9 @@ struct SurvivorJob {
     uint64_t lo, hi;  // flat survivor range of job j
     const uint64_t* keys;
     const uint64_t* vals;
-    int shift;
+    int key_bits, bits;
+    bool even;
     uint64_t n_buckets, bucket_base;
-    uint64_t* res_keys;
-    uint64_t* res_vals;
     uint64_t res_cap;
     __device__ void load(const BatchDesc* D, uint32_t jj) {
         j = jj;
@@ -493,13 +492,14 @@ struct SurvivorJob {
         hi = jj + 1 < D->n_jobs ? D->jobs[jj + 1].flat_base : D->n_flat;
         keys = J.sv_keys;
         vals = J.sv_vals;
-        shift = J.key_bits - J.sort_bits;
+        key_bits = J.key_bits;
+        bits = J.sort_bits;
+        even = J.even != 0;
         n_buckets = J.n_buckets;
         bucket_base = J.bucket_base;
-        res_keys = J.res_keys;
-        res_vals = J.res_vals;
         res_cap = J.res_cap;
     }
+    __device__ uint64_t bucket(uint64_t key) const { return key_bucket(key, key_bits, bits, even); }
     __device__ void seek(const BatchDesc* D, uint64_t i) {
         while (i >= hi && j + 1 < D->n_jobs) load(D, j + 1);
     }
@@ -508,7 +508,6 @@ struct SurvivorJob {
 // The survivors of all jobs as one flat range: every thread takes survivors
 // across job boundaries, so one job or many keep the whole grid busy.
 __global__ void k_prefix_hist_q(const BatchDesc* __restrict__ D) {
-    if (D->hist_early) return;  // counted by the consumer
     const uint64_t n = D->n_flat;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -517,7 +516,7 @@ __global__ void k_prefix_hist_q(const BatchDesc* __restrict__ D) {
     S.load(D, job_of_survivor(D, i));
     for (; i < n; i += stride) {
         S.seek(D, i);
-        const uint64_t b = S.keys[i - S.lo] >> S.shift;
+        const uint64_t b = S.bucket(S.keys[i - S.lo]);
         if (b < S.n_buckets) atomicAdd(D->hist + S.bucket_base + b, 1u);
         else atomicOr(D->err, DERR_INTERNAL);
     }
@@ -619,7 +618,7 @@ __global__ void k_scatter_q(const BatchDesc* __restrict__ D) {
         const uint64_t k = i - S.lo;
         const uint64_t key = S.keys[k];
         const uint64_t val = S.vals[k];
-        const uint64_t b = key >> S.shift;
+        const uint64_t b = S.bucket(key);
         if (b >= S.n_buckets) {
             atomicOr(D->err, DERR_INTERNAL);
             continue;
@@ -644,12 +643,11 @@ __device__ __forceinline__ uint32_t job_of_bucket(const BatchDesc* D, uint64_t f
     return lo;
 }
 
-// Buckets of 2..64 keys (nearly all of them: the bits are chosen for about
-// 32 keys a bucket on average, and canonical keys, the smaller of two
-// orientations, are up to twice as dense at the low end of the key space):
-// one warp each, packed (warp_sort32_packed / warp_sort64_packed), small
-// enough in registers for six 256-thread CTAs per SM, so the loads of many
-// buckets are in flight.
+// Buckets of 2..64 keys (nearly all of them: the bits are chosen for 16 to 32
+// keys a bucket, and key_bucket's even shares keep them there): one warp each,
+// packed (warp_sort32_core / warp_sort64_core, from the smallest key's top
+// bits on), small enough in registers for six 256-thread CTAs per SM, so the
+// loads of many buckets are in flight.
 __global__ void __launch_bounds__(256, 6) k_warp_sort_q(const BatchDesc* __restrict__ D) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -665,6 +663,7 @@ __global__ void __launch_bounds__(256, 6) k_warp_sort_q(const BatchDesc* __restr
         if (!packable || n64 == 1 || n64 > 64) {
             // one key, or sorted later in place (k_warp_sort_big_q): the pairs
             // into the result arrays as they are
+            if (n64 > 1 && lane == 0 && !(*(volatile unsigned*)D->err & DERR_SORT_BIG)) atomicOr(D->err, DERR_SORT_BIG);
             for (uint64_t i = lane; i < n64; i += 32) {
                 const ulonglong2 q = src[i];
                 J.res_keys[lo + i] = q.x;
@@ -672,28 +671,25 @@ __global__ void __launch_bounds__(256, 6) k_warp_sort_q(const BatchDesc* __restr
             }
             continue;
         }
-        const int shift = J.key_bits - J.sort_bits;  // the bucket's keys share the bits above shift (<= 58)
+        const bool in = lane < (int)n64, in1 = 32 + lane < (int)n64;
+        const ulonglong2 q0 = in ? src[lane] : make_ulonglong2(~0ull, 0ull);
+        const ulonglong2 q1 = in1 ? src[32 + lane] : make_ulonglong2(~0ull, 0ull);
+        uint64_t k0 = q0.x, v0 = q0.y, k1 = q1.x, v1 = q1.y;
+        // keys have at most 62 bits; the bucket spans less than 2^57 of them
+        const uint64_t kmin = k0 < k1 ? k0 : k1;
+        const uint64_t base = (uint64_t)__reduce_min_sync(kFull, (unsigned)min((unsigned long long)(kmin >> 30), 0xffffffffull)) << 30;
         if (n64 <= 32) {
-            const bool in = lane < (int)n64;
-            const ulonglong2 q = in ? src[lane] : make_ulonglong2(0ull, 0ull);
-            uint64_t k = q.x, v = q.y;
-            warp_sort32_core(k, v, in, lane, shift);
-            if (in) {
-                J.res_keys[lo + lane] = k;
-                J.res_vals[lo + lane] = v;
-            }
+            warp_sort32_core(k0, v0, in, lane, base);
         } else {
-            const bool in1 = 32 + lane < (int)n64;
-            const ulonglong2 q0 = src[lane];
-            const ulonglong2 q1 = in1 ? src[32 + lane] : make_ulonglong2(0ull, 0ull);
-            uint64_t k0 = q0.x, v0 = q0.y, k1 = q1.x, v1 = q1.y;
-            warp_sort64_core(k0, v0, k1, v1, true, in1, lane, shift);
+            warp_sort64_core(k0, v0, k1, v1, in, in1, lane, base);
+        }
+        if (in) {
             J.res_keys[lo + lane] = k0;
             J.res_vals[lo + lane] = v0;
-            if (in1) {
-                J.res_keys[lo + 32 + lane] = k1;
-                J.res_vals[lo + 32 + lane] = v1;
-            }
+        }
+        if (in1) {
+            J.res_keys[lo + 32 + lane] = k1;
+            J.res_vals[lo + 32 + lane] = v1;
         }
     }
 }
@@ -707,6 +703,7 @@ __global__ void __launch_bounds__(256, 2) k_warp_sort_big_q(const BatchDesc* __r
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    if (!(*D->err & DERR_SORT_BIG)) return;
     const uint64_t nb = D->n_buckets;
     const bool all_pack = D->all_packable != 0;
     for (uint64_t base = warp * 32; base < nb; base += n_warps * 32) {
@@ -813,7 +810,7 @@ struct kc_batch_ctx {
     uint64_t* d_cursor = nullptr;
     unsigned long long* d_tiles = nullptr;
     uint64_t buckets_cap = 0, tiles_cap = 0;
-    cudaGraphExec_t sort_graph = nullptr;
+    cudaGraphExec_t sort_graph[2] = {nullptr, nullptr};  // [1]: the consumer has counted the buckets
     // captured consumer launches, one per launch shape
     struct ConsumeGraph {
         bool one;  // one sample in every job
@@ -901,22 +898,27 @@ kc_status ensure_buckets(kc_batch_ctx* b, uint64_t n_buckets) {
     KC_CUDA(cudaMalloc(&b->d_tiles, tiles * 8));
     b->buckets_cap = n;
     b->tiles_cap = tiles;
-    if (b->sort_graph) {  // the graph holds the old capacities
-        cudaGraphExecDestroy(b->sort_graph);
-        b->sort_graph = nullptr;
-    }
+    for (cudaGraphExec_t& g : b->sort_graph)
+        if (g) {  // the graph holds the old capacities
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
     return KC_OK;
 }
 
-// Capture the sort sequence once; it reads everything else from d_desc.
-kc_status capture_sort_graph(kc_batch_ctx* b) {
+// Capture the sort sequence once (early: without the histogram the consumer
+// has taken); it reads everything else from d_desc.
+kc_status capture_sort_graph(kc_batch_ctx* b, int early) {
+    if (b->sort_graph[early]) return KC_OK;
     std::lock_guard<std::mutex> lk(kc::sync_api_mutex());
     cudaGraph_t g = nullptr;
     KC_CUDA(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
     const unsigned grid2 = (unsigned)b->sm_count * 16;  // latency-bound atomics: many threads in flight
     kc::k_plan_q<<<1, 32, 0, b->st>>>(b->d_desc);
-    kc::k_zero_hist_q<<<(unsigned)b->sm_count * 4, 256, 0, b->st>>>(b->d_desc);
-    kc::k_prefix_hist_q<<<grid2, 256, 0, b->st>>>(b->d_desc);
+    if (!early) {
+        kc::k_zero_hist_q<<<(unsigned)b->sm_count * 4, 256, 0, b->st>>>(b->d_desc);
+        kc::k_prefix_hist_q<<<grid2, 256, 0, b->st>>>(b->d_desc);
+    }
     kc::k_scan_tiles_q<<<(unsigned)b->tiles_cap, 1024, 0, b->st>>>(b->d_desc);
     kc::k_scan_top_q<<<1, 1024, 0, b->st>>>(b->d_desc);
     kc::k_scan_apply_q<<<(unsigned)b->tiles_cap, 1024, 0, b->st>>>(b->d_desc);
@@ -925,15 +927,14 @@ kc_status capture_sort_graph(kc_batch_ctx* b) {
     kc::k_warp_sort_big_q<<<(unsigned)b->sm_count * 2, 256, 0, b->st>>>(b->d_desc);
     cudaError_t e = cudaStreamEndCapture(b->st, &g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture(sort)");
-    e = cudaGraphInstantiate(&b->sort_graph, g, 0);
+    e = cudaGraphInstantiate(&b->sort_graph[early], g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate(sort)");
     return KC_OK;
 }
 
-kc_status upload_desc(kc_batch_ctx* b, uint32_t n_jobs, uint32_t n_items, uint64_t n_buckets, int hist_early = 0) {
+kc_status upload_desc(kc_batch_ctx* b, uint32_t n_jobs, uint32_t n_items, uint64_t n_buckets) {
     kc::BatchDesc d{};
-    d.hist_early = hist_early;
     d.pairs = b->d_pairs;
     d.pairs_cap = b->pairs_cap;
     d.buckets_cap = b->buckets_cap;
@@ -1143,7 +1144,8 @@ kc_status kc_batch_create_internal(cudaStream_t st, kc_batch_ctx** out) {
 void kc_batch_destroy_internal(kc_batch_ctx* b) {
     if (!b) return;
     if (b->st) cudaStreamSynchronize(b->st);
-    if (b->sort_graph) cudaGraphExecDestroy(b->sort_graph);
+    for (cudaGraphExec_t g : b->sort_graph)
+        if (g) cudaGraphExecDestroy(g);
     for (auto& g : b->consume_graphs) cudaGraphExecDestroy(g.exec);
     std::lock_guard<std::mutex> lk(kc::sync_api_mutex());
     cudaFree(b->d_desc);
@@ -1364,7 +1366,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         for (int j = 0; j < n; ++j) {
             kc::JobDesc& J = b->jobs[j];
             J.fixed_bits = sort_bits_for(std::min<uint64_t>(hs[j]->res_cap, J.sv_cap), J.key_bits);
-            J.hist_shift = J.key_bits - J.fixed_bits;
             spec_buckets += 1ull << J.fixed_bits;
             J.res_keys = hs[j]->res_keys;
             J.res_vals = hs[j]->res_vals;
@@ -1373,7 +1374,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         uint64_t spec_pairs = 0;
         for (int j = 0; j < n; ++j) spec_pairs += hs[j]->res_cap;
         if ((s = ensure_buckets(b, spec_buckets)) != KC_OK || (s = grow(b->d_pairs, b->pairs_cap, spec_pairs)) != KC_OK ||
-            (!b->sort_graph && (s = capture_sort_graph(b)) != KC_OK)) {
+            (s = capture_sort_graph(b, 1)) != KC_OK) {
             release_work(b, work);
             return s;
         }
@@ -1384,7 +1385,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         }
         KC_CUDA(cudaMemsetAsync(b->d_hist, 0, spec_buckets * 4, st));
     }
-    if ((s = upload_desc(b, (uint32_t)n, n_items, 0, spec ? 1 : 0)) != KC_OK) {
+    if ((s = upload_desc(b, (uint32_t)n, n_items, 0)) != KC_OK) {
         release_work(b, work);
         return s;
     }
@@ -1415,7 +1416,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     err = 0;
     if (spec) {
         t0 = timed ? phase_begin(hs[0], st) : nullptr;
-        KC_CUDA(cudaGraphLaunch(b->sort_graph, st));
+        KC_CUDA(cudaGraphLaunch(b->sort_graph[1], st));
         if (timed) phase_end(hs[0], kSort, t0, st);
         KC_CUDA(cudaMemcpyAsync(&err, b->d_flags + 1, 4, cudaMemcpyDeviceToHost, st));
     }
@@ -1423,7 +1424,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     if (fast)
         for (int j = 0; j < n; ++j) KC_CUDA(cudaMemcpyAsync(&hc[j], hs[j]->ctr, sizeof(kc::DevCounters), cudaMemcpyDeviceToHost, st));
     KC_CUDA(cudaStreamSynchronize(st));
-    for (int j = 0; j < n; ++j) work[j].h->launches += spec ? 11 : 2;
+    for (int j = 0; j < n; ++j) work[j].h->launches += spec ? 9 : 2;
     if (fast) {
         for (int j = 0; j < n; ++j) {
             hs[j]->host_ctr = hc[j];
@@ -1504,12 +1505,12 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     if ((s = ensure_buckets(b, bucket_need)) != KC_OK ||
         (s = grow(b->d_pairs, b->pairs_cap, std::max<uint64_t>(1, pairs_need))) != KC_OK ||
         (s = upload_desc(b, (uint32_t)n, n_items, 0)) != KC_OK ||
-        (!b->sort_graph && (s = capture_sort_graph(b)) != KC_OK)) {
+        (s = capture_sort_graph(b, 0)) != KC_OK) {
         release_work(b, work);
         return s;
     }
     t0 = timed ? phase_begin(hs[0], st) : nullptr;
-    KC_CUDA(cudaGraphLaunch(b->sort_graph, st));
+    KC_CUDA(cudaGraphLaunch(b->sort_graph[0], st));
     if (timed) phase_end(hs[0], kSort, t0, st);
     KC_CUDA(cudaMemcpyAsync(&err, b->d_flags + 1, 4, cudaMemcpyDeviceToHost, st));
     KC_CUDA(cudaStreamSynchronize(st));

@@ -40,6 +40,7 @@ enum : unsigned int {
     DERR_SORT_BUCKET = 8u,     // a sort bucket exceeded the shared-memory tile
     DERR_INTERNAL = 16u,       // a self-check failed (index out of range)
     DERR_SORT_MEDIUM = 32u,    // a sort bucket exceeded one warp's registers
+    DERR_SORT_BIG = 64u,       // a sort bucket is left to the second warp sort (not an error)
 };
 
 // Parameters shared by the extraction passes.
@@ -301,17 +302,32 @@ __device__ __forceinline__ void warp_sort_bucket(uint64_t* __restrict__ keys, ui
     }
 }
 
-// Warp sort of a bucket of n <= 32 (key, value) pairs whose keys all share
-// the bits above bit `shift` (shift <= 59: the bucket is a key-prefix range),
-// one pair per lane (k, v; in = lane < n).  Each lane packs its key's low
-// `shift` bits with its lane index into one word, the bitonic network
-// exchanges that single word (the lane index breaks ties between equal keys),
-// and each value then follows its key through the lane index.  Lanes >= n
-// hold ~0, which sorts last (a packed word equals ~0 only at lane 31, i.e.
-// when n = 32 and no lane is empty).  On return lane i holds the i-th pair.
-__device__ __forceinline__ void warp_sort32_core(uint64_t& k, uint64_t& v, bool in, int lane, int shift) {
-    const uint64_t low_mask = (1ull << shift) - 1ull;
-    uint64_t p = in ? (((k & low_mask) << 5) | (uint64_t)lane) : ~0ull;
+// Bucket of a key among 2^bits buckets in key order.  Canonical keys, the
+// smaller of two orientations, are not uniform: with x the key as a fraction
+// of the key space their density is 2 (1 - x), so plain key prefixes give
+// buckets from twice the mean down to none.  even: the buckets are equal parts
+// of the distribution function x (2 - x), from the key's top 32 bits (the
+// floor of x^2 grows by at most 2 a step, so the map never decreases).
+__device__ __forceinline__ uint32_t key_bucket(uint64_t key, int key_bits, int bits, bool even) {
+    if (!even) return (uint32_t)(key >> (key_bits - bits));
+    const uint32_t x = (uint32_t)(key >> (key_bits - 32));
+    const uint64_t y = 2ull * x - __umulhi(x, x);
+    return (uint32_t)(y >> 32 ? 0xffffffffull : y) >> (32 - bits);
+}
+// Even buckets of 2^bits: the widest (the last) spans 2^(key_bits - bits / 2)
+// keys, which has to leave the 6 index bits of the packed sorts.
+__host__ __device__ __forceinline__ bool even_buckets(int key_bits, int bits) {
+    return key_bits >= 32 && bits >= 1 && key_bits - bits / 2 <= 56;
+}
+
+// Warp sort of a bucket of n <= 32 (key, value) pairs whose keys lie less than
+// 2^58 above `base`, one pair per lane (k, v; in = lane < n).  Each lane packs
+// its key's distance from base with its lane index into one word, the bitonic
+// network exchanges that single word (the lane index breaks ties between equal
+// keys), and each value then follows its key through the lane index.  Lanes >=
+// n hold ~0, which sorts last.  On return lane i holds the i-th pair.
+__device__ __forceinline__ void warp_sort32_core(uint64_t& k, uint64_t& v, bool in, int lane, uint64_t base) {
+    uint64_t p = in ? (((k - base) << 5) | (uint64_t)lane) : ~0ull;
 #pragma unroll
     for (int size = 2; size <= 32; size <<= 1) {
 #pragma unroll
@@ -324,7 +340,7 @@ __device__ __forceinline__ void warp_sort32_core(uint64_t& k, uint64_t& v, bool 
         }
     }
     v = __shfl_sync(0xffffffffu, v, (int)(p & 31ull));
-    k = (k & ~low_mask) | (p >> 5);
+    k = base + (p >> 5);
 }
 
 __device__ __forceinline__ void warp_sort32_packed(uint64_t* __restrict__ keys, uint64_t* __restrict__ vals,
@@ -332,22 +348,21 @@ __device__ __forceinline__ void warp_sort32_packed(uint64_t* __restrict__ keys, 
     const bool in = lane < n;
     uint64_t k = in ? keys[lo + lane] : 0ull;
     uint64_t v = in ? vals[lo + lane] : 0ull;
-    warp_sort32_core(k, v, in, lane, shift);
+    warp_sort32_core(k, v, in, lane, __shfl_sync(0xffffffffu, k, 0) & ~((1ull << shift) - 1ull));
     if (in) {
         keys[lo + lane] = k;
         vals[lo + lane] = v;
     }
 }
 
-// The same for 33..64 pairs (shift <= 58): two packed words per lane, element
+// The same for 33..64 pairs: two packed words per lane, element
 // i = 32 r + lane in register r (k0, v0: element lane; k1, v1: element 32 +
-// lane; n > 32, so lane 0 holds a key); 6 index bits.  Compare-exchanges
+// lane); 6 index bits.  Compare-exchanges
 // across the two registers of a lane (stride 32) need no shuffle.
 __device__ __forceinline__ void warp_sort64_core(uint64_t& k0, uint64_t& v0, uint64_t& k1, uint64_t& v1, bool in0,
-                                                 bool in1, int lane, int shift) {
-    const uint64_t low_mask = (1ull << shift) - 1ull;
-    uint64_t p0 = in0 ? (((k0 & low_mask) << 6) | (uint64_t)lane) : ~0ull;
-    uint64_t p1 = in1 ? (((k1 & low_mask) << 6) | (uint64_t)(32 + lane)) : ~0ull;
+                                                 bool in1, int lane, uint64_t base) {
+    uint64_t p0 = in0 ? (((k0 - base) << 6) | (uint64_t)lane) : ~0ull;
+    uint64_t p1 = in1 ? (((k1 - base) << 6) | (uint64_t)(32 + lane)) : ~0ull;
 #pragma unroll
     for (int size = 2; size <= 64; size <<= 1) {
 #pragma unroll
@@ -371,10 +386,9 @@ __device__ __forceinline__ void warp_sort64_core(uint64_t& k0, uint64_t& v0, uin
     const int i0 = (int)(p0 & 63ull), i1 = (int)(p1 & 63ull);
     const uint64_t a0 = __shfl_sync(0xffffffffu, v0, i0 & 31), b0 = __shfl_sync(0xffffffffu, v1, i0 & 31);
     const uint64_t a1 = __shfl_sync(0xffffffffu, v0, i1 & 31), b1 = __shfl_sync(0xffffffffu, v1, i1 & 31);
-    const uint64_t prefix = __shfl_sync(0xffffffffu, k0, 0) & ~low_mask;
-    k0 = prefix | (p0 >> 6);
+    k0 = base + (p0 >> 6);
     v0 = (i0 >> 5) ? b0 : a0;
-    k1 = prefix | (p1 >> 6);
+    k1 = base + (p1 >> 6);
     v1 = (i1 >> 5) ? b1 : a1;
 }
 
@@ -383,7 +397,7 @@ __device__ __forceinline__ void warp_sort64_packed(uint64_t* __restrict__ keys, 
     const bool in0 = lane < n, in1 = 32 + lane < n;
     uint64_t k0 = in0 ? keys[lo + lane] : 0ull, v0 = in0 ? vals[lo + lane] : 0ull;
     uint64_t k1 = in1 ? keys[lo + 32 + lane] : 0ull, v1 = in1 ? vals[lo + 32 + lane] : 0ull;
-    warp_sort64_core(k0, v0, k1, v1, in0, in1, lane, shift);
+    warp_sort64_core(k0, v0, k1, v1, in0, in1, lane, __shfl_sync(0xffffffffu, k0, 0) & ~((1ull << shift) - 1ull));
     if (in0) {
         keys[lo + lane] = k0;
         vals[lo + lane] = v0;

@@ -168,3 +168,24 @@ def test_blocks_kept_between_jobs(oracle_mod):
             _same(c, oracles[k, i])
     for c in handles.values():
         c.close()
+
+
+def test_sort_buckets_at_both_ends_of_the_key_space():
+    """150,000 keys (even-share sort buckets), thousands of them at the very top and
+    bottom of the canonical keys: ascending, each with its own count."""
+    rng = np.random.default_rng(8)
+    codes, _ = _canonical_31mers(rng, 150_000)
+    top = rng.integers(0, 4, (3000, 31), dtype=np.uint8)
+    top[:, :14], top[:, 17:] = 3, 0  # T...T xyz A...A: both orientations near the top
+    low = rng.integers(0, 4, (3000, 31), dtype=np.uint8)
+    low[:, :24] = 0
+    codes = np.concatenate([codes, top, low])
+    w = np.uint64(2)
+    fwd = np.zeros(len(codes), np.uint64)
+    rev = np.zeros(len(codes), np.uint64)
+    for i in range(31):
+        fwd = (fwd << w) | codes[:, i].astype(np.uint64)
+        rev |= (np.uint64(3) - codes[:, i].astype(np.uint64)) << np.uint64(2 * i)
+    keys, at = np.unique(np.minimum(fwd, rev), return_index=True)
+    repeats = [rng.integers(1, 4, len(keys))]
+    _count(codes[at], keys, repeats, 1, 1)
