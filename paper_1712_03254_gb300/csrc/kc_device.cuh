@@ -149,6 +149,46 @@ __device__ __forceinline__ void rolling_step_k(RollingWindow& r) {
     r.y <<= 2;
 }
 
+// Forward codes of eight windows at a time, cut out of the unit's bases at
+// constant places: f holds the bases from the first of the eight windows on,
+// as 32-bit words, first base on top.  Two funnel shifts and a mask a window
+// (K = k at compile time; K = 0: one 64-bit shift by rc_shift more), where the
+// rolling code takes nine operations.
+struct WindowWords {
+    uint32_t f[6];
+};
+
+__device__ __forceinline__ WindowWords window_words(uint64_t w0, uint64_t w1, uint64_t w2) {
+    return WindowWords{{(uint32_t)(w0 >> 32), (uint32_t)w0, (uint32_t)(w1 >> 32), (uint32_t)w1, (uint32_t)(w2 >> 32),
+                        (uint32_t)w2}};
+}
+
+__device__ __forceinline__ void next_windows(WindowWords& w) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w.f[i] = __funnelshift_l(w.f[i + 1], w.f[i], 16);
+    w.f[5] <<= 16;
+}
+
+// Window J (0..7) of the eight.
+template <int K, int J>
+__device__ __forceinline__ uint64_t forward_code(const WindowWords& w, int rc_shift) {
+    constexpr int drop = K > 16 ? 64 - 2 * K : 0;  // bits after the window in the 64 cut out
+    constexpr int off = 2 * J - drop;
+    uint32_t hi, lo;
+    if (off > 0) {
+        hi = __funnelshift_l(w.f[1], w.f[0], off);
+        lo = __funnelshift_l(w.f[2], w.f[1], off);
+    } else if (off == 0) {
+        hi = w.f[0];
+        lo = w.f[1];
+    } else {
+        hi = w.f[0] >> -off;
+        lo = __funnelshift_r(w.f[1], w.f[0], -off);
+    }
+    if (K > 16) return ((uint64_t)(hi & (0xffffffffu >> drop)) << 32) | lo;
+    return (((uint64_t)hi << 32) | lo) >> rc_shift;
+}
+
 // shl.b32 clamps its shift amount at 32: x << b is 0 for b >= 32.
 __device__ __forceinline__ uint32_t shl_clamped(uint32_t x, uint32_t b) {
     uint32_t r;

@@ -146,10 +146,16 @@ struct SelTable {
 
 __device__ __forceinline__ uint64_t sel_h(uint64_t code) { return code * 0x9e3779b97f4a7c15ull; }
 
+// Bucket and fingerprint of a hash, 8 <= lb <= 32: both from 32-bit shifts.
+__device__ __forceinline__ uint32_t sel_bucket(uint64_t h, int lb) { return (uint32_t)(h >> 32) >> (32 - lb); }
+__device__ __forceinline__ unsigned sel_fp(uint64_t h, int lb) {
+    return __funnelshift_rc((uint32_t)h, (uint32_t)(h >> 32), 32 - lb) | 1u;  // never 0 (0 marks a free slot)
+}
+
 __device__ __forceinline__ void sel_hash(uint64_t code, int lb, uint64_t& bucket, unsigned& fp) {
     const uint64_t h = sel_h(code);
-    bucket = h >> (64 - lb);
-    fp = (unsigned)(h >> (32 - lb)) | 1u;  // never 0 (0 marks a free slot)
+    bucket = sel_bucket(h, lb);
+    fp = sel_fp(h, lb);
 }
 
 __device__ __forceinline__ uint32_t pre_word(uint64_t h) {
@@ -212,9 +218,15 @@ __device__ __forceinline__ bool sel_probe_rest(const SelTable& T, uint64_t b, un
     return false;
 }
 
-// Filter rescan: one lane per 64-base unit; the lane walks its unit's 64
-// window starts with the rolling forward code and probes the selection for
-// four windows at a time (four 16-byte bucket loads in flight).  PRE: one
+// Whether both prefilter bits of h are set in word (in bit 0): the word rotated
+// by the two bit numbers.
+__device__ __forceinline__ uint32_t pre_test(uint32_t word, uint64_t h) {
+    return __funnelshift_r(word, word, (uint32_t)h >> 20) & __funnelshift_r(word, word, (uint32_t)h >> 14);
+}
+
+// Filter rescan: one lane per 64-base unit; the lane cuts the forward codes of
+// its unit's 64 window starts out of the unit's words (forward_code) and probes
+// the selection for four windows at a time (four 16-byte bucket loads in flight).  PRE: one
 // 1024-thread CTA per SM holds the prefilter in shared memory and loads a
 // bucket only for windows that pass it.  Hits go to the unit's hit mask (bit
 // 63 - j: the window starting at base j of the unit, as the valid-window
@@ -223,7 +235,39 @@ __device__ __forceinline__ bool sel_probe_rest(const SelTable& T, uint64_t b, un
 constexpr int kFilterThreads = 256;
 constexpr int kFilterThreadsPre = 1024;
 
-template <bool PRE>
+template <bool PRE, int K, int J0>
+__device__ __forceinline__ void filter_four(const WindowWords& w, unsigned valid, int rc_shift, const SelTable& T,
+                                            const uint32_t* s_pre, unsigned& hits) {
+    const uint64_t code[4] = {forward_code<K, J0>(w, rc_shift), forward_code<K, J0 + 1>(w, rc_shift),
+                              forward_code<K, J0 + 2>(w, rc_shift), forward_code<K, J0 + 3>(w, rc_shift)};
+    uint64_t h[4];
+    bool probe[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        h[t] = sel_h(code[t]);
+        probe[t] = (valid >> (7 - J0 - t)) & 1u;
+        if (PRE && probe[t]) probe[t] = pre_test(s_pre[pre_word(h[t])], h[t]) & 1u;
+    }
+    if (!(probe[0] || probe[1] || probe[2] || probe[3])) return;
+    uint4 q[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        q[t] = make_uint4(0u, 0u, 0u, 0u);
+        if (probe[t]) q[t] = __ldg(reinterpret_cast<const uint4*>(T.fp) + sel_bucket(h[t], T.lb));
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const unsigned fp = sel_fp(h[t], T.lb);
+        const bool match = q[t].x == fp || q[t].y == fp || q[t].z == fp || q[t].w == fp;
+        if (!match && q[t].w == 0u) continue;  // not in the table (skipped windows read as empty)
+        const uint64_t b = sel_bucket(h[t], T.lb);
+        bool hit = match && sel_confirm(T, b, q[t], fp, code[t]);
+        if (!hit && q[t].w != 0u) hit = sel_probe_rest(T, b, fp, code[t]);
+        if (hit) hits |= 1u << (7 - J0 - t);
+    }
+}
+
+template <bool PRE, int K>
 __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE ? 1 : 4)
     k_filter_hits(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw, uint64_t n_units, PassParams p,
                   SelTable T, uint64_t* __restrict__ hitmask, DevCounters* __restrict__ ctr) {
@@ -237,51 +281,21 @@ __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE 
     const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const int kk = 64 - p.rc_shift;  // 2k
-    const uint4* fpw = reinterpret_cast<const uint4*>(T.fp);
     unsigned long long found = 0;
     for (uint64_t base = warp * 32; base < n_units; base += n_warps * 32) {
         const uint64_t u = base + lane;
         const UnitWords uw = load_unit(pw, vw, u, n_units, lane);
         uint64_t vm = uw.v, hm = 0;
-        // forward code of window j, and the bases entering at the next steps
-        uint64_t fwd = uw.w0 >> p.rc_shift;
-        uint64_t x = (uw.w0 << kk) | (uw.w1 >> p.rc_shift);
-        uint64_t y = (uw.w1 << kk) | (uw.w2 >> p.rc_shift);
-        for (int j0 = 0; j0 < 64 && vm; j0 += 4, vm <<= 4) {
-            uint64_t code[4], b[4];
-            unsigned fp[4];
-            bool probe[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                code[t] = fwd;
-                const uint64_t h = sel_h(fwd);
-                b[t] = h >> (64 - T.lb);
-                fp[t] = (unsigned)(h >> (32 - T.lb)) | 1u;
-                probe[t] = (vm >> (63 - t)) & 1ull;
-                if (PRE && probe[t]) {
-                    const uint32_t m = pre_bits(h);
-                    probe[t] = (s_pre[pre_word(h)] & m) == m;
-                }
-                fwd = ((fwd << 2) | (x >> 62)) & p.kmask;
-                x = (x << 2) | (y >> 62);
-                y <<= 2;
+        WindowWords w = window_words(uw.w0, uw.w1, uw.w2);
+        for (int j0 = 0; j0 < 64; j0 += 8, vm <<= 8) {  // eight windows: their bits on top of vm
+            unsigned hits = 0;
+            const unsigned valid = (unsigned)(vm >> 56);
+            if (valid) {
+                filter_four<PRE, K, 0>(w, valid, p.rc_shift, T, s_pre, hits);
+                filter_four<PRE, K, 4>(w, valid, p.rc_shift, T, s_pre, hits);
             }
-            if (!(probe[0] || probe[1] || probe[2] || probe[3])) continue;
-            uint4 q[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                q[t] = make_uint4(0u, 0u, 0u, 0u);
-                if (probe[t]) q[t] = __ldg(fpw + b[t]);
-            }
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const bool match = q[t].x == fp[t] || q[t].y == fp[t] || q[t].z == fp[t] || q[t].w == fp[t];
-                if (!match && q[t].w == 0u) continue;  // not in the table (skipped windows read as empty)
-                bool hit = match && sel_confirm(T, b[t], q[t], fp[t], code[t]);
-                if (!hit && q[t].w != 0u) hit = sel_probe_rest(T, b[t], fp[t], code[t]);
-                if (hit) hm |= 0x8000000000000000ull >> (j0 + t);
-            }
+            hm = (hm << 8) | hits;
+            next_windows(w);
         }
         if (u < n_units) hitmask[u] = hm;
         found += __popcll(hm);
@@ -457,13 +471,13 @@ unsigned grid_of(uint64_t n, unsigned block, unsigned cap) {
     return (unsigned)g;
 }
 
-// Resident CTAs of k_filter_hits<false> per SM: its grid fills the SMs
+// Resident CTAs of k_filter_hits<false, K> per SM: its grid fills the SMs
 // once, no partial second wave.
 int filter_blocks_per_sm() {
     static std::atomic<int> cached{0};
     int v = cached.load(std::memory_order_relaxed);
     if (!v) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_filter_hits<false>, kFilterThreads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_filter_hits<false, 31>, kFilterThreads, 0) !=
                 cudaSuccess ||
             v < 1) {
             cudaGetLastError();
@@ -474,14 +488,15 @@ int filter_blocks_per_sm() {
     return v;
 }
 
-// k_filter_hits<true> takes 192 KiB of dynamic shared memory (set once per
+// k_filter_hits<true, K> takes 192 KiB of dynamic shared memory (set once per
 // device; the value is the same for every caller).
 cudaError_t filter_pre_smem_attr() {
     static std::atomic<int> done[64];
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
-    cudaError_t e = allow_max_dynamic_smem(k_filter_hits<true>);
+    cudaError_t e = allow_max_dynamic_smem(k_filter_hits<true, 31>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_filter_hits<true, 0>);
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(1, std::memory_order_relaxed);
     return e;
 }
@@ -863,15 +878,23 @@ kc_status kc_filter_reads(kc_handle h, const uint64_t* packed_reads, const uint6
             KC_CUDA(kc::filter_pre_smem_attr());
             const unsigned grid = kc::grid_of(n_units, kc::kFilterThreadsPre, (unsigned)h->grid.sm_count);
             cudaEvent_t t0 = phase_begin(h);
-            kc::k_filter_hits<true><<<grid, kc::kFilterThreadsPre, kc::kPreWords * 4, st>>>(
-                pw, vw, n_units, h->params(0), T, hitmask, fctr);
+            if (h->k == 31)  // (the longest k, the one the paper's configurations use)
+                kc::k_filter_hits<true, 31><<<grid, kc::kFilterThreadsPre, kc::kPreWords * 4, st>>>(
+                    pw, vw, n_units, h->params(0), T, hitmask, fctr);
+            else
+                kc::k_filter_hits<true, 0><<<grid, kc::kFilterThreadsPre, kc::kPreWords * 4, st>>>(
+                    pw, vw, n_units, h->params(0), T, hitmask, fctr);
             phase_end(h, kFilterReads, t0);
         } else {
             const unsigned grid = kc::grid_of(n_units, kc::kFilterThreads,
                                               (unsigned)(h->grid.sm_count * kc::filter_blocks_per_sm()));
             cudaEvent_t t0 = phase_begin(h);
-            kc::k_filter_hits<false><<<grid, kc::kFilterThreads, 0, st>>>(pw, vw, n_units, h->params(0), T,
-                                                                         hitmask, fctr);
+            if (h->k == 31)
+                kc::k_filter_hits<false, 31><<<grid, kc::kFilterThreads, 0, st>>>(pw, vw, n_units, h->params(0), T,
+                                                                                 hitmask, fctr);
+            else
+                kc::k_filter_hits<false, 0><<<grid, kc::kFilterThreads, 0, st>>>(pw, vw, n_units, h->params(0), T,
+                                                                                hitmask, fctr);
             phase_end(h, kFilterReads, t0);
         }
         kc::k_read_hits<<<kc::grid_of(n_reads, 256, h->grid.sm_count * 8), 256, 0, st>>>(doff, n_reads, B, n_units,
