@@ -146,8 +146,9 @@ struct kc_ctx {
     // per chunk; a device word for the check's error bits and its pinned copy
     cudaEvent_t ev_chunk[kcapi::kMaxChunks + 1] = {};
     kc::DevCounters* chk_ctr = nullptr;
-    // pinned host words small readbacks land in ([0] the offsets check's
-    // error bits, [1..2] the first and last offset of device offsets)
+    // pinned host words small readbacks land in (kc_add_reads: [0] the offsets
+    // check's error bits, [1..2] the first and last offset of device offsets;
+    // kc_filter_reads: [0..3])
     uint64_t* pinned = nullptr;
     kc::Grid grid;
     int log2_words = 0, log2_slots = 0;
@@ -280,6 +281,8 @@ void free_spill_chunks(kc_handle h);
 uint64_t* spill_alloc(kc_handle h, uint64_t words);  // nullptr when pinning fails
 kc_status check_open(kc_handle h);                   // KC_ERR_ARG / KC_ERR_STATE for null or poisoned
 bool is_device_ptr(const void* p);
+bool is_local_device_ptr(const void* p, int device);
+cudaError_t pinned_words(kc_handle h);
 // Copy a spilled result back to the device and sort it there
 // (KC_ERR_OOM_DEVICE, nothing changed, when it does not fit).
 kc_status resort_spilled(kc_handle h);

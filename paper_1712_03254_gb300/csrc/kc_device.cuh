@@ -175,18 +175,18 @@ __device__ __forceinline__ uint64_t forward_code(const WindowWords& w, int rc_sh
     constexpr int drop = K > 16 ? 64 - 2 * K : 0;  // bits after the window in the 64 cut out
     constexpr int off = 2 * J - drop;
     uint32_t hi, lo;
-    if (off > 0) {
+    if constexpr (off > 0) {
         hi = __funnelshift_l(w.f[1], w.f[0], off);
         lo = __funnelshift_l(w.f[2], w.f[1], off);
-    } else if (off == 0) {
+    } else if constexpr (off == 0) {
         hi = w.f[0];
         lo = w.f[1];
     } else {
         hi = w.f[0] >> -off;
         lo = __funnelshift_r(w.f[1], w.f[0], -off);
     }
-    if (K > 16) return ((uint64_t)(hi & (0xffffffffu >> drop)) << 32) | lo;
-    return (((uint64_t)hi << 32) | lo) >> rc_shift;
+    if constexpr (K > 16) return ((uint64_t)(hi & (0xffffffffu >> drop)) << 32) | lo;
+    else return (((uint64_t)hi << 32) | lo) >> rc_shift;
 }
 
 // shl.b32 clamps its shift amount at 32: x << b is 0 for b >= 32.
@@ -229,18 +229,24 @@ struct UnitWords {
 // Units at or beyond u_end are inactive (zero words); the last active lane
 // loads its successor word itself, since that unit may belong to another
 // lane group or CTA.  All 32 lanes must call this together.
+// n_words: the words there are at pw (a caller's array read in place, without
+// the padding); words past them read as zero.
 __device__ __forceinline__ UnitWords load_unit(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw,
-                                               uint64_t u, uint64_t u_end, int lane) {
+                                               uint64_t u, uint64_t u_end, int lane, uint64_t n_words = ~0ull) {
     UnitWords r{0, 0, 0, 0};
     const bool in = u < u_end;
     if (in) {
         r.v = __ldg(vw + u);
-        const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(pw) + u);
-        r.w0 = p.x;
-        r.w1 = p.y;
+        if (2 * u + 1 < n_words) {
+            const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(pw) + u);
+            r.w0 = p.x;
+            r.w1 = p.y;
+        } else if (2 * u < n_words) {
+            r.w0 = __ldg(pw + 2 * u);
+        }
     }
     r.w2 = __shfl_down_sync(0xffffffffu, r.w0, 1);
-    if (in && (lane == 31 || u + 1 >= u_end)) r.w2 = __ldg(pw + 2 * u + 2);
+    if (in && (lane == 31 || u + 1 >= u_end)) r.w2 = 2 * u + 2 < n_words ? __ldg(pw + 2 * u + 2) : 0ull;
     return r;
 }
 

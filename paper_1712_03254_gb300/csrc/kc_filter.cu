@@ -58,16 +58,29 @@ struct HitPred {
     __device__ bool operator()(uint64_t i) const { return hits[i] != 0u; }
 };
 
+// Sum of a value over the CTA's THREADS threads, in thread 0.
+template <int THREADS>
+__device__ __forceinline__ uint32_t tile_sum(uint32_t v) {
+    __shared__ uint32_t s_sum[THREADS / 32];
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < THREADS / 32; ++w) v += s_sum[w];
+    return v;
+}
+
 template <typename Pred>
 __global__ void __launch_bounds__(kTileThreads) k_tile_count(Pred pred, uint64_t n, uint32_t* __restrict__ counts) {
     const uint64_t base = (uint64_t)blockIdx.x * kTileItems;
-    int total = 0;
-#pragma unroll 4
+    uint32_t mine = 0;
+#pragma unroll 8
     for (int r = 0; r < kTileRounds; ++r) {
         const uint64_t i = base + (uint64_t)r * kTileThreads + threadIdx.x;
-        total += __syncthreads_count(i < n && pred(i));
+        mine += i < n && pred(i);
     }
-    if (threadIdx.x == 0) counts[blockIdx.x] = (uint32_t)total;
+    const uint32_t total = tile_sum<kTileThreads>(mine);
+    if (threadIdx.x == 0) counts[blockIdx.x] = total;
 }
 
 // Writer for the selection: key and packed counts.
@@ -88,32 +101,35 @@ struct IndexWrite {
     __device__ void operator()(uint64_t i, uint64_t pos) const { out[pos] = i; }
 };
 
+// Each warp a row of kTileRounds * 32 items of the tile: the ballots of its
+// rounds stay in its lanes (lane r: round r), one barrier gives the warps their
+// output starts, then the kept items are written in order.  (A barrier pair
+// and a prefix a round took 40 us where this takes 37 for 5.5 M keys, 151 k
+// kept, and 13 against 5 for the candidates of 600 k reads.)
 template <typename Pred, typename Write>
 __global__ void __launch_bounds__(kTileThreads) k_tile_write(Pred pred, Write write, uint64_t n,
                                                              const uint64_t* __restrict__ starts) {
-    __shared__ uint32_t warp_base[kTileThreads / 32 + 1];
+    __shared__ uint32_t warp_n[kTileThreads / 32];
+    static_assert(kTileRounds <= 32, "a lane per round");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * kTileItems;
-    uint64_t out = starts[blockIdx.x];
+    const uint64_t base = (uint64_t)blockIdx.x * kTileItems + (uint64_t)warp * (kTileRounds * 32) + lane;
+    unsigned mine = 0;
+#pragma unroll 8
     for (int r = 0; r < kTileRounds; ++r) {
-        const uint64_t i = base + (uint64_t)r * kTileThreads + threadIdx.x;
-        const bool keep = i < n && pred(i);
-        const unsigned ballot = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) warp_base[warp] = (uint32_t)__popc(ballot);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t acc = 0;
-            for (int w = 0; w < kTileThreads / 32; ++w) {
-                const uint32_t c = warp_base[w];
-                warp_base[w] = acc;
-                acc += c;
-            }
-            warp_base[kTileThreads / 32] = acc;
-        }
-        __syncthreads();
-        if (keep) write(i, out + warp_base[warp] + (uint32_t)__popc(ballot & ((1u << lane) - 1u)));
-        out += warp_base[kTileThreads / 32];
-        __syncthreads();  // warp_base is rewritten by the next round
+        const uint64_t i = base + r * 32;
+        const unsigned ballot = __ballot_sync(0xffffffffu, i < n && pred(i));
+        if (lane == r) mine = ballot;
+    }
+    const uint32_t total = __reduce_add_sync(0xffffffffu, (unsigned)__popc(mine));
+    if (lane == 0) warp_n[warp] = total;
+    __syncthreads();
+    uint64_t out = starts[blockIdx.x];
+    for (int w = 0; w < warp; ++w) out += warp_n[w];
+    if (total == 0) return;
+    for (int r = 0; r < kTileRounds; ++r) {
+        const unsigned ballot = __shfl_sync(0xffffffffu, mine, r);
+        if ((ballot >> lane) & 1u) write(base + r * 32, out + (uint32_t)__popc(ballot & ((1u << lane) - 1u)));
+        out += __popc(ballot);
     }
 }
 
@@ -269,8 +285,8 @@ __device__ __forceinline__ void filter_four(const WindowWords& w, unsigned valid
 
 template <bool PRE, int K>
 __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE ? 1 : 4)
-    k_filter_hits(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw, uint64_t n_units, PassParams p,
-                  SelTable T, uint64_t* __restrict__ hitmask, DevCounters* __restrict__ ctr) {
+    k_filter_hits(const uint64_t* __restrict__ pw, uint64_t n_words, const uint64_t* __restrict__ vw, uint64_t n_units,
+                  PassParams p, SelTable T, uint64_t* __restrict__ hitmask, DevCounters* __restrict__ ctr) {
     extern __shared__ uint4 s_pre4[];
     const uint32_t* s_pre = reinterpret_cast<const uint32_t*>(s_pre4);
     if (PRE) {
@@ -284,7 +300,7 @@ __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE 
     unsigned long long found = 0;
     for (uint64_t base = warp * 32; base < n_units; base += n_warps * 32) {
         const uint64_t u = base + lane;
-        const UnitWords uw = load_unit(pw, vw, u, n_units, lane);
+        const UnitWords uw = load_unit(pw, vw, u, n_units, lane, n_words);
         uint64_t vm = uw.v, hm = 0;
         WindowWords w = window_words(uw.w0, uw.w1, uw.w2);
         for (int j0 = 0; j0 < 64; j0 += 8, vm <<= 8) {  // eight windows: their bits on top of vm
@@ -305,26 +321,39 @@ __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE 
 }
 
 // hits[r] = hit-mask bits inside read r's bases (local positions o0 .. o1 - 1;
-// the mask has bits only at valid window starts, which lie inside reads).
-// Thread per read.
-__global__ void k_read_hits(const uint64_t* __restrict__ offsets, uint64_t n_reads, uint64_t base,
-                            uint64_t n_units, const uint64_t* __restrict__ hitmask, unsigned int* __restrict__ hits) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_reads; r += stride) {
-        const uint64_t o0 = offsets[r] - base, o1 = offsets[r + 1] - base;
+// the mask has bits only at valid window starts, which lie inside reads), and
+// per tile of kTileItems reads how many of them have hits (the compaction's
+// counts).  Thread per read, CTA per tile.
+constexpr int kReadThreads = 1024;
+
+__global__ void __launch_bounds__(kReadThreads) k_read_hits(const uint64_t* __restrict__ offsets, uint64_t n_reads,
+                                                            uint64_t base, uint64_t n_units,
+                                                            const uint64_t* __restrict__ hitmask,
+                                                            unsigned int* __restrict__ hits,
+                                                            uint32_t* __restrict__ counts) {
+    uint32_t mine = 0;
+#pragma unroll 4
+    for (int round = 0; round < (int)(kTileItems / kReadThreads); ++round) {
+        const uint64_t r = (uint64_t)blockIdx.x * kTileItems + (uint64_t)round * kReadThreads + threadIdx.x;
         unsigned n = 0;
-        if (o1 > o0) {
-            const uint64_t u0 = o0 >> 6, u1 = (o1 - 1) >> 6;
-            for (uint64_t u = u0; u <= u1 && u < n_units; ++u) {
-                uint64_t m = hitmask[u];
-                if (u == u0) m &= ~0ull >> (o0 & 63);                 // from base o0 on
-                const int e = (int)((o1 - 1) & 63);
-                if (u == u1 && e < 63) m &= ~(~0ull >> (e + 1));      // up to base o1 - 1
-                n += (unsigned)__popcll(m);
+        if (r < n_reads) {
+            const uint64_t o0 = offsets[r] - base, o1 = offsets[r + 1] - base;
+            if (o1 > o0) {
+                const uint64_t u0 = o0 >> 6, u1 = (o1 - 1) >> 6;
+                for (uint64_t u = u0; u <= u1 && u < n_units; ++u) {
+                    uint64_t m = hitmask[u];
+                    if (u == u0) m &= ~0ull >> (o0 & 63);                 // from base o0 on
+                    const int e = (int)((o1 - 1) & 63);
+                    if (u == u1 && e < 63) m &= ~(~0ull >> (e + 1));      // up to base o1 - 1
+                    n += (unsigned)__popcll(m);
+                }
             }
+            hits[r] = n;
         }
-        hits[r] = n;
+        mine += n != 0u;
     }
+    const uint32_t total = tile_sum<kReadThreads>(mine);
+    if (threadIdx.x == 0) counts[blockIdx.x] = total;
 }
 
 __global__ void k_items16(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ vals, uint64_t n,
@@ -554,39 +583,44 @@ kc_status device_result(kc_handle h, const char* who) {
     return s;
 }
 
+// The tiles of an ordered compaction of n items: per tile its kept items and
+// the output start (one block; starts[n_tiles] is the total).
+struct Tiles {
+    uint64_t n = 0;
+    uint64_t *starts = nullptr, *cursor = nullptr;
+    uint32_t* counts = nullptr;
+    cudaError_t take(uint64_t items, cudaStream_t st) {
+        n = std::max<uint64_t>(1, (items + kc::kTileItems - 1) / kc::kTileItems);
+        cudaError_t e = cudaMallocAsync(&starts, (n + 1) * 8 + n * 12, st);
+        if (e != cudaSuccess) return e;
+        cursor = starts + n + 1;
+        counts = reinterpret_cast<uint32_t*>(cursor + n);
+        return cudaSuccess;
+    }
+    void leave(cudaStream_t st) {
+        if (starts) cudaFreeAsync(starts, st);
+        starts = nullptr;
+    }
+};
+
 // Ordered compaction of n items into the writer's arrays; *kept = how many.
 template <typename Pred, typename Write>
-kc_status compact_ordered(kc_handle h, Pred pred, Write write, uint64_t n, uint64_t* kept, bool do_write) {
+kc_status compact_ordered(kc_handle h, Pred pred, Write write, uint64_t n, uint64_t* kept) {
     cudaStream_t st = h->stream;
-    const uint64_t n_tiles = std::max<uint64_t>(1, (n + kc::kTileItems - 1) / kc::kTileItems);
-    uint32_t* counts = nullptr;
-    uint64_t *starts = nullptr, *cursor = nullptr;
-    cudaError_t e;
-    if ((e = cudaMallocAsync(&counts, n_tiles * 4, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&starts, (n_tiles + 1) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&cursor, n_tiles * 8, st)) != cudaSuccess) {
-        if (counts) cudaFreeAsync(counts, st);
-        if (starts) cudaFreeAsync(starts, st);
-        return cuda_fail(e, "cudaMallocAsync(compaction tiles)");
-    }
-    kc::k_tile_count<Pred><<<(unsigned)n_tiles, kc::kTileThreads, 0, st>>>(pred, n, counts);
-    e = kc::launch_scan(counts, n_tiles, starts, cursor, st);
+    Tiles t;
+    cudaError_t e = t.take(n, st);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(compaction tiles)");
+    kc::k_tile_count<Pred><<<(unsigned)t.n, kc::kTileThreads, 0, st>>>(pred, n, t.counts);
+    e = kc::launch_scan(t.counts, t.n, t.starts, t.cursor, st);
     if (e != cudaSuccess) {
-        cudaFreeAsync(counts, st);
-        cudaFreeAsync(starts, st);
-        cudaFreeAsync(cursor, st);
+        t.leave(st);
         return cuda_fail(e, "tile scan");
     }
-    h->launches += 2;
-    if (do_write) {
-        kc::k_tile_write<Pred, Write><<<(unsigned)n_tiles, kc::kTileThreads, 0, st>>>(pred, write, n, starts);
-        h->launches += 1;
-    }
+    kc::k_tile_write<Pred, Write><<<(unsigned)t.n, kc::kTileThreads, 0, st>>>(pred, write, n, t.starts);
+    h->launches += 3;
     KC_LAUNCHED("ordered compaction launches");
-    KC_CUDA(cudaMemcpyAsync(kept, starts + n_tiles, 8, cudaMemcpyDeviceToHost, st));
-    cudaFreeAsync(counts, st);
-    cudaFreeAsync(starts, st);
-    cudaFreeAsync(cursor, st);
+    KC_CUDA(cudaMemcpyAsync(kept, t.starts + t.n, 8, cudaMemcpyDeviceToHost, st));
+    t.leave(st);
     KC_CUDA(cudaStreamSynchronize(st));
     return KC_OK;
 }
@@ -687,7 +721,7 @@ static kc_status build_stems(kc_handle h) {
         KC_CUDA(cudaMallocAsync(&starts, std::max<uint64_t>(1, n_rec) * 8, st));
         uint64_t n_items = 0;
         t0 = phase_begin(h);
-        s = compact_ordered(h, kc::StemStartPred{sk}, kc::IndexWrite{starts}, n_rec, &n_items, true);
+        s = compact_ordered(h, kc::StemStartPred{sk}, kc::IndexWrite{starts}, n_rec, &n_items);
         if (s != KC_OK) return s;
         KC_CUDA(cudaMallocAsync(&h->stem_items, std::max<uint64_t>(1, n_items) * sizeof(kc_stem_item), st));
         if (n_items)
@@ -738,21 +772,34 @@ kc_status kc_filter_select(kc_handle h, const kc_filter_spec* spec, uint64_t* n_
     uint64_t kept = 0;
     cudaEvent_t t0 = phase_begin(h);
     // count first, then allocate exactly and write
-    s = compact_ordered(h, pred, kc::SelectWrite{}, n, &kept, false);
-    if (s != KC_OK) return s;
+    Tiles tiles;
+    cudaError_t e = tiles.take(n, st);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(compaction tiles)");
+    kc::k_tile_count<kc::SelectPred><<<(unsigned)tiles.n, kc::kTileThreads, 0, st>>>(pred, n, tiles.counts);
+    if ((e = kc::launch_scan(tiles.counts, tiles.n, tiles.starts, tiles.cursor, st)) != cudaSuccess) {
+        tiles.leave(st);
+        return cuda_fail(e, "tile scan");
+    }
+    h->launches += 2;
+    KC_LAUNCHED("selection count launches");
+    KC_CUDA(cudaMemcpyAsync(&kept, tiles.starts + tiles.n, 8, cudaMemcpyDeviceToHost, st));
+    KC_CUDA(cudaStreamSynchronize(st));
     const uint64_t cap = std::max<uint64_t>(1, kept);
     // buckets of four slots for both orientations of every key, at most a
     // quarter full: about 2 % of the buckets are full and make a miss probe on
     int lb = 8;
     while ((1ull << lb) < 2 * kept) ++lb;
-    if (lb > 32) return fail(KC_ERR_CAPACITY, "selection larger than 2^31 keys");
+    if (lb > 32) {
+        tiles.leave(st);
+        return fail(KC_ERR_CAPACITY, "selection larger than 2^31 keys");
+    }
     const uint64_t n_buckets = 1ull << lb;
-    cudaError_t e;
     const bool pre = 2 * kept <= kc::kPreMaxEntries;
     const uint64_t table_bytes = n_buckets * kSelBucketBytes + (pre ? kc::kPreWords * 4ull : 0);
     if ((e = cudaMallocAsync(&h->sel_keys, cap * 8, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&h->sel_vals, cap * 8, st)) != cudaSuccess ||
         (e = cudaMallocAsync(&h->sel_table, table_bytes, st)) != cudaSuccess) {
+        tiles.leave(st);
         free_selection(h);
         return cuda_fail(e, "cudaMallocAsync(selection)");
     }
@@ -763,17 +810,14 @@ kc_status kc_filter_select(kc_handle h, const kc_filter_spec* spec, uint64_t* n_
         KC_CUDA(cudaMemsetAsync(reinterpret_cast<char*>(h->sel_table) + n_buckets * kSelBucketBytes, 0,
                                 kc::kPreWords * 4ull, st));
     if (kept) {
-        s = compact_ordered(h, pred, kc::SelectWrite{h->res_keys, h->res_vals, h->sel_keys, h->sel_vals}, n, &kept,
-                            true);
-        if (s != KC_OK) {
-            free_selection(h);
-            return s;
-        }
+        kc::k_tile_write<kc::SelectPred, kc::SelectWrite><<<(unsigned)tiles.n, kc::kTileThreads, 0, st>>>(
+            pred, kc::SelectWrite{h->res_keys, h->res_vals, h->sel_keys, h->sel_vals}, n, tiles.starts);
         kc::k_sel_insert<<<kc::grid_of(kept, 256, h->grid.sm_count * 8), 256, 0, st>>>(
             h->sel_keys, kept, sel_table_of(h), h->params(0), h->ctr);
-        h->launches += 1;
-        KC_LAUNCHED("selection table launch");
+        h->launches += 2;
+        KC_LAUNCHED("selection table launches");
     }
+    tiles.leave(st);
     phase_end(h, kFilterSelect, t0);
     s = read_counters(h);
     if (s != KC_OK) return s;
@@ -815,12 +859,12 @@ kc_status kc_filter_reads(kc_handle h, const uint64_t* packed_reads, const uint6
     const bool off_dev = is_device_ptr(offsets);
     uint64_t b0, b1;
     if (off_dev) {
-        uint64_t ends[2];
-        KC_CUDA(cudaMemcpyAsync(&ends[0], offsets, 8, cudaMemcpyDeviceToHost, st));
-        KC_CUDA(cudaMemcpyAsync(&ends[1], offsets + n_reads, 8, cudaMemcpyDeviceToHost, st));
+        KC_CUDA(pinned_words(h));
+        KC_CUDA(cudaMemcpyAsync(h->pinned + 1, offsets, 8, cudaMemcpyDeviceToHost, st));
+        KC_CUDA(cudaMemcpyAsync(h->pinned + 2, offsets + n_reads, 8, cudaMemcpyDeviceToHost, st));
         KC_CUDA(cudaStreamSynchronize(st));
-        b0 = ends[0];
-        b1 = ends[1];
+        b0 = h->pinned[1];
+        b1 = h->pinned[2];
     } else {
         b0 = offsets[0];
         b1 = offsets[n_reads];
@@ -836,85 +880,108 @@ kc_status kc_filter_reads(kc_handle h, const uint64_t* packed_reads, const uint6
     const uint64_t B = (b0 / 64) * 64;
     const uint64_t n_local = b1 - B;
     const uint64_t n_units = std::max<uint64_t>(1, (n_local + 63) / 64);
-    const uint64_t n_pwords_src = (n_local + 31) / 32;
+    const bool any = b1 > b0;  // else no word is read
+    const uint64_t n_pwords_src = any ? (n_local + 31) / 32 : 0;
     const uint64_t n_pwords = 2 * n_units + 2;
 
-    uint64_t *pw = nullptr, *vw = nullptr, *nm = nullptr, *bd = nullptr, *doff = nullptr, *dcand = nullptr;
-    uint32_t* dhits = hits_dev ? hits : nullptr;
-    uint64_t* hitmask = nullptr;
-    kc::DevCounters* fctr = nullptr;
+    // Device arrays are read where they are (the packed words where 16-byte
+    // loads can reach them), host ones copied; everything of this call lies in
+    // one block.
+    const uint64_t* const src_pw = any ? packed_reads + B / 32 : nullptr;
+    const bool own_pw = !any || !is_local_device_ptr(packed_reads, h->device) || reinterpret_cast<uintptr_t>(src_pw) % 16 != 0;
+    const bool own_nm = !any || !is_local_device_ptr(n_mask, h->device);
+    const bool own_off = !is_local_device_ptr(offsets, h->device);
+    const bool own_cand = candidates && !cand_dev;
+    char* block = nullptr;
+    uint64_t* hmask = nullptr;  // pinned words the call's small readbacks land in
+    Tiles tiles;
     auto release = [&]() {
-        for (void* q : {(void*)pw, (void*)vw, (void*)nm, (void*)bd, (void*)doff, (void*)fctr, (void*)hitmask})
-            if (q) cudaFreeAsync(q, st);
-        if (dhits && !hits_dev) cudaFreeAsync(dhits, st);
-        if (dcand && !cand_dev) cudaFreeAsync(dcand, st);
+        if (block) cudaFreeAsync(block, st);
+        tiles.leave(st);
     };
+    const size_t bytes = (own_pw ? n_pwords * 8 : 0) + n_units * 8 * (3 + (own_nm ? 1 : 0)) + (own_off ? (n_reads + 1) * 8 : 0) +
+                         (own_cand ? n_reads * 8 : 0) + (hits_dev ? 0 : n_reads * 4) + sizeof(kc::DevCounters) + 16;
     cudaError_t e = cudaSuccess;
-    if ((e = cudaMallocAsync(&pw, n_pwords * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&vw, n_units * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&nm, n_units * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&bd, n_units * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&doff, (n_reads + 1) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&fctr, sizeof(kc::DevCounters), st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&hitmask, n_units * 8, st)) != cudaSuccess ||
-        (!hits_dev && (e = cudaMallocAsync(&dhits, n_reads * 4, st)) != cudaSuccess) ||
-        (candidates && !cand_dev && (e = cudaMallocAsync(&dcand, n_reads * 8, st)) != cudaSuccess)) {
+    if ((e = cudaMallocAsync(&block, bytes, st)) != cudaSuccess || (e = tiles.take(n_reads, st)) != cudaSuccess ||
+        (e = pinned_words(h)) != cudaSuccess) {
         release();
         return cuda_fail(e, "cudaMallocAsync(filter reads)");
     }
-    if (cand_dev) dcand = candidates;
+    hmask = h->pinned;
+    char* q = block;
+    const auto part = [&](size_t n) {
+        char* p = q;
+        q += n;
+        return p;
+    };
+    kc::DevCounters* fctr = reinterpret_cast<kc::DevCounters*>(part(sizeof(kc::DevCounters)));
+    uint64_t* bd = reinterpret_cast<uint64_t*>(part(n_units * 8));  // (cleared with the counters)
+    uint64_t* pw = own_pw ? reinterpret_cast<uint64_t*>(part(n_pwords * 8 + (n_units % 2 ? 8 : 0))) : nullptr;
+    if (pw && reinterpret_cast<uintptr_t>(pw) % 16 != 0) ++pw;  // 16-byte loads
+    uint64_t* vw = reinterpret_cast<uint64_t*>(part(n_units * 8));
+    uint64_t* hitmask = reinterpret_cast<uint64_t*>(part(n_units * 8));
+    uint64_t* nm = own_nm ? reinterpret_cast<uint64_t*>(part(n_units * 8)) : nullptr;
+    uint64_t* doff = own_off ? reinterpret_cast<uint64_t*>(part((n_reads + 1) * 8)) : nullptr;
+    uint64_t* dcand = own_cand ? reinterpret_cast<uint64_t*>(part(n_reads * 8)) : candidates;
+    uint32_t* dhits = hits_dev ? hits : reinterpret_cast<uint32_t*>(part(n_reads * 4));
     auto run = [&]() -> kc_status {
-        KC_CUDA(cudaMemsetAsync(fctr, 0, sizeof(kc::DevCounters), st));
-        KC_CUDA(cudaMemsetAsync(pw, 0, n_pwords * 8, st));
-        KC_CUDA(cudaMemsetAsync(nm, 0, n_units * 8, st));
-        if (n_pwords_src) KC_CUDA(cudaMemcpyAsync(pw, packed_reads + B / 32, n_pwords_src * 8, cudaMemcpyDefault, st));
-        if (n_local) KC_CUDA(cudaMemcpyAsync(nm, n_mask + B / 64, ((n_local + 63) / 64) * 8, cudaMemcpyDefault, st));
-        KC_CUDA(cudaMemcpyAsync(doff, offsets, (n_reads + 1) * 8, cudaMemcpyDefault, st));
-        KC_CUDA(cudaMemsetAsync(bd, 0, n_units * 8, st));
-        kc::launch_mark_read_starts(doff, n_reads, B, n_local, bd, fctr, st);
-        kc::launch_build_valid(nm, bd, n_units, b0 - B, n_local, h->k, vw, fctr, h->grid, st);
+        KC_CUDA(cudaMemsetAsync(fctr, 0, sizeof(kc::DevCounters) + n_units * 8, st));
+        if (own_pw) {
+            KC_CUDA(cudaMemsetAsync(pw + n_pwords_src, 0, (n_pwords - n_pwords_src) * 8, st));
+            if (n_pwords_src) KC_CUDA(cudaMemcpyAsync(pw, src_pw, n_pwords_src * 8, cudaMemcpyDefault, st));
+        }
+        if (own_nm) {
+            if (any) KC_CUDA(cudaMemcpyAsync(nm, n_mask + B / 64, n_units * 8, cudaMemcpyDefault, st));
+            else KC_CUDA(cudaMemsetAsync(nm, 0, n_units * 8, st));
+        }
+        if (own_off) KC_CUDA(cudaMemcpyAsync(doff, offsets, (n_reads + 1) * 8, cudaMemcpyDefault, st));
+        const uint64_t* off_in = own_off ? doff : offsets;
+        const uint64_t* pw_in = own_pw ? pw : src_pw;
+        const uint64_t n_words = own_pw ? n_pwords : n_pwords_src;
+        kc::launch_mark_read_starts(off_in, n_reads, B, n_local, bd, fctr, st);
+        kc::launch_build_valid(own_nm ? nm : n_mask + B / 64, bd, n_units, b0 - B, n_local, h->k, vw, fctr, h->grid, st);
         const kc::SelTable T = sel_table_of(h);
+        const auto rescan = [&](auto kern, unsigned grid, int threads, size_t smem) {
+            cudaEvent_t t0 = phase_begin(h);
+            kern<<<grid, threads, smem, st>>>(pw_in, n_words, vw, n_units, h->params(0), T, hitmask, fctr);
+            phase_end(h, kFilterReads, t0);
+        };
+        // k = 31 (the longest k, the one the paper's configurations use): constant shifts
         if (T.pre) {
             KC_CUDA(kc::filter_pre_smem_attr());
             const unsigned grid = kc::grid_of(n_units, kc::kFilterThreadsPre, (unsigned)h->grid.sm_count);
-            cudaEvent_t t0 = phase_begin(h);
-            if (h->k == 31)  // (the longest k, the one the paper's configurations use)
-                kc::k_filter_hits<true, 31><<<grid, kc::kFilterThreadsPre, kc::kPreWords * 4, st>>>(
-                    pw, vw, n_units, h->params(0), T, hitmask, fctr);
-            else
-                kc::k_filter_hits<true, 0><<<grid, kc::kFilterThreadsPre, kc::kPreWords * 4, st>>>(
-                    pw, vw, n_units, h->params(0), T, hitmask, fctr);
-            phase_end(h, kFilterReads, t0);
+            if (h->k == 31) rescan(kc::k_filter_hits<true, 31>, grid, kc::kFilterThreadsPre, kc::kPreWords * 4);
+            else rescan(kc::k_filter_hits<true, 0>, grid, kc::kFilterThreadsPre, kc::kPreWords * 4);
         } else {
             const unsigned grid = kc::grid_of(n_units, kc::kFilterThreads,
                                               (unsigned)(h->grid.sm_count * kc::filter_blocks_per_sm()));
-            cudaEvent_t t0 = phase_begin(h);
-            if (h->k == 31)
-                kc::k_filter_hits<false, 31><<<grid, kc::kFilterThreads, 0, st>>>(pw, vw, n_units, h->params(0), T,
-                                                                                 hitmask, fctr);
-            else
-                kc::k_filter_hits<false, 0><<<grid, kc::kFilterThreads, 0, st>>>(pw, vw, n_units, h->params(0), T,
-                                                                                hitmask, fctr);
-            phase_end(h, kFilterReads, t0);
+            if (h->k == 31) rescan(kc::k_filter_hits<false, 31>, grid, kc::kFilterThreads, 0);
+            else rescan(kc::k_filter_hits<false, 0>, grid, kc::kFilterThreads, 0);
         }
-        kc::k_read_hits<<<kc::grid_of(n_reads, 256, h->grid.sm_count * 8), 256, 0, st>>>(doff, n_reads, B, n_units,
-                                                                                         hitmask, dhits);
+        kc::k_read_hits<<<(unsigned)tiles.n, kc::kReadThreads, 0, st>>>(off_in, n_reads, B, n_units, hitmask, dhits, tiles.counts);
         h->launches += 4;
         KC_LAUNCHED("filter rescan launches");
-        kc::DevCounters c{};
-        KC_CUDA(cudaMemcpyAsync(&c, fctr, sizeof(c), cudaMemcpyDeviceToHost, st));
+        KC_CUDA(kc::launch_scan(tiles.counts, tiles.n, tiles.starts, tiles.cursor, st));
+        h->launches += 1;
+        if (candidates) {
+            kc::k_tile_write<kc::HitPred, kc::IndexWrite><<<(unsigned)tiles.n, kc::kTileThreads, 0, st>>>(
+                kc::HitPred{dhits}, kc::IndexWrite{dcand}, n_reads, tiles.starts);
+            h->launches += 1;
+        }
+        KC_LAUNCHED("candidate list launches");
+        // one readback: windows, hits and error bits, the number of candidates
+        KC_CUDA(cudaMemcpyAsync(hmask, fctr, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+        KC_CUDA(cudaMemcpyAsync(hmask + 2, &fctr->err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+        KC_CUDA(cudaMemcpyAsync(hmask + 3, tiles.starts + tiles.n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
         KC_CUDA(cudaStreamSynchronize(st));
-        if (c.err & kc::DERR_OFFSETS) return fail(KC_ERR_ARG, "read offsets decrease or start before the first word");
-        h->filter_windows += c.windows;
-        h->filter_hits += c.candidates;
-        uint64_t n_cand = 0;
-        kc_status s2 = compact_ordered(h, kc::HitPred{dhits}, kc::IndexWrite{dcand}, n_reads, &n_cand,
-                                       candidates != nullptr);
-        if (s2 != KC_OK) return s2;
+        const unsigned err = *reinterpret_cast<unsigned*>(hmask + 2);
+        const uint64_t n_cand = hmask[3];
+        if (err & kc::DERR_OFFSETS) return fail(KC_ERR_ARG, "read offsets decrease or start before the first word");
+        h->filter_windows += hmask[0];
+        h->filter_hits += hmask[1];
         if (!hits_dev) KC_CUDA(cudaMemcpyAsync(hits, dhits, n_reads * 4, cudaMemcpyDeviceToHost, st));
-        if (candidates && !cand_dev && n_cand)
-            KC_CUDA(cudaMemcpyAsync(candidates, dcand, n_cand * 8, cudaMemcpyDeviceToHost, st));
-        KC_CUDA(cudaStreamSynchronize(st));
+        if (own_cand && n_cand) KC_CUDA(cudaMemcpyAsync(candidates, dcand, n_cand * 8, cudaMemcpyDeviceToHost, st));
+        if (!hits_dev || (own_cand && n_cand)) KC_CUDA(cudaStreamSynchronize(st));
         phase_collect(h);
         if (n_candidates) *n_candidates = n_cand;
         return KC_OK;

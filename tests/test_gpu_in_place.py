@@ -1,0 +1,77 @@
+"""Reads given in device memory are read where they are: without the padding of
+the library's own copy, at any 8-byte alignment, up to the last base exactly."""
+import numpy as np
+import pytest
+
+import synth
+import paper_1712_03254_gb300 as kc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kc.lib()
+
+
+def _on_device(a, shift):
+    """The array on the device, `shift` words behind a 16-byte boundary, with no word after it."""
+    import torch
+
+    t = torch.empty(len(a) + shift, dtype=torch.int64, device="cuda")
+    t[shift:] = torch.from_numpy(np.ascontiguousarray(a).view(np.int64))
+    return t[shift:]
+
+
+@pytest.mark.parametrize("k", [5, 16, 17, 25, 31])
+@pytest.mark.parametrize("tail", [1, 31, 32, 33, 63, 64])
+def test_filter_reads_in_place(oracle_mod, k, tail):
+    """Hits of device reads (aligned and not) are those of host reads, and their
+    sum is the selected keys' counts; the last unit holds `tail` bases."""
+    import torch
+
+    g = synth.genome(41, 3_000 if k > 5 else 120)
+    normal = synth.reads(42, g, 400, 60, 100, 0.01, 0.002)
+    rs = synth.reads(43, synth.mutate(44, g, 0.02, 0.0), 400, 60, 100, 0.01, 0.002)
+    keep = rs.n_reads
+    cut = int(rs.offsets[-1]) - (int(rs.offsets[-1]) - tail) % 64  # bases = tail mod 64
+    rs = synth.ReadSet(rs.ascii[:cut], np.minimum(rs.offsets, np.uint64(cut)))
+    c = kc.KmerCounter(k, 2, 1 << 18, 4, 2)
+    c.add_readset(0, normal)
+    c.add_readset(1, rs)
+    c.finalize()
+    n_sel = c.filter_select(tumor=1, min_tumor=2, max_normal=3)
+    packed, mask = kc.pack_ascii(rs.ascii)
+    want, cand, n = c.filter_reads(packed, rs.offsets, mask)
+    if n_sel:
+        assert int(want.sum()) == int(c.filter_keys()[1][:, 1].sum())
+    assert np.array_equal(cand, np.flatnonzero(want)) and n == len(cand)
+    for shift in (0, 1):
+        torch.cuda.synchronize()
+        args = [_on_device(packed, shift), _on_device(rs.offsets, shift), _on_device(mask, shift)]
+        torch.cuda.synchronize()
+        hits = torch.full((keep,), -1, dtype=torch.int32, device="cuda")
+        which = torch.full((keep,), -1, dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        _, _, m = c.filter_reads(*args, hits=hits, candidates=which)
+        assert m == n
+        assert np.array_equal(hits.cpu().numpy(), want.astype(np.int32))
+        assert np.array_equal(which[:m].cpu().numpy(), cand.astype(np.int64))
+    c.close()
+
+
+def test_filter_reads_without_bases():
+    """Reads that are all empty behind a base offset: no word is read, no hit."""
+    c = kc.KmerCounter(5, 2, 1 << 12, 4, 1)
+    rs = synth.ReadSet.from_strings(["ACGTTGCA", "ACGTAGCA"])
+    c.add_readset(0, rs)
+    c.add_readset(1, rs)
+    c.finalize()
+    c.filter_select(tumor=1, min_tumor=1, max_normal=5)
+    offsets = np.full(4, 100, dtype=np.uint64)
+    hits, cand, n = c.filter_reads(np.zeros(1, np.uint64), offsets, np.zeros(1, np.uint64))
+    assert n == 0 and len(cand) == 0 and not hits.any()
+    c.close()
