@@ -107,56 +107,47 @@ __device__ __forceinline__ uint64_t canonical_key(uint64_t fwd, const PassParams
     return fwd < rc ? fwd : rc;
 }
 
-// Rolling codes over the 64 window starts of a unit: the forward and
-// reverse-complement codes of window j, updated by one base per step instead
-// of being cut out of the unit's words for every window.  `x` and `y` hold the
-// bases entering at the next steps (base j + k first, as the top two bits of
-// x), taken from the unit's words w0, w1 and the following word w2.
-struct RollingWindow {
-    uint64_t fwd, rc, x, y;
-};
-
-__device__ __forceinline__ RollingWindow rolling_start(uint64_t w0, uint64_t w1, uint64_t w2, const PassParams& p) {
-    RollingWindow r;
-    const int kk = 64 - p.rc_shift;  // 2k, in 2..62
-    r.fwd = w0 >> p.rc_shift;
-    r.rc = reverse_pairs(r.fwd ^ p.kmask) >> p.rc_shift;
-    r.x = (w0 << kk) | (w1 >> p.rc_shift);
-    r.y = (w1 << kk) | (w2 >> p.rc_shift);
-    return r;
-}
-
-// Window j -> window j + 1: the base leaving is dropped by the mask (forward)
-// or shifted out (reverse complement), the entering base b adds b at the low
-// end of the forward code and its complement 3 - b at the high end of the
-// reverse complement.
-__device__ __forceinline__ void rolling_step(RollingWindow& r, const PassParams& p) {
-    const uint64_t b = r.x >> 62;
-    r.fwd = ((r.fwd << 2) | b) & p.kmask;
-    r.rc = (r.rc >> 2) | ((b ^ 3ull) << (62 - p.rc_shift));
-    r.x = (r.x << 2) | (r.y >> 62);
-    r.y <<= 2;
-}
-
-// rolling_step with k = K a compile-time constant (every shift an immediate).
-template <int K>
-__device__ __forceinline__ void rolling_step_k(RollingWindow& r) {
-    constexpr uint64_t kmask = K >= 32 ? ~0ull : (1ull << (2 * K)) - 1ull;
-    const uint64_t b = r.x >> 62;
-    r.fwd = ((r.fwd << 2) | b) & kmask;
-    r.rc = (r.rc >> 2) | ((b ^ 3ull) << (2 * K - 2));
-    r.x = (r.x << 2) | (r.y >> 62);
-    r.y <<= 2;
-}
-
-// Forward codes of eight windows at a time, cut out of the unit's bases at
-// constant places: f holds the bases from the first of the eight windows on,
-// as 32-bit words, first base on top.  Two funnel shifts and a mask a window
-// (K = k at compile time; K = 0: one 64-bit shift by rc_shift more), where the
-// rolling code takes nine operations.
+// Codes of eight windows at a time, cut out of the unit's bases at constant
+// places: f holds the bases from the first of the eight windows on, as 32-bit
+// words, first base on top.  Two funnel shifts and a mask a window (K = k at
+// compile time; K = 0: one 64-bit shift by rc_shift more), where the rolling
+// code takes nine operations.
 struct WindowWords {
     uint32_t f[6];
 };
+
+// The reverse complements of the same windows: r holds the reverse complement
+// of all bases from the first of the eight windows on, its lowest word first,
+// so that window J's code begins at bit 2 J.
+struct ReverseWords {
+    uint32_t r[6];
+};
+
+__device__ __forceinline__ ReverseWords reverse_words(uint64_t w0, uint64_t w1, uint64_t w2) {
+    const uint64_t a = reverse_pairs(~w0), b = reverse_pairs(~w1), c = reverse_pairs(~w2);
+    return ReverseWords{{(uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32), (uint32_t)c,
+                         (uint32_t)(c >> 32)}};
+}
+
+__device__ __forceinline__ void next_windows(ReverseWords& w) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w.r[i] = __funnelshift_r(w.r[i], w.r[i + 1], 16);
+    w.r[5] >>= 16;
+}
+
+template <int K, int J>
+__device__ __forceinline__ uint64_t reverse_code(const ReverseWords& w, uint64_t kmask) {
+    uint32_t lo, hi;
+    if constexpr (J == 0) {
+        lo = w.r[0];
+        hi = w.r[1];
+    } else {
+        lo = __funnelshift_r(w.r[0], w.r[1], 2 * J);
+        hi = __funnelshift_r(w.r[1], w.r[2], 2 * J);
+    }
+    if constexpr (K > 16) return ((uint64_t)(hi & (0xffffffffu >> (64 - 2 * K))) << 32) | lo;
+    else return (((uint64_t)hi << 32) | lo) & kmask;
+}
 
 __device__ __forceinline__ WindowWords window_words(uint64_t w0, uint64_t w1, uint64_t w2) {
     return WindowWords{{(uint32_t)(w0 >> 32), (uint32_t)w0, (uint32_t)(w1 >> 32), (uint32_t)w1, (uint32_t)(w2 >> 32),

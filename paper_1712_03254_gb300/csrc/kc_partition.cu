@@ -274,16 +274,13 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
             if (lane == 0) wb = atomicAdd(&s_pos, tot);
             wb = __shfl_sync(kFull, wb, 0);
         }
-        // every lane walks the 64 window starts of its unit with rolling codes
-        RollingWindow rw = rolling_start(uw.w0, uw.w1, uw.w2, p);
-        uint64_t vbits = vm;  // window start j's bit at the top at step j
-#pragma unroll 4
-        for (int j = 0; j < 64; ++j) {
-            bool has = (int64_t)vbits < 0;
-            vbits <<= 1;
+        // every lane walks the 64 window starts of its unit, eight at a time
+        WindowWords fw = window_words(uw.w0, uw.w1, uw.w2);
+        ReverseWords rv = reverse_words(uw.w0, uw.w1, uw.w2);
+        const auto window = [&](uint64_t fwd, uint64_t rc, bool has) {
             uint64_t h = 0;
             if (has) {
-                h = mixer64(rw.fwd < rw.rc ? rw.fwd : rw.rc);
+                h = mixer64(fwd < rc ? fwd : rc);
                 if (kRange) has = h >= p.h_lo && h <= p.h_hi;
                 if (has) atomicAdd(&s_cnt[(uint32_t)(h >> 32) >> hist_shift], 1u);
             }
@@ -294,8 +291,20 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
             }
             if (has) lin[base + wb + __popc(ballot & lt)] = h;
             if (!kRange) wb += __popc(ballot);
-            if (K > 0) rolling_step_k<(K > 0 ? K : 1)>(rw);
-            else rolling_step(rw, p);
+        };
+        uint64_t vbits = vm;  // the eight windows' valid bits on top
+        for (int j = 0; j < 64; j += 8, vbits <<= 8) {
+            const unsigned valid = (unsigned)(vbits >> 56);
+            window(forward_code<K, 0>(fw, p.rc_shift), reverse_code<K, 0>(rv, p.kmask), valid & 128u);
+            window(forward_code<K, 1>(fw, p.rc_shift), reverse_code<K, 1>(rv, p.kmask), valid & 64u);
+            window(forward_code<K, 2>(fw, p.rc_shift), reverse_code<K, 2>(rv, p.kmask), valid & 32u);
+            window(forward_code<K, 3>(fw, p.rc_shift), reverse_code<K, 3>(rv, p.kmask), valid & 16u);
+            window(forward_code<K, 4>(fw, p.rc_shift), reverse_code<K, 4>(rv, p.kmask), valid & 8u);
+            window(forward_code<K, 5>(fw, p.rc_shift), reverse_code<K, 5>(rv, p.kmask), valid & 4u);
+            window(forward_code<K, 6>(fw, p.rc_shift), reverse_code<K, 6>(rv, p.kmask), valid & 2u);
+            window(forward_code<K, 7>(fw, p.rc_shift), reverse_code<K, 7>(rv, p.kmask), valid & 1u);
+            next_windows(fw);
+            next_windows(rv);
         }
     }
     __syncthreads();
