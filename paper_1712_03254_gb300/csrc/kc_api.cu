@@ -397,9 +397,8 @@ kc_status regroup_batch(kc_handle h, Batch& b, cudaStream_t st) {
     kc::launch_count_seg(b.hdata, dsegs, (int)nv, a1, a2, counts, st);
     kc::launch_regroup_offsets(counts, dvlo, a1, a2, rel, total, st);
     if ((e = kc::launch_scan(total, P, starts, cursor, st)) != cudaSuccess) return bail(e);
-    kc::launch_regroup_base(rel, starts, dsegs, nv, a2, st);
-    kc::launch_scatter_staged_seg(b.hdata, dsegs, (int)nv, 1, a1, a2, rel, out, st);
-    h->launches += 5;
+    kc::launch_scatter_staged_seg(b.hdata, dsegs, (int)nv, 1, a1, a2, rel, starts, out, st);
+    h->launches += 4;
     KC_LAUNCHED("second-level bucketing launches");
     cudaFreeAsync(scratch, st);
     if (st == h->stream) {
@@ -507,10 +506,10 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
         b.hash_bytes = std::max<uint64_t>(1, need) * 8;
         if ((e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess) return bail(e);
     }
-    if (mode != 1) kc::launch_bucket_base(rel, b.hstarts, n_ctas, a, st);
-    if (mode == 4) kc::launch_scatter_staged_seg(lin, seg, n_ctas, n_pieces, 0, a, rel, b.hdata, st);
+    if (mode == 2 || mode == 3) kc::launch_bucket_base(rel, b.hstarts, n_ctas, a, st);
+    if (mode == 4) kc::launch_scatter_staged_seg(lin, seg, n_ctas, n_pieces, 0, a, rel, b.hstarts, b.hdata, st);
     else kc::launch_bucket_scatter(b.pw, b.vw, b.n_units, upc, n_ctas, p, a, mode, rel, cursor, b.hdata, st);
-    h->launches += mode != 1 ? 5 : 4;
+    h->launches += mode == 2 || mode == 3 ? 5 : 4;
     leave_block(h, scratch, scratch_bytes, st);  // every caller's st is the handle's stream
     if (h->l1_bits != h->part_bits) return regroup_batch(h, b, st);
     return KC_OK;
@@ -573,9 +572,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         B.upi = upi;
         B.ctr = h->ctr;
         B.bucket_off = plan.n_buckets;
-        B.rel_off = plan.n_rel;
         plan.n_buckets += P;
-        plan.n_rel += (uint64_t)B.n_items * P;
         plan.max_a = std::max(plan.max_a, B.a);
         item_batch.insert(item_batch.end(), B.n_items, (uint32_t)i);
         // scratch: counts, relative bases, segments, totals, cursor, linear hashes
@@ -639,7 +636,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         b.pw = b.vw = nullptr;
         b.pending = false;
     }
-    for (int j = 0; j < n; ++j) hs[j]->launches += 5;
+    for (int j = 0; j < n; ++j) hs[j]->launches += 4;
     for (const Ref& r : refs) {
         kc_handle h = r.h;
         if (h->l1_bits != h->part_bits) {

@@ -121,11 +121,12 @@ void launch_extract_count(const uint64_t* pw, const uint64_t* vw, uint64_t n_uni
                           int n_ctas, const PassParams& p, int a, uint32_t* counts, uint64_t* g_cursor, SegDesc* seg,
                           uint64_t* lin, DevCounters* ctr, cudaStream_t st,
                           bool accumulate = false);
-// Staged scatter of segment c into its runs: bucket (h >> (64 - a1 - a2)) mod
+// Staged scatter of segment c into its runs (base: within their buckets,
+// which begin at starts): bucket (h >> (64 - a1 - a2)) mod
 // 2^a2; with a1 > 0 only hashes of the segment's level-1 group.  Segment c
 // comes in n_pieces pieces segs[c], segs[c + n_segs], ...
 void launch_scatter_staged_seg(const uint64_t* src, const SegDesc* segs, int n_segs, int n_pieces, int a1, int a2,
-                               const uint64_t* base, uint64_t* out, cudaStream_t st);
+                               const uint64_t* base, const uint64_t* starts, uint64_t* out, cudaStream_t st);
 // Batched ingest: the read batches of several jobs extracted and grouped by
 // one set of launches.  Each batch is cut into items of whole units; the
 // extraction and the staged scatter are persistent kernels over the item
@@ -147,12 +148,11 @@ struct IngestBatch {
     uint64_t* lin;      // linear hashes
     unsigned long long* g_cursor;
     DevCounters* ctr;
-    uint64_t* rel;      // [n_items][2^a]: run starts, relative, then absolute
+    uint64_t* rel;      // [n_items][2^a]: run starts within their bucket
     uint32_t* total;    // [2^a]
     uint64_t* starts;   // [2^a + 1]
     uint64_t* out;      // grouped hashes
     uint64_t bucket_off;  // first (batch, bucket) index of the batch: sum of 2^a over earlier batches
-    uint64_t rel_off;     // first (item, bucket) index: sum of n_items 2^a over earlier batches
 };
 struct IngestPlan {
     const IngestBatch* batches;
@@ -160,22 +160,19 @@ struct IngestPlan {
     unsigned int* head;          // [0] extraction queue, [1] scatter queue
     uint32_t n_batches, n_items;
     uint64_t n_buckets;  // sum of 2^a
-    uint64_t n_rel;      // sum of n_items 2^a
     int max_a;
 };
 size_t ingest_scatter_smem(int max_a);
-// The five launches; `plan` is on the device, its arrays too.  ranged: some
+// The four launches; `plan` is on the device, its arrays too.  ranged: some
 // batch keeps only a hash range; all_k31: every batch has k = 31.
 void launch_ingest(const IngestPlan* plan, const IngestPlan& host_plan, bool ranged, bool all_k31, int sm_count,
                    cudaStream_t st);
 // Level-2 re-bucketing of level-1 groups: per-segment counts, per-(group,
-// partition) offsets and totals (padded to 4), absolute run starts.
+// partition) offsets and totals (padded to 4).
 void launch_count_seg(const uint64_t* src, const SegDesc* segs, int n_segs, int a1, int a2, uint32_t* counts,
                       cudaStream_t st);
 void launch_regroup_offsets(const uint32_t* counts, const uint32_t* vlo, int a1, int a2, uint64_t* rel,
                             uint32_t* total, cudaStream_t st);
-void launch_regroup_base(uint64_t* rel, const uint64_t* starts, const SegDesc* segs, uint64_t n_segs, int a2,
-                         cudaStream_t st);
 void launch_bucket_scatter(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, uint64_t units_per_cta,
                            int n_ctas, const PassParams& p, int a, int mode, const uint64_t* base, uint64_t* cursor,
                            uint64_t* out, cudaStream_t st);

@@ -195,15 +195,17 @@ __global__ void k_compact(const Slot* __restrict__ table, uint64_t n_slots, int 
     }
 }
 
-// Exclusive scan of n counters with one CTA of 1024 threads.
+// Exclusive scan of n <= 4096 counters with one CTA of 1024 threads, four
+// consecutive ones a thread (all loads in flight at once).
 __global__ void __launch_bounds__(1024) k_scan(const uint32_t* __restrict__ hist, uint64_t n,
                                                uint64_t* __restrict__ starts, uint64_t* __restrict__ cursor) {
     __shared__ unsigned long long warp_tot[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const uint64_t chunk = (n + blockDim.x - 1) / blockDim.x;
-    const uint64_t lo = (uint64_t)t * chunk, hi = lo + chunk < n ? lo + chunk : n;
-    unsigned long long sum = 0;
-    for (uint64_t i = lo; i < hi; ++i) sum += hist[i];
+    const uint64_t lo = 4ull * t;
+    uint32_t c[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[j] = lo + j < n ? hist[lo + j] : 0u;
+    const unsigned long long sum = (unsigned long long)c[0] + c[1] + c[2] + c[3];
     // inclusive warp scan
     unsigned long long x = sum;
 #pragma unroll
@@ -224,10 +226,13 @@ __global__ void __launch_bounds__(1024) k_scan(const uint32_t* __restrict__ hist
     }
     __syncthreads();
     unsigned long long run = x - sum + (wid ? warp_tot[wid - 1] : 0ull);
-    for (uint64_t i = lo; i < hi; ++i) {
-        starts[i] = run;
-        cursor[i] = run;
-        run += hist[i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (lo + j < n) {
+            starts[lo + j] = run;
+            cursor[lo + j] = run;
+        }
+        run += c[j];
     }
     if (t == (int)blockDim.x - 1) starts[n] = warp_tot[(blockDim.x >> 5) - 1];
 }
