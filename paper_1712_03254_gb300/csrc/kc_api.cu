@@ -828,7 +828,7 @@ kc_status finalize_direct(kc_handle h) {
     }
     KC_CUDA(cudaMemsetAsync(&h->ctr->survivors, 0, 8, st));
     t0 = phase_begin(h);
-    kc::launch_compact(h->table, h->n_slots, h->n_samples, h->min_count, tk, tv, h->ctr, nullptr, 0, h->grid, st);
+    kc::launch_compact(h->table, h->n_slots, h->n_samples, h->min_count, tk, tv, h->ctr, h->grid, st);
     phase_end(h, kCompact, t0);
     h->launches += 1;
     KC_LAUNCHED("direct compaction launches");

@@ -260,6 +260,29 @@ __device__ __forceinline__ int table_claim(Slot* __restrict__ table, uint64_t ma
     return 0;
 }
 
+// Insert key (stored as key + 1) and add one occurrence to it, from slot s on,
+// whose key1 the caller has read as cur.  Returns 1 if this call claimed a new
+// slot.
+__device__ __forceinline__ int table_add(Slot* __restrict__ table, uint64_t mask, uint64_t s, uint64_t stored,
+                                         unsigned long long cur, int sample, DevCounters* ctr) {
+    for (uint64_t i = 0;; ) {
+        int claimed = 0;
+        if (cur == 0ull) {
+            cur = atomicCAS(&table[s].key1, 0ull, (unsigned long long)stored);
+            claimed = cur == 0ull;
+        }
+        if (claimed || cur == stored) {
+            if (atomicAdd(&table[s].cnt[sample], 1u) == 0xffffffffu) atomicOr(&ctr->err, DERR_COUNT_OVERFLOW);
+            return claimed;
+        }
+        if (++i > mask) break;
+        s = (s + 1) & mask;
+        cur = __ldcg(&table[s].key1);
+    }
+    atomicOr(&ctr->err, DERR_TABLE_FULL);
+    return 0;
+}
+
 // Add one occurrence of key to its slot if the key is in the table.
 __device__ __forceinline__ void table_count(Slot* __restrict__ table, uint64_t mask, uint64_t s, uint64_t stored,
                                             int sample, DevCounters* ctr) {

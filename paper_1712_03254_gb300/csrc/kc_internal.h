@@ -45,11 +45,9 @@ void launch_pass1(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, cons
 void launch_pass2(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, const PassParams& p, Slot* table,
                   DevCounters* ctr, const Grid& g, cudaStream_t st);
 
-// Compaction of slots with summed count >= min_count, with a histogram of the
-// survivors' top key bits (bucket = key >> prefix_shift).
+// Compaction of slots with summed count >= min_count.
 void launch_compact(const Slot* table, uint64_t n_slots, int n_samples, uint32_t min_count, uint64_t* keys,
-                    uint64_t* vals, DevCounters* ctr, uint32_t* hist, int prefix_shift, const Grid& g,
-                    cudaStream_t st);
+                    uint64_t* vals, DevCounters* ctr, const Grid& g, cudaStream_t st);
 // starts[0..n] = exclusive scan of hist[0..n); cursor[0..n) = starts[0..n).
 // Above 4096 counters a three-kernel multi-CTA scan with a small stream-
 // ordered temporary (n <= 2^25).

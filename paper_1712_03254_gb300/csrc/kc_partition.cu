@@ -574,8 +574,8 @@ __global__ void k_regroup_offsets(const uint32_t* __restrict__ counts, const uin
 // 32 buckets a block, eight warps sharing the CTAs' rows: each warp adds up its
 // rows, the warps' sums give it its first offset, then it writes its rows'.
 // (One thread a bucket walked all rows: 4096 buckets of 152 rows 17.7 us, 64
-// blocks; now 6.4 us for 256 buckets, from 16.4.)  With pad4, every count is rounded up to a multiple of 4
-// first.
+// blocks; 256 buckets 16.4 us, now 6.4.)  With pad4, every count is rounded up
+// to a multiple of 4 first.
 constexpr int kOffsetWarps = 8;
 
 __global__ void __launch_bounds__(32 * kOffsetWarps) k_bucket_offsets(const uint32_t* __restrict__ counts, int n_ctas,
