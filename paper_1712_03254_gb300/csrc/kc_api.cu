@@ -431,8 +431,93 @@ int scatter_mode_of(kc_handle h) {
     return mode;
 }
 
+// Two levels at once (launch_extract_groups): *done unless a stream of some CTA
+// overflowed, which leaves the batch ungrouped (its valid-window bits are built).
+kc_status bucket_two_levels(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st, const kc::PassParams& p,
+                            const ChunkedReads* chunks, bool* done) {
+    const int a = h->part_bits, a1 = h->l1_bits, a2 = a - a1;
+    const uint64_t P = 1ull << a;
+    const int max_ctas = h->grid.sm_count * (h->cfg.ctas_per_sm ? (int)h->cfg.ctas_per_sm : 1);
+    const uint64_t upc = std::max<uint64_t>(1, (b.n_units + max_ctas - 1) / max_ctas);
+    const int n_ctas = (int)((b.n_units + upc - 1) / upc);
+    const int n_pieces = chunks ? chunks->n : 1;
+    const uint64_t n_segs = (uint64_t)n_ctas << a1;
+    // the pieces' units, units a CTA and room a stream
+    uint64_t u[kMaxChunks + 1] = {0, b.n_units}, upc_c[kMaxChunks], lin_off[kMaxChunks + 1] = {0};
+    uint32_t cap[kMaxChunks];
+    for (int c = 0; c < n_pieces; ++c) {
+        if (chunks) u[c + 1] = chunks->u[c + 1];
+        upc_c[c] = std::max<uint64_t>(1, (u[c + 1] - u[c] + n_ctas - 1) / n_ctas);
+        cap[c] = kc::extract_groups_cap(upc_c[c], a1);
+        lin_off[c + 1] = lin_off[c] + n_segs * cap[c];
+    }
+    *done = false;
+    b.hcap = n_local + 3ull * (uint64_t)n_ctas * P;
+    const uint64_t cells = (uint64_t)n_ctas * P, n_lin = lin_off[n_pieces];
+    size_t scratch_bytes = n_lin * 8 + cells * 12 + P * 12 + n_segs * n_pieces * sizeof(kc::SegDesc) + 64;
+    void* scratch = nullptr;
+    cudaError_t e = cudaSuccess;
+    auto drop = [&]() {
+        if (b.hstarts) cudaFreeAsync(b.hstarts, st);
+        if (b.hdata) cudaFreeAsync(b.hdata, st);
+        b.hstarts = b.hdata = nullptr;
+        b.hash_bytes = 0;
+    };
+    auto bail = [&](cudaError_t err) {
+        if (scratch) cudaFreeAsync(scratch, st);
+        drop();
+        return cuda_fail(err, "cudaMallocAsync(partition buckets)");
+    };
+    b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
+    if ((e = take_block(h, &scratch, &scratch_bytes, st)) != cudaSuccess || (e = pinned_words(h)) != cudaSuccess ||
+        (e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
+        (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess)
+        return bail(e);
+    char* q = static_cast<char*>(scratch);
+    kc::SegDesc* seg = reinterpret_cast<kc::SegDesc*>(q);
+    uint64_t* lin = reinterpret_cast<uint64_t*>(q += n_segs * n_pieces * sizeof(kc::SegDesc));
+    uint64_t* rel = reinterpret_cast<uint64_t*>(q += n_lin * 8);
+    uint64_t* cursor = reinterpret_cast<uint64_t*>(q += cells * 8);
+    unsigned* overflow = reinterpret_cast<unsigned*>(q += P * 8);
+    uint32_t* counts = reinterpret_cast<uint32_t*>(q += 8);
+    uint32_t* total = reinterpret_cast<uint32_t*>(q += cells * 4);
+    unsigned* flag = reinterpret_cast<unsigned*>(h->pinned + 3);
+    KC_CUDA(cudaMemsetAsync(overflow, 0, 4, st));
+    for (int c = 0; c < n_pieces; ++c) {
+        const uint64_t nu = u[c + 1] - u[c];
+        if (chunks) {
+            KC_CUDA(cudaStreamWaitEvent(st, chunks->ev[c], 0));
+            kc::launch_build_valid_range(chunks->nm, chunks->bd, b.n_units, u[c], u[c + 1], chunks->start_local,
+                                         chunks->n_local, h->k, b.vw, h->ctr, h->grid, st);
+        }
+        kc::launch_extract_groups(b.pw + 2 * u[c], b.vw + u[c], nu, upc_c[c], n_ctas, p, a1, a, counts, cap[c],
+                                  seg + (size_t)c * n_segs, lin_off[c], lin, overflow, st, c > 0);
+    }
+    KC_CUDA(cudaMemcpyAsync(flag, overflow, 4, cudaMemcpyDeviceToHost, st));
+    KC_CUDA(cudaEventRecord(h->ev_main, st));
+    // the rest is queued before the flag is known (the segments stay within
+    // their streams' room in any case)
+    kc::launch_bucket_offsets(counts, n_ctas, a, 1, rel, total, st);
+    if ((e = kc::launch_scan(total, P, b.hstarts, cursor, st)) != cudaSuccess) return bail(e);
+    kc::launch_scatter_staged_seg(lin, seg, (int)n_segs, n_pieces, a1, a2, rel, b.hstarts, b.hdata, st);
+    h->launches += 3 + (chunks ? 2 : 1) * n_pieces;
+    KC_LAUNCHED("two-level bucketing launches");
+    KC_CUDA(cudaEventSynchronize(h->ev_main));
+    leave_block(h, scratch, scratch_bytes, st);
+    if (*flag) drop();
+    else *done = true;
+    return KC_OK;
+}
+
 kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st, const kc::PassParams& p,
                        bool exact, const ChunkedReads* chunks) {
+    if (h->l1_bits != h->part_bits && h->l1_bits <= kc::kStreamBits && !exact && p.h_lo == 0ull && p.h_hi == ~0ull &&
+        b.n_units < 1ull << 30) {  // (positions within a stream are 32-bit numbers)
+        bool done = false;
+        const kc_status s = bucket_two_levels(h, b, n_local, st, p, chunks, &done);
+        if (s != KC_OK || done) return s;
+        chunks = nullptr;  // every chunk is there, its valid-window bits built
+    }
     const int a = h->l1_bits;
     const uint64_t P = 1ull << a;
     const int mode = scatter_mode_of(h);
@@ -697,8 +782,12 @@ bool fits_device(kc_handle h, uint64_t bytes) { return small_need(h, bytes) || b
 uint64_t bucket_bytes(kc_handle h, uint64_t n_local) {
     const int max_ctas = h->grid.sm_count * (h->cfg.ctas_per_sm ? (int)h->cfg.ctas_per_sm : 1);
     if (n_local + 3ull * (uint64_t)max_ctas * (1ull << h->l1_bits) > kMaxGroupedHashes) return ~0ull;
+    // (two levels at once: streams of 9/8 of the hashes, rows over both levels)
+    const uint64_t streams = h->l1_bits != h->part_bits && h->l1_bits <= kc::kStreamBits
+                                 ? n_local + (uint64_t)max_ctas * ((1ull << h->part_bits) * 36 + (32ull * 128 * 8 << h->l1_bits))
+                                 : 0;
     return 16 * n_local + 24ull * (uint64_t)max_ctas * (1ull << h->l1_bits) +
-           (uint64_t)max_ctas * (1ull << h->l1_bits) * 12;
+           (uint64_t)max_ctas * (1ull << h->l1_bits) * 12 + streams;
 }
 
 // Sort n (key, value) pairs held in tk/tv, keys below 2^key_bits, into

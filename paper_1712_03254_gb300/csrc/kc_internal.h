@@ -119,6 +119,16 @@ void launch_extract_count(const uint64_t* pw, const uint64_t* vw, uint64_t n_uni
                           int n_ctas, const PassParams& p, int a, uint32_t* counts, uint64_t* g_cursor, SegDesc* seg,
                           uint64_t* lin, DevCounters* ctr, cudaStream_t st,
                           bool accumulate = false);
+// Two grouping levels with a first one of a1 <= kStreamBits bits: CTA c's hashes
+// of group g go to a stream of at most cap hashes at lin_off + (c 2^a1 + g) cap
+// (segment seg[c 2^a1 + g]); counts rows over all 2^a partitions.  *overflow is
+// set when a stream had no room for all.
+constexpr int kStreamBits = 2;
+uint32_t extract_groups_cap(uint64_t units_per_cta, int a1);
+void launch_extract_groups(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, uint64_t units_per_cta,
+                           int n_ctas, const PassParams& p, int a1, int a, uint32_t* counts, uint32_t cap,
+                           SegDesc* seg, uint64_t lin_off, uint64_t* lin, unsigned* overflow, cudaStream_t st,
+                           bool accumulate);
 // Staged scatter of segment c into its runs (base: within their buckets,
 // which begin at starts): bucket (h >> (64 - a1 - a2)) mod
 // 2^a2; with a1 > 0 only hashes of the segment's level-1 group.  Segment c

@@ -329,6 +329,101 @@ __global__ void __launch_bounds__(kExtractThreads) k_extract_count(const uint64_
                           ctr, accumulate != 0);
 }
 
+// Extraction for two grouping levels of which the first has A1 = 1 or 2 bits:
+// each CTA writes the hashes of each first-level group to a stream of its own,
+// and its histogram covers the partitions of both levels, so the staged scatter
+// of the second level follows at once (without a scatter by the first level's
+// bits and without counting what that wrote: 2.4e8 windows of 2^14 partitions
+// 3.5 -> 2.5 ms).  A warp takes kStreamChunk positions of a stream
+// at a time; the ends of its last chunks get padding of another group.  A
+// stream has room for 9/8 of its even share of the CTA's window starts; a CTA
+// that needs more (few keys making up most of the reads) sets *overflow and
+// drops the rest, and the caller groups the batch the other way.
+constexpr unsigned kStreamChunk = 128;
+
+template <int K, int A1>
+__global__ void __launch_bounds__(kExtractThreads) k_extract_groups(
+    const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw, uint64_t n_units, uint64_t units_per_cta,
+    PassParams p, int a, uint32_t* __restrict__ counts, uint32_t cap, SegDesc* __restrict__ seg, uint64_t lin_off,
+    uint64_t* __restrict__ lin, unsigned* __restrict__ overflow, int accumulate) {
+    constexpr int G = 1 << A1;
+    extern __shared__ uint32_t s_cnt[];
+    __shared__ unsigned s_cur[G];
+    const uint32_t P = 1u << a;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) s_cnt[i] = 0;
+    if (threadIdx.x < G) s_cur[threadIdx.x] = 0;
+    __syncthreads();
+    const uint64_t lo = min((uint64_t)blockIdx.x * units_per_cta, n_units);
+    const uint64_t hi = min(lo + units_per_cta, n_units);
+    const uint64_t off = lin_off + (uint64_t)blockIdx.x * G * cap;  // the CTA's streams
+    const int hist_shift = 32 - a;
+    const unsigned lt = (1u << lane) - 1u;
+    // the warp's current chunk of stream g and what is used of it: held by the
+    // lanes l with l mod G = g
+    const int gl = lane & (G - 1);
+    const unsigned flip0 = gl & 1 ? 0u : kFull, flip1 = A1 > 1 && !(gl & 2) ? kFull : 0u;
+    unsigned used = kStreamChunk, chunk = 0;
+    for (uint64_t u = lo + (uint64_t)wid * 32; u < hi; u += (uint64_t)nwarps * 32) {
+        const UnitWords uw = load_unit(pw, vw, u + lane, hi, lane);
+        WindowWords fw = window_words(uw.w0, uw.w1, uw.w2);
+        ReverseWords rv = reverse_words(uw.w0, uw.w1, uw.w2);
+        const auto window = [&](uint64_t fwd, uint64_t rc, bool has) {
+            uint64_t h = 0;
+            if (has) {
+                h = mixer64(fwd < rc ? fwd : rc);
+                atomicAdd(&s_cnt[(uint32_t)(h >> 32) >> hist_shift], 1u);
+            }
+            const unsigned own = (unsigned)(h >> (64 - A1));
+            const unsigned all = __ballot_sync(kFull, has);
+            const unsigned b0 = __ballot_sync(kFull, own & 1u), b1 = A1 > 1 ? __ballot_sync(kFull, own & 2u) : 0u;
+            // the windows of this lane's group, and of the group whose chunk it holds
+            const unsigned m = all & (b0 ^ (own & 1u ? 0u : kFull)) & (A1 == 1 ? kFull : b1 ^ (own & 2u ? 0u : kFull));
+            const unsigned mg = all & (b0 ^ flip0) & (A1 == 1 ? kFull : b1 ^ flip1);
+            const unsigned idx = __shfl_sync(kFull, used, (int)own) + __popc(m & lt);
+            unsigned at = __shfl_sync(kFull, chunk, (int)own) + idx;
+            used += __popc(mg);
+            if (__any_sync(kFull, used > kStreamChunk)) {  // some group's next chunk
+                unsigned next = 0;
+                if (lane < G && used > kStreamChunk) next = atomicAdd(&s_cur[lane], kStreamChunk);
+                const unsigned mine = __shfl_sync(kFull, next, (int)own);
+                if (idx >= kStreamChunk) at = mine + idx - kStreamChunk;
+                next = __shfl_sync(kFull, next, gl);
+                if (used > kStreamChunk) {
+                    chunk = next;
+                    used -= kStreamChunk;
+                }
+            }
+            if (has && at < cap) lin[off + (uint64_t)own * cap + at] = h;
+        };
+        uint64_t vbits = uw.v;  // the eight windows' valid bits on top
+        for (int j = 0; j < 64; j += 8, vbits <<= 8) {
+            const unsigned valid = (unsigned)(vbits >> 56);
+            window(forward_code<K, 0>(fw, p.rc_shift), reverse_code<K, 0>(rv, p.kmask), valid & 128u);
+            window(forward_code<K, 1>(fw, p.rc_shift), reverse_code<K, 1>(rv, p.kmask), valid & 64u);
+            window(forward_code<K, 2>(fw, p.rc_shift), reverse_code<K, 2>(rv, p.kmask), valid & 32u);
+            window(forward_code<K, 3>(fw, p.rc_shift), reverse_code<K, 3>(rv, p.kmask), valid & 16u);
+            window(forward_code<K, 4>(fw, p.rc_shift), reverse_code<K, 4>(rv, p.kmask), valid & 8u);
+            window(forward_code<K, 5>(fw, p.rc_shift), reverse_code<K, 5>(rv, p.kmask), valid & 4u);
+            window(forward_code<K, 6>(fw, p.rc_shift), reverse_code<K, 6>(rv, p.kmask), valid & 2u);
+            window(forward_code<K, 7>(fw, p.rc_shift), reverse_code<K, 7>(rv, p.kmask), valid & 1u);
+            next_windows(fw);
+            next_windows(rv);
+        }
+    }
+    // the rest of the warp's chunks: padding of another group
+    for (unsigned i = used + lane / G; i < kStreamChunk; i += 32 / G)
+        if (chunk + i < cap) lin[off + (uint64_t)gl * cap + chunk + i] = (uint64_t)(gl ^ 1) << (64 - A1);
+    __syncthreads();
+    uint32_t* const row = counts + ((uint64_t)blockIdx.x << a);
+    for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) row[i] = (accumulate ? row[i] : 0u) + s_cnt[i];
+    if (threadIdx.x < G) {
+        const unsigned n = s_cur[threadIdx.x];
+        seg[blockIdx.x * G + threadIdx.x] = SegDesc{off + (uint64_t)threadIdx.x * cap, min(n, cap), threadIdx.x, 0ull};
+        if (n > cap) *overflow = 1u;
+    }
+}
+
 constexpr int kLinThreads = 1024;
 constexpr int kLinPerThread = 5;
 constexpr uint32_t kRetryCap = 2048;  // hashes one retry list holds
@@ -849,6 +944,29 @@ void launch_extract_count(const uint64_t* pw, const uint64_t* vw, uint64_t n_uni
         extract_count_k<false>(pw, vw, n_units, units_per_cta, n_ctas, p, a, counts, cur, seg, lin, ctr, st, accumulate);
     else
         extract_count_k<true>(pw, vw, n_units, units_per_cta, n_ctas, p, a, counts, cur, seg, lin, ctr, st, accumulate);
+}
+
+uint32_t extract_groups_cap(uint64_t units_per_cta, int a1) {
+    return (uint32_t)((units_per_cta * 64 * 9 / 8 >> a1) + kStreamChunk - 1) / kStreamChunk * kStreamChunk +
+           kExtractThreads / 32 * kStreamChunk;
+}
+
+void launch_extract_groups(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, uint64_t units_per_cta,
+                           int n_ctas, const PassParams& p, int a1, int a, uint32_t* counts, uint32_t cap,
+                           SegDesc* seg, uint64_t lin_off, uint64_t* lin, unsigned* overflow, cudaStream_t st,
+                           bool accumulate) {
+    const auto go = [&](auto kern) {
+        allow_max_dynamic_smem(kern);
+        kern<<<n_ctas, kExtractThreads, bucket_pass_smem(a), st>>>(pw, vw, n_units, units_per_cta, p, a, counts, cap, seg,
+                                                                   lin_off, lin, overflow, accumulate);
+    };
+    if (p.k == 31) {
+        if (a1 == 1) go(k_extract_groups<31, 1>);
+        else go(k_extract_groups<31, 2>);
+    } else {
+        if (a1 == 1) go(k_extract_groups<0, 1>);
+        else go(k_extract_groups<0, 2>);
+    }
 }
 
 // stage, fill count and output cursor (in sectors) per bucket, then the two retry lists

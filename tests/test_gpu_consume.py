@@ -189,3 +189,34 @@ def test_sort_buckets_at_both_ends_of_the_key_space():
     keys, at = np.unique(np.minimum(fwd, rev), return_index=True)
     repeats = [rng.integers(1, 4, len(keys))]
     _count(codes[at], keys, repeats, 1, 1)
+
+
+@pytest.mark.parametrize("k", [31, 20])
+@pytest.mark.parametrize("part_bits", [13, 14])
+@pytest.mark.parametrize("place", ["device", "chunked"])
+def test_two_levels_at_once(oracle_mod, k, part_bits, place):
+    """13 and 14 partition bits, reads on the device and host reads copied in
+    chunks: streams by the first level's bits, with and without overflow (reads
+    that are one key nearly all), and a small batch behind a large one."""
+    import torch
+
+    g = synth.genome(51, 100_000)
+    poly = synth.ReadSet.from_strings(["A" * 150] * 3_000)
+    plain = synth.reads(52, g, 32_000, 120, 160, 0.01, 0.001)
+    few = synth.reads(53, g, 40, 20, 90, 0.01, 0.001)
+    for sets in ([plain, few], [plain, poly, few]):
+        both = synth.ReadSet(np.concatenate([r.ascii for r in sets]),
+                             np.concatenate([[0], np.cumsum(np.concatenate([np.diff(r.offsets) for r in sets]))]).astype(np.uint64))
+        o = oracle_mod.count(synth.Workload("two", [both], k, 1 << 26, 4, 2))
+        c = kc.KmerCounter(k, 1, 1 << 26, 4, 2, strategy="partitioned", part_bits=part_bits)
+        for rs in sets:
+            packed, mask = kc.pack_ascii(rs.ascii)
+            arrays = [packed, np.ascontiguousarray(rs.offsets, dtype=np.uint64), mask]
+            if place == "device":
+                arrays = [torch.from_numpy(a.view(np.int64)).cuda() for a in arrays]
+                torch.cuda.synchronize()
+            c.add_reads(0, *arrays)
+        assert c.stats()["windows"] == o.windows
+        c.finalize()
+        _same(c, o)
+        c.close()
