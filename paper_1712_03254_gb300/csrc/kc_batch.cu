@@ -83,7 +83,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kConsumeThreads = 512;      // consumer CTAs, two an SM
 constexpr int kConsumeThreadsWide = 1024;  // when the shared memory has room for one alone
-constexpr int kAhead = 4;                  // hashes a consumer thread has in flight
+constexpr int kAhead = 3;                  // hashes a consumer thread has in flight
 constexpr unsigned long long kTopBit = 1ull << 63;
 constexpr int kTile = 4096;
 constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32 bits
@@ -95,16 +95,16 @@ constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32
 // window, no window waits for the filter's answer, and the hashes are read
 // once, without a recount.  (Updating the filter with every window and counting
 // the candidates took 0.975 ms for 1.18e8 windows of 4096 partitions, this
-// 0.745 ms: the instructions per window fell from 206 to about 130.  It is
-// bound by instruction issue; reading the hashes alone takes 0.17 ms, with one
-// probe each 0.21, with the queue's probes 0.36, the writing 0.09 and the
-// filter 0.11 more.)
+// 0.645 ms.  It is bound by instruction issue, at two thirds of the issue
+// slots: reading the hashes alone takes 0.17 ms, with one probe each 0.21, with
+// the queue's probes 0.36, the writing 0.08 and the filter 0.09 more.)
 //
 //   count    each window's first probe; a window that finds its key adds one
 //            to its count.  The others (new keys and displaced ones, about one
 //            in four at 30x coverage) go to a queue of the warp; 32 of them at a
-//            time take one probe (and claim) each and go back to the queue if
-//            it failed, so every probe step has all its lanes.
+//            time take two probes (and a claim) each and go back to the queue if
+//            both failed, so every probe step has all its lanes.  (One probe a
+//            step and four hashes in flight instead of three: 0.680 ms.)
 //   emit     keys of at least min_count, one position claim per warp
 //   filter   the counts are no longer needed: their memory takes the filter
 //            words, every key sets its bits, the words are written out
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                 uint32_t* const scol = ONE ? sc : sc + J.samples[bt];  // this batch's count column
                 unsigned q = 0;                             // entries in the warp's queue
                 // The queue's last n (at most 32) windows, one per lane, take their
-                // next probe: slots home, home + 1, home + 3, home + 6, ... (every
+                // next two probes: slots home, home + 1, home + 3, home + 6, ... (every
                 // slot of a power-of-two table in turn).
                 const auto step = [&](unsigned n) {
                     __syncwarp();
@@ -212,18 +212,27 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                     if ((unsigned)lane < n) {
                         h = wq[q + lane];
                         next = ws[q + lane];
-                        const uint32_t slot = next & tmask;
-                        unsigned long long cur = sk[slot];
-                        if (cur == empty) {
-                            cur = atomicCAS(sk + slot, empty, h);
-                            if (cur == empty) cur = h;
+                        const auto probe = [&](uint32_t slot) {
+                            unsigned long long cur = sk[slot];
+                            if (cur == empty) {
+                                cur = atomicCAS(sk + slot, empty, h);
+                                if (cur == empty) cur = h;
+                            }
+                            return cur == h;
+                        };
+                        uint32_t slot = next & tmask;
+                        bool found = probe(slot);
+                        if (!found) {
+                            next += 0x10000u;
+                            slot = (slot + (next >> 16)) & tmask;
+                            found = probe(slot);
                         }
-                        again = cur != h;
-                        if (!again) atomicAdd(scol + (slot << s2), 1u);
-                        next = ((next & 0xffff0000u) + 0x10000u) | ((slot + (next >> 16) + 1) & tmask);
-                        if (again && next >= (unsigned)kProbeLimit << 16) {
-                            s_fail = 1;
-                            again = false;
+                        if (found) {
+                            atomicAdd(scol + (slot << s2), 1u);
+                        } else {
+                            next = ((next & 0xffff0000u) + 0x10000u) | ((slot + (next >> 16) + 1) & tmask);
+                            again = next < (unsigned)kProbeLimit << 16;
+                            if (!again) s_fail = 1;
                         }
                     }
                     const unsigned back = __ballot_sync(kFull, again);

@@ -468,7 +468,7 @@ __device__ __forceinline__ void warp_sort64_packed(uint64_t* __restrict__ keys, 
     }
 }
 
-constexpr int kProbeLimit = 64;  // shared-memory table probes before a partition splits or falls back
+constexpr int kProbeLimit = 64;  // shared-memory table probes (taken in pairs) before a partition splits or falls back
 
 // Filter pattern with the number of bits chosen at run time.
 __device__ __forceinline__ uint64_t bloom_pattern_rt(uint64_t g, int n_hashes) {

@@ -124,10 +124,11 @@ def test_table_from_one_key_to_overfull(n, samples, min_count):
         assert st["split_partitions"] == 1
 
 
-@pytest.mark.parametrize("n_same", [2, 33, 64, 65, 90])
+@pytest.mark.parametrize("n_same", [2, 33, 64, 66, 90])
 def test_keys_of_one_home_slot(n_same):
     """Keys whose hashes end in the same bits as the table's last slot: the probes
-    wrap round, and past the probe limit the partition splits."""
+    wrap round, and past the probe limit (64, or 65 where the pairs of probes
+    begin at an odd one) the partition splits."""
     rng = np.random.default_rng(n_same)
     codes, keys = _canonical_31mers(rng, 400_000)
     h = _mixer(keys)
