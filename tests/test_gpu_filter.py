@@ -352,6 +352,19 @@ def test_stems_clamp_device_buffer_and_errors(oracle_mod):
     assert e.value.name == "KC_ERR_STATE"
 
 
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 513])
+def test_stems_at_the_edges_of_a_block(oracle_mod, n):
+    """Result keys and items just below, at and above the 256 of one block
+    (random 31-mers: a stem each but for chance)."""
+    rng = random.Random(n)
+    reads = ["".join(rng.choice("ACGT") for _ in range(31)) for _ in range(n)]
+    w = synth.Workload("edges", [synth.ReadSet.from_strings(reads)], 31, 1 << 16, 4, 1)
+    o = oracle_mod.count(w)
+    c = gpu_count(w)
+    assert c.dump()[0].size == n
+    assert c.export_stems().tobytes() == o.stems().tobytes()
+
+
 @pytest.mark.parametrize("spill", [1, 2])
 def test_stems_of_a_spilled_result(paired_small, spill):
     w, o = paired_small
