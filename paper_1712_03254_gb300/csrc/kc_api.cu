@@ -804,7 +804,6 @@ kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64
     int bits = 0;
     while (bits < 24 && bits < key_bits && (cap >> bits) > 32) ++bits;
     const uint64_t n_buckets = 1ull << bits;
-    const int prefix_shift = key_bits - bits;
     uint64_t *starts = nullptr, *cursor = nullptr;
     uint32_t* hist = nullptr;
     cudaError_t e;
@@ -822,12 +821,12 @@ kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64
     };
     cudaEvent_t t0 = phase_begin(h);
     KC_CUDA(cudaMemsetAsync(hist, 0, n_buckets * 4, st));
-    kc::launch_prefix_hist(tk, ctr, n, prefix_shift, n_buckets, hist, h->grid, st);
+    kc::launch_prefix_hist(tk, ctr, n, key_bits, bits, hist, h->grid, st);
     KC_CUDA(kc::launch_scan(hist, n_buckets, starts, cursor, st));
-    kc::launch_scatter(tk, tv, ctr, n, prefix_shift, n_buckets, cursor, out_k, out_v, h->grid, st);
-    kc::launch_bucket_sort_warp(out_k, out_v, starts, n_buckets, prefix_shift, ctr, h->grid, st);
+    kc::launch_scatter(tk, tv, ctr, n, key_bits, bits, cursor, out_k, out_v, h->grid, st);
+    kc::launch_bucket_sort_warp(out_k, out_v, starts, n_buckets, key_bits, ctr, h->grid, st);
     phase_end(h, phase, t0);
-    h->launches += 4;
+    h->launches += 5;
     KC_LAUNCHED("sort launches");
     unsigned err = 0;
     KC_CUDA(cudaMemcpyAsync(&err, &ctr->err, 4, cudaMemcpyDeviceToHost, st));
@@ -861,8 +860,9 @@ kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64
             }
         KC_LAUNCHED("global sort launches");
     }
-    if (err & (kc::DERR_SORT_MEDIUM | kc::DERR_SORT_BUCKET)) {
-        const unsigned keep = err & ~(kc::DERR_SORT_MEDIUM | kc::DERR_SORT_BUCKET);
+    constexpr unsigned kSortFlags = kc::DERR_SORT_BIG | kc::DERR_SORT_MEDIUM | kc::DERR_SORT_BUCKET;
+    if (err & kSortFlags) {
+        const unsigned keep = err & ~kSortFlags;
         KC_CUDA(cudaMemcpyAsync(&ctr->err, &keep, 4, cudaMemcpyHostToDevice, st));
     }
     release();

@@ -374,98 +374,75 @@ __device__ __forceinline__ uint32_t key_bucket(uint64_t key, int key_bits, int b
     const uint64_t y = 2ull * x - __umulhi(x, x);
     return (uint32_t)(y >> 32 ? 0xffffffffull : y) >> (32 - bits);
 }
-// Even buckets of 2^bits: the widest (the last) spans 2^(key_bits - bits / 2)
-// keys, which has to leave the 6 index bits of the packed sorts.
+// The map needs the 32 bits; one bucket needs no map.
 __host__ __device__ __forceinline__ bool even_buckets(int key_bits, int bits) {
-    return key_bits >= 32 && bits >= 1 && key_bits - bits / 2 <= 56;
+    return key_bits >= 32 && bits >= 1;
 }
 
-// Warp sort of a bucket of n <= 32 (key, value) pairs whose keys lie less than
-// 2^58 above `base`, one pair per lane (k, v; in = lane < n).  Each lane packs
-// its key's distance from base with its lane index into one word, the bitonic
-// network exchanges that single word (the lane index breaks ties between equal
-// keys), and each value then follows its key through the lane index.  Lanes >=
-// n hold ~0, which sorts last.  On return lane i holds the i-th pair.
-__device__ __forceinline__ void warp_sort32_core(uint64_t& k, uint64_t& v, bool in, int lane, uint64_t base) {
-    uint64_t p = in ? (((k - base) << 5) | (uint64_t)lane) : ~0ull;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const uint64_t o = __shfl_xor_sync(0xffffffffu, p, stride);
-            const bool asc = (lane & size) == 0;
-            const bool lower = (lane & stride) == 0;
-            const bool take = (lower == asc) ? (o < p) : (o > p);
-            p = take ? o : p;
-        }
-    }
-    v = __shfl_sync(0xffffffffu, v, (int)(p & 31ull));
-    k = base + (p >> 5);
+// Ranks of a bucket's n <= 64 distinct keys, two a lane (k0: element lane, k1:
+// element 32 + lane; in0, in1: whether there is one; two: n > 32), by one warp.
+// The keys of a bucket lie nearly evenly between its smallest and its largest,
+// so 64 equal ranges of them (by the keys' top 32 bits) hold about one key
+// each: a count per range, a scan over the counts, and each key is compared
+// with the few of its own range only.  240 instructions a bucket of 26 keys where a
+// bitonic network over packed words took 350 (15 or 21 steps of two shuffles, a
+// 64-bit compare and two selects, 80 % of the ALU pipe).  The counts are zero
+// before and after.  A range's first place and end share a word: two words cost
+// the warp three more shared-memory wavefronts.
+struct WarpRankTile {
+    uint64_t key[64];
+    uint32_t count[64];
+    uint32_t place[64];  // a range's first place, and its end in the upper half
+};
+__device__ __forceinline__ uint32_t rank_in_range(const WarpRankTile& t, uint64_t k, uint32_t place) {
+    uint32_t r = place & 0xffffu;
+    const uint64_t *p = t.key + r, *const e = t.key + (place >> 16);
+#pragma unroll 1
+    for (; p < e; ++p) r += *p < k ? 1u : 0u;
+    return r;
 }
-
-__device__ __forceinline__ void warp_sort32_packed(uint64_t* __restrict__ keys, uint64_t* __restrict__ vals,
-                                                   uint64_t lo, int n, int lane, int shift) {
-    const bool in = lane < n;
-    uint64_t k = in ? keys[lo + lane] : 0ull;
-    uint64_t v = in ? vals[lo + lane] : 0ull;
-    warp_sort32_core(k, v, in, lane, __shfl_sync(0xffffffffu, k, 0) & ~((1ull << shift) - 1ull));
-    if (in) {
-        keys[lo + lane] = k;
-        vals[lo + lane] = v;
-    }
-}
-
-// The same for 33..64 pairs: two packed words per lane, element
-// i = 32 r + lane in register r (k0, v0: element lane; k1, v1: element 32 +
-// lane); 6 index bits.  Compare-exchanges
-// across the two registers of a lane (stride 32) need no shuffle.
-__device__ __forceinline__ void warp_sort64_core(uint64_t& k0, uint64_t& v0, uint64_t& k1, uint64_t& v1, bool in0,
-                                                 bool in1, int lane, uint64_t base) {
-    uint64_t p0 = in0 ? (((k0 - base) << 6) | (uint64_t)lane) : ~0ull;
-    uint64_t p1 = in1 ? (((k1 - base) << 6) | (uint64_t)(32 + lane)) : ~0ull;
-#pragma unroll
-    for (int size = 2; size <= 64; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride == 32) {  // size 64: element lane against element lane + 32, ascending
-                const uint64_t a = p0 < p1 ? p0 : p1, b = p0 < p1 ? p1 : p0;
-                p0 = a;
-                p1 = b;
-            } else {
-                const uint64_t o0 = __shfl_xor_sync(0xffffffffu, p0, stride);
-                const uint64_t o1 = __shfl_xor_sync(0xffffffffu, p1, stride);
-                const bool lower = (lane & stride) == 0;
-                const bool asc0 = (lane & size) == 0, asc1 = ((32 + lane) & size) == 0;
-                const bool t0 = (lower == asc0) ? (o0 < p0) : (o0 > p0);
-                const bool t1 = (lower == asc1) ? (o1 < p1) : (o1 > p1);
-                p0 = t0 ? o0 : p0;
-                p1 = t1 ? o1 : p1;
-            }
-        }
-    }
-    const int i0 = (int)(p0 & 63ull), i1 = (int)(p1 & 63ull);
-    const uint64_t a0 = __shfl_sync(0xffffffffu, v0, i0 & 31), b0 = __shfl_sync(0xffffffffu, v1, i0 & 31);
-    const uint64_t a1 = __shfl_sync(0xffffffffu, v0, i1 & 31), b1 = __shfl_sync(0xffffffffu, v1, i1 & 31);
-    k0 = base + (p0 >> 6);
-    v0 = (i0 >> 5) ? b0 : a0;
-    k1 = base + (p1 >> 6);
-    v1 = (i1 >> 5) ? b1 : a1;
-}
-
-__device__ __forceinline__ void warp_sort64_packed(uint64_t* __restrict__ keys, uint64_t* __restrict__ vals,
-                                                   uint64_t lo, int n, int lane, int shift) {
-    const bool in0 = lane < n, in1 = 32 + lane < n;
-    uint64_t k0 = in0 ? keys[lo + lane] : 0ull, v0 = in0 ? vals[lo + lane] : 0ull;
-    uint64_t k1 = in1 ? keys[lo + 32 + lane] : 0ull, v1 = in1 ? vals[lo + 32 + lane] : 0ull;
-    warp_sort64_core(k0, v0, k1, v1, in0, in1, lane, __shfl_sync(0xffffffffu, k0, 0) & ~((1ull << shift) - 1ull));
-    if (in0) {
-        keys[lo + lane] = k0;
-        vals[lo + lane] = v0;
-    }
+__device__ __forceinline__ void warp_rank64(WarpRankTile& t, uint64_t k0, uint64_t k1, bool in0, bool in1, bool two,
+                                            int key_bits, int lane, uint32_t& r0, uint32_t& r1) {
+    const int top = key_bits > 32 ? key_bits - 32 : 0;
+    const uint32_t x0 = (uint32_t)(k0 >> top), x1 = (uint32_t)(k1 >> top);
+    uint32_t lo = in0 ? x0 : 0xffffffffu, hi = in0 ? x0 : 0u;
     if (in1) {
-        keys[lo + 32 + lane] = k1;
-        vals[lo + 32 + lane] = v1;
+        lo = min(lo, x1);
+        hi = max(hi, x1);
     }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    const int shift = max(0, 26 - __clz((int)(hi - lo)));  // (hi - lo) >> shift < 64
+    const uint32_t b0 = (x0 - lo) >> shift, b1 = (x1 - lo) >> shift;
+    uint32_t o0 = 0, o1 = 0;
+    if (in0) o0 = atomicAdd(&t.count[b0], 1u);
+    if (two && in1) o1 = atomicAdd(&t.count[b1], 1u);
+    __syncwarp();
+    const uint2 c = *reinterpret_cast<const uint2*>(&t.count[2 * lane]);
+    *reinterpret_cast<uint2*>(&t.count[2 * lane]) = make_uint2(0u, 0u);
+    uint32_t incl = c.x + c.y;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        // the shuffle's own predicate: whether the lane has a source
+        asm volatile(
+            "{ .reg .b32 y; .reg .pred p; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
+            : "+r"(incl)
+            : "r"(o));
+    const uint32_t mid = incl - c.y;
+    *reinterpret_cast<uint2*>(&t.place[2 * lane]) = make_uint2((mid - c.x) | mid << 16, mid | incl << 16);
+    __syncwarp();
+    uint32_t p0 = 0, p1 = 0;
+    if (in0) {
+        p0 = t.place[b0];
+        t.key[(p0 & 0xffffu) + o0] = k0;
+    }
+    if (two && in1) {
+        p1 = t.place[b1];
+        t.key[(p1 & 0xffffu) + o1] = k1;
+    }
+    __syncwarp();
+    r0 = rank_in_range(t, k0, p0);
+    if (two) r1 = rank_in_range(t, k1, p1);
 }
 
 constexpr int kProbeLimit = 64;  // shared-memory table probes (taken in pairs) before a partition splits or falls back

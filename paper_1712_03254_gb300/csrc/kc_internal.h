@@ -54,12 +54,13 @@ void launch_compact(const Slot* table, uint64_t n_slots, int n_samples, uint32_t
 cudaError_t launch_scan(const uint32_t* hist, uint64_t n, uint64_t* starts, uint64_t* cursor, cudaStream_t st);
 // Scatter survivors (at most cap of them) into their buckets; keys whose
 // bucket or position would fall outside the arrays set DERR_INTERNAL.
-void launch_scatter(const uint64_t* keys, const uint64_t* vals, DevCounters* ctr, uint64_t cap, int prefix_shift,
-                    uint64_t n_buckets, uint64_t* cursor, uint64_t* out_keys, uint64_t* out_vals, const Grid& g,
+void launch_scatter(const uint64_t* keys, const uint64_t* vals, DevCounters* ctr, uint64_t cap, int key_bits,
+                    int bits, uint64_t* cursor, uint64_t* out_keys, uint64_t* out_vals, const Grid& g,
                     cudaStream_t st);
 // Sort every bucket of at most warp_sort_capacity() keys in place, one warp
-// per bucket; larger buckets set DERR_SORT_MEDIUM and are left alone.
-void launch_bucket_sort_warp(uint64_t* keys, uint64_t* vals, const uint64_t* starts, uint64_t n_buckets, int shift,
+// per bucket (two launches: up to 64 keys, and the larger ones if there are any,
+// told by DERR_SORT_BIG); larger buckets set DERR_SORT_MEDIUM and are left alone.
+void launch_bucket_sort_warp(uint64_t* keys, uint64_t* vals, const uint64_t* starts, uint64_t n_buckets, int key_bits,
                              DevCounters* ctr, const Grid& g, cudaStream_t st);
 int warp_sort_capacity();
 // Sort buckets of warp_sort_capacity()+1 .. bucket_sort_capacity() keys in
@@ -193,7 +194,7 @@ size_t consume_queue_smem(int threads);
 void launch_fb_claim(const FallbackArgs& F, int bt, cudaStream_t st);
 void launch_fb_recount(const FallbackArgs& F, int bt, cudaStream_t st);
 void launch_fb_compact(const FallbackArgs& F, cudaStream_t st);
-void launch_prefix_hist(const uint64_t* keys, DevCounters* ctr, uint64_t cap, int shift, uint64_t n_buckets,
+void launch_prefix_hist(const uint64_t* keys, DevCounters* ctr, uint64_t cap, int key_bits, int bits,
                         uint32_t* hist, const Grid& g, cudaStream_t st);
 
 // The device's opt-in shared memory per block (cached per device).

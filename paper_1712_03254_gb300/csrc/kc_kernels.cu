@@ -340,15 +340,16 @@ __global__ void __launch_bounds__(1024) k_scan_apply(const uint32_t* __restrict_
 }
 
 __global__ void k_scatter(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ vals,
-                          DevCounters* __restrict__ ctr, uint64_t cap, int prefix_shift, uint64_t n_buckets,
+                          DevCounters* __restrict__ ctr, uint64_t cap, int key_bits, int bits,
                           unsigned long long* __restrict__ cursor, uint64_t* __restrict__ out_keys,
                           uint64_t* __restrict__ out_vals) {
     const uint64_t n = ctr->survivors < cap ? ctr->survivors : cap;
+    const bool even = even_buckets(key_bits, bits);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint64_t key = keys[i];
-        const uint64_t b = key >> prefix_shift;
-        if (b >= n_buckets) {
+        const uint64_t b = key_bucket(key, key_bits, bits, even);
+        if (b >> bits) {
             atomicOr(&ctr->err, DERR_INTERNAL);
             continue;
         }
@@ -425,29 +426,74 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(uint64_t* __restri
     }
 }
 
-// shift: the keys of a bucket share their bits above `shift` (buckets are
-// key-prefix ranges); buckets of up to 32 keys then sort packed.
-__global__ void __launch_bounds__(256, 2) k_bucket_sort_warp(uint64_t* __restrict__ keys, uint64_t* __restrict__ vals,
-                                                          const uint64_t* __restrict__ starts, uint64_t n_buckets,
-                                                          int shift, DevCounters* __restrict__ ctr) {
+// Buckets of up to 64 keys ranked (warp_rank64) and stored in place; larger
+// ones set DERR_SORT_BIG.  1.05 M pairs: 11 us; one kernel with the networks
+// for the larger buckets, at two CTAs an SM for their registers and on plain
+// key prefixes (buckets of up to twice the mean), 40.
+__global__ void __launch_bounds__(256, 6) k_bucket_sort_warp(uint64_t* keys, uint64_t* vals,
+                                                             const uint64_t* __restrict__ starts, uint64_t n_buckets,
+                                                             int key_bits, DevCounters* __restrict__ ctr) {
+    __shared__ __align__(16) WarpRankTile tiles[256 / 32];
     const int lane = threadIdx.x & 31;
+    WarpRankTile& tile = tiles[threadIdx.x >> 5];
+    *reinterpret_cast<uint2*>(&tile.count[2 * lane]) = make_uint2(0u, 0u);
+    __syncwarp();
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < n_buckets; b += n_warps) {
         const uint64_t lo = starts[b];
-        const uint64_t n64 = starts[b + 1] - lo;
-        if (n64 <= 1) continue;
-        if (n64 > (uint64_t)kWarpSortMax) {
-            if (lane == 0) atomicOr(&ctr->err, DERR_SORT_MEDIUM);
+        const uint64_t n = starts[b + 1] - lo;
+        if (n <= 1) continue;
+        if (n > 64) {
+            if (lane == 0 && !(*(volatile unsigned*)&ctr->err & DERR_SORT_BIG)) atomicOr(&ctr->err, DERR_SORT_BIG);
             continue;
         }
-        const int n = (int)n64;
-        if (n <= 32 && shift <= 59) warp_sort32_packed(keys, vals, lo, n, lane, shift);
-        else if (n <= 64 && shift <= 58) warp_sort64_packed(keys, vals, lo, n, lane, shift);
-        else if (n <= 32) warp_sort_bucket<1>(keys, vals, lo, n, lane);
-        else if (n <= 64) warp_sort_bucket<2>(keys, vals, lo, n, lane);
-        else if (n <= 128) warp_sort_bucket<4>(keys, vals, lo, n, lane);
-        else warp_sort_bucket<8>(keys, vals, lo, n, lane);
+        const bool in0 = lane < (int)n, in1 = 32 + lane < (int)n;
+        const uint64_t k0 = in0 ? keys[lo + lane] : 0ull, v0 = in0 ? vals[lo + lane] : 0ull;
+        const uint64_t k1 = in1 ? keys[lo + 32 + lane] : 0ull, v1 = in1 ? vals[lo + 32 + lane] : 0ull;
+        uint32_t r0 = 0, r1 = 0;
+        // every pair is read before the first is stored: the ranks wait for all keys, and __syncwarp orders the values
+        warp_rank64(tile, k0, k1, in0, in1, n > 32, key_bits, lane, r0, r1);
+        __syncwarp();
+        if (in0) {
+            keys[lo + r0] = k0;
+            vals[lo + r0] = v0;
+        }
+        if (in1) {
+            keys[lo + r1] = k1;
+            vals[lo + r1] = v1;
+        }
+    }
+}
+
+// The buckets of 65..256 keys by a network in one warp's registers; larger
+// ones set DERR_SORT_MEDIUM.
+__global__ void __launch_bounds__(256, 2) k_bucket_sort_warp_big(uint64_t* __restrict__ keys,
+                                                                 uint64_t* __restrict__ vals,
+                                                                 const uint64_t* __restrict__ starts,
+                                                                 uint64_t n_buckets, DevCounters* __restrict__ ctr) {
+    if (!(*(volatile unsigned*)&ctr->err & DERR_SORT_BIG)) return;
+    const int lane = threadIdx.x & 31;
+    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    // a lane looks at a bucket, the warp sorts the ones it has to
+    for (uint64_t base = warp * 32; base < n_buckets; base += n_warps * 32) {
+        const uint64_t b = base + (uint64_t)lane;
+        const uint64_t lo_b = b < n_buckets ? starts[b] : 0ull;
+        const uint64_t n_b = b < n_buckets ? starts[b + 1] - lo_b : 0ull;
+        unsigned todo = __ballot_sync(0xffffffffu, n_b > 64);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const uint64_t lo = __shfl_sync(0xffffffffu, lo_b, src), n = __shfl_sync(0xffffffffu, n_b, src);
+            if (n > (uint64_t)kWarpSortMax) {
+                if (lane == 0) atomicOr(&ctr->err, DERR_SORT_MEDIUM);
+            } else if (n <= 128) {
+                warp_sort_bucket<4>(keys, vals, lo, (int)n, lane);
+            } else {
+                warp_sort_bucket<8>(keys, vals, lo, (int)n, lane);
+            }
+        }
     }
 }
 
@@ -541,23 +587,25 @@ cudaError_t launch_scan(const uint32_t* hist, uint64_t n, uint64_t* starts, uint
     return cudaFreeAsync(tile, st);
 }
 
-void launch_scatter(const uint64_t* keys, const uint64_t* vals, DevCounters* ctr, uint64_t cap, int prefix_shift,
-                    uint64_t n_buckets, uint64_t* cursor, uint64_t* out_keys, uint64_t* out_vals, const Grid& g,
+void launch_scatter(const uint64_t* keys, const uint64_t* vals, DevCounters* ctr, uint64_t cap, int key_bits,
+                    int bits, uint64_t* cursor, uint64_t* out_keys, uint64_t* out_vals, const Grid& g,
                     cudaStream_t st) {
-    k_scatter<<<g.sm_count * 8, 256, 0, st>>>(keys, vals, ctr, cap, prefix_shift, n_buckets,
+    k_scatter<<<g.sm_count * 8, 256, 0, st>>>(keys, vals, ctr, cap, key_bits, bits,
                                                reinterpret_cast<unsigned long long*>(cursor), out_keys, out_vals);
 }
 
 int bucket_sort_capacity() { return kSortCap; }
 
-void launch_bucket_sort_warp(uint64_t* keys, uint64_t* vals, const uint64_t* starts, uint64_t n_buckets, int shift,
+void launch_bucket_sort_warp(uint64_t* keys, uint64_t* vals, const uint64_t* starts, uint64_t n_buckets, int key_bits,
                              DevCounters* ctr, const Grid& g, cudaStream_t st) {
     const uint64_t warps = n_buckets;
     unsigned grid = (unsigned)((warps + 7) / 8);
-    const unsigned cap = (unsigned)g.sm_count * 8;
+    const unsigned cap = (unsigned)g.sm_count * 6;  // one wave
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    k_bucket_sort_warp<<<grid, 256, 0, st>>>(keys, vals, starts, n_buckets, shift, ctr);
+    k_bucket_sort_warp<<<grid, 256, 0, st>>>(keys, vals, starts, n_buckets, key_bits, ctr);
+    grid = (unsigned)std::min<uint64_t>((n_buckets + 255) / 256, (uint64_t)g.sm_count * 2);
+    k_bucket_sort_warp_big<<<grid, 256, 0, st>>>(keys, vals, starts, n_buckets, ctr);
 }
 
 int warp_sort_capacity() { return kWarpSortMax; }

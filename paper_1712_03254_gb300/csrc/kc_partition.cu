@@ -784,12 +784,13 @@ __global__ void k_fb_compact(FallbackArgs F) {
 }
 
 __global__ void k_prefix_hist(const uint64_t* __restrict__ keys, DevCounters* __restrict__ ctr, uint64_t cap,
-                              int shift, uint64_t n_buckets, uint32_t* __restrict__ hist) {
+                              int key_bits, int bits, uint32_t* __restrict__ hist) {
     const uint64_t n = ctr->survivors < cap ? ctr->survivors : cap;
+    const bool even = even_buckets(key_bits, bits);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint64_t b = keys[i] >> shift;
-        if (b < n_buckets) atomicAdd(hist + b, 1u);
+        const uint64_t b = key_bucket(keys[i], key_bits, bits, even);
+        if (!(b >> bits)) atomicAdd(hist + b, 1u);
         else atomicOr(&ctr->err, DERR_INTERNAL);
     }
 }
@@ -1070,9 +1071,9 @@ void launch_fb_recount(const FallbackArgs& F, int bt, cudaStream_t st) {
 }
 void launch_fb_compact(const FallbackArgs& F, cudaStream_t st) { k_fb_compact<<<1024, 256, 0, st>>>(F); }
 
-void launch_prefix_hist(const uint64_t* keys, DevCounters* ctr, uint64_t cap, int shift, uint64_t n_buckets,
+void launch_prefix_hist(const uint64_t* keys, DevCounters* ctr, uint64_t cap, int key_bits, int bits,
                         uint32_t* hist, const Grid& g, cudaStream_t st) {
-    k_prefix_hist<<<g.sm_count * 4, 256, 0, st>>>(keys, ctr, cap, shift, n_buckets, hist);
+    k_prefix_hist<<<g.sm_count * 4, 256, 0, st>>>(keys, ctr, cap, key_bits, bits, hist);
 }
 
 }  // namespace kc

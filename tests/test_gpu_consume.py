@@ -192,6 +192,33 @@ def test_sort_buckets_at_both_ends_of_the_key_space():
     _count(codes[at], keys, repeats, 1, 1)
 
 
+@pytest.mark.parametrize("strategy", ["partitioned", "direct"])
+@pytest.mark.parametrize("same", [24, 20, 8])
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 63, 64, 65, 256, 257])
+def test_sort_bucket_of_n_keys(oracle_mod, n, same, strategy):
+    """n keys that begin with `same` As: they share the first sort bucket, spread over
+    its ranges (8) or all in one (20, where the keys' top 32 bits are equal, and 24)."""
+    rng = np.random.default_rng(1000 * same + n)
+    codes = rng.integers(0, 4, (4 * n, 31), dtype=np.uint8)
+    codes[:, :same], codes[:, 30] = 0, 1  # the reverse complement begins with G: these are the canonical ones
+    codes = np.unique(codes, axis=0)
+    codes = codes[np.sort(rng.permutation(len(codes))[:n])]
+    assert len(codes) == n
+    rows = np.repeat(np.arange(n), rng.integers(1, 5, n))
+    rng.shuffle(rows)
+    ascii = np.frombuffer(b"ACGT", np.uint8)[codes[rows]].reshape(-1)
+    rs = synth.ReadSet(ascii, np.arange(len(rows) + 1, dtype=np.uint64) * np.uint64(31))
+    w = synth.Workload("bucket", [rs], 31, 1 << 16, 4, 1)
+    o = oracle_mod.count(w)
+    kw = dict(table_slots=1 << 12) if strategy == "direct" else {}
+    c = kc.KmerCounter(31, 1, 1 << 16, 4, 1, strategy=strategy, **kw)
+    c.add_readset(0, rs)
+    c.finalize()
+    assert len(c.dump()[0]) == n
+    _same(c, o)
+    c.close()
+
+
 @pytest.mark.parametrize("k", [31, 20])
 @pytest.mark.parametrize("part_bits", [13, 14])
 @pytest.mark.parametrize("place", ["device", "chunked"])
