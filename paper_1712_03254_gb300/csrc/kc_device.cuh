@@ -379,6 +379,109 @@ __host__ __device__ __forceinline__ bool even_buckets(int key_bits, int bits) {
     return key_bits >= 32 && bits >= 1;
 }
 
+// Exclusive scan of n counters into starts (and starts[n], the total) and
+// cursor, in one launch: each CTA takes the next tile by ticket, adds it up,
+// publishes the sum and looks back over the tiles before it, 32 at a time,
+// until one has published its whole prefix (Merrill and Garland's decoupled
+// look-back).  A tile waits only for tiles of smaller tickets, whose CTAs run
+// already; the wait is bounded all the same, and a tile that gives up adds the
+// counters before it itself.  state, a word per tile, and ticket are zero
+// before.
+constexpr int kScanThreads = 256;
+constexpr uint64_t kScanTile = 4 * kScanThreads;
+constexpr int kScanPolls = 1 << 22;
+__device__ __forceinline__ void scan_lookback(const uint32_t* __restrict__ hist, uint64_t n,
+                                              uint64_t* __restrict__ starts, uint64_t* __restrict__ cursor,
+                                              unsigned long long* state, unsigned long long* ticket) {
+    constexpr unsigned long long kSum = 1ull << 62, kPrefix = 2ull << 62, kValue = kSum - 1;
+    constexpr int nw = kScanThreads / 32;
+    __shared__ unsigned long long s_w[nw];
+    __shared__ unsigned long long s_prefix, s_tile;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1ull);
+    __syncthreads();
+    const uint64_t tile = s_tile;
+    if (tile * kScanTile >= n) return;
+    const uint64_t i0 = tile * kScanTile + 4 * threadIdx.x;
+    const bool wide = i0 + 4 <= n && !((reinterpret_cast<uintptr_t>(hist) | reinterpret_cast<uintptr_t>(starts) |
+                                        reinterpret_cast<uintptr_t>(cursor)) & 15u);
+    uint32_t c[4];
+    if (wide) {
+        const uint4 q = *reinterpret_cast<const uint4*>(hist + i0);
+        c[0] = q.x, c[1] = q.y, c[2] = q.z, c[3] = q.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c[j] = i0 + j < n ? hist[i0 + j] : 0u;
+    }
+    const unsigned long long sum = (unsigned long long)c[0] + c[1] + c[2] + c[3];
+    unsigned long long incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_w[wid] = incl;
+    __syncthreads();
+    unsigned long long before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < nw; ++w) {
+        if (w < wid) before += s_w[w];
+        total += s_w[w];
+    }
+    volatile unsigned long long* const st = state;
+    if (wid == 0) {
+        if (lane == 0) st[tile] = (tile ? kSum : kPrefix) | total;
+        unsigned long long prefix = 0;
+        for (uint64_t at = tile; at > 0;) {  // tiles [0, at) are still to be added
+            unsigned long long v = kPrefix;  // before the first tile: nothing
+            for (int polls = 0; polls < kScanPolls; ++polls) {
+                if ((uint64_t)lane < at) v = st[at - 1 - lane];
+                if (__all_sync(0xffffffffu, v >> 62)) break;
+            }
+            if (__any_sync(0xffffffffu, !(v >> 62))) {
+                prefix = 0;
+                for (uint64_t i = lane; i < tile * kScanTile; i += 32) prefix += hist[i];
+#pragma unroll
+                for (int o = 16; o; o >>= 1) prefix += __shfl_xor_sync(0xffffffffu, prefix, o);
+                break;
+            }
+            const unsigned whole = __ballot_sync(0xffffffffu, v >> 63);
+            const int last = whole ? __ffs(whole) - 1 : 31;
+            unsigned long long x = lane <= last ? v & kValue : 0ull;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            prefix += x;
+            if (whole) break;
+            at -= 32;  // every lane had a tile
+        }
+        if (lane == 0) {
+            if (tile) st[tile] = kPrefix | (prefix + total);
+            s_prefix = prefix;
+        }
+    }
+    __syncthreads();
+    uint64_t run = s_prefix + before + incl - sum;
+    if (wide) {
+        const ulonglong2 a = make_ulonglong2(run, run + c[0]);
+        const ulonglong2 b = make_ulonglong2(a.y + c[1], a.y + c[1] + c[2]);
+        reinterpret_cast<ulonglong2*>(starts + i0)[0] = a;
+        reinterpret_cast<ulonglong2*>(starts + i0)[1] = b;
+        reinterpret_cast<ulonglong2*>(cursor + i0)[0] = a;
+        reinterpret_cast<ulonglong2*>(cursor + i0)[1] = b;
+        run += sum;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (i0 + j < n) {
+                starts[i0 + j] = run;
+                cursor[i0 + j] = run;
+            }
+            run += c[j];
+        }
+    }
+    if (i0 < n && i0 + 4 >= n) starts[n] = run;  // the thread holding the last counter
+}
+
 // Ranks of a bucket's n <= 64 distinct keys, two a lane (k0: element lane, k1:
 // element 32 + lane; in0, in1: whether there is one; two: n > 32), by one warp.
 // The keys of a bucket lie nearly evenly between its smallest and its largest,

@@ -192,6 +192,25 @@ def test_sort_buckets_at_both_ends_of_the_key_space():
     _count(codes[at], keys, repeats, 1, 1)
 
 
+@pytest.mark.parametrize("sizes", [[32768], [32768, 1], [1, 32768], [31 * 32] * 32 + [1], [32768] * 33 + [40]])
+def test_sort_starts_over_several_tiles(sizes):
+    """Batches whose sort buckets (sizes / 32 each, at least one) fill one tile of 1024
+    counters exactly, pass it by one, and take more tiles than one look-back step."""
+    rng = np.random.default_rng(len(sizes))
+    jobs = []
+    for n in sizes:
+        codes, keys = _canonical_31mers(rng, n)
+        c = kc.KmerCounter(31, 1, 1 << 20, 4, 1, strategy="partitioned")
+        ascii = np.frombuffer(b"ACGT", np.uint8)[codes[rng.permutation(n)]].reshape(-1)
+        c.add_readset(0, synth.ReadSet(ascii, np.arange(n + 1, dtype=np.uint64) * np.uint64(31)))
+        jobs.append((c, keys))
+    kc.KcBatch().finalize([c for c, _ in jobs])
+    for c, keys in jobs:
+        got, counts = c.dump()
+        assert np.array_equal(got, keys) and np.all(counts == 1)
+        c.close()
+
+
 @pytest.mark.parametrize("strategy", ["partitioned", "direct"])
 @pytest.mark.parametrize("same", [24, 20, 8])
 @pytest.mark.parametrize("n", [2, 31, 32, 33, 63, 64, 65, 256, 257])
