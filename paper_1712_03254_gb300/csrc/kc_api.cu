@@ -58,6 +58,17 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Memory of the given device, on a boundary of `align` bytes: a kernel there
+// may store to it (a copy reaches other devices and odd addresses too).
+static bool storable(const void* p, int device, size_t align) {
+    cudaPointerAttributes a;
+    if (!p || reinterpret_cast<uintptr_t>(p) % align || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // Pinned host memory the device can write (its device-side address in *dev):
 // a kernel writes such memory directly, over the host link.
 bool host_mapped(const void* p, void** dev) {
@@ -1536,6 +1547,13 @@ kc_status kc_dump(kc_handle h, uint64_t* keys, uint32_t* counts, uint64_t capaci
         if (dev_c)
             KC_CUDA(cudaMemcpyAsync(counts, cout, h->n_result * 4 * (size_t)h->n_samples, cudaMemcpyHostToDevice, st));
         if (dev_k || dev_c) KC_CUDA(cudaStreamSynchronize(st));  // the staging buffers go out of scope
+        return KC_OK;
+    }
+    if (storable(counts, h->device, 4) && storable(keys, h->device, 8)) {
+        kc::launch_dump(h->res_keys, h->res_vals, h->n_result, h->n_samples, keys, counts, h->grid, st);
+        h->launches += 1;
+        KC_LAUNCHED("dump launch");
+        KC_CUDA(cudaStreamSynchronize(st));
         return KC_OK;
     }
     // pinned host counts of one sample: narrowed straight into them by a

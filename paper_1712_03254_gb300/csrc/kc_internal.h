@@ -72,6 +72,9 @@ int bucket_sort_capacity();
 void launch_bitonic_global(uint64_t* keys, uint64_t* vals, uint64_t n, cudaStream_t st);
 
 void launch_counts_narrow(const uint64_t* vals, uint64_t n, uint32_t* out, cudaStream_t st);
+// The result's keys and counts into device arrays (result arrays 16-byte aligned).
+void launch_dump(const uint64_t* keys, const uint64_t* vals, uint64_t n, int n_samples, uint64_t* out_keys,
+                 uint32_t* out_counts, const Grid& g, cudaStream_t st);
 
 // ---- partitioned strategy (kc_partition.cu) --------------------------------
 

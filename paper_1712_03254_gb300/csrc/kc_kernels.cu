@@ -456,6 +456,45 @@ __global__ void k_counts_narrow(const uint64_t* __restrict__ vals, uint64_t n, u
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = (uint32_t)vals[i];
 }
 
+// The result table into device arrays: keys as they are, the packed counts as
+// S 32-bit counts a key, in one pass (a copy of the keys and k_counts_narrow
+// read and wrote the same bytes one after the other).  Four keys a thread, 16
+// bytes at a time, where the caller's arrays are aligned for it.  Bound by the
+// memory: 6.8 M keys 27 us, 12.3 M of two samples 67 us (5.9 TB/s); a dump call
+// of 5.3 M keys 72 -> 58 us.
+template <int S>
+__global__ void __launch_bounds__(256) k_dump(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ vals,
+                                              uint64_t n, uint64_t* __restrict__ out_keys,
+                                              uint32_t* __restrict__ out_counts) {
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    uint64_t done = 0;
+    if (!((reinterpret_cast<uintptr_t>(out_keys) | reinterpret_cast<uintptr_t>(out_counts)) & 15u)) {
+        const ulonglong2 *k2 = reinterpret_cast<const ulonglong2*>(keys), *v2 = reinterpret_cast<const ulonglong2*>(vals);
+        ulonglong2* ok = reinterpret_cast<ulonglong2*>(out_keys);
+        const uint64_t quads = n >> 2;
+        for (uint64_t q = t; q < quads; q += stride) {
+            const ulonglong2 a = k2[2 * q], b = k2[2 * q + 1], x = v2[2 * q], y = v2[2 * q + 1];
+            ok[2 * q] = a;
+            ok[2 * q + 1] = b;
+            if (S == 1) {
+                reinterpret_cast<uint4*>(out_counts)[q] =
+                    make_uint4((uint32_t)x.x, (uint32_t)x.y, (uint32_t)y.x, (uint32_t)y.y);
+            } else {
+                reinterpret_cast<ulonglong2*>(out_counts)[2 * q] = x;
+                reinterpret_cast<ulonglong2*>(out_counts)[2 * q + 1] = y;
+            }
+        }
+        done = quads << 2;
+    }
+    for (uint64_t i = done + t; i < n; i += stride) {
+        const uint64_t v = vals[i];
+        out_keys[i] = keys[i];
+        out_counts[S * i] = (uint32_t)v;
+        if (S == 2) out_counts[S * i + 1] = (uint32_t)(v >> 32);
+    }
+}
+
 unsigned grid_for(uint64_t work, int block, int max_ctas) {
     uint64_t g = (work + block - 1) / block;
     if (g < 1) g = 1;
@@ -559,6 +598,13 @@ void launch_bitonic_global(uint64_t* keys, uint64_t* vals, uint64_t n, cudaStrea
         for (uint64_t stride = size >> 2; stride > 0; stride >>= 1)
             k_bitonic_step<<<grid, 256, 0, st>>>(keys, vals, n, n2, size, stride, 0);
     }
+}
+
+void launch_dump(const uint64_t* keys, const uint64_t* vals, uint64_t n, int n_samples, uint64_t* out_keys,
+                 uint32_t* out_counts, const Grid& g, cudaStream_t st) {
+    const unsigned grid = grid_for((n + 3) / 4, 256, g.sm_count * 8);
+    if (n_samples == 2) k_dump<2><<<grid, 256, 0, st>>>(keys, vals, n, out_keys, out_counts);
+    else k_dump<1><<<grid, 256, 0, st>>>(keys, vals, n, out_keys, out_counts);
 }
 
 void launch_counts_narrow(const uint64_t* vals, uint64_t n, uint32_t* out, cudaStream_t st) {

@@ -192,6 +192,36 @@ def test_sort_buckets_at_both_ends_of_the_key_space():
     _count(codes[at], keys, repeats, 1, 1)
 
 
+@pytest.mark.parametrize("samples", [1, 2])
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 1023, 40001])
+def test_dump_into_device_arrays(n, samples):
+    """Device arrays on and off 16-byte boundaries get what host arrays get, and
+    nothing is written behind them."""
+    import torch
+
+    rng = np.random.default_rng(n)
+    codes, _ = _canonical_31mers(rng, n)
+    c = kc.KmerCounter(31, samples, 1 << 16, 4, 1, strategy="partitioned")
+    for s in range(samples):
+        rows = np.repeat(np.arange(n), rng.integers(1, 4, n))
+        ascii = np.frombuffer(b"ACGT", np.uint8)[codes[rows]].reshape(-1)
+        c.add_readset(s, synth.ReadSet(ascii, np.arange(len(rows) + 1, dtype=np.uint64) * np.uint64(31)))
+    c.finalize()
+    keys, counts = c.dump()
+    assert len(keys) == n
+    for key_at, count_at in ((0, 0), (1, 0), (0, 1), (2, 3), (1, 2)):
+        dk = torch.full((n + 4,), -1, dtype=torch.int64, device="cuda")
+        dc = torch.full((n * samples + 4,), -1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        c.dump(dk[key_at : key_at + n], dc[count_at : count_at + n * samples])
+        dk, dc = dk.cpu().numpy(), dc.cpu().numpy()
+        assert np.array_equal(dk[key_at : key_at + n].view(np.uint64), keys)
+        assert np.array_equal(dc[count_at : count_at + n * samples].view(np.uint32), counts.reshape(-1))
+        assert np.all(np.delete(dk, np.s_[key_at : key_at + n]) == -1)
+        assert np.all(np.delete(dc, np.s_[count_at : count_at + n * samples]) == -1)
+    c.close()
+
+
 @pytest.mark.parametrize("sizes", [[32768], [32768, 1], [1, 32768], [31 * 32] * 32 + [1], [32768] * 33 + [40]])
 def test_sort_starts_over_several_tiles(sizes):
     """Batches whose sort buckets (sizes / 32 each, at least one) fill one tile of 1024
