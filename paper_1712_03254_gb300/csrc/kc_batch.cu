@@ -102,7 +102,11 @@ constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32
 //            in four at 30x coverage) go to a queue of the warp; 32 of them at a
 //            time take two probes (and a claim) each and go back to the queue if
 //            both failed, so every probe step has all its lanes.  (One probe a
-//            step and four hashes in flight instead of three: 0.680 ms.)
+//            step and four hashes in flight instead of three: 0.680 ms.)  With
+//            one sample a new key whose first slot is free claims it at once:
+//            2.9e7 windows of which 64 % are new keys 0.435 -> 0.412 ms, 1.2e8
+//            of which 18 % are as before; with two samples, where fewer warps
+//            run, 4.7e8 windows took 2.95 ms without and 2.99 with it.
 //   emit     keys of at least min_count, one position claim per warp
 //   filter   the counts are no longer needed: their memory takes the filter
 //            words, every key sets its bits, the words are written out
@@ -133,6 +137,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
     __shared__ int s_fail, s_hint;
     __shared__ unsigned s_item;
     constexpr int kWarps = THREADS / 32;
+    constexpr bool kClaimAtOnce = ONE;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t n_items = D->n_items;
@@ -188,8 +193,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             // a + sl <= 32 bits of its hash equal those of `range`
             const uint64_t range = hpre | ((uint64_t)sub << sub_shift);
             const uint32_t rhi = (uint32_t)(range >> 32), rmask = ~0u << (32 - a - sl);
-            for (uint32_t i = threadIdx.x; i < T; i += THREADS) sk[i] = empty;
-            for (uint32_t i = threadIdx.x; i < (T << s2); i += THREADS) sc[i] = 0u;
+            for (uint32_t i = threadIdx.x; i < T / 2; i += THREADS)
+                reinterpret_cast<ulonglong2*>(sk)[i] = make_ulonglong2(empty, empty);
+            for (uint32_t i = threadIdx.x; i < (T << s2) / 4; i += THREADS)
+                reinterpret_cast<uint4*>(sc)[i] = make_uint4(0u, 0u, 0u, 0u);
             if (threadIdx.x == 0) s_fail = 0;
             __syncthreads();
             bool stop = false;  // the same in all lanes of a warp
@@ -265,7 +272,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                             const uint64_t h = hc[e];
                             const bool in = ((((uint32_t)(h >> 32)) ^ rhi) & rmask) == 0u;  // else run padding, or another sub-range
                             const uint32_t s = (uint32_t)h & tmask;
-                            const unsigned long long cur = sk[s];
+                            unsigned long long cur = sk[s];
+                            if (kClaimAtOnce && in && cur == empty) {
+                                cur = atomicCAS(sk + s, empty, h);
+                                if (cur == empty) cur = h;
+                            }
                             const bool hit = in && cur == h;  // (padding may hold the empty mark)
                             if (hit) atomicAdd(scol + (s << s2), 1u);
                             const unsigned miss = __ballot_sync(kFull, in && !hit);
@@ -273,7 +284,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                                 if (in && !hit) {
                                     const unsigned pos = q + __popc(miss & lt);
                                     wq[pos] = h;
-                                    ws[pos] = cur == empty ? s : 0x10000u | ((s + 1) & tmask);
+                                    ws[pos] = !kClaimAtOnce && cur == empty ? s : 0x10000u | ((s + 1) & tmask);
                                 }
                                 q += __popc(miss);
                                 while (q >= 32) step(32);
@@ -300,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             // emit: each warp its slots [wid * T / kWarps, ...), at most 32 rows of 32
             const uint32_t rows = T / THREADS;  // T >= 1024
             const uint32_t slot0 = wid * rows * 32 + lane;
-            unsigned kept = 0, n_kept = 0;  // lane r: the ballot of row r
+            unsigned kept = 0, n_kept = 0, once = 0;  // kept, once: lane r has the ballot of row r
             uint64_t n_win = 0;
             const uint32_t min_count = J.min_count;
             for (uint32_t r = 0; r < rows; ++r) {
@@ -308,11 +319,12 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                 const uint64_t sum = s2 ? (uint64_t)sc[2 * i] + sc[2 * i + 1] : (uint64_t)sc[i];
                 n_win += sum;
                 const unsigned ballot = __ballot_sync(kFull, sum != 0 && sum >= min_count);
-                if (lane == (int)r) kept = ballot;
+                const unsigned ones = __ballot_sync(kFull, sum == 1);
+                if (lane == (int)r) {
+                    kept = ballot;
+                    once = ones;
+                }
                 n_kept += __popc(ballot);
-                // a key seen once is marked by its top bit (unless that makes it the
-                // empty mark): the filter's candidates do not count it if its bits are new
-                if (sum == 1 && (sk[i] ^ kTopBit) != empty) sk[i] ^= kTopBit;
             }
             unsigned long long pos0 = 0;
             if (n_kept) {
@@ -331,9 +343,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                     const uint64_t pos = pos0 + lane;
                     if ((unsigned)lane < n && pos < sv_cap) {
                         const uint32_t i = ws[qn + lane];
-                        uint64_t h = sk[i];
-                        if ((h ^ hpre) & kTopBit) h ^= kTopBit;
-                        const uint64_t key = unmixer64(h);
+                        const uint64_t key = unmixer64(sk[i]);
                         sv_keys[pos] = key;
                         sv_vals[pos] = s2 ? (uint64_t)sc[2 * i] | ((uint64_t)sc[2 * i + 1] << 32) : (uint64_t)sc[i];
                         if (hist) atomicAdd(hist + key_bucket(key, key_bits, hist_bits, even), 1u);
@@ -379,7 +389,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
             for (uint32_t r = 0; r < rows; ++r) {
                 const uint64_t h = sk[slot0 + r * 32];
                 const unsigned used = __ballot_sync(kFull, h != empty);
-                if (h != empty) wq[qn + __popc(used & lt)] = h;
+                // a key seen once is queued with its top bit flipped: the filter's
+                // candidates do not count it if its bits are new
+                const unsigned ones = __shfl_sync(kFull, once, r);
+                if (h != empty) wq[qn + __popc(used & lt)] = (ones >> lane) & 1u ? h ^ kTopBit : h;
                 qn += __popc(used);
                 if (qn >= 32) set_bits(32);
             }
