@@ -178,6 +178,7 @@ void free_idle(kc_handle h) {
 
 cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
     *bytes = std::max<size_t>(*bytes, 16);
+    h->job_blocks += *bytes;
     size_t best = h->idle.size();
     for (size_t i = 0; i < h->idle.size(); ++i) {
         const size_t have = h->idle[i].bytes;
@@ -203,7 +204,7 @@ cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
 
 void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st) {
     if (!p) return;
-    if (h->reused && !h->cfg.device_budget && bytes >= kIdleMinBytes && h->idle.size() < kMaxIdleBlocks &&
+    if (h->keep_blocks && !h->cfg.device_budget && bytes >= kIdleMinBytes && h->idle.size() < kMaxIdleBlocks &&
         g_idle_bytes.load() + bytes <= idle_limit(h)) {
         h->idle.push_back({p, bytes});
         h->idle_bytes += bytes;
@@ -1179,6 +1180,9 @@ kc_status kc_create_ex(int k, int n_samples, uint64_t bloom_bits, int n_hashes, 
 kc_status kc_reset(kc_handle h) {
     if (!h) return fail(KC_ERR_ARG, "null handle");
     h->reused = h->reused || !h->batches.empty();
+    h->keep_blocks = h->reused && h->job_blocks <= idle_limit(h) / 2;
+    h->job_blocks = 0;
+    if (!h->keep_blocks) free_idle(h);
     free_batches(h);
     h->n_result = 0;  // the result arrays stay allocated for the next job (finalize reuses them)
     free_selection(h);
@@ -1216,7 +1220,7 @@ kc_status kc_reset(kc_handle h) {
 void kc_destroy(kc_handle h) {
     if (!h) return;
     if (h->stream) {
-        h->reused = false;
+        h->keep_blocks = false;
         free_batches(h);
         free_idle(h);
         free_result(h);

@@ -87,18 +87,19 @@ struct SpillRun {
     uint64_t n_items = 0;
 };
 
-// Pinned host memory the spilled runs are placed in; kept across kc_reset so
-// a repeated out-of-core job does not pin memory again.
 // Device blocks a handle keeps for its next job (idle between their uses): the
 // grouped hashes and the scratch of the grouping and the finalize, a few bytes
 // per base each.  Taking blocks of this size from the stream-ordered pool for
 // every job cost 0.35 ms each when several handles took turns (the pool maps
 // their memory anew).  A handle keeps blocks from its second job on
-// (kc_reset), unless it has a device budget, and all handles together at most
-// kIdleShare of the device's memory; kc_destroy gives them back, and so does a
-// failed allocation of the handle.  A block is taken for work ordered after
-// the handle's stream and left when the handle's stream is ordered after its
-// last use.
+// (kc_reset), unless it has a device budget or its last job took more than half
+// the share, and all handles together at most a kIdleShare-th of the device's
+// memory; kc_destroy gives them back, and so does a failed allocation of the
+// handle.  (A job that passes the share would keep some blocks and give others
+// back, in an order that has the pool map memory for every job: two samples of
+// 10,000,000 reads took 51 to 70 ms a job so, 55 with none kept.)  A block is
+// taken for work ordered after the handle's stream and left when the handle's
+// stream is ordered after its last use.
 struct IdleBlock {
     void* p = nullptr;
     size_t bytes = 0;
@@ -110,6 +111,8 @@ constexpr size_t kIdleMinBytes = 1ull << 20;  // smaller blocks come from the po
 // (cudaMemGetInfo takes 16 us); if that fails, they are handled as not fitting.
 constexpr uint64_t kSmallNeed = 64ull << 20;  // (below any batch copied in chunks)
 
+// Pinned host memory the spilled runs are placed in; kept across kc_reset so
+// a repeated out-of-core job does not pin memory again.
 struct PinnedChunk {
     uint64_t* p = nullptr;
     uint64_t words = 0, used = 0;
@@ -180,6 +183,8 @@ struct kc_ctx {
     std::vector<kcapi::IdleBlock> idle;
     size_t idle_bytes = 0;
     bool reused = false;
+    bool keep_blocks = false;
+    size_t job_blocks = 0;  // bytes of blocks the job has taken
 
     kc::DevCounters host_ctr{};
     kcapi::State state = kcapi::State::Open;
