@@ -8,18 +8,21 @@
 // structures live in shared memory:
 //
 //   ingest (per kc_add_reads call)
-//     k_bucket_pass<count>  per window: canonical key, h = mixer64(key),
-//                           bucket = top a bits of h; per-CTA histogram in
-//                           shared memory, written out CTA-major
+//     k_extract_count       per window: canonical key, h = mixer64(key), into the
+//                           CTA's segment; bucket = top a bits of h; per-CTA
+//                           histogram in shared memory, written out CTA-major
+//                           (k_extract_groups: the same for two levels at once)
 //     k_bucket_offsets      per bucket: exclusive prefix over CTAs, totals
 //     (scan)                bucket starts
-//     k_bucket_pass<scatter> the same windows again; each h is stored at the
-//                           next position of its CTA's run of its bucket (or
-//                           at a position from a global per-bucket cursor)
+//     k_scatter_staged_seg  each segment into its CTA's runs of the buckets, in
+//                           whole sectors
+//     k_bucket_pass         the other scatter modes: the windows counted, then
+//                           extracted again and stored one by one at the next
+//                           position of the run (or from a global cursor)
 //   finalize (the consumer itself is k_consume_q in kc_batch.cu: one CTA per
-//   partition holds the partition's filter words -- a contiguous slice, since
-//   the filter word is also a prefix of h -- and an open-addressing table in
-//   shared memory)
+//   partition holds an open-addressing table and then the partition's filter
+//   words -- a contiguous slice, since the filter word is also a prefix of h --
+//   in shared memory)
 //     k_fb_*                fallback for partitions whose shared-memory table
 //                           overflowed: the same steps with the partition's
 //                           filter slice and a table in global memory.
@@ -229,7 +232,7 @@ constexpr int kExtractThreads = 1024;
 // Units [lo, hi) by one CTA: its histogram row goes to counts[0 .. 2^a)
 // (added to it with accumulate: a later piece of the same segment) and its
 // segment (piece) descriptor to *seg.  K > 0: k = K known at compile time
-// (every shift of the rolling codes a constant); K = 0: k from p.
+// (the codes cut out at constant places); K = 0: k from p.
 template <bool kRange, int K>
 __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw,
                                               uint64_t lo, uint64_t hi, const PassParams& p, int a,
@@ -431,8 +434,10 @@ constexpr uint32_t kPieceMax = 1u << 31;  // hashes a scatter loop indexes with 
 
 // Bound by the shared-memory staging and the stores' requests: without its
 // stores a round takes two thirds of the time.  1.2e8 hashes into 4096 buckets
-// take 0.69 ms (2.7 TB/s read and written); 0.76 with two 16-byte stores a
-// sector, four hashes a thread placed one after the other and 64-bit cursors.
+// take 0.65 ms (2.9 TB/s read and written); 0.67 with every bucket's stage read
+// front half first (neighbouring lanes' 16-byte reads lie 32 bytes apart, so half
+// the buckets begin with the other half), 0.76 with two 16-byte stores a sector,
+// four hashes a thread placed one after the other and 64-bit cursors.
 //
 // Staged scatter of hashes already in memory.  CTA c moves segment c
 // (seg[c] = {offset into src, length, group}) into its padded runs, 5 hashes
@@ -567,7 +572,8 @@ __device__ __forceinline__ void scatter_segment(const uint64_t* __restrict__ src
                     if (fill[b] >= 4) {
                         const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(s_stage + (size_t)b * 4);
                         const uint32_t c = cursor[b];
-                        st_sector(out + ((uint64_t)c << 2), sp[0], sp[1]);
+                        const uint32_t first = (b >> 2) & 1u;  // the order within a sector is free
+                        st_sector(out + ((uint64_t)c << 2), sp[first], sp[first ^ 1u]);
                         cursor[b] = c + 1;
                         fill[b] = 0;
                     }
