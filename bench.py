@@ -5,8 +5,8 @@ A step is one whole counting job on the "mid" workload: a 5 Mbp i.i.d.
 uniform genome sequenced at 30x as 1,000,000 x 150 bp reads from both strands
 with 0.5 % substitutions and 0.05 % N; k = 31, a 2^30-bit filter with 4 bits
 per key, a 2^24-slot table, min_count 2.  The step is reset (filter and table
-zeroed), ingest, pass 1 (filter + candidate claims), finalize (exact recount,
-compaction, sort) and dump.  The unit of work is one valid window (an N-free
+zeroed), ingest (windows extracted and grouped), finalize (exact counting,
+filter, compaction, sort) and dump.  The unit of work is one valid window (an N-free
 k-window inside one read).  Before the warm-up, kc_autotune picks the
 strategy and its knobs on the same device-resident reads (untimed; the
 choice and every trial are in the "tuning" field); --no-tune keeps the
@@ -274,8 +274,8 @@ def algorithmic_bytes(n_bases: int, windows: int, bloom_bits: int, table_slots: 
 def atomic_ceiling(rates: dict, strategy: int) -> dict:
     """Windows per second the random updates allow.  Per window the partitioned
     path makes 3 random shared-memory 32-bit adds (extraction histogram,
-    scatter stage fill, recount) and 1 shared-memory 64-bit OR (the filter
-    slice); the direct strategy makes 1 global 64-bit OR into the filter
+    scatter stage fill, count) and at most 1 shared-memory 64-bit OR (the
+    filter slice, updated once per distinct key); the direct strategy makes 1 global 64-bit OR into the filter
     (beyond L2) and its table probes."""
     if strategy == 1:
         per = {"hbm_or64": 1}

@@ -167,8 +167,8 @@ typedef struct kc_config {
                                      of the batch together: one persistent launch
                                      over a queue of (batch, unit range) items per
                                      phase (extraction, bucket offsets, starts,
-                                     run bases, staged scatter) instead of a set
-                                     of launches per kc_add_reads call.  The
+                                     staged scatter) instead of a set of launches
+                                     per kc_add_reads call.  The
                                      result is the same.                          */
     uint32_t reserved32;
 } kc_config;
@@ -214,7 +214,7 @@ typedef struct kc_stats {
      * extraction, inside pass1); sort = key-prefix bucketing and bucket sorts.  DIRECT: pass1 = filter update and
      * candidate claims, pass2 = exact recount, compact = survivor compaction.
      * PARTITIONED: pass1 = hash bucketing (count and scatter), pass2 = the
-     * shared-memory partition consumer (filter, claims, recount, compaction),
+     * shared-memory partition consumer (counting, compaction, filter),
      * compact = fallback partitions. */
     double ms_ingest, ms_pass1, ms_pass2, ms_compact, ms_sort;
     uint32_t strategy;              /* KC_STRATEGY_DIRECT or KC_STRATEGY_PARTITIONED */
@@ -264,7 +264,7 @@ kc_status kc_batch_finalize(kc_batch b, kc_handle* handles, int n);
  * and group the reads that the n handles' kc_add_reads calls kept, all
  * together on the batch's stream -- a persistent extraction launch over a
  * queue of (read batch, unit range) items of every job, one launch each for
- * the bucket offsets, starts and run bases of all of them, and a persistent
+ * the bucket offsets and the starts of all of them, and a persistent
  * staged-scatter launch over the same items.  Handles without kept reads, or
  * not partitioned or open, are left alone.  The call does not wait for the
  * device: each handle's stream is ordered after the work, so a later

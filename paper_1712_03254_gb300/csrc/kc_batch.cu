@@ -5,9 +5,9 @@
 // partition's keys in a shared-memory table, writes the survivors and the
 // partition's filter words and moves on, so uneven jobs share the GPU without a
 // launch each.
-// Sort: every job's survivors are bucketed by the top bits of their key into
-// one flat bucket array covering all jobs, scanned once, scattered into each
-// job's own result arrays, and each bucket sorted by one warp.  These launches
+// Sort: every job's survivors are bucketed by key (key_bucket) into one flat
+// bucket array covering all jobs, scanned once, scattered as pairs, and each
+// bucket sorted by one warp into its job's result arrays.  These launches
 // read every size and pointer from a device-side batch descriptor, so the
 // sequence is captured once in a CUDA graph and replayed for every batch.
 // A single kc_finalize is a batch of one.

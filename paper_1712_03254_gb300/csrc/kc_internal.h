@@ -142,10 +142,9 @@ void launch_scatter_staged_seg(const uint64_t* src, const SegDesc* segs, int n_s
 // Batched ingest: the read batches of several jobs extracted and grouped by
 // one set of launches.  Each batch is cut into items of whole units; the
 // extraction and the staged scatter are persistent kernels over the item
-// queue, the per-bucket offsets, scans and run bases cover every batch in one
-// launch each.  Per batch: histogram rows and segments of its items, its
-// linear hashes, the runs' relative and absolute bases, its bucket totals and
-// starts (the batch's partition starts) and its grouped hashes.
+// queue, the per-bucket offsets and scans cover every batch in one launch each.  Per batch: histogram rows and segments of its items, its
+// linear hashes, the runs' bases in their buckets, its bucket totals and starts
+// (the batch's partition starts) and its grouped hashes.
 struct IngestBatch {
     const uint64_t* pw;
     const uint64_t* vw;

@@ -11,8 +11,8 @@
 //             input).
 // Compaction  keys whose summed count reaches min_count (this removes the
 //             filter's false positives, Section III, Unify).
-// Sort        bucket by top key bits, then sort each bucket in shared memory
-//             (bitonic network), giving ascending keys.
+// Sort        bucket by key, then sort each bucket: a warp ranks up to 64 keys
+//             by key range, larger ones take bitonic networks; ascending keys.
 
 #include <atomic>
 
