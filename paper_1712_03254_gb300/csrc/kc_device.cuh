@@ -241,6 +241,28 @@ __device__ __forceinline__ UnitWords load_unit(const uint64_t* __restrict__ pw, 
     return r;
 }
 
+// Part `part` of 2^lp of unit u: the windows that start in its 64 >> lp bases,
+// moved to the front.  The words are padded as above.
+__device__ __forceinline__ UnitWords load_part(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw,
+                                               uint64_t u, int part, int lp) {
+    const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(pw) + u);
+    UnitWords r{p.x, p.y, __ldg(pw + 2 * u + 2), __ldg(vw + u)};
+    int skip = part << (6 - lp);  // bases
+    r.v = (r.v << skip) & (~0ull << (64 - (64 >> lp)));
+    if (skip >= 32) {
+        r.w0 = r.w1;
+        r.w1 = r.w2;
+        r.w2 = 0;
+        skip -= 32;
+    }
+    if (skip) {
+        r.w0 = r.w0 << 2 * skip | r.w1 >> (64 - 2 * skip);
+        r.w1 = r.w1 << 2 * skip | r.w2 >> (64 - 2 * skip);
+        r.w2 <<= 2 * skip;
+    }
+    return r;
+}
+
 // Insert key (stored as key + 1) by linear probing.  Returns 1 if this call
 // claimed a new slot.  A probe sequence that wraps the whole table sets
 // DERR_TABLE_FULL and gives up.

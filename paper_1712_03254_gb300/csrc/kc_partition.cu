@@ -263,8 +263,14 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
     const uint64_t base = s_base;
     const int hist_shift = 32 - a;  // a <= 20: the partition is the top a bits of h's high word
     const unsigned lt = (1u << lane) - 1u;
-    for (uint64_t g = lo + (uint64_t)wid * 32; g < hi; g += (uint64_t)nwarps * 32) {
-        const UnitWords uw = load_unit(pw, vw, g + lane, hi, lane);
+    // lanes of a short range take a half to an eighth of a unit each, so that more
+    // than a few of the CTA's warps have one (1.4 M windows: 14.3 -> 10.4 us)
+    int lp = 0;
+    while (lp < 3 && (hi - lo) << (lp + 1) <= blockDim.x) ++lp;
+    for (uint64_t g = (lo << lp) + (uint64_t)wid * 32; g < hi << lp; g += (uint64_t)nwarps * 32) {
+        UnitWords uw{0, 0, 0, 0};
+        if (lp == 0) uw = load_unit(pw, vw, g + lane, hi, lane);
+        else if (g + lane < hi << lp) uw = load_part(pw, vw, (g + lane) >> lp, (int)(g + lane) & ((1 << lp) - 1), lp);
         const uint64_t vm = uw.v;
         const unsigned nv = (unsigned)__popcll(vm);
         // the warp's windows of these 32 units get consecutive positions,
@@ -276,7 +282,7 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
             if (lane == 0) wb = atomicAdd(&s_pos, tot);
             wb = __shfl_sync(kFull, wb, 0);
         }
-        // every lane walks the 64 window starts of its unit, eight at a time
+        // every lane walks the window starts of its unit, eight at a time
         WindowWords fw = window_words(uw.w0, uw.w1, uw.w2);
         ReverseWords rv = reverse_words(uw.w0, uw.w1, uw.w2);
         const auto window = [&](uint64_t fwd, uint64_t rc, bool has) {
@@ -295,7 +301,7 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
             if (!kRange) wb += __popc(ballot);
         };
         uint64_t vbits = vm;  // the eight windows' valid bits on top
-        for (int j = 0; j < 64; j += 8, vbits <<= 8) {
+        for (int j = 0; j < 64 >> lp; j += 8, vbits <<= 8) {
             const unsigned valid = (unsigned)(vbits >> 56);
             window(forward_code<K, 0>(fw, p.rc_shift), reverse_code<K, 0>(rv, p.kmask), valid & 128u);
             window(forward_code<K, 1>(fw, p.rc_shift), reverse_code<K, 1>(rv, p.kmask), valid & 64u);

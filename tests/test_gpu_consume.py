@@ -192,6 +192,32 @@ def test_sort_buckets_at_both_ends_of_the_key_space():
     _count(codes[at], keys, repeats, 1, 1)
 
 
+@pytest.mark.parametrize("k", [31, 17, 4])
+@pytest.mark.parametrize("units", [1, 2, 152 * 128, 152 * 128 + 1, 152 * 256, 152 * 512, 152 * 512 + 1])
+def test_units_in_parts(oracle_mod, k, units):
+    """Reads of so many 64-base units that each CTA's share lies at and above the
+    bounds where its lanes take an eighth, a quarter, a half of a unit or all of it."""
+    rng = np.random.default_rng(units)
+    genome = rng.integers(0, 4, 30_000, dtype=np.uint8)
+    n = units * 64 - 21
+    lengths = rng.integers(1, 200, n // 60 + 2)
+    offsets = np.concatenate([[0], np.minimum(np.cumsum(lengths), n)]).astype(np.uint64)
+    offsets = offsets[: int(np.searchsorted(offsets, n)) + 1]
+    offsets[-1] = n
+    starts = rng.integers(0, len(genome) - 6500, len(offsets) - 1)
+    codes = np.concatenate([genome[a : a + int(e - b)] for a, b, e in zip(starts, offsets[:-1], offsets[1:])])
+    ascii = np.frombuffer(b"ACGT", np.uint8)[codes].copy()
+    ascii[rng.integers(0, n, n // 500 + 1)] = ord("N")
+    w = synth.Workload("parts", [synth.ReadSet(ascii, offsets)], k, 1 << 16, 4, 2)
+    o = oracle_mod.count(w)
+    c = kc.KmerCounter(k, 1, 1 << 16, 4, 2, strategy="partitioned", part_bits=6)
+    c.add_readset(0, w.samples[0])
+    c.finalize()
+    _same(c, o)
+    assert c.stats()["windows"] == o.windows
+    c.close()
+
+
 @pytest.mark.parametrize("samples", [1, 2])
 @pytest.mark.parametrize("n", [1, 3, 4, 5, 1023, 40001])
 def test_dump_into_device_arrays(n, samples):
