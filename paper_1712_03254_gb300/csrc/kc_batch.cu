@@ -435,7 +435,6 @@ __global__ void k_reset_q(const BatchDesc* __restrict__ D) {
 // the flat arrays; the total into D->n_buckets.  More buckets than the arrays
 // hold (never, when the host sized them from the survivor capacities) is an
 // internal error and sorts nothing.
-// Then the scan's state is cleared.
 __device__ void plan_sort(BatchDesc* __restrict__ D) {
     JobDesc* jobs = const_cast<JobDesc*>(D->jobs);
     uint64_t total = 0, flat = 0;
@@ -474,10 +473,8 @@ __device__ void plan_sort(BatchDesc* __restrict__ D) {
 }
 __global__ void k_plan_q(BatchDesc* __restrict__ D) {
     if (threadIdx.x == 0) plan_sort(D);
-    __syncthreads();
-    const uint64_t n_tiles = (*(volatile uint64_t*)&D->n_buckets + kScanTile - 1) / kScanTile;
-    for (uint64_t i = threadIdx.x; i < n_tiles; i += blockDim.x) D->tiles[i] = 0ull;
-    if (threadIdx.x == 0) D->tiles[D->n_tiles] = 0ull;
+    if (threadIdx.x >= 32)  // meanwhile the other warps clear the scan's state (all of it: the plan is not known yet)
+        for (uint64_t i = threadIdx.x - 32; i <= D->n_tiles; i += blockDim.x - 32) D->tiles[i] = 0ull;
 }
 
 __global__ void k_zero_hist_q(const BatchDesc* __restrict__ D) {
@@ -877,7 +874,7 @@ kc_status capture_sort_graph(kc_batch_ctx* b, int early) {
     cudaGraph_t g = nullptr;
     KC_CUDA(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
     const unsigned grid2 = (unsigned)b->sm_count * 16;  // latency-bound atomics: many threads in flight
-    kc::k_plan_q<<<1, 128, 0, b->st>>>(b->d_desc);
+    kc::k_plan_q<<<1, 512, 0, b->st>>>(b->d_desc);
     if (!early) {
         kc::k_zero_hist_q<<<(unsigned)b->sm_count * 4, 256, 0, b->st>>>(b->d_desc);
         kc::k_prefix_hist_q<<<grid2, 256, 0, b->st>>>(b->d_desc);
