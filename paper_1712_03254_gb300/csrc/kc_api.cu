@@ -634,7 +634,17 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
                 total_units += hs[j]->batches[t].n_units;
             }
     if (refs.empty()) return KC_OK;
-    const uint64_t upi = std::max<uint64_t>(1ull << 12, (total_units + sm_count - 1) / sm_count);
+    // Units an item: the fewest for which all items run at once, one CTA an SM.
+    // (Rounded up batch by batch, an even share gave 12 batches 159 items, and the
+    // seven left over a second round: extraction 517 -> 384 us, scatter 969 -> 811.)
+    uint64_t upi = std::max<uint64_t>(1ull << 12, (total_units + sm_count - 1) / sm_count);
+    const auto n_items = [&](const Ref& r) { return (r.h->batches[r.t].n_units + upi - 1) / upi; };
+    const uint64_t max_items = std::max<uint64_t>(sm_count, refs.size());
+    for (;; upi += upi / 64) {
+        uint64_t items = 0;
+        for (const Ref& r : refs) items += n_items(r);
+        if (items <= max_items) break;
+    }
     std::vector<kc::IngestBatch> ib(refs.size());
     std::vector<uint32_t> item_batch;
     std::vector<void*> scratch(refs.size(), nullptr);
@@ -665,8 +675,8 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         all_k31 &= h->k == 31;
         B.a = h->l1_bits;
         B.item0 = (uint32_t)item_batch.size();
-        B.n_items = (uint32_t)((b.n_units + upi - 1) / upi);
-        B.upi = upi;
+        B.n_items = (uint32_t)n_items(refs[i]);
+        B.upi = B.n_items ? (b.n_units + B.n_items - 1) / B.n_items : upi;  // even shares of the batch
         B.ctr = h->ctr;
         B.bucket_off = plan.n_buckets;
         plan.n_buckets += P;

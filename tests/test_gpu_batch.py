@@ -157,6 +157,33 @@ def test_batched_ingest_equals_oracle(oracle_mod):
         assert c.stats()["windows"] == o.windows
 
 
+@pytest.mark.parametrize("bases", [[24_100_000, 20_300_000, 5_000], [45_000_000], [9_000_000] * 5])
+def test_batched_ingest_items_fill_the_sms_once(bases):
+    """Batches large enough that their items are cut for one per SM, even and uneven:
+    each job's table and filter equal those of the job grouped at kc_add_reads."""
+    rng = np.random.default_rng(len(bases))
+    g = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, 400_000, dtype=np.uint8)]
+    jobs = []
+    for i, n in enumerate(bases):
+        n_reads = n // 1000
+        starts = rng.integers(0, len(g) - 1000, n_reads)
+        ascii = g[(starts[:, None] + np.arange(1000)).reshape(-1)]
+        jobs.append((31 - 6 * (i % 2), synth.ReadSet(ascii, np.arange(n_reads + 1, dtype=np.uint64) * np.uint64(1000))))
+    counters = {}
+    for batched in (True, False):
+        counters[batched] = [kc.KmerCounter(k, 1, 1 << 24, 4, 2, strategy="partitioned", batched_ingest=batched)
+                             for k, _ in jobs]
+        for c, (_, rs) in zip(counters[batched], jobs):
+            c.add_readset(0, rs)
+    kc.KcBatch().finalize(counters[True])
+    for c, d in zip(counters[True], counters[False]):
+        d.finalize()
+        for x, y in zip(c.dump(), d.dump()):
+            assert np.array_equal(x, y)
+        assert np.array_equal(c.export_bloom(), d.export_bloom())
+        assert c.stats()["windows"] == d.stats()["windows"]
+
+
 def test_batched_ingest_alone_mixed_and_reused(oracle_mod):
     """A batched-ingest job finalized alone (kc_finalize), a batch mixing
     batched-ingest jobs with jobs grouped at kc_add_reads, and a handle reset
