@@ -242,11 +242,18 @@ __device__ __forceinline__ UnitWords load_unit(const uint64_t* __restrict__ pw, 
 }
 
 // Part `part` of 2^lp of unit u: the windows that start in its 64 >> lp bases,
-// moved to the front.  The words are padded as above.
+// moved to the front.  n_words as above.
 __device__ __forceinline__ UnitWords load_part(const uint64_t* __restrict__ pw, const uint64_t* __restrict__ vw,
-                                               uint64_t u, int part, int lp) {
-    const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(pw) + u);
-    UnitWords r{p.x, p.y, __ldg(pw + 2 * u + 2), __ldg(vw + u)};
+                                               uint64_t u, int part, int lp, uint64_t n_words = ~0ull) {
+    UnitWords r{0, 0, 0, __ldg(vw + u)};
+    if (2 * u + 1 < n_words) {
+        const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(pw) + u);
+        r.w0 = p.x;
+        r.w1 = p.y;
+        if (2 * u + 2 < n_words) r.w2 = __ldg(pw + 2 * u + 2);
+    } else if (2 * u < n_words) {
+        r.w0 = __ldg(pw + 2 * u);
+    }
     int skip = part << (6 - lp);  // bases
     r.v = (r.v << skip) & (~0ull << (64 - (64 >> lp)));
     if (skip >= 32) {
@@ -261,6 +268,14 @@ __device__ __forceinline__ UnitWords load_part(const uint64_t* __restrict__ pw, 
         r.w2 <<= 2 * skip;
     }
     return r;
+}
+
+// log2 of the parts, at most eight a unit, that give n units' lanes something to
+// do without passing `lanes`.
+__device__ __forceinline__ int parts_log2(uint64_t n, uint64_t lanes) {
+    int lp = 0;
+    while (lp < 3 && n << (lp + 1) <= lanes) ++lp;
+    return lp;
 }
 
 // Insert key (stored as key + 1) by linear probing.  Returns 1 if this call

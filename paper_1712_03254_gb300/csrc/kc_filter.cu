@@ -298,12 +298,21 @@ __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE 
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     unsigned long long found = 0;
-    for (uint64_t base = warp * 32; base < n_units; base += n_warps * 32) {
+    // The units in whole rounds of the grid's lanes, then the rest, whose lanes take
+    // a half to an eighth of a unit each if they are few (9.03 rounds: 188 -> 176 us
+    // and 285 -> 278, no hits and 1.5 M).
+    const uint64_t rest = n_units / (n_warps * 32) * (n_warps * 32);
+    for (int lp = 0, at_rest = rest == 0; at_rest < 2; ++at_rest) {
+    if (at_rest) lp = parts_log2(n_units - rest, n_warps * 32);
+    const uint64_t end = at_rest ? n_units : rest;
+    for (uint64_t base = ((at_rest ? rest : 0) << lp) + warp * 32; base < end << lp; base += n_warps * 32) {
         const uint64_t u = base + lane;
-        const UnitWords uw = load_unit(pw, vw, u, n_units, lane, n_words);
+        UnitWords uw{0, 0, 0, 0};
+        if (lp == 0) uw = load_unit(pw, vw, u, end, lane, n_words);
+        else if (u < end << lp) uw = load_part(pw, vw, u >> lp, (int)u & ((1 << lp) - 1), lp, n_words);
         uint64_t vm = uw.v, hm = 0;
         WindowWords w = window_words(uw.w0, uw.w1, uw.w2);
-        for (int j0 = 0; j0 < 64; j0 += 8, vm <<= 8) {  // eight windows: their bits on top of vm
+        for (int j0 = 0; j0 < 64 >> lp; j0 += 8, vm <<= 8) {  // eight windows: their bits on top of vm
             unsigned hits = 0;
             const unsigned valid = (unsigned)(vm >> 56);
             if (valid) {
@@ -313,8 +322,14 @@ __global__ void __launch_bounds__(PRE ? kFilterThreadsPre : kFilterThreads, PRE 
             hm = (hm << 8) | hits;
             next_windows(w);
         }
-        if (u < n_units) hitmask[u] = hm;
+        if (u < end << lp) {  // the first window's bit is the unit's highest: part 0 is its last bytes
+            if (lp == 0) hitmask[u] = hm;
+            else if (lp == 1) reinterpret_cast<uint32_t*>(hitmask)[u ^ 1] = (uint32_t)hm;
+            else if (lp == 2) reinterpret_cast<uint16_t*>(hitmask)[u ^ 3] = (uint16_t)hm;
+            else reinterpret_cast<uint8_t*>(hitmask)[u ^ 7] = (uint8_t)hm;
+        }
         found += __popcll(hm);
+    }
     }
     found = warp_sum(found);
     if (lane == 0 && found) atomicAdd(&ctr->candidates, found);

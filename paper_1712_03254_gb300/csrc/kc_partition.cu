@@ -265,8 +265,7 @@ __device__ __forceinline__ void extract_range(const uint64_t* __restrict__ pw, c
     const unsigned lt = (1u << lane) - 1u;
     // lanes of a short range take a half to an eighth of a unit each, so that more
     // than a few of the CTA's warps have one (1.4 M windows: 14.3 -> 10.4 us)
-    int lp = 0;
-    while (lp < 3 && (hi - lo) << (lp + 1) <= blockDim.x) ++lp;
+    const int lp = parts_log2(hi - lo, blockDim.x);
     for (uint64_t g = (lo << lp) + (uint64_t)wid * 32; g < hi << lp; g += (uint64_t)nwarps * 32) {
         UnitWords uw{0, 0, 0, 0};
         if (lp == 0) uw = load_unit(pw, vw, g + lane, hi, lane);

@@ -75,3 +75,32 @@ def test_filter_reads_without_bases():
     hits, cand, n = c.filter_reads(np.zeros(1, np.uint64), offsets, np.zeros(1, np.uint64))
     assert n == 0 and len(cand) == 0 and not hits.any()
     c.close()
+
+
+@pytest.mark.parametrize("units", [155648 // 8, 155648 // 8 + 1, 155648 // 4, 155648 // 4 + 1, 155648 // 2,
+                                   155648 // 2 + 1, 155648 + 5])
+def test_filter_units_in_parts(units):
+    """Rescans whose units fill the lanes an eighth, a quarter, half or a whole time, exactly
+    and passed by one: the hits of every read are those of the reads scanned in pieces, and add
+    up to the selected keys' counts."""
+    rng = np.random.default_rng(units)
+    genome = rng.integers(0, 4, 20_000, dtype=np.uint8)
+    letters = np.frombuffer(b"ACGT", np.uint8)
+    n = units * 64 - 13
+    bounds = np.append(np.arange(0, n - 300, 150), n).astype(np.uint64)
+    starts = rng.integers(0, len(genome) - 500, len(bounds) - 1)
+    lengths = np.diff(bounds).astype(np.int64)
+    at = np.repeat(starts, lengths) + np.arange(n) - np.repeat(bounds[:-1].astype(np.int64), lengths)
+    tumour = synth.ReadSet(letters[genome[at]], bounds)
+    normal = synth.ReadSet.from_strings([letters[genome[:15_000]].tobytes().decode()])
+    c = kc.KmerCounter(25, 2, 1 << 20, 4, 2)
+    c.add_readset(0, normal)
+    c.add_readset(1, tumour)
+    c.finalize()
+    assert c.filter_select(tumor=1, min_tumor=2, max_normal=0) > 0
+    hits, _, _ = c.filter_readset(tumour)
+    assert int(hits.sum()) == int(c.filter_keys()[1][:, 1].sum())
+    pieces = np.array_split(np.arange(tumour.n_reads), 7)
+    parts = [c.filter_readset(tumour.slice(int(p[0]), int(p[-1]) + 1))[0] for p in pieces]
+    assert np.array_equal(hits, np.concatenate(parts))
+    c.close()
