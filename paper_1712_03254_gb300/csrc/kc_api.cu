@@ -61,8 +61,9 @@ bool is_device_ptr(const void* p) {
 // Memory of the given device, on a boundary of `align` bytes: a kernel there
 // may store to it (a copy reaches other devices and odd addresses too).
 static bool storable(const void* p, int device, size_t align) {
+    if (!p || reinterpret_cast<uintptr_t>(p) % align) return false;
     cudaPointerAttributes a;
-    if (!p || reinterpret_cast<uintptr_t>(p) % align || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
