@@ -107,7 +107,47 @@ std::mutex& sync_api_mutex() {
     static std::mutex m;
     return m;
 }
+
+namespace {
+// Allocations of this thread made to fail (kc_test_fail_alloc).
+struct AllocFaults {
+    uint64_t seen = 0, skip = 0, fails = 0;
+    bool next() {
+        ++seen;
+        if (!fails) return false;
+        if (skip) {
+            --skip;
+            return false;
+        }
+        --fails;
+        return true;
+    }
+};
+thread_local AllocFaults t_alloc_faults;
+}  // namespace
+
+cudaError_t dev_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = t_alloc_faults.next() ? cudaErrorMemoryAllocation : cudaMallocAsync(p, bytes, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+cudaError_t dev_alloc_fixed_bytes(void** p, size_t bytes) {
+    const cudaError_t e = t_alloc_faults.next() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
 }  // namespace kc
+
+// For the tests of the out-of-memory paths (not part of kc.h): of the calling
+// thread's device allocations the next `skip` are made as usual and the `fails`
+// after them report cudaErrorMemoryAllocation.  Returns how many the thread has
+// tried since the last call.
+extern "C" uint64_t kc_test_fail_alloc(uint64_t skip, uint64_t fails) {
+    const uint64_t seen = kc::t_alloc_faults.seen;
+    kc::t_alloc_faults = {0, skip, fails};
+    return seen;
+}
 
 
 namespace kcapi {
@@ -193,12 +233,11 @@ cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
         h->idle.erase(h->idle.begin() + best);
         return cudaSuccess;
     }
-    cudaError_t e = cudaMallocAsync(p, *bytes, st);
+    cudaError_t e = kc::dev_alloc(p, *bytes, st);
     if (e == cudaErrorMemoryAllocation && !h->idle.empty()) {
-        cudaGetLastError();
         free_idle(h);
         cudaStreamSynchronize(h->stream);
-        e = cudaMallocAsync(p, *bytes, st);
+        e = kc::dev_alloc(p, *bytes, st);
     }
     return e;
 }
@@ -395,8 +434,8 @@ kc_status regroup_batch(kc_handle h, Batch& b, cudaStream_t st) {
         return cuda_fail(err, "cudaMallocAsync(second partitioning level)");
     };
     if ((e = take_block(h, reinterpret_cast<void**>(&out), &out_bytes, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&starts, (P + 1) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&scratch, scratch_bytes, st)) != cudaSuccess)
+        (e = kc::dev_alloc(&starts, (P + 1) * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&scratch, scratch_bytes, st)) != cudaSuccess)
         return bail(e);
     char* q = static_cast<char*>(scratch);
     kc::SegDesc* dsegs = reinterpret_cast<kc::SegDesc*>(q);
@@ -483,7 +522,7 @@ kc_status bucket_two_levels(kc_handle h, Batch& b, uint64_t n_local, cudaStream_
     };
     b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
     if ((e = take_block(h, &scratch, &scratch_bytes, st)) != cudaSuccess || (e = pinned_words(h)) != cudaSuccess ||
-        (e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
         (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess)
         return bail(e);
     char* q = static_cast<char*>(scratch);
@@ -565,7 +604,7 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
     };
     b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
     if ((e = take_block(h, &scratch, &scratch_bytes, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
         (!exact && (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess))
         return bail(e);
     char* q = static_cast<char*>(scratch);
@@ -702,7 +741,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
         B.total = reinterpret_cast<uint32_t*>(q);
         b.hcap = b.n_local + 3 * cells;
         b.hash_bytes = std::max<uint64_t>(1, b.hcap) * 8;
-        if ((e = cudaMallocAsync(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
+        if ((e = kc::dev_alloc(&b.hstarts, (P + 1) * 8, st)) != cudaSuccess ||
             (e = take_block(h, reinterpret_cast<void**>(&b.hdata), &b.hash_bytes, st)) != cudaSuccess)
             return bail(e);
         B.starts = b.hstarts;
@@ -715,7 +754,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
     const size_t bytes = sizeof(kc::IngestPlan) + ib.size() * sizeof(kc::IngestBatch) + item_batch.size() * 4 + 16;
     char* blk = nullptr;
     cudaError_t e;
-    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&blk), bytes, st)) != cudaSuccess) return bail(e);
+    if ((e = kc::dev_alloc(reinterpret_cast<void**>(&blk), bytes, st)) != cudaSuccess) return bail(e);
     kc::IngestPlan* dplan = reinterpret_cast<kc::IngestPlan*>(blk);
     kc::IngestBatch* dbat = reinterpret_cast<kc::IngestBatch*>(blk + sizeof(kc::IngestPlan));
     unsigned* dhead = reinterpret_cast<unsigned*>(blk + sizeof(kc::IngestPlan) + ib.size() * sizeof(kc::IngestBatch));
@@ -830,9 +869,9 @@ kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64
     uint64_t *starts = nullptr, *cursor = nullptr;
     uint32_t* hist = nullptr;
     cudaError_t e;
-    if ((e = cudaMallocAsync(&hist, n_buckets * 4, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&starts, (n_buckets + 1) * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&cursor, n_buckets * 8, st)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&hist, n_buckets * 4, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&starts, (n_buckets + 1) * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&cursor, n_buckets * 8, st)) != cudaSuccess) {
         if (hist) cudaFreeAsync(hist, st);
         if (starts) cudaFreeAsync(starts, st);
         return cuda_fail(e, "cudaMallocAsync(sort buffers)");
@@ -901,8 +940,8 @@ kc_status sort_result(kc_handle h, uint64_t* tk, uint64_t* tv) {
     const uint64_t cap = std::max<uint64_t>(1, n);
     free_result(h);
     cudaError_t e;
-    if ((e = cudaMallocAsync(&h->res_keys, cap * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&h->res_vals, cap * 8, st)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&h->res_keys, cap * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&h->res_vals, cap * 8, st)) != cudaSuccess) {
         free_result(h);
         return cuda_fail(e, "cudaMallocAsync(result)");
     }
@@ -934,7 +973,7 @@ kc_status finalize_direct(kc_handle h) {
     const uint64_t cap = std::max<uint64_t>(1, h->host_ctr.claimed);
     uint64_t *tk = nullptr, *tv = nullptr;
     cudaError_t e;
-    if ((e = cudaMallocAsync(&tk, cap * 8, st)) != cudaSuccess || (e = cudaMallocAsync(&tv, cap * 8, st)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&tk, cap * 8, st)) != cudaSuccess || (e = kc::dev_alloc(&tv, cap * 8, st)) != cudaSuccess) {
         if (tk) cudaFreeAsync(tk, st);
         return cuda_fail(e, "cudaMallocAsync(compaction)");
     }
@@ -975,8 +1014,7 @@ kc_status resort_spilled(kc_handle h) {
     const uint64_t n = h->n_result;
     cudaStream_t st = h->stream;
     uint64_t *tk = nullptr, *tv = nullptr;
-    if (cudaMallocAsync(&tk, n * 8, st) != cudaSuccess || cudaMallocAsync(&tv, n * 8, st) != cudaSuccess) {
-        cudaGetLastError();
+    if (kc::dev_alloc(&tk, n * 8, st) != cudaSuccess || kc::dev_alloc(&tv, n * 8, st) != cudaSuccess) {
         if (tk) cudaFreeAsync(tk, st);
         return KC_ERR_OOM_DEVICE;
     }
@@ -1174,12 +1212,12 @@ kc_status kc_create_ex(int k, int n_samples, uint64_t bloom_bits, int n_hashes, 
     }
     const size_t bloom_bytes = bloom_bits / 8, table_bytes = slots * sizeof(kc::Slot);
     // stream-ordered pool allocations: no device-wide synchronisation
-    if ((e = cudaMallocAsync(&h->bloom, bloom_bytes + sizeof(kc::DevCounters), h->stream)) != cudaSuccess)
+    if ((e = kc::dev_alloc(&h->bloom, bloom_bytes + sizeof(kc::DevCounters), h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(filter)"));
     h->ctr = reinterpret_cast<kc::DevCounters*>(reinterpret_cast<char*>(h->bloom) + bloom_bytes);  // behind the filter
-    if (table_bytes && (e = cudaMallocAsync(&h->table, table_bytes, h->stream)) != cudaSuccess)
+    if (table_bytes && (e = kc::dev_alloc(&h->table, table_bytes, h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(table)"));
-    if (c.prune_chain && (e = cudaMallocAsync(&h->bloom2, bloom_bytes, h->stream)) != cudaSuccess)
+    if (c.prune_chain && (e = kc::dev_alloc(&h->bloom2, bloom_bytes, h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(second filter)"));
     h->fixed_bytes = bloom_bytes * (c.prune_chain ? 2 : 1) + table_bytes + sizeof(kc::DevCounters);
     kc_status s = kc_reset(h);
@@ -1296,7 +1334,7 @@ kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* p
     cudaError_t e = cudaSuccess;
     // the check's device counters (stream-ordered on the copy stream) and the
     // pinned word its error bits come back to, both kept with the handle
-    if (!h->chk_ctr && (e = cudaMallocAsync(&h->chk_ctr, sizeof(kc::DevCounters), cs)) != cudaSuccess) {
+    if (!h->chk_ctr && (e = kc::dev_alloc(&h->chk_ctr, sizeof(kc::DevCounters), cs)) != cudaSuccess) {
         release();
         return cuda_fail(e, "cudaMallocAsync(offsets check)");
     }
@@ -1428,8 +1466,8 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     // the read store (packed words, valid-window bits) and, for this call, the
     // read-start bits and the copies of the N mask and offsets
     void* temp = nullptr;
-    if ((e = cudaMallocAsync(&b.pw, (n_pwords + n_units) * 8, cs)) != cudaSuccess ||
-        (e = cudaMallocAsync(&temp, (n_units + (own_nm ? n_units : 0) + (own_off ? n_reads + 1 : 0)) * 8, cs)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&b.pw, (n_pwords + n_units) * 8, cs)) != cudaSuccess ||
+        (e = kc::dev_alloc(&temp, (n_units + (own_nm ? n_units : 0) + (own_off ? n_reads + 1 : 0)) * 8, cs)) != cudaSuccess) {
         if (b.pw) cudaFreeAsync(b.pw, cs);
         return cuda_fail(e, "cudaMallocAsync(read store)");
     }
@@ -1488,7 +1526,6 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     } else {
         s = bucket_batch(h, b, n_local, st, h->params(sample), false);
         if (s == KC_ERR_OOM_DEVICE && small_need(h, bucket_bytes(h, n_local))) {
-            cudaGetLastError();
             leave_hashes(h, b);  // no room after all: kept as reads
             b.deferred = true;
             ++h->deferred;
@@ -1591,7 +1628,7 @@ kc_status kc_dump(kc_handle h, uint64_t* keys, uint32_t* counts, uint64_t capaci
             h->launches += 1;
         } else {
             uint32_t* narrow = nullptr;
-            KC_CUDA(cudaMallocAsync(&narrow, h->n_result * 4, st));
+            KC_CUDA(kc::dev_alloc(&narrow, h->n_result * 4, st));
             kc::launch_counts_narrow(h->res_vals, h->n_result, narrow, st);
             h->launches += 1;
             KC_CUDA(cudaMemcpyAsync(counts, narrow, h->n_result * 4, cudaMemcpyDefault, st));

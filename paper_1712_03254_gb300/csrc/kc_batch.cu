@@ -801,7 +801,7 @@ kc_status grow(T*& p, size_t& cap, size_t need) {
     if (p) cudaFree(p);
     p = nullptr;
     cap = 0;
-    KC_CUDA(cudaMalloc(&p, n * sizeof(T)));
+    KC_CUDA(kc::dev_alloc_fixed(&p, n * sizeof(T)));
     cap = n;
     return KC_OK;
 }
@@ -815,8 +815,8 @@ kc_status ensure_jobs(kc_batch_ctx* b, size_t n_jobs, size_t n_items) {
         b->d_jobs = nullptr;
         b->d_counters = nullptr;
         b->jobs_cap = 0;
-        KC_CUDA(cudaMalloc(&b->d_jobs, n * sizeof(kc::JobDesc)));
-        KC_CUDA(cudaMalloc(&b->d_counters, 2 * n * sizeof(unsigned long long)));
+        KC_CUDA(kc::dev_alloc_fixed(&b->d_jobs, n * sizeof(kc::JobDesc)));
+        KC_CUDA(kc::dev_alloc_fixed(&b->d_counters, 2 * n * sizeof(unsigned long long)));
         b->jobs_cap = n;
     }
     size_t cap = b->items_cap;
@@ -852,10 +852,10 @@ kc_status ensure_buckets(kc_batch_ctx* b, uint64_t n_buckets) {
     b->d_tiles = nullptr;
     b->buckets_cap = 0;
     const uint64_t tiles = (n + kc::kScanTile - 1) / kc::kScanTile;
-    KC_CUDA(cudaMalloc(&b->d_hist, n * 4));
-    KC_CUDA(cudaMalloc(&b->d_starts, (n + 1) * 8));
-    KC_CUDA(cudaMalloc(&b->d_cursor, n * 8));
-    KC_CUDA(cudaMalloc(&b->d_tiles, (tiles + 1) * 8));
+    KC_CUDA(kc::dev_alloc_fixed(&b->d_hist, n * 4));
+    KC_CUDA(kc::dev_alloc_fixed(&b->d_starts, (n + 1) * 8));
+    KC_CUDA(kc::dev_alloc_fixed(&b->d_cursor, n * 8));
+    KC_CUDA(kc::dev_alloc_fixed(&b->d_tiles, (tiles + 1) * 8));
     b->buckets_cap = n;
     b->tiles_cap = tiles;
     for (cudaGraphExec_t& g : b->sort_graph)
@@ -1013,7 +1013,7 @@ kc_status run_fallbacks(kc_batch_ctx* b, JobWork& x, uint32_t j, uint32_t n_fail
     const uint64_t need = n_sv + extra;
     if (need > x.sv_cap) {
         uint64_t* nk = nullptr;
-        cudaError_t e = cudaMallocAsync(&nk, need * 16, b->st);
+        cudaError_t e = kc::dev_alloc(&nk, need * 16, b->st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(fallback survivors)");
         uint64_t* nv = nk + need;
         const uint64_t have = std::min<uint64_t>(n_sv, x.sv_cap);
@@ -1032,7 +1032,7 @@ kc_status run_fallbacks(kc_batch_ctx* b, JobWork& x, uint32_t j, uint32_t n_fail
         uint64_t slots = 1024;
         while (slots < 2 * windows_of(p)) slots <<= 1;
         kc::Slot* table = nullptr;
-        cudaError_t e = cudaMallocAsync(&table, slots * sizeof(kc::Slot), b->st);
+        cudaError_t e = kc::dev_alloc(&table, slots * sizeof(kc::Slot), b->st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(fallback table)");
         KC_CUDA(cudaMemsetAsync(table, 0, slots * sizeof(kc::Slot), b->st));
         KC_CUDA(cudaMemsetAsync(h->bloom + p * n_sw + w_lo, 0, (n_sw - w_lo) * 8, b->st));
@@ -1091,10 +1091,10 @@ kc_status kc_batch_create_internal(cudaStream_t st, kc_batch_ctx** out) {
     }
     {
         std::lock_guard<std::mutex> lk(kc::sync_api_mutex());
-        if ((e = cudaMalloc(&b->d_desc, sizeof(kc::BatchDesc))) != cudaSuccess ||
-            (e = cudaMalloc(&b->d_flags, 2 * sizeof(unsigned int))) != cudaSuccess)
-            return bail(cuda_fail(e, "cudaMalloc(batch descriptor)"));
+        if ((e = kc::dev_alloc_fixed(&b->d_desc, sizeof(kc::BatchDesc))) == cudaSuccess)
+            e = kc::dev_alloc_fixed(&b->d_flags, 2 * sizeof(unsigned int));
     }
+    if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc(batch descriptor)"));  // after the lock: bail takes it again
     *out = b;
     return KC_OK;
 }
@@ -1257,7 +1257,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         // handle's stream; the other one is written at once)
         x.sv_bytes = x.sv_cap * 16;
         if ((e = take_block(h, reinterpret_cast<void**>(&x.sv_keys), &x.sv_bytes, st)) != cudaSuccess ||
-            (e = cudaMallocAsync(&x.failed, P * 8 + meta_bytes, st)) != cudaSuccess) {
+            (e = kc::dev_alloc(&x.failed, P * 8 + meta_bytes, st)) != cudaSuccess) {
             release_work(b, work);
             return cuda_fail(e, "cudaMallocAsync(batch consumer)");
         }
@@ -1447,8 +1447,8 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         if (!h->res_keys || h->res_cap < cap) {
             free_result(h);
             cudaError_t e;
-            if ((e = cudaMallocAsync(&h->res_keys, cap * 8, st)) != cudaSuccess ||
-                (e = cudaMallocAsync(&h->res_vals, cap * 8, st)) != cudaSuccess) {
+            if ((e = kc::dev_alloc(&h->res_keys, cap * 8, st)) != cudaSuccess ||
+                (e = kc::dev_alloc(&h->res_vals, cap * 8, st)) != cudaSuccess) {
                 free_result(h);
                 release_work(b, work);
                 return cuda_fail(e, "cudaMallocAsync(result)");
@@ -1718,7 +1718,7 @@ kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
         if (!fits_device(h, need)) return finalize_spilled(b, h);
         kc_status s = finalize_core(b, hs, n, 0, 0xffffffffu, true);
         if (s != KC_ERR_OOM_DEVICE || !small_need(h, need)) return s;
-        cudaGetLastError();  // no room after all: counted again, group by group
+        // no room after all: counted again, group by group
         KC_CUDA(cudaMemsetAsync(&h->ctr->candidates, 0, 2 * sizeof(unsigned long long), b->st));  // and claimed
         KC_CUDA(cudaMemsetAsync(&h->ctr->split_parts, 0, sizeof(unsigned), b->st));
         return finalize_spilled(b, h);

@@ -628,7 +628,7 @@ struct Tiles {
     uint32_t* counts = nullptr;
     cudaError_t take(uint64_t items, cudaStream_t st) {
         n = std::max<uint64_t>(1, (items + kc::kTileItems - 1) / kc::kTileItems);
-        cudaError_t e = cudaMallocAsync(&starts, (n + 1) * 8 + n * 12, st);
+        cudaError_t e = kc::dev_alloc(&starts, (n + 1) * 8 + n * 12, st);
         if (e != cudaSuccess) return e;
         cursor = starts + n + 1;
         counts = reinterpret_cast<uint32_t*>(cursor + n);
@@ -681,7 +681,7 @@ kc_status kc_export_items(kc_handle h, kc_item16* items, uint64_t capacity, uint
     const bool dev = is_device_ptr(items);
     if (dev && reinterpret_cast<uintptr_t>(items) % 16 != 0) return fail(KC_ERR_ARG, "device items must be 16-byte aligned");
     ulonglong2* out = reinterpret_cast<ulonglong2*>(items);
-    if (!dev) KC_CUDA(cudaMallocAsync(&out, n * 16, st));
+    if (!dev) KC_CUDA(kc::dev_alloc(&out, n * 16, st));
     kc::k_items16<<<kc::grid_of(n, 256, h->grid.sm_count * 8), 256, 0, st>>>(h->res_keys, h->res_vals, n,
                                                                              h->n_samples, out);
     h->launches += 1;
@@ -703,7 +703,7 @@ kc_status kc_spectrum(kc_handle h, uint32_t cap, uint64_t* hist) {
     cudaStream_t st = h->stream;
     const bool dev = is_device_ptr(hist);
     uint64_t* out = hist;
-    if (!dev) KC_CUDA(cudaMallocAsync(&out, n_bins * 8, st));
+    if (!dev) KC_CUDA(kc::dev_alloc(&out, n_bins * 8, st));
     KC_CUDA(cudaMemsetAsync(out, 0, n_bins * 8, st));
     if (h->n_result) {
         kc::k_spectrum<<<kc::grid_of(h->n_result, 256, h->grid.sm_count * 2), 256, 0, st>>>(
@@ -731,9 +731,9 @@ static kc_status build_stems(kc_handle h) {
             if (q) cudaFreeAsync(q, st);
     };
     cudaError_t e;
-    if ((e = cudaMallocAsync(&rk, cap * 8, st)) != cudaSuccess || (e = cudaMallocAsync(&rv, cap * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&sk, cap * 8, st)) != cudaSuccess || (e = cudaMallocAsync(&sv, cap * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&sctr, sizeof(kc::DevCounters), st)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&rk, cap * 8, st)) != cudaSuccess || (e = kc::dev_alloc(&rv, cap * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&sk, cap * 8, st)) != cudaSuccess || (e = kc::dev_alloc(&sv, cap * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&sctr, sizeof(kc::DevCounters), st)) != cudaSuccess) {
         release();
         return cuda_fail(e, "cudaMallocAsync(stem records)");
     }
@@ -755,12 +755,12 @@ static kc_status build_stems(kc_handle h) {
         }
         kc_status s = sort_pairs(h, rk, rv, n_rec, 2 * (h->k - 2) + 4, sctr, sk, sv, kStems);
         if (s != KC_OK) return s;
-        KC_CUDA(cudaMallocAsync(&starts, std::max<uint64_t>(1, n_rec) * 8, st));
+        KC_CUDA(kc::dev_alloc(&starts, std::max<uint64_t>(1, n_rec) * 8, st));
         uint64_t n_items = 0;
         t0 = phase_begin(h);
         s = compact_ordered(h, kc::StemStartPred{sk}, kc::IndexWrite{starts}, n_rec, &n_items);
         if (s != KC_OK) return s;
-        KC_CUDA(cudaMallocAsync(&h->stem_items, std::max<uint64_t>(1, n_items) * sizeof(kc_stem_item), st));
+        KC_CUDA(kc::dev_alloc(&h->stem_items, std::max<uint64_t>(1, n_items) * sizeof(kc_stem_item), st));
         if (n_items)
             kc::k_stem_items<<<kc::grid_of(n_items, kc::kTileThreads, h->grid.sm_count * 8), kc::kTileThreads, 0, st>>>(
                 sk, sv, n_rec, starts, n_items, h->n_samples, reinterpret_cast<uint64_t*>(h->stem_items));
@@ -833,9 +833,9 @@ kc_status kc_filter_select(kc_handle h, const kc_filter_spec* spec, uint64_t* n_
     const uint64_t n_buckets = 1ull << lb;
     const bool pre = 2 * kept <= kc::kPreMaxEntries;
     const uint64_t table_bytes = n_buckets * kSelBucketBytes + (pre ? kc::kPreWords * 4ull : 0);
-    if ((e = cudaMallocAsync(&h->sel_keys, cap * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&h->sel_vals, cap * 8, st)) != cudaSuccess ||
-        (e = cudaMallocAsync(&h->sel_table, table_bytes, st)) != cudaSuccess) {
+    if ((e = kc::dev_alloc(&h->sel_keys, cap * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&h->sel_vals, cap * 8, st)) != cudaSuccess ||
+        (e = kc::dev_alloc(&h->sel_table, table_bytes, st)) != cudaSuccess) {
         tiles.leave(st);
         free_selection(h);
         return cuda_fail(e, "cudaMallocAsync(selection)");
@@ -939,7 +939,7 @@ kc_status kc_filter_reads(kc_handle h, const uint64_t* packed_reads, const uint6
     const size_t bytes = (own_pw ? n_pwords * 8 : 0) + n_units * 8 * (3 + (own_nm ? 1 : 0)) + (own_off ? (n_reads + 1) * 8 : 0) +
                          (own_cand ? n_reads * 8 : 0) + (hits_dev ? 0 : n_reads * 4) + sizeof(kc::DevCounters) + 16;
     cudaError_t e = cudaSuccess;
-    if ((e = cudaMallocAsync(&block, bytes, st)) != cudaSuccess || (e = tiles.take(n_reads, st)) != cudaSuccess ||
+    if ((e = kc::dev_alloc(&block, bytes, st)) != cudaSuccess || (e = tiles.take(n_reads, st)) != cudaSuccess ||
         (e = pinned_words(h)) != cudaSuccess) {
         release();
         return cuda_fail(e, "cudaMallocAsync(filter reads)");

@@ -20,6 +20,20 @@ void set_last_error(const std::string& msg);
 // lands inside another host thread's capture.
 std::mutex& sync_api_mutex();
 
+// Every device allocation of the library: stream-ordered from the pool, and
+// fixed (cudaMalloc, with sync_api_mutex() held).  A failure leaves no error
+// behind for a later cudaGetLastError to find.
+cudaError_t dev_alloc_bytes(void** p, size_t bytes, cudaStream_t st);
+cudaError_t dev_alloc_fixed_bytes(void** p, size_t bytes);
+template <class T>
+cudaError_t dev_alloc(T** p, size_t bytes, cudaStream_t st) {
+    return dev_alloc_bytes(reinterpret_cast<void**>(p), bytes, st);
+}
+template <class T>
+cudaError_t dev_alloc_fixed(T** p, size_t bytes) {
+    return dev_alloc_fixed_bytes(reinterpret_cast<void**>(p), bytes);
+}
+
 struct Grid {
     int sm_count = 152;
     int block = 256;

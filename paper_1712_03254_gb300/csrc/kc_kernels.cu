@@ -546,7 +546,7 @@ cudaError_t launch_scan(const uint32_t* hist, uint64_t n, uint64_t* starts, uint
     }
     const uint64_t n_tiles = (n + kScanTile - 1) / kScanTile;
     unsigned long long* state = nullptr;
-    cudaError_t e = cudaMallocAsync(&state, (n_tiles + 1) * 8, st);
+    cudaError_t e = dev_alloc(&state, (n_tiles + 1) * 8, st);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(state, 0, (n_tiles + 1) * 8, st);
     if (e == cudaSuccess) k_scan_long<<<(unsigned)n_tiles, kScanThreads, 0, st>>>(hist, n, starts, cursor, state, n_tiles);
