@@ -927,15 +927,27 @@ struct JobWork {
     void* meta = nullptr;
 };
 
-void release_work(kc_batch_ctx* b, std::vector<JobWork>& w) {
-    for (auto& x : w) {
-        if (x.sv_keys) cudaFreeAsync(x.sv_keys, b->st);
-        if (x.failed) cudaFreeAsync(x.failed, b->st);
-        x.sv_keys = x.sv_vals = nullptr;
-        x.failed = nullptr;
-        x.meta = nullptr;
+// The jobs' blocks of one finalize, given back when it returns.  They go to the
+// batch's stream, so that stream must be ordered after the handles' by then: a
+// survivors' block may be the scratch of a grouping still queued on its handle's
+// stream.  A finalize that fails before it has queued that order waits for the
+// handles here.
+struct WorkSet {
+    kc_batch_ctx* b;
+    std::vector<JobWork> jobs;
+    bool ordered = false;
+    WorkSet(kc_batch_ctx* batch, size_t n) : b(batch), jobs(n) {}
+    WorkSet(const WorkSet&) = delete;
+    WorkSet& operator=(const WorkSet&) = delete;
+    JobWork& operator[](size_t j) { return jobs[j]; }
+    ~WorkSet() {
+        for (auto& x : jobs) {
+            if (x.sv_keys && !ordered) cudaStreamSynchronize(x.h->stream);
+            if (x.sv_keys) cudaFreeAsync(x.sv_keys, b->st);
+            if (x.failed) cudaFreeAsync(x.failed, b->st);
+        }
     }
-}
+};
 
 // prepare: set the kernel's shared-memory limit (before any capture);
 // otherwise launch it.
@@ -1127,7 +1139,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     if (!b || !hs || n < 0) return fail(KC_ERR_ARG, "null argument");
     if (n == 0) return KC_OK;
     cudaStream_t st = b->st;
-    std::vector<JobWork> work((size_t)n);
+    WorkSet work(b, (size_t)n);
     const bool one = n == 1 && hs[0]->stream == st;  // no cross-stream ordering needed
     const bool timed = n == 1;                         // phase times go to the only handle
     bool fast = true;  // every job whole: sized from host counts (below)
@@ -1151,6 +1163,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
                 KC_CUDA(cudaEventRecord(hs[j]->ev_main, hs[j]->stream));
                 KC_CUDA(cudaStreamWaitEvent(st, hs[j]->ev_main, 0));
             }
+        work.ordered = true;
         return KC_OK;
     };
     if (!fast) {
@@ -1230,7 +1243,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         while (tl > 10 && kc::consume_smem(h->slice_log2 - split_min, tl, h->n_samples) + queue > (size_t)b->max_optin) --tl;
         const size_t smem = kc::consume_smem(h->slice_log2 - split_min, tl, h->n_samples);
         if (smem + queue > (size_t)b->max_optin) {
-            release_work(b, work);
             return fail(KC_ERR_INTERNAL, "partition does not fit shared memory");
         }
         smem_max = std::max(smem_max, smem);
@@ -1258,7 +1270,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         x.sv_bytes = x.sv_cap * 16;
         if ((e = take_block(h, reinterpret_cast<void**>(&x.sv_keys), &x.sv_bytes, st)) != cudaSuccess ||
             (e = kc::dev_alloc(&x.failed, P * 8 + meta_bytes, st)) != cudaSuccess) {
-            release_work(b, work);
             return cuda_fail(e, "cudaMallocAsync(batch consumer)");
         }
         x.sv_vals = x.sv_keys + x.sv_cap;
@@ -1304,7 +1315,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     const uint32_t n_items = (uint32_t)b->item_job.size();
     kc_status s = ensure_jobs(b, (size_t)n, n_items);
     if (s != KC_OK) {
-        release_work(b, work);
         return s;
     }
     KC_CUDA(cudaMemcpyAsync(b->d_item_job, b->item_job.data(), n_items * 4, cudaMemcpyHostToDevice, st));
@@ -1333,7 +1343,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         for (int j = 0; j < n; ++j) spec_pairs += hs[j]->res_cap;
         if ((s = ensure_buckets(b, spec_buckets)) != KC_OK || (s = grow(b->d_pairs, b->pairs_cap, spec_pairs)) != KC_OK ||
             (s = capture_sort_graph(b, 1)) != KC_OK) {
-            release_work(b, work);
             return s;
         }
         uint64_t first = 0;  // the plan gives the jobs their buckets in this order
@@ -1344,7 +1353,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         KC_CUDA(cudaMemsetAsync(b->d_hist, 0, spec_buckets * 4, st));
     }
     if ((s = upload_desc(b, (uint32_t)n, n_items, 0)) != KC_OK) {
-        release_work(b, work);
         return s;
     }
     bool one_sample = true;
@@ -1359,12 +1367,10 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     const int n_ctas = b->sm_count * per_sm;
     cudaGraphExec_t cons = nullptr;
     if ((s = consume_graph(b, one_sample, threads, n_ctas, smem_max, &cons)) != KC_OK) {
-        release_work(b, work);
         return s;
     }
 
     if (fast && (s = order_after_handles()) != KC_OK) {
-        release_work(b, work);
         return s;
     }
     // consume: one persistent launch over the (job, partition) queue
@@ -1388,7 +1394,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
             hs[j]->host_ctr = hc[j];
             kc_status s = device_errors(hs[j]);
             if (s != KC_OK) {
-                release_work(b, work);
                 return s;
             }
         }
@@ -1408,7 +1413,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
             s = run_fallbacks(b, work[j], (uint32_t)j, (uint32_t)cnt[2 * j + 1]);
             if (timed) phase_end(hs[0], kCompact, t0, st);
             if (s != KC_OK) {
-                release_work(b, work);
                 return s;
             }
             kc::JobDesc& J = b->jobs[j];
@@ -1422,7 +1426,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         for (int j = 0; j < n; ++j) {
             hs[j]->host_ctr = hc[j];
             if ((s = device_errors(hs[j])) != KC_OK) {
-                release_work(b, work);
                 return s;
             }
         }
@@ -1450,7 +1453,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
             if ((e = kc::dev_alloc(&h->res_keys, cap * 8, st)) != cudaSuccess ||
                 (e = kc::dev_alloc(&h->res_vals, cap * 8, st)) != cudaSuccess) {
                 free_result(h);
-                release_work(b, work);
                 return cuda_fail(e, "cudaMallocAsync(result)");
             }
             h->res_cap = cap;
@@ -1464,7 +1466,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         (s = grow(b->d_pairs, b->pairs_cap, std::max<uint64_t>(1, pairs_need))) != KC_OK ||
         (s = upload_desc(b, (uint32_t)n, n_items, 0)) != KC_OK ||
         (s = capture_sort_graph(b, 0)) != KC_OK) {
-        release_work(b, work);
         return s;
     }
     t0 = timed ? phase_begin(hs[0], st) : nullptr;
@@ -1475,7 +1476,6 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     for (int j = 0; j < n; ++j) work[j].h->launches += 7;
     }  // !sorted
     if (err & kc::DERR_INTERNAL) {
-        release_work(b, work);
         for (int j = 0; j < n; ++j) hs[j]->state = State::Poisoned;
         return fail(KC_ERR_INTERNAL, "sort: key outside its bucket range");
     }
@@ -1512,11 +1512,10 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
     }
     if (t0) phase_end(hs[0], kSort, t0, st);
     KC_CUDA(cudaStreamSynchronize(st));
-    for (JobWork& x : work) {  // nothing uses them any more
+    for (JobWork& x : work.jobs) {  // nothing uses them any more
         leave_block(x.h, x.sv_keys, x.sv_bytes, st);
         x.sv_keys = x.sv_vals = nullptr;
     }
-    release_work(b, work);
     for (int j = 0; j < n; ++j) {
         kc_handle h = hs[j];
         h->host_ctr.survivors = h->n_result;

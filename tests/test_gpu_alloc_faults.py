@@ -3,8 +3,10 @@ filled): a call either reports KC_ERR_OOM_DEVICE and works when it is made again
 or gives the result it gives with memory to spare."""
 import ctypes
 
+import numpy as np
 import pytest
 
+import synth
 import paper_1712_03254_gb300 as kc
 
 pytestmark = pytest.mark.gpu
@@ -38,3 +40,84 @@ def test_batch_object_that_cannot_be_made(fail_alloc, n):
     assert e.value.name == "KC_ERR_OOM_DEVICE"
     fail_alloc(0, 0)
     kc.KcBatch()
+
+
+def _device(rs):
+    import torch
+
+    packed, mask = kc.pack_ascii(rs.ascii)
+    arrays = [packed, np.ascontiguousarray(rs.offsets, dtype=np.uint64), mask]
+    arrays = [torch.from_numpy(a.view(np.int64)).cuda() for a in arrays]
+    torch.cuda.synchronize()
+    return arrays
+
+
+def _expect(o):
+    return (*o.result(), o.bloom())
+
+
+def _same(c, want):
+    for x, y in zip((*c.dump(), c.export_bloom()), want):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("how", ["alone", "batch", "batched_ingest"])
+def test_finalize_fails_and_is_made_again(oracle_mod, fail_alloc, how):
+    """Each allocation of a finalize in turn fails, and all after it, while the handle's
+    grouping may still run; another handle's job then takes memory at once, and the
+    first one's finalize is made again: both results are the oracle's.  (The reads are
+    too many for the finalize to fall back on spilling, and the handle holds blocks from
+    earlier jobs, so the survivors' block is the grouping's scratch.)"""
+    sets, want = [], []
+    for i in range(2):
+        g = synth.genome(300 + i, 200_000)
+        sets.append(synth.reads(310 + i, g, 40_000, 140, 150, 0.005, 0.0005))
+        want.append(_expect(oracle_mod.count(synth.Workload("job", [sets[i]], 31, 1 << 24, 4, 2))))
+    dev = [_device(rs) for rs in sets]
+
+    def handle():
+        return kc.KmerCounter(31, 1, 1 << 24, 4, 2, strategy="partitioned", batched_ingest=how == "batched_ingest")
+
+    b = handle()
+    batch = kc.KcBatch()
+
+    def finalize(c):
+        c.finalize() if how == "alone" else batch.finalize([c])
+
+    failed = 0
+    for kept in (False, True):  # a handle's first job (result arrays to be made), and its later ones
+        for n in range(100):
+            if n == 0 or not kept:
+                a = handle()
+            for _ in range(2 if kept and n == 0 else 0):
+                a.add_reads(0, *dev[0])
+                finalize(a)
+                a.reset()
+            a.add_reads(0, *dev[0])
+            fail_alloc(n, 1 << 40)
+            try:
+                finalize(a)
+                done = True
+            except kc.KcError as e:
+                assert e.name == "KC_ERR_OOM_DEVICE"
+                done = False
+            tried = fail_alloc(0, 0)
+            b.reset()
+            b.add_reads(0, *dev[1])
+            finalize(b)
+            if not done:
+                failed += 1
+                finalize(a)
+            _same(a, want[0])
+            _same(b, want[1])
+            if done and tried <= n:  # every allocation has had its turn
+                break
+            if kept:
+                a.reset()
+            else:
+                a.close()
+        else:
+            raise AssertionError("a finalize of more than 100 allocations")
+    assert failed > 0
+    a.close()
+    b.close()
