@@ -195,11 +195,11 @@ kc_status check_open(kc_handle h) {
 }
 
 // Bytes all handles of the process keep idle.
-std::atomic<size_t> g_idle_bytes{0};
+IdleTotals g_idle;
 
 size_t idle_limit(kc_handle h) {
-    static std::atomic<size_t> cached[64];
-    const int dev = h->device >= 0 && h->device < 64 ? h->device : 0;
+    static std::atomic<size_t> cached[kMaxDevices];
+    const int dev = h->device >= 0 && h->device < kMaxDevices ? h->device : 0;
     size_t v = cached[dev].load(std::memory_order_relaxed);
     if (!v) {
         size_t free_b = 0, total_b = 0;
@@ -212,7 +212,7 @@ size_t idle_limit(kc_handle h) {
 
 void free_idle(kc_handle h) {
     for (const IdleBlock& b : h->idle) cudaFreeAsync(b.p, h->stream);
-    g_idle_bytes -= h->idle_bytes;
+    g_idle.release(h->device, h->idle_bytes);
     h->idle.clear();
     h->idle_bytes = 0;
 }
@@ -229,7 +229,7 @@ cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
         *p = h->idle[best].p;
         *bytes = h->idle[best].bytes;
         h->idle_bytes -= *bytes;
-        g_idle_bytes -= *bytes;
+        g_idle.release(h->device, *bytes);
         h->idle.erase(h->idle.begin() + best);
         return cudaSuccess;
     }
@@ -245,10 +245,9 @@ cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
 void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st) {
     if (!p) return;
     if (h->keep_blocks && !h->cfg.device_budget && bytes >= kIdleMinBytes && h->idle.size() < kMaxIdleBlocks &&
-        g_idle_bytes.load() + bytes <= idle_limit(h)) {
+        g_idle.reserve(h->device, bytes, idle_limit(h))) {
         h->idle.push_back({p, bytes});
         h->idle_bytes += bytes;
-        g_idle_bytes += bytes;
         return;
     }
     cudaFreeAsync(p, st);
@@ -993,10 +992,10 @@ kc_status finalize_direct(kc_handle h) {
 // One finalize engine per device, shared by every handle (its buffers and
 // captured sort graph are reused); calls on it are serialised.
 std::mutex g_engine_mutex;
-kc_batch_ctx* g_engines[64] = {};
+kc_batch_ctx* g_engines[kMaxDevices] = {};
 
 kc_status finalize_partitioned(kc_handle h) {
-    if (h->device < 0 || h->device >= 64) return fail(KC_ERR_ARG, "device index out of range");
+    if (h->device < 0 || h->device >= kMaxDevices) return fail(KC_ERR_ARG, "device index out of range");
     std::lock_guard<std::mutex> lock(g_engine_mutex);
     if (!g_engines[h->device]) {
         kc_status s = kc_batch_create_internal(nullptr, &g_engines[h->device]);

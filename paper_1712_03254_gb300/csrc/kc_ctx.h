@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/kc.h"
+#include "kc_idle.h"
 #include "kc_internal.h"
 
 struct kc_batch_ctx;
@@ -93,8 +94,8 @@ struct SpillRun {
 // every job cost 0.35 ms each when several handles took turns (the pool maps
 // their memory anew).  A handle keeps blocks from its second job on
 // (kc_reset), unless it has a device budget or its last job took more than half
-// the share, and all handles together at most a kIdleShare-th of the device's
-// memory; kc_destroy gives them back, and so does a failed allocation of the
+// the share, and all handles of a device together at most a kIdleShare-th of its
+// memory (IdleTotals); kc_destroy gives them back, and so does a failed allocation of the
 // handle.  (A job that passes the share would keep some blocks and give others
 // back, in an order that has the pool map memory for every job: two samples of
 // 10,000,000 reads took 51 to 70 ms a job so, 55 with none kept.)  A block is
