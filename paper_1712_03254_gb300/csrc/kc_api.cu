@@ -100,6 +100,12 @@ bool is_local_device_ptr(const void* p, int device) {
 
 }  // namespace kcapi
 
+namespace kcapi {
+namespace {
+bool reclaim_idle(bool locked);
+}
+}  // namespace kcapi
+
 namespace kc {
 void set_last_error(const std::string& msg) { kcapi::g_last_error = msg; }
 
@@ -126,16 +132,26 @@ struct AllocFaults {
 thread_local AllocFaults t_alloc_faults;
 }  // namespace
 
-cudaError_t dev_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
-    const cudaError_t e = t_alloc_faults.next() ? cudaErrorMemoryAllocation : cudaMallocAsync(p, bytes, st);
-    if (e != cudaSuccess) cudaGetLastError();
+namespace {
+template <class Alloc>
+cudaError_t alloc_or_reclaim(const Alloc& alloc, bool locked) {
+    const auto attempt = [&] {
+        const cudaError_t e = t_alloc_faults.next() ? cudaErrorMemoryAllocation : alloc();
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
+    };
+    cudaError_t e = attempt();
+    if (e == cudaErrorMemoryAllocation && kcapi::reclaim_idle(locked)) e = attempt();
     return e;
+}
+}  // namespace
+
+cudaError_t dev_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
+    return alloc_or_reclaim([&] { return cudaMallocAsync(p, bytes, st); }, false);
 }
 
 cudaError_t dev_alloc_fixed_bytes(void** p, size_t bytes) {
-    const cudaError_t e = t_alloc_faults.next() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
-    if (e != cudaSuccess) cudaGetLastError();
-    return e;
+    return alloc_or_reclaim([&] { return cudaMalloc(p, bytes); }, true);
 }
 }  // namespace kc
 
@@ -197,6 +213,26 @@ kc_status check_open(kc_handle h) {
 // Bytes all handles of the process keep idle.
 IdleTotals g_idle;
 
+// Every handle, and every handle's idle blocks, under one lock: an allocation
+// that fails gives back the idle blocks of all of them (reclaim_idle).
+std::mutex g_idle_mutex;
+kc_ctx* g_handles = nullptr;
+
+void list_handle(kc_handle h) {
+    std::lock_guard<std::mutex> lk(g_idle_mutex);
+    h->next_handle = g_handles;
+    g_handles = h;
+}
+
+void unlist_handle(kc_handle h) {
+    std::lock_guard<std::mutex> lk(g_idle_mutex);
+    for (kc_ctx** at = &g_handles; *at; at = &(*at)->next_handle)
+        if (*at == h) {
+            *at = h->next_handle;
+            return;
+        }
+}
+
 size_t idle_limit(kc_handle h) {
     static std::atomic<size_t> cached[kMaxDevices];
     const int dev = h->device >= 0 && h->device < kMaxDevices ? h->device : 0;
@@ -210,45 +246,74 @@ size_t idle_limit(kc_handle h) {
     return v;
 }
 
-void free_idle(kc_handle h) {
+namespace {
+
+// With g_idle_mutex held.
+void free_idle_locked(kc_handle h) {
     for (const IdleBlock& b : h->idle) cudaFreeAsync(b.p, h->stream);
     g_idle.release(h->device, h->idle_bytes);
     h->idle.clear();
     h->idle_bytes = 0;
 }
 
+// Gives the idle blocks of every handle of the current device back to the pool
+// and waits until they are there; false if there were none.  locked: the caller
+// holds sync_api_mutex(), without which a handle's stream may be in the middle of
+// a capture on another thread.
+bool reclaim_idle(bool locked) {
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess || !g_idle.held(device)) return false;
+    std::unique_lock<std::mutex> sync(kc::sync_api_mutex(), std::defer_lock);
+    if (!locked) sync.lock();
+    std::lock_guard<std::mutex> lk(g_idle_mutex);
+    bool any = false;
+    for (kc_ctx* h = g_handles; h; h = h->next_handle) {
+        if (h->device != device || h->idle.empty()) continue;
+        free_idle_locked(h);
+        cudaStreamSynchronize(h->stream);
+        any = true;
+    }
+    return any;
+}
+
+}  // namespace
+
+void free_idle(kc_handle h) {
+    std::lock_guard<std::mutex> lk(g_idle_mutex);
+    free_idle_locked(h);
+}
+
 cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st) {
     *bytes = std::max<size_t>(*bytes, 16);
     h->job_blocks += *bytes;
-    size_t best = h->idle.size();
-    for (size_t i = 0; i < h->idle.size(); ++i) {
-        const size_t have = h->idle[i].bytes;
-        if (have >= *bytes && have / 4 <= *bytes && (best == h->idle.size() || have < h->idle[best].bytes)) best = i;
+    {
+        std::lock_guard<std::mutex> lk(g_idle_mutex);
+        size_t best = h->idle.size();
+        for (size_t i = 0; i < h->idle.size(); ++i) {
+            const size_t have = h->idle[i].bytes;
+            if (have >= *bytes && have / 4 <= *bytes && (best == h->idle.size() || have < h->idle[best].bytes)) best = i;
+        }
+        if (best < h->idle.size()) {
+            *p = h->idle[best].p;
+            *bytes = h->idle[best].bytes;
+            h->idle_bytes -= *bytes;
+            g_idle.release(h->device, *bytes);
+            h->idle.erase(h->idle.begin() + best);
+            return cudaSuccess;
+        }
     }
-    if (best < h->idle.size()) {
-        *p = h->idle[best].p;
-        *bytes = h->idle[best].bytes;
-        h->idle_bytes -= *bytes;
-        g_idle.release(h->device, *bytes);
-        h->idle.erase(h->idle.begin() + best);
-        return cudaSuccess;
-    }
-    cudaError_t e = kc::dev_alloc(p, *bytes, st);
-    if (e == cudaErrorMemoryAllocation && !h->idle.empty()) {
-        free_idle(h);
-        cudaStreamSynchronize(h->stream);
-        e = kc::dev_alloc(p, *bytes, st);
-    }
-    return e;
+    return kc::dev_alloc(p, *bytes, st);
 }
 
 void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st) {
     if (!p) return;
-    if (h->keep_blocks && !h->cfg.device_budget && bytes >= kIdleMinBytes && h->idle.size() < kMaxIdleBlocks &&
-        g_idle.reserve(h->device, bytes, idle_limit(h))) {
-        h->idle.push_back({p, bytes});
-        h->idle_bytes += bytes;
-        return;
+    if (h->keep_blocks && !h->cfg.device_budget && bytes >= kIdleMinBytes) {
+        std::lock_guard<std::mutex> lk(g_idle_mutex);
+        if (h->idle.size() < kMaxIdleBlocks && g_idle.reserve(h->device, bytes, idle_limit(h))) {
+            h->idle.push_back({p, bytes});
+            h->idle_bytes += bytes;
+            return;
+        }
     }
     cudaFreeAsync(p, st);
 }
@@ -659,7 +724,7 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
 // hashes (at most one per base plus run padding of 3 per (item, partition))
 // and partition starts stay with the batch.  Batches of handles with two
 // grouping levels are re-bucketed afterwards (regroup_batch).
-kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
+kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count, std::vector<LeftBlock>* left) {
     struct Ref {
         kc_handle h;
         size_t t;
@@ -775,7 +840,7 @@ kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count) {
     bool keep = true;
     for (const Ref& r : refs) keep = keep && r.h->l1_bits == r.h->part_bits;
     for (size_t i = 0; i < refs.size(); ++i) {
-        if (keep) leave_block(refs[i].h, scratch[i], scratch_bytes[i], st);  // the handle's stream will wait for st
+        if (keep) left->push_back({refs[i].h, scratch[i], scratch_bytes[i]});
         else cudaFreeAsync(scratch[i], st);
         Batch& b = refs[i].h->batches[refs[i].t];
         cudaFreeAsync(b.pw, st);  // the hashes replace the reads
@@ -809,7 +874,8 @@ uint64_t held_bytes(kc_handle h) {
 
 // Bytes the handle may still allocate: kc_config.device_budget minus what it
 // holds, or (no budget) the device's free memory plus what the stream-ordered
-// pool has cached and not handed out, less a 1 GiB margin.
+// pool has cached and not handed out and what the handles keep idle (a failed
+// allocation has them give it back), less a 1 GiB margin.
 uint64_t room_bytes(kc_handle h) {
     const uint64_t held = held_bytes(h);
     if (h->cfg.device_budget) return h->cfg.device_budget > held ? h->cfg.device_budget - held : 0;
@@ -828,7 +894,7 @@ uint64_t room_bytes(kc_handle h) {
         else
             cudaGetLastError();
     }
-    const uint64_t avail = (uint64_t)free_b + cached + h->idle_bytes, margin = 1ull << 30;
+    const uint64_t avail = (uint64_t)free_b + cached + g_idle.held(h->device), margin = 1ull << 30;
     return avail > margin ? avail - margin : 0;
 }
 
@@ -1219,6 +1285,7 @@ kc_status kc_create_ex(int k, int n_samples, uint64_t bloom_bits, int n_hashes, 
     if (c.prune_chain && (e = kc::dev_alloc(&h->bloom2, bloom_bytes, h->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocAsync(second filter)"));
     h->fixed_bytes = bloom_bytes * (c.prune_chain ? 2 : 1) + table_bytes + sizeof(kc::DevCounters);
+    list_handle(h);
     kc_status s = kc_reset(h);
     if (s != KC_OK) return bail(s);
     *out = h;
@@ -1271,6 +1338,7 @@ void kc_destroy(kc_handle h) {
         h->keep_blocks = false;
         free_batches(h);
         free_idle(h);
+        unlist_handle(h);
         free_result(h);
         free_selection(h);
         free_stems(h);
@@ -1687,7 +1755,10 @@ kc_status kc_stats_get(kc_handle h, kc_stats* out) {
         if (b.pw) bytes += (2 * b.n_units + 2) * 8 + b.n_units * 8;
         if (b.hdata) bytes += b.hcap * 8 + ((1ull << h->part_bits) + 1) * 8;
     }
-    out->device_bytes = bytes + h->idle_bytes;
+    {
+        std::lock_guard<std::mutex> lk(g_idle_mutex);
+        out->device_bytes = bytes + h->idle_bytes;
+    }
     out->launches = h->launches;
     out->ms_ingest = h->ms[kIngest];
     out->ms_pass1 = h->ms[kPass1];

@@ -1693,11 +1693,13 @@ kc_status ingest_batches(kc_batch_ctx* b, kc_handle* hs, int n) {
         KC_CUDA(cudaEventRecord(h->ev_main, h->stream));
         KC_CUDA(cudaStreamWaitEvent(b->st, h->ev_main, 0));
     }
-    kc_status s = ingest_pending(open.data(), (int)open.size(), b->st, b->sm_count);
+    std::vector<LeftBlock> left;
+    kc_status s = ingest_pending(open.data(), (int)open.size(), b->st, b->sm_count, &left);
     for (kc_handle h : open) {
         KC_CUDA(cudaEventRecord(h->ev_main, b->st));
         KC_CUDA(cudaStreamWaitEvent(h->stream, h->ev_main, 0));
     }
+    for (const LeftBlock& x : left) leave_block(x.h, x.p, x.bytes, x.h->stream);
     return s;
 }
 

@@ -95,15 +95,22 @@ struct SpillRun {
 // their memory anew).  A handle keeps blocks from its second job on
 // (kc_reset), unless it has a device budget or its last job took more than half
 // the share, and all handles of a device together at most a kIdleShare-th of its
-// memory (IdleTotals); kc_destroy gives them back, and so does a failed allocation of the
-// handle.  (A job that passes the share would keep some blocks and give others
+// memory (IdleTotals); kc_destroy gives them back, and so does a failed device
+// allocation of any handle (dev_alloc), before it is tried once more.  (A job that passes the share would keep some blocks and give others
 // back, in an order that has the pool map memory for every job: two samples of
 // 10,000,000 reads took 51 to 70 ms a job so, 55 with none kept.)  A block is
 // taken for work ordered after the handle's stream and left when the handle's
-// stream is ordered after its last use.
+// stream is ordered after its last use: from then on another thread's failed
+// allocation may free it there.
 struct IdleBlock {
     void* p = nullptr;
     size_t bytes = 0;
+};
+// A block to be left once the handle's stream is ordered after its last use.
+struct LeftBlock {
+    kc_handle h;
+    void* p;
+    size_t bytes;
 };
 constexpr size_t kMaxIdleBlocks = 12;
 constexpr size_t kIdleShare = 8;
@@ -183,6 +190,7 @@ struct kc_ctx {
     // blocks kept for the next job (IdleBlock); reused: a job has been reset
     std::vector<kcapi::IdleBlock> idle;
     size_t idle_bytes = 0;
+    kc_ctx* next_handle = nullptr;  // in the list of all handles
     bool reused = false;
     bool keep_blocks = false;
     size_t job_blocks = 0;  // bytes of blocks the job has taken
@@ -276,8 +284,8 @@ void free_result(kc_handle h);
 // after the handle's stream: an idle block of the handle (*bytes becomes its
 // size) or one from the pool.
 cudaError_t take_block(kc_handle h, void** p, size_t* bytes, cudaStream_t st);
-// Give a block back, last used on stream st, which the handle's stream is (or
-// will be, before its next work) ordered after: kept idle, or to the pool.
+// Give a block back, last used on stream st, which the handle's stream is
+// ordered after: kept idle, or to the pool.
 void leave_block(kc_handle h, void* p, size_t bytes, cudaStream_t st);
 // The batch's grouped hashes and their starts, last used on the handle's stream.
 void leave_hashes(kc_handle h, Batch& b);
@@ -303,8 +311,9 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
 int scatter_mode_of(kc_handle h);
 uint64_t held_bytes(kc_handle h);
 // Extract and group every pending batch (kc_config.batched_ingest) of the
-// handles on stream st, ordered after each handle's stream by the caller.
-kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count);
+// handles on stream st, ordered after each handle's stream by the caller; *left
+// are the blocks to give back when the handles' streams are ordered after st.
+kc_status ingest_pending(kc_handle* hs, int n, cudaStream_t st, int sm_count, std::vector<LeftBlock>* left);
 uint64_t room_bytes(kc_handle h);
 // Whether the handle may allocate `bytes` (a small need: try it and see).
 bool fits_device(kc_handle h, uint64_t bytes);

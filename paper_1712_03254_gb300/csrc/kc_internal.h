@@ -21,8 +21,10 @@ void set_last_error(const std::string& msg);
 std::mutex& sync_api_mutex();
 
 // Every device allocation of the library: stream-ordered from the pool, and
-// fixed (cudaMalloc, with sync_api_mutex() held).  A failure leaves no error
-// behind for a later cudaGetLastError to find.
+// fixed (cudaMalloc, with sync_api_mutex() held).  One that finds no memory has
+// all handles give back their idle blocks and is tried once more.  A failure
+// leaves no error behind for a later cudaGetLastError to find.  (Not with
+// sync_api_mutex() held, and never during a capture: dev_alloc.)
 cudaError_t dev_alloc_bytes(void** p, size_t bytes, cudaStream_t st);
 cudaError_t dev_alloc_fixed_bytes(void** p, size_t bytes);
 template <class T>

@@ -121,3 +121,100 @@ def test_finalize_fails_and_is_made_again(oracle_mod, fail_alloc, how):
     assert failed > 0
     a.close()
     b.close()
+
+
+def _keep_blocks(c, arrays):
+    """Two jobs and a reset: the handle keeps blocks for its next job."""
+    for _ in range(2):
+        c.reset()
+        c.add_reads(0, *arrays)
+        c.finalize()
+    c.reset()
+
+
+def test_any_allocation_may_take_what_idle_handles_keep(oracle_mod, fail_alloc):
+    """Each allocation of a handle's life in turn fails once while another handle keeps
+    blocks idle: the blocks are given back and the call goes on, result unchanged."""
+    g = synth.genome(330, 60_000)
+    normal = synth.reads(331, g, 8_000, 90, 120, 0.005, 0.0005)
+    tumour = synth.reads(332, synth.mutate(333, g, 0.01, 0.0), 8_000, 90, 120, 0.005, 0.0005)
+    o = oracle_mod.count(synth.Workload("job", [normal, tumour], 31, 1 << 22, 4, 2))
+    want = _expect(o)
+    arrays = [_device(normal), _device(tumour)]
+    packed, mask = kc.pack_ascii(tumour.ascii)
+    keeper_reads = _device(synth.reads(334, g, 30_000, 90, 120, 0.005, 0.0005))
+    keeper = kc.KmerCounter(31, 1, 1 << 22, 4, 2, strategy="partitioned")
+
+    def life(strategy):
+        c = kc.KmerCounter(31, 2, 1 << 22, 4, 2, strategy=strategy)
+        for s, a in enumerate(arrays):
+            c.add_reads(s, *a)
+        c.finalize()
+        _same(c, want)
+        out = [c.export_items(), c.spectrum(15), c.export_stems()]
+        c.filter_select(tumor=1, min_tumor=3, max_normal=0)
+        out += [*c.filter_keys(), *c.filter_reads(packed, tumour.offsets, mask)]
+        c.close()
+        return out
+
+    for strategy in ("partitioned", "direct"):
+        first = life(strategy)
+        for n in range(200):
+            _keep_blocks(keeper, keeper_reads)
+            kept = keeper.stats()["device_bytes"]
+            fail_alloc(n, 1)
+            again = life(strategy)
+            tried = fail_alloc(0, 0)
+            for x, y in zip(first, again):
+                assert np.array_equal(x, y)
+            if tried <= n:
+                break
+            assert keeper.stats()["device_bytes"] <= kept - (1 << 20)
+        assert 10 < n < 199
+    keeper.close()
+
+
+def test_blocks_taken_back_from_a_busy_handle(oracle_mod, fail_alloc):
+    """A handle works job after job on one thread while another thread's allocations
+    fail, each taking back what the first one keeps idle at that moment."""
+    import threading
+
+    g = synth.genome(340, 200_000)
+    rs = synth.reads(341, g, 40_000, 90, 120, 0.005, 0.0005)
+    want = _expect(oracle_mod.count(synth.Workload("job", [rs], 31, 1 << 22, 4, 2)))
+    arrays = _device(rs)
+    stop, wrong = threading.Event(), []
+
+    def busy():
+        try:
+            c = kc.KmerCounter(31, 1, 1 << 22, 4, 2, strategy="partitioned", batched_ingest=True)
+            batch = kc.KcBatch()
+            jobs = 0
+            while not stop.is_set() or jobs < 3:
+                c.reset()
+                c.add_reads(0, *arrays)
+                batch.ingest([c])
+                batch.finalize([c])
+                _same(c, want)
+                jobs += 1
+            c.close()
+        except BaseException as e:  # noqa: BLE001 -- reported by the test's own thread
+            wrong.append(e)
+
+    t = threading.Thread(target=busy)
+    t.start()
+    c = kc.KmerCounter(31, 1, 1 << 22, 4, 2, strategy="partitioned")
+    for n in range(120):
+        c.reset()
+        fail_alloc(n % 12, 1)
+        try:
+            c.add_reads(0, *arrays)
+            c.finalize()
+            _same(c, want)
+        except kc.KcError as e:
+            assert e.name == "KC_ERR_OOM_DEVICE"  # nothing was idle at that moment
+        fail_alloc(0, 0)
+    stop.set()
+    t.join()
+    assert not wrong, wrong
+    c.close()
