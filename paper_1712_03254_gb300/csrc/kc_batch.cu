@@ -1703,7 +1703,17 @@ kc_status ingest_batches(kc_batch_ctx* b, kc_handle* hs, int n) {
     return s;
 }
 
-kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
+// A finalize of the handle has failed and it stays open: what its consumer and
+// fallbacks have added to the handle's counts is taken back, since the next
+// finalize counts every partition again.
+static void uncount(kc_batch_ctx* b, kc_handle h) {
+    h->fallback_partitions = 0;
+    cudaMemsetAsync(&h->ctr->candidates, 0, 2 * sizeof(unsigned long long), b->st);  // and claimed
+    cudaMemsetAsync(&h->ctr->split_parts, 0, sizeof(unsigned), b->st);
+    cudaStreamSynchronize(b->st);
+}
+
+static kc_status finalize_jobs(kc_batch_ctx* b, kc_handle* hs, int n) {
     if (b && hs && n > 0) {
         kc_status s = ingest_batches(b, hs, n);
         if (s != KC_OK) return s;
@@ -1719,10 +1729,8 @@ kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
         if (!fits_device(h, need)) return finalize_spilled(b, h);
         kc_status s = finalize_core(b, hs, n, 0, 0xffffffffu, true);
         if (s != KC_ERR_OOM_DEVICE || !small_need(h, need)) return s;
-        // no room after all: counted again, group by group
-        KC_CUDA(cudaMemsetAsync(&h->ctr->candidates, 0, 2 * sizeof(unsigned long long), b->st));  // and claimed
-        KC_CUDA(cudaMemsetAsync(&h->ctr->split_parts, 0, sizeof(unsigned), b->st));
-        return finalize_spilled(b, h);
+        uncount(b, h);
+        return finalize_spilled(b, h);  // no room after all: counted again, group by group
     }
     if (!hs || n <= 1) return finalize_core(b, hs, n, 0, 0xffffffffu, true);
     // handles whose reads passed the device budget are finalized alone, in
@@ -1737,6 +1745,14 @@ kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
         }
     }
     return finalize_core(b, rest.data(), (int)rest.size(), 0, 0xffffffffu, true);
+}
+
+kc_status kc_batch_finalize_internal(kc_batch_ctx* b, kc_handle* hs, int n) {
+    const kc_status s = finalize_jobs(b, hs, n);
+    if (s != KC_OK && b && hs)
+        for (int j = 0; j < n; ++j)
+            if (hs[j] && hs[j]->state == State::Open && hs[j]->strategy == KC_STRATEGY_PARTITIONED) uncount(b, hs[j]);
+    return s;
 }
 
 extern "C" {

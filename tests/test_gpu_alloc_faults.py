@@ -218,3 +218,63 @@ def test_blocks_taken_back_from_a_busy_handle(oracle_mod, fail_alloc):
     t.join()
     assert not wrong, wrong
     c.close()
+
+
+def _take_back_idle_blocks(fail_alloc):
+    """No handle keeps blocks afterwards (a failed allocation takes them back)."""
+    fail_alloc(0, 1)
+    try:
+        kc.KcBatch()
+    except kc.KcError:
+        pass
+    fail_alloc(0, 0)
+
+
+@pytest.mark.parametrize("call", ["add_reads", "finalize"])
+def test_small_job_without_room(oracle_mod, fail_alloc, call):
+    """A small job asks for memory without looking whether there is room.  Where there is
+    none, its reads are kept and its result spilled: result, filter and counts are those
+    of the job that had room, fallback partitions counted once."""
+    g = synth.genome(350, 20_000)
+    rs = synth.reads(351, g, 6_000, 90, 120, 0.005, 0.0005)
+    o = oracle_mod.count(synth.Workload("job", [rs], 31, 1 << 20, 4, 1))
+    want = _expect(o)
+    arrays = _device(rs)
+
+    def handle():  # every partition too large for its table: global tables
+        return kc.KmerCounter(31, 1, 1 << 20, 4, 1, strategy="partitioned", part_bits=2, smem_table_log2=10, split_max=-1)
+
+    c = handle()
+    c.add_reads(0, *arrays)
+    c.finalize()
+    plain = c.stats()
+    assert plain["fallback_partitions"] == 4 and plain["candidates"] == o.windows
+    c.close()
+    spilled = deferred = again = 0
+    for n in range(100):
+        _take_back_idle_blocks(fail_alloc)
+        c = handle()
+        for step in ("add_reads", "finalize"):
+            def go():
+                c.add_reads(0, *arrays) if step == "add_reads" else c.finalize()
+
+            if step == call:
+                fail_alloc(n, 1)
+            try:
+                go()
+            except kc.KcError as e:
+                assert e.name == "KC_ERR_OOM_DEVICE"
+                go()
+                again += 1
+            if step == call:
+                tried = fail_alloc(0, 0)
+        st = c.stats()
+        for name in ("windows", "candidates", "table_keys", "result_keys", "fallback_partitions", "split_partitions"):
+            assert st[name] == plain[name], name
+        spilled += st["spilled_bytes"] > 0
+        deferred += st["deferred_batches"]
+        _same(c, want)
+        c.close()
+        if tried <= n:
+            break
+    assert deferred > 0 if call == "add_reads" else spilled > 0
