@@ -96,7 +96,11 @@ bool is_local_device_ptr(const void* p, int device) {
     return (a.type == cudaMemoryTypeDevice && a.device == device) || a.type == cudaMemoryTypeManaged;
 }
 
-
+// The same for 64-bit words read one by one: an array at an odd address is
+// copied instead (a copy reaches any address).
+bool words_in_place(const uint64_t* p, int device) {
+    return reinterpret_cast<uintptr_t>(p) % sizeof(uint64_t) == 0 && is_local_device_ptr(p, device);
+}
 
 }  // namespace kcapi
 
@@ -1527,8 +1531,8 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     // read where they are (in stream order), host ones copied.  The packed
     // words are always copied: the store is padded for the kernels' loads and
     // may outlive the call.
-    const bool own_nm = chunked || !is_local_device_ptr(n_mask, h->device);
-    const bool own_off = chunked || !is_local_device_ptr(offsets, h->device);
+    const bool own_nm = chunked || !words_in_place(n_mask, h->device);
+    const bool own_off = chunked || !words_in_place(offsets, h->device);
     cudaError_t e;
     // the read store (packed words, valid-window bits) and, for this call, the
     // read-start bits and the copies of the N mask and offsets

@@ -296,6 +296,7 @@ uint64_t* spill_alloc(kc_handle h, uint64_t words);  // nullptr when pinning fai
 kc_status check_open(kc_handle h);                   // KC_ERR_ARG / KC_ERR_STATE for null or poisoned
 bool is_device_ptr(const void* p);
 bool is_local_device_ptr(const void* p, int device);
+bool words_in_place(const uint64_t* p, int device);
 cudaError_t pinned_words(kc_handle h);
 // Copy a spilled result back to the device and sort it there
 // (KC_ERR_OOM_DEVICE, nothing changed, when it does not fit).

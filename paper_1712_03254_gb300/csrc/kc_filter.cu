@@ -926,8 +926,8 @@ kc_status kc_filter_reads(kc_handle h, const uint64_t* packed_reads, const uint6
     // one block.
     const uint64_t* const src_pw = any ? packed_reads + B / 32 : nullptr;
     const bool own_pw = !any || !is_local_device_ptr(packed_reads, h->device) || reinterpret_cast<uintptr_t>(src_pw) % 16 != 0;
-    const bool own_nm = !any || !is_local_device_ptr(n_mask, h->device);
-    const bool own_off = !is_local_device_ptr(offsets, h->device);
+    const bool own_nm = !any || !words_in_place(n_mask, h->device);
+    const bool own_off = !words_in_place(offsets, h->device);
     const bool own_cand = candidates && !cand_dev;
     char* block = nullptr;
     uint64_t* hmask = nullptr;  // pinned words the call's small readbacks land in

@@ -104,3 +104,44 @@ def test_filter_units_in_parts(units):
     parts = [c.filter_readset(tumour.slice(int(p[0]), int(p[-1]) + 1))[0] for p in pieces]
     assert np.array_equal(hits, np.concatenate(parts))
     c.close()
+
+
+@pytest.mark.parametrize("shift", [1, 4, 6])
+def test_device_arrays_at_odd_addresses(oracle_mod, shift):
+    """Packed words, offsets and N mask in device memory, `shift` bytes behind an 8-byte
+    boundary, are copied: the counts are the oracle's, the hits those of host reads."""
+    import ctypes
+
+    import torch
+
+    g = synth.genome(45, 5_000)
+    rs = synth.reads(46, g, 700, 60, 100, 0.01, 0.002)
+    other = synth.reads(47, g, 300, 60, 100, 0.01, 0.002)
+    w = synth.Workload("odd", [other, rs], 31, 1 << 18, 4, 2)
+    o = oracle_mod.count(w)
+    packed, mask = kc.pack_ascii(rs.ascii)
+    held = []
+
+    def odd(a):
+        raw = np.ascontiguousarray(a).view(np.uint8)
+        t = torch.zeros(len(raw) + 16, dtype=torch.uint8, device="cuda")
+        assert t.data_ptr() % 8 == 0
+        t[shift : shift + len(raw)] = torch.from_numpy(raw.copy())
+        held.append(t)
+        return ctypes.c_void_p(t.data_ptr() + shift)
+
+    args = [odd(packed), odd(rs.offsets.astype(np.uint64)), odd(mask)]
+    torch.cuda.synchronize()
+    for strategy in ("partitioned", "direct"):
+        c = kc.KmerCounter(31, 2, 1 << 18, 4, 2, strategy=strategy)
+        c.add_readset(0, other)
+        assert c._L.kc_add_reads(c._h, 1, *args, rs.n_reads) == 0
+        c.finalize()
+        for x, y in zip(c.dump(), o.result()):
+            assert np.array_equal(x, y)
+        c.filter_select(tumor=1, min_tumor=2, max_normal=1)
+        want, _, n = c.filter_reads(packed, rs.offsets, mask)
+        hits, m = np.zeros(rs.n_reads, np.uint32), ctypes.c_uint64()
+        assert c._L.kc_filter_reads(c._h, *args, rs.n_reads, hits.ctypes.data_as(ctypes.c_void_p), None, ctypes.byref(m)) == 0
+        assert m.value == n > 0 and np.array_equal(hits, want)
+        c.close()
