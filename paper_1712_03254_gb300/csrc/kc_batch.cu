@@ -376,11 +376,11 @@ __global__ void __launch_bounds__(THREADS, THREADS == kConsumeThreads ? 2 : 1)
                     if (once) h ^= kTopBit;
                     const uint64_t g = mixer64(h);
                     const uint64_t pat = n_hashes == 4 ? bloom_pattern_n<4>(g) : bloom_pattern_rt(g, n_hashes);  // (4: every configuration's)
-                    // two 32-bit updates: a shared 64-bit one takes three times as long as a 32-bit one
-                    uint32_t* const word = reinterpret_cast<uint32_t*>(sb + ((uint32_t)(h >> bloom_shift) & (w_n - 1)));
-                    const uint32_t p_lo = (uint32_t)pat, p_hi = (uint32_t)(pat >> 32);
-                    const uint32_t o_lo = atomicOr(word, p_lo), o_hi = atomicOr(word + 1, p_hi);
-                    const bool fresh = (p_lo & ~o_lo) != 0u || (p_hi & ~o_hi) != 0u;
+                    // one 64-bit update, so that of the keys with equal bits one alone finds them new (an
+                    // update a half, where two keys can each be first in one, saves 0.5 to 1 % of a job)
+                    const unsigned long long old =
+                        atomicOr(sb + ((uint32_t)(h >> bloom_shift) & (w_n - 1)), (unsigned long long)pat);
+                    const bool fresh = (pat & ~old) != 0ull;
                     n_new += fresh;
                     n_seen += all_cand || !(fresh && once);
                 }

@@ -323,3 +323,38 @@ def test_two_levels_at_once(oracle_mod, k, part_bits, place):
         c.finalize()
         _same(c, o)
         c.close()
+
+
+@pytest.mark.parametrize("samples", [1, 2])
+def test_candidates_of_equal_patterns(samples):
+    """Keys seen once that share a filter word and its two bits, one in each half of the
+    word: whatever their order, the first is new to the filter and every other one a
+    candidate."""
+    bits, hashes = 1 << 12, 2
+    rng = np.random.default_rng(12)
+    codes, keys = _canonical_31mers(rng, 1_500_000)
+    h = _mixer(keys)
+    g = _mixer(h)
+    word = (h >> np.uint64(58)).astype(np.int64)
+    b0, b1 = (g & np.uint64(63)).astype(np.int64), ((g >> np.uint64(6)) & np.uint64(63)).astype(np.int64)
+    lo, hi = np.minimum(b0, b1), np.maximum(b0, b1)
+    pick = []
+    for w in range(64):  # per word its most frequent pattern over both halves
+        at = np.flatnonzero((word == w) & (lo < 32) & (hi >= 32))
+        pattern = lo[at] * 64 + hi[at]
+        best = np.bincount(pattern).argmax()
+        pick.append(at[pattern == best][:40])
+    rows = np.concatenate(pick)
+    assert all(len(p) > 15 for p in pick)
+    reads = np.frombuffer(b"ACGT", np.uint8)[codes[rows]]
+    for seed in range(40):
+        c = kc.KmerCounter(31, samples, bits, hashes, 2, strategy="partitioned", part_bits=1, smem_table_log2=13)
+        order = np.random.default_rng(seed).permutation(len(rows))
+        for s, part in enumerate(np.array_split(order, samples)):
+            c.add_readset(s, synth.ReadSet(reads[part].reshape(-1), np.arange(len(part) + 1, dtype=np.uint64) * np.uint64(31)))
+        c.finalize()
+        st = c.stats()
+        assert st["windows"] == len(rows) and st["split_partitions"] == 0
+        assert st["candidates"] == st["table_keys"] == len(rows) - 64
+        assert st["result_keys"] == 0
+        c.close()
