@@ -120,7 +120,10 @@ typedef struct kc_config {
                                      again as 2, 4, ... 2^split_max sub-ranges of
                                      its filter slice before it falls back to a
                                      global table (0 = 8; at most the slice's
-                                     log2 words; KC_SPLIT_NONE = never split)       */
+                                     log2 words; KC_SPLIT_NONE = never split).  With
+                                     smem_table_log2 = 0 a limit set here is about
+                                     the keys seen more than once: five levels
+                                     more make room for the others             */
     uint32_t prune_chain;         /* 1: the paper's two-filter Prune chain (direct
                                      strategy; KC_ERR_ARG with the partitioned one):
                                      kc_add_reads puts every window into the filter

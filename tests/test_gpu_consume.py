@@ -358,3 +358,20 @@ def test_candidates_of_equal_patterns(samples):
         assert st["candidates"] == st["table_keys"] == len(rows) - 64
         assert st["result_keys"] == 0
         c.close()
+
+
+@pytest.mark.parametrize("samples,split_max", [(1, -1), (1, 1), (2, -1), (2, 2)])
+def test_split_limit_is_about_repeated_keys(samples, split_max):
+    """70,000 keys of one partition, one in twelve of them more than once: the repeated
+    ones fit a table of the library's own size, so a limit on the splits (none at all)
+    sends nothing to the global tables."""
+    rng = np.random.default_rng(70)
+    n = 70_000
+    codes, keys = _canonical_31mers(rng, 2 * n + 2000)
+    own = (_mixer(keys) >> np.uint64(63)) == 0
+    codes, keys = codes[own][:n], keys[own][:n]
+    assert len(keys) == n
+    repeats = [np.ones(n, np.int64), np.zeros(n, np.int64)]
+    repeats[samples - 1][::12] += 2
+    st = _count(codes, keys, repeats, samples, 2, part_bits=1, split_max=split_max)
+    assert st["fallback_partitions"] == 0 and st["split_partitions"] == 1
