@@ -630,9 +630,9 @@ kc_status bucket_two_levels(kc_handle h, Batch& b, uint64_t n_local, cudaStream_
 }
 
 kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st, const kc::PassParams& p,
-                       bool exact, const ChunkedReads* chunks) {
-    if (h->l1_bits != h->part_bits && h->l1_bits <= kc::kStreamBits && !exact && p.h_lo == 0ull && p.h_hi == ~0ull &&
-        b.n_units < 1ull << 30) {  // (positions within a stream are 32-bit numbers)
+                       Grouping how, const ChunkedReads* chunks) {
+    const bool exact = how == Grouping::Exact;
+    if (how == Grouping::AtOnce && p.h_lo == 0ull && p.h_hi == ~0ull && b.n_units < 1ull << 30) {  // (positions within a stream are 32-bit numbers)
         bool done = false;
         const kc_status s = bucket_two_levels(h, b, n_local, st, p, chunks, &done);
         if (s != KC_OK || done) return s;
@@ -913,12 +913,24 @@ bool fits_device(kc_handle h, uint64_t bytes) { return small_need(h, bytes) || b
 uint64_t bucket_bytes(kc_handle h, uint64_t n_local) {
     const int max_ctas = h->grid.sm_count * (h->cfg.ctas_per_sm ? (int)h->cfg.ctas_per_sm : 1);
     if (n_local + 3ull * (uint64_t)max_ctas * (1ull << h->l1_bits) > kMaxGroupedHashes) return ~0ull;
-    // (two levels at once: streams of 9/8 of the hashes, rows over both levels)
-    const uint64_t streams = h->l1_bits != h->part_bits && h->l1_bits <= kc::kStreamBits
-                                 ? n_local + (uint64_t)max_ctas * ((1ull << h->part_bits) * 36 + (32ull * 128 * 8 << h->l1_bits))
-                                 : 0;
     return 16 * n_local + 24ull * (uint64_t)max_ctas * (1ull << h->l1_bits) +
-           (uint64_t)max_ctas * (1ull << h->l1_bits) * 12 + streams;
+           (uint64_t)max_ctas * (1ull << h->l1_bits) * 12;
+}
+
+// What two levels at once take beyond that (streams of 9/8 of the hashes, rows
+// over both levels); 0 for a handle that cannot.
+uint64_t stream_bytes(kc_handle h, uint64_t n_local) {
+    if (h->l1_bits == h->part_bits || h->l1_bits > kc::kStreamBits) return 0;
+    const int max_ctas = h->grid.sm_count * (h->cfg.ctas_per_sm ? (int)h->cfg.ctas_per_sm : 1);
+    return n_local + (uint64_t)max_ctas * ((1ull << h->part_bits) * 36 + (32ull * 128 * 8 << h->l1_bits));
+}
+
+// The grouping of a batch that there is room for: two levels at once where the
+// handle has two, else one after the other, else none (the reads are kept).
+Grouping grouping_for(kc_handle h, uint64_t n_local) {
+    const uint64_t need = bucket_bytes(h, n_local), streams = stream_bytes(h, n_local);
+    if (streams && need != ~0ull && fits_device(h, need + streams)) return Grouping::AtOnce;
+    return fits_device(h, need) ? Grouping::ByLevels : Grouping::None;
 }
 
 // Sort n (key, value) pairs held in tk/tv, keys below 2^key_bits, into
@@ -1391,7 +1403,7 @@ cudaError_t pinned_words(kc_handle h) {
 // check: per chunk its valid-window bits and extraction, then the grouping.
 kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* packed_reads, const uint64_t* offsets,
                             const uint64_t* n_mask, uint64_t n_reads, uint64_t b0, uint64_t b1, int n_chunks,
-                            uint64_t* nm, uint64_t* bd, uint64_t* doff, void* temp) {
+                            uint64_t* nm, uint64_t* bd, uint64_t* doff, void* temp, Grouping how) {
     cudaStream_t st = h->stream, cs = h->copy_stream;
     const uint64_t B = (b0 / 64) * 64;
     const uint64_t n_local = b1 - B;
@@ -1454,7 +1466,7 @@ kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* p
     // handle's stream: the chunks' valid bits and extraction, the grouping
     KC_CUDA(cudaStreamWaitEvent(st, h->ev_chunk[n_chunks], 0));
     cudaEvent_t t0 = phase_begin(h);
-    kc_status s = bucket_batch(h, b, n_local, st, h->params(sample), false, &ch);
+    kc_status s = bucket_batch(h, b, n_local, st, h->params(sample), how, &ch);
     phase_end(h, kPass1, t0);
     if (s != KC_OK) {
         KC_CUDA(cudaStreamSynchronize(cs));
@@ -1525,8 +1537,10 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     // offsets go first and are checked on the device before anything touches
     // the handle.
     const int n_chunks = (int)std::min<uint64_t>(kMaxChunks, n_units / kChunkUnits);
+    Grouping how = Grouping::None;
     const bool chunked = !data_dev && !mask_dev && n_chunks >= 2 && h->strategy != KC_STRATEGY_DIRECT &&
-                         !h->cfg.batched_ingest && scatter_mode_of(h) == 4 && fits_device(h, bucket_bytes(h, n_local));
+                         !h->cfg.batched_ingest && scatter_mode_of(h) == 4 &&
+                         (how = grouping_for(h, n_local)) != Grouping::None;
     // The N mask and offsets serve this call's kernels only: device ones are
     // read where they are (in stream order), host ones copied.  The packed
     // words are always copied: the store is padded for the kernels' loads and
@@ -1547,7 +1561,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
     if (own_nm) nm = bd + n_units;
     if (own_off) doff = bd + (own_nm ? 2 : 1) * n_units;
     if (chunked) {
-        s = add_reads_chunked(h, b, sample, packed_reads, offsets, n_mask, n_reads, b0, b1, n_chunks, nm, bd, doff, temp);
+        s = add_reads_chunked(h, b, sample, packed_reads, offsets, n_mask, n_reads, b0, b1, n_chunks, nm, bd, doff, temp, how);
         if (s != KC_OK) return s;
         h->batches.push_back(b);
         h->bases += b1 - b0;
@@ -1585,7 +1599,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
         else
             kc::launch_pass1(b.pw, b.vw, n_units, h->params(sample), h->bloom, h->table, h->ctr, h->grid, st);
         h->launches += 3;
-    } else if (!fits_device(h, bucket_bytes(h, n_local))) {
+    } else if ((how = grouping_for(h, n_local)) == Grouping::None) {
         // the window hashes would not fit the device budget: keep the packed
         // reads (about 3 bits per base), extracted again at kc_finalize one
         // hash range at a time
@@ -1595,7 +1609,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
         b.pending = true;  // extracted and grouped at kc_finalize, with the batch's other jobs
         b.n_local = n_local;
     } else {
-        s = bucket_batch(h, b, n_local, st, h->params(sample), false);
+        s = bucket_batch(h, b, n_local, st, h->params(sample), how);
         if (s == KC_ERR_OOM_DEVICE && small_need(h, bucket_bytes(h, n_local))) {
             leave_hashes(h, b);  // no room after all: kept as reads
             b.deferred = true;

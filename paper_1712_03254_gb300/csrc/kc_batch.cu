@@ -1656,7 +1656,7 @@ kc_status finalize_grouped(kc_batch_ctx* b, kc_handle h) {
                 pc.n_units = std::min(piece_units, bt.n_units - u0);
                 kc::PassParams p = base;
                 p.sample = bt.sample;
-                s = bucket_batch(h, pc, pc.n_units * 64, st, p, true);
+                s = bucket_batch(h, pc, pc.n_units * 64, st, p, Grouping::Exact);
                 h->launches += 5;
                 pc.pw = pc.vw = nullptr;  // the piece borrows the kept reads
                 pc.deferred = true;       // marks hashes to free after the range

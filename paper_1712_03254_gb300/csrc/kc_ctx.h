@@ -303,10 +303,13 @@ cudaError_t pinned_words(kc_handle h);
 kc_status resort_spilled(kc_handle h);
 void free_selection(kc_handle h);
 void free_stems(kc_handle h);
+// How a batch is grouped: not at all, one level after the other, two levels at
+// once (kStreamBits), or one after the other with b.hdata sized after a read-back.
+enum class Grouping { None, ByLevels, AtOnce, Exact };
 // Group a batch's window hashes (those in [p.h_lo, p.h_hi]) by partition
-// into b.hdata / b.hstarts; exact: size b.hdata after one read-back.
+// into b.hdata / b.hstarts.
 kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st, const kc::PassParams& p,
-                       bool exact, const ChunkedReads* chunks = nullptr);
+                       Grouping how, const ChunkedReads* chunks = nullptr);
 // The ingest scatter mode bucket_batch uses for the handle (kc_config.scatter_mode
 // resolved against the grouping levels and the shared memory).
 int scatter_mode_of(kc_handle h);

@@ -196,3 +196,28 @@ def test_budget_reuse_after_reset(oracle_mod):
         keys, counts = c.dump()
         assert np.array_equal(keys, ok) and np.array_equal(counts, oc)
         assert np.array_equal(c.export_bloom(), o.bloom())
+
+
+@pytest.mark.parametrize("part_bits", [13, 14])
+@pytest.mark.parametrize("batched", [False, True])
+def test_budget_without_room_for_both_levels_at_once(oracle_mod, part_bits, batched):
+    """A budget that holds the grouping one level after the other, but not the streams and
+    rows of both at once: the reads are grouped as they come, none kept to be read again."""
+    import torch
+
+    g = synth.genome(57, 100_000)
+    rs = synth.reads(58, g, 32_000, 120, 160, 0.01, 0.001)
+    o = oracle_mod.count(synth.Workload("two", [rs], 31, 1 << 26, 4, 2))
+    bases = int(rs.offsets[-1])
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count
+    budget = (1 << 26) // 8 + 16 * bases + ctas * 36 * (1 << (part_bits - 12)) + (16 << 20)
+    c = kc.KmerCounter(31, 1, 1 << 26, 4, 2, strategy="partitioned", part_bits=part_bits, device_budget=budget,
+                       batched_ingest=batched)
+    c.add_readset(0, rs)
+    assert c.stats()["deferred_batches"] == 0
+    c.finalize()
+    ok, oc = o.result()
+    keys, counts = c.dump()
+    assert np.array_equal(keys, ok) and np.array_equal(counts, oc)
+    assert np.array_equal(c.export_bloom(), o.bloom())
+    c.close()
