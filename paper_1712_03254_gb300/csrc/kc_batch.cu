@@ -1496,7 +1496,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         KC_CUDA(cudaStreamSynchronize(st));
         for (int j = 0; j < n; ++j) hs[j]->launches += 1;
     }
-    if (err & kc::DERR_SORT_BUCKET) {  // rare: buckets above 2048 keys, sorted in global memory
+    if (err & kc::DERR_SORT_BUCKET) {  // buckets above 2048 keys, sorted in global memory
         // the plan is on the device: read back the jobs' bucket ranges and the starts
         std::vector<kc::JobDesc> jd((size_t)n);
         uint64_t nbk = 0;
@@ -1506,18 +1506,18 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
         std::vector<uint64_t> starts(nbk + 1);
         KC_CUDA(cudaMemcpyAsync(starts.data(), b->d_starts, (nbk + 1) * 8, cudaMemcpyDeviceToHost, st));
         KC_CUDA(cudaStreamSynchronize(st));
+        std::vector<kc::SortRange> large;
         for (int j = 0; j < n; ++j) {
             const kc::JobDesc& J = jd[j];
             const uint64_t job0 = starts[J.bucket_base];
             for (uint64_t q = 0; q < J.n_buckets; ++q) {
                 const uint64_t lo = starts[J.bucket_base + q], m = starts[J.bucket_base + q + 1] - lo;
-                if (m > 2048) {
-                    kc::launch_bitonic_global(J.res_keys + (lo - job0), J.res_vals + (lo - job0), m, st);
-                    hs[j]->launches += 1;
-                }
+                if (m > (uint64_t)kc::kMedCap) large.push_back({J.res_keys + (lo - job0), J.res_vals + (lo - job0), m});
             }
         }
-        KC_LAUNCHED("batched global sort launches");
+        uint64_t steps = 0;
+        if ((s = sort_ranges(large, st, &steps)) != KC_OK) return s;
+        for (int j = 0; j < n; ++j) hs[j]->launches += steps;
     }
     if (t0) phase_end(hs[0], kSort, t0, st);
     KC_CUDA(cudaStreamSynchronize(st));

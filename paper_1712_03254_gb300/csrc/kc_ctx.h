@@ -322,6 +322,8 @@ uint64_t room_bytes(kc_handle h);
 // Whether the handle may allocate `bytes` (a small need: try it and see).
 bool fits_device(kc_handle h, uint64_t bytes);
 bool small_need(kc_handle h, uint64_t bytes);
+// Sort each range in global memory; adds the launches to *launches.
+kc_status sort_ranges(std::vector<kc::SortRange>& ranges, cudaStream_t st, uint64_t* launches);
 // Sort n (key, value) pairs (keys below 2^key_bits) from tk/tv into out_k/out_v;
 // ctr->survivors holds n on the device; synchronises the stream.
 kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64_t n, int key_bits,

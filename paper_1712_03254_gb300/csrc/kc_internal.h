@@ -85,7 +85,14 @@ int warp_sort_capacity();
 void launch_bucket_sort(uint64_t* keys, uint64_t* vals, const uint64_t* starts, uint64_t n_buckets,
                         DevCounters* ctr, cudaStream_t st);
 int bucket_sort_capacity();
-void launch_bitonic_global(uint64_t* keys, uint64_t* vals, uint64_t n, cudaStream_t st);
+struct SortRange {
+    uint64_t* keys;
+    uint64_t* vals;
+    uint64_t n;
+};
+// Sort ranges of about the same size (the largest has `largest` pairs) in global
+// memory, all of them with the same launches; returns how many.
+uint64_t launch_bitonic_global(const SortRange* ranges, uint64_t n_ranges, uint64_t largest, cudaStream_t st);
 
 void launch_counts_narrow(const uint64_t* vals, uint64_t n, uint32_t* out, cudaStream_t st);
 // The result's keys and counts into device arrays (result arrays 16-byte aligned).

@@ -14,6 +14,7 @@
 // Sort        bucket by key, then sort each bucket: a warp ranks up to 64 keys
 //             by key range, larger ones take bitonic networks; ascending keys.
 
+#include <algorithm>
 #include <atomic>
 
 #include "kc_internal.h"
@@ -426,27 +427,34 @@ __global__ void __launch_bounds__(256, 2) k_bucket_sort_warp_big(uint64_t* __res
     }
 }
 
-// One comparator stage of the same network over global memory.
-__global__ void k_bitonic_step(uint64_t* __restrict__ keys, uint64_t* __restrict__ vals, uint64_t n,
-                               uint64_t n2, uint64_t size, uint64_t stride, int mirror) {
-    const uint64_t pairs = n2 >> 1;
+// One comparator stage of the same network over global memory, for every bucket
+// of the list that still has stages of this size (a row of the grid each).
+__global__ void __launch_bounds__(256) k_bitonic_step(const SortRange* __restrict__ ranges, uint64_t n_ranges,
+                                                      uint64_t size, uint64_t stride, int mirror) {
     const uint64_t gstride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gstride) {
-        uint64_t a, b;
-        if (mirror) {
-            const uint64_t half = size >> 1, blk = i / half, off = i % half;
-            a = blk * size + off;
-            b = blk * size + size - 1 - off;
-        } else {
-            a = 2 * i - (i & (stride - 1));
-            b = a + stride;
-        }
-        if (b < n && keys[a] > keys[b]) {
-            const uint64_t tk = keys[a], tv = vals[a];
-            keys[a] = keys[b];
-            vals[a] = vals[b];
-            keys[b] = tk;
-            vals[b] = tv;
+    for (uint64_t r = blockIdx.y; r < n_ranges; r += gridDim.y) {
+        const uint64_t n = ranges[r].n;
+        uint64_t* const keys = ranges[r].keys;
+        uint64_t* const vals = ranges[r].vals;
+        if (size >= 2 * n) continue;  // the bucket's network, of the next power of two, ends before
+        const uint64_t pairs = (n + size - 1) / size * (size >> 1);  // blocks of `size` that hold a key
+        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gstride) {
+            uint64_t a, b;
+            if (mirror) {
+                const uint64_t half = size >> 1, blk = i / half, off = i % half;
+                a = blk * size + off;
+                b = blk * size + size - 1 - off;
+            } else {
+                a = 2 * i - (i & (stride - 1));
+                b = a + stride;
+            }
+            if (b < n && keys[a] > keys[b]) {
+                const uint64_t tk = keys[a], tv = vals[a];
+                keys[a] = keys[b];
+                vals[a] = vals[b];
+                keys[b] = tk;
+                vals[b] = tv;
+            }
         }
     }
 }
@@ -588,16 +596,18 @@ void launch_bucket_sort(uint64_t* keys, uint64_t* vals, const uint64_t* starts, 
     k_bucket_sort<<<(unsigned)n_buckets, kSortThreads, smem, st>>>(keys, vals, starts, ctr);
 }
 
-void launch_bitonic_global(uint64_t* keys, uint64_t* vals, uint64_t n, cudaStream_t st) {
-    if (n <= 1) return;
-    uint64_t n2 = 1;
-    while (n2 < n) n2 <<= 1;
-    const unsigned grid = grid_for(n2 >> 1, 256, 152 * 16);
+uint64_t launch_bitonic_global(const SortRange* ranges, uint64_t n_ranges, uint64_t largest, cudaStream_t st) {
+    uint64_t n2 = 1, launches = 0;
+    while (n2 < largest) n2 <<= 1;
+    const unsigned rows = (unsigned)std::min<uint64_t>(n_ranges, 4096);
+    const dim3 grid(grid_for(n2 >> 1, 256, std::max(1, 152 * 16 / (int)rows)), rows);
     for (uint64_t size = 2; size <= n2; size <<= 1) {
-        k_bitonic_step<<<grid, 256, 0, st>>>(keys, vals, n, n2, size, 0, 1);
-        for (uint64_t stride = size >> 2; stride > 0; stride >>= 1)
-            k_bitonic_step<<<grid, 256, 0, st>>>(keys, vals, n, n2, size, stride, 0);
+        k_bitonic_step<<<grid, 256, 0, st>>>(ranges, n_ranges, size, 0, 1);
+        ++launches;
+        for (uint64_t stride = size >> 2; stride > 0; stride >>= 1, ++launches)
+            k_bitonic_step<<<grid, 256, 0, st>>>(ranges, n_ranges, size, stride, 0);
     }
+    return launches;
 }
 
 void launch_dump(const uint64_t* keys, const uint64_t* vals, uint64_t n, int n_samples, uint64_t* out_keys,

@@ -1,0 +1,96 @@
+"""Reads far from uniform: the same results, and no cost out of all proportion to a
+uniform job of the same size (the times are minima of several runs, the bounds wide)."""
+import time
+
+import numpy as np
+import pytest
+
+import synth
+import paper_1712_03254_gb300 as kc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kc.lib()
+
+
+def _device(rs):
+    import torch
+
+    packed, mask = kc.pack_ascii(rs.ascii)
+    arrays = [packed, np.ascontiguousarray(rs.offsets, dtype=np.uint64), mask]
+    arrays = [torch.from_numpy(a.view(np.int64)).cuda() for a in arrays]
+    torch.cuda.synchronize()
+    return arrays
+
+
+def _seconds(c, arrays, runs=4):
+    import torch
+
+    best = 1e9
+    for _ in range(runs):
+        c.reset()
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        c.add_reads(0, *arrays)
+        c.finalize()
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+def _genome(seed, n, at):
+    rng = np.random.default_rng(seed)
+    return np.frombuffer(b"ACGT", np.uint8)[rng.choice(4, n, p=[at / 2, (1 - at) / 2, (1 - at) / 2, at / 2])]
+
+
+@pytest.mark.parametrize("strategy", ["partitioned", "direct"])
+@pytest.mark.parametrize("min_count", [1, 2])
+def test_genome_of_few_letters(oracle_mod, strategy, min_count):
+    """A genome of 97 % A and T: hundreds of sort buckets of thousands of keys, of many
+    sizes, are sorted in global memory; result, filter and stem table are the oracle's."""
+    rs = synth.reads(401, _genome(400, 400_000, 0.97), 20_000, 90, 130, 0.005, 0.0005)
+    o = oracle_mod.count(synth.Workload("at", [rs], 31, 1 << 22, 4, min_count))
+    c = kc.KmerCounter(31, 1, 1 << 22, 4, min_count, strategy=strategy, table_slots=1 << 23 if strategy == "direct" else 0)
+    c.add_readset(0, rs)
+    c.finalize()
+    assert c.stats()["launches"] > 78  # the global-memory networks ran: 12 * 13 / 2 stages for up to 4096 keys
+    ok, oc = o.result()
+    keys, counts = c.dump()
+    assert np.array_equal(keys, ok) and np.array_equal(counts, oc)
+    assert np.array_equal(c.export_bloom(), o.bloom())
+    assert c.export_stems().tobytes() == o.stems().tobytes()
+    c.close()
+
+
+def test_batch_of_genomes_of_few_letters(oracle_mod):
+    """The same in a batch, beside a uniform job: each job's large buckets in its own arrays."""
+    counters, oracles = [], []
+    for i, at in enumerate((0.97, 0.5, 0.99)):
+        rs = synth.reads(411 + i, _genome(410 + i, 300_000, at), 15_000, 90, 130, 0.005, 0.0005)
+        oracles.append(oracle_mod.count(synth.Workload("at", [rs], 31, 1 << 22, 4, 1)))
+        c = kc.KmerCounter(31, 1, 1 << 22, 4, 1, strategy="partitioned")
+        c.add_readset(0, rs)
+        counters.append(c)
+    kc.KcBatch().finalize(counters)
+    for c, o in zip(counters, oracles):
+        ok, oc = o.result()
+        keys, counts = c.dump()
+        assert np.array_equal(keys, ok) and np.array_equal(counts, oc)
+        c.close()
+
+
+def test_sort_of_a_genome_of_few_letters_in_proportion():
+    """One network after the other for each large bucket took more than a hundred times a
+    uniform job's time."""
+    at = _device(synth.reads(421, _genome(420, 3_000_000, 0.95), 300_000, 150, 150, 0.005, 0.0005))
+    uniform = _device(synth.reads(422, _genome(423, 3_000_000, 0.5), 300_000, 150, 150, 0.005, 0.0005))
+    c = kc.KmerCounter(31, 1, 1 << 28, 4, 1, strategy="partitioned")
+    base, skewed = _seconds(c, uniform), _seconds(c, at)
+    c.close()
+    assert skewed < 20 * base, (skewed, base)
