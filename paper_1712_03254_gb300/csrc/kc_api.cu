@@ -616,10 +616,11 @@ kc_status bucket_two_levels(kc_handle h, Batch& b, uint64_t n_local, cudaStream_
     KC_CUDA(cudaMemcpyAsync(flag, overflow, 4, cudaMemcpyDeviceToHost, st));
     KC_CUDA(cudaEventRecord(h->ev_main, st));
     // the rest is queued before the flag is known (the segments stay within
-    // their streams' room in any case)
+    // their streams' room in any case); the scatter reads it.  A scatter of streams
+    // that overflow has most of them in one bucket: 4.8e7 windows of one key 270 ms
     kc::launch_bucket_offsets(counts, n_ctas, a, 1, rel, total, st);
     if ((e = kc::launch_scan(total, P, b.hstarts, cursor, st)) != cudaSuccess) return bail(e);
-    kc::launch_scatter_staged_seg(lin, seg, (int)n_segs, n_pieces, a1, a2, rel, b.hstarts, b.hdata, st);
+    kc::launch_scatter_staged_seg(lin, seg, (int)n_segs, n_pieces, a1, a2, rel, b.hstarts, b.hdata, st, overflow);
     h->launches += 3 + (chunks ? 2 : 1) * n_pieces;
     KC_LAUNCHED("two-level bucketing launches");
     KC_CUDA(cudaEventSynchronize(h->ev_main));

@@ -159,9 +159,11 @@ void launch_extract_groups(const uint64_t* pw, const uint64_t* vw, uint64_t n_un
 // Staged scatter of segment c into its runs (base: within their buckets,
 // which begin at starts): bucket (h >> (64 - a1 - a2)) mod
 // 2^a2; with a1 > 0 only hashes of the segment's level-1 group.  Segment c
-// comes in n_pieces pieces segs[c], segs[c + n_segs], ...
+// comes in n_pieces pieces segs[c], segs[c + n_segs], ...  Nothing is moved where
+// *skip is set by then.
 void launch_scatter_staged_seg(const uint64_t* src, const SegDesc* segs, int n_segs, int n_pieces, int a1, int a2,
-                               const uint64_t* base, const uint64_t* starts, uint64_t* out, cudaStream_t st);
+                               const uint64_t* base, const uint64_t* starts, uint64_t* out, cudaStream_t st,
+                               const unsigned* skip = nullptr);
 // Batched ingest: the read batches of several jobs extracted and grouped by
 // one set of launches.  Each batch is cut into items of whole units; the
 // extraction and the staged scatter are persistent kernels over the item

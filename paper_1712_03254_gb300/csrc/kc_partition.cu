@@ -346,7 +346,8 @@ __global__ void __launch_bounds__(kExtractThreads) k_extract_count(const uint64_
 // at a time; the ends of its last chunks get padding of another group.  A
 // stream has room for 9/8 of its even share of the CTA's window starts; a CTA
 // that needs more (few keys making up most of the reads) sets *overflow and
-// drops the rest, and the caller groups the batch the other way.
+// drops the rest, the scatter behind it does nothing, and the caller groups the
+// batch the other way.
 constexpr unsigned kStreamChunk = 128;
 
 template <int K, int A1>
@@ -634,7 +635,9 @@ __global__ void __launch_bounds__(kLinThreads) k_scatter_staged_seg(const uint64
                                                                     int a1, int a2,
                                                                     const uint64_t* __restrict__ base,
                                                                     const uint64_t* __restrict__ starts,
-                                                                    uint64_t* __restrict__ out) {
+                                                                    uint64_t* __restrict__ out,
+                                                                    const unsigned* __restrict__ skip) {
+    if (skip && *skip) return;
     scatter_segment(src, segs + blockIdx.x, n_pieces, gridDim.x, a1, a2, base + ((uint64_t)blockIdx.x << a2), starts, out);
 }
 
@@ -988,10 +991,11 @@ size_t staged_seg_smem(int a) {
 }
 
 void launch_scatter_staged_seg(const uint64_t* src, const SegDesc* segs, int n_segs, int n_pieces, int a1, int a2,
-                               const uint64_t* base, const uint64_t* starts, uint64_t* out, cudaStream_t st) {
+                               const uint64_t* base, const uint64_t* starts, uint64_t* out, cudaStream_t st,
+                               const unsigned* skip) {
     const size_t smem = staged_seg_smem(a2);
     allow_max_dynamic_smem(k_scatter_staged_seg);
-    k_scatter_staged_seg<<<n_segs, kLinThreads, smem, st>>>(src, segs, n_pieces, a1, a2, base, starts, out);
+    k_scatter_staged_seg<<<n_segs, kLinThreads, smem, st>>>(src, segs, n_pieces, a1, a2, base, starts, out, skip);
 }
 
 void launch_count_seg(const uint64_t* src, const SegDesc* segs, int n_segs, int a1, int a2, uint32_t* counts,
