@@ -145,3 +145,15 @@ def test_device_arrays_at_odd_addresses(oracle_mod, shift):
         assert c._L.kc_filter_reads(c._h, *args, rs.n_reads, hits.ctypes.data_as(ctypes.c_void_p), None, ctypes.byref(m)) == 0
         assert m.value == n > 0 and np.array_equal(hits, want)
         c.close()
+
+
+@pytest.mark.parametrize("rest", [1, 155648 // 8, 155648 // 8 + 1, 155648 // 4, 155648 // 4 + 1, 155648 // 2,
+                                  155648 // 2 + 1])
+def test_filter_rest_of_units_in_parts(rest):
+    """The same behind a whole round of the lanes (152 CTAs of 1024): a rest whose units are
+    taken in eighths, quarters, halves and whole, so that the hit mask is written in bytes,
+    in 16 and in 32 bits."""
+    import torch
+
+    lanes = torch.cuda.get_device_properties(0).multi_processor_count * 1024
+    test_filter_units_in_parts(lanes + rest * lanes // 155648)
