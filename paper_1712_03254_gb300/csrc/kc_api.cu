@@ -1061,6 +1061,8 @@ kc_status sort_result(kc_handle h, uint64_t* tk, uint64_t* tv) {
 kc_status finalize_direct(kc_handle h) {
     cudaStream_t st = h->stream;
     cudaEvent_t t0 = phase_begin(h);
+    if (h->recounted) kc::launch_clear_counts(h->table, h->n_slots, h->grid, st);  // a finalize made again
+    h->recounted = true;
     for (const auto& b : h->batches) {
         if (h->bloom2)
             kc::launch_count_chain(b.pw, b.vw, b.n_units, h->params(b.sample), h->bloom2, h->table, h->ctr, h->grid,
@@ -1367,6 +1369,7 @@ kc_status kc_reset(kc_handle h) {
     h->launches = 0;
     h->fallback_partitions = 0;
     h->deferred = h->scan_groups = 0;
+    h->recounted = false;
     h->state = State::Open;
     return KC_OK;
 }

@@ -211,6 +211,8 @@ struct kc_ctx {
     uint64_t launches = 0;
     uint32_t fallback_partitions = 0;
 
+    bool recounted = false;  // direct: a kc_finalize has counted reads into the table
+
     // out-of-core results (kc_config.spill)
     bool spilled = false;
     std::vector<kcapi::SpillRun> spill_dir;

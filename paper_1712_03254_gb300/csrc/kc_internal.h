@@ -61,6 +61,9 @@ void launch_pass1(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, cons
 void launch_pass2(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, const PassParams& p, Slot* table,
                   DevCounters* ctr, const Grid& g, cudaStream_t st);
 
+// The table's counts set back to zero, its keys kept.
+void launch_clear_counts(Slot* table, uint64_t n_slots, const Grid& g, cudaStream_t st);
+
 // Compaction of slots with summed count >= min_count.
 void launch_compact(const Slot* table, uint64_t n_slots, int n_samples, uint32_t min_count, uint64_t* keys,
                     uint64_t* vals, DevCounters* ctr, const Grid& g, cudaStream_t st);

@@ -160,6 +160,12 @@ __global__ void __launch_bounds__(256) k_pass2(const uint64_t* __restrict__ pw, 
     }
 }
 
+__global__ void k_clear_counts(Slot* __restrict__ table, uint64_t n_slots) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += stride)
+        table[i].cnt[0] = table[i].cnt[1] = 0u;
+}
+
 // Survivors of the table.  A warp queues the kept slots of its rows in shared
 // memory and writes 32 at a time behind one claim of the output: a claim a row
 // of 32 slots was one atomic on one address for each of 2.6e5 rows (2^23 slots,
@@ -539,6 +545,10 @@ void launch_pass1(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, cons
 void launch_pass2(const uint64_t* pw, const uint64_t* vw, uint64_t n_units, const PassParams& p, Slot* table,
                   DevCounters* ctr, const Grid& g, cudaStream_t st) {
     k_pass2<<<grid_for(n_units, 256, g.ctas()), 256, 0, st>>>(pw, vw, n_units, p, table, ctr);
+}
+
+void launch_clear_counts(Slot* table, uint64_t n_slots, const Grid& g, cudaStream_t st) {
+    k_clear_counts<<<grid_for(n_slots, 256, g.sm_count * 8), 256, 0, st>>>(table, n_slots);
 }
 
 void launch_compact(const Slot* table, uint64_t n_slots, int n_samples, uint32_t min_count, uint64_t* keys,

@@ -278,3 +278,42 @@ def test_small_job_without_room(oracle_mod, fail_alloc, call):
         if tried <= n:
             break
     assert deferred > 0 if call == "add_reads" else spilled > 0
+
+
+@pytest.mark.parametrize("chain", [False, True])
+def test_direct_finalize_made_again(oracle_mod, fail_alloc, chain):
+    """The direct strategy counts the reads into its table before the allocations of its
+    finalize: a finalize made again does not count them twice, nor where reads are added
+    in between."""
+    g = synth.genome(360, 30_000)
+    rs = synth.reads(361, g, 6_000, 90, 120, 0.005, 0.0005)
+    want = _expect(oracle_mod.count(synth.Workload("job", [rs], 31, 1 << 20, 4, 2)))
+    arrays, halves = _device(rs), [_device(rs.slice(0, 2_500)), _device(rs.slice(2_500, 6_000))]
+    c = kc.KmerCounter(31, 1, 1 << 20, 4, 2, strategy="direct", table_slots=1 << 20, prune_chain=chain)
+    again = 0
+    for n in range(100):
+        _take_back_idle_blocks(fail_alloc)
+        c.reset()
+        c.add_reads(0, *arrays)
+        fail_alloc(n, 1)
+        try:
+            c.finalize()
+        except kc.KcError as e:
+            assert e.name == "KC_ERR_OOM_DEVICE"
+            c.finalize()
+            again += 1
+        tried = fail_alloc(0, 0)
+        _same(c, want)
+        if tried <= n:
+            break
+        c.reset()
+        c.add_reads(0, *halves[0])
+        fail_alloc(0, 1 << 40)
+        with pytest.raises(kc.KcError):
+            c.finalize()
+        fail_alloc(0, 0)
+        c.add_reads(0, *halves[1])
+        c.finalize()
+        _same(c, want)
+    assert again > 0
+    c.close()
