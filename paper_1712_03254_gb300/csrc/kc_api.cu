@@ -988,7 +988,10 @@ kc_status sort_pairs(kc_handle h, const uint64_t* tk, const uint64_t* tv, uint64
     cudaEvent_t t0 = phase_begin(h);
     KC_CUDA(cudaMemsetAsync(hist, 0, n_buckets * 4, st));
     kc::launch_prefix_hist(tk, ctr, n, key_bits, bits, hist, h->grid, st);
-    KC_CUDA(kc::launch_scan(hist, n_buckets, starts, cursor, st));
+    if ((e = kc::launch_scan(hist, n_buckets, starts, cursor, st)) != cudaSuccess) {
+        release();
+        return cuda_fail(e, "cudaMallocAsync(scan)");
+    }
     kc::launch_scatter(tk, tv, ctr, n, key_bits, bits, cursor, out_k, out_v, h->grid, st);
     kc::launch_bucket_sort_warp(out_k, out_v, starts, n_buckets, key_bits, ctr, h->grid, st);
     phase_end(h, phase, t0);
@@ -1495,6 +1498,7 @@ kc_status add_reads_chunked(kc_handle h, Batch& b, int sample, const uint64_t* p
     kc_status s = bucket_batch(h, b, n_local, st, h->params(sample), how, &ch);
     phase_end(h, kPass1, t0);
     if (s != KC_OK) {
+        leave_hashes(h, b);  // (of a first level whose second found no room)
         KC_CUDA(cudaStreamSynchronize(cs));
         for (void* q : {temp, (void*)b.pw}) cudaFreeAsync(q, st);
         b.pw = b.vw = nullptr;
@@ -1643,6 +1647,7 @@ kc_status kc_add_reads(kc_handle h, int sample, const uint64_t* packed_reads, co
             s = KC_OK;
         }
         if (s != KC_OK) {
+            leave_hashes(h, b);  // (of a first level whose second found no room)
             for (void* q : {temp, (void*)b.pw}) cudaFreeAsync(q, st);
             if (any_host) cudaEventSynchronize(h->ev_copy);  // the caller's arrays are no longer read
             return s;

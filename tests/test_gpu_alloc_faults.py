@@ -317,3 +317,48 @@ def test_direct_finalize_made_again(oracle_mod, fail_alloc, chain):
         _same(c, want)
     assert again > 0
     c.close()
+
+
+@pytest.mark.parametrize("place", ["device", "host"])
+def test_failed_calls_keep_no_memory(fail_alloc, place):
+    """Many kc_add_reads calls that fail in every place of a two-level grouping, and many
+    failed sorts, leave the device's free memory where it was."""
+    import torch
+
+    g = synth.genome(370, 300_000)
+    rs = synth.reads(371, g, 120_000, 150, 150, 0.005, 0.0005)
+    packed, mask = kc.pack_ascii(rs.ascii)
+    arrays = _device(rs) if place == "device" else [packed, rs.offsets.astype(np.uint64), mask]
+    c = kc.KmerCounter(31, 1, 1 << 28, 4, 2, strategy="partitioned", part_bits=15)
+    d = kc.KmerCounter(31, 1, 1 << 24, 4, 1, strategy="direct", table_slots=1 << 23)
+
+    def failing(rounds):
+        for n in range(14):
+            for _ in range(rounds):
+                c.reset()
+                fail_alloc(n, 1 << 40)
+                try:
+                    c.add_reads(0, *arrays)
+                except kc.KcError as e:
+                    assert e.name == "KC_ERR_OOM_DEVICE"
+                fail_alloc(0, 0)
+        d.reset()
+        d.add_reads(0, *arrays)
+        for n in range(10):
+            for _ in range(rounds):
+                fail_alloc(n, 1 << 40)
+                try:
+                    d.finalize()
+                except kc.KcError as e:
+                    assert e.name == "KC_ERR_OOM_DEVICE"
+                fail_alloc(0, 0)
+        torch.cuda.synchronize()
+
+    c.add_reads(0, *arrays)
+    c.finalize()
+    failing(1)
+    before = torch.cuda.mem_get_info()[0]
+    failing(8)
+    assert torch.cuda.mem_get_info()[0] > before - (1 << 29)
+    c.close()
+    d.close()
