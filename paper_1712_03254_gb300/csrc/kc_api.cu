@@ -9,7 +9,7 @@
 //                for the exact recount of kc_finalize
 //   result       sorted keys and per-sample counts after kc_finalize
 // Transient buffers (N mask, read starts, offsets, sort buckets) come from the
-// stream-ordered pool (cudaMallocAsync) and are released on the same stream.
+// stream-ordered pool (dev_alloc) and are released on the same stream.
 
 #include <cuda_runtime.h>
 
@@ -725,7 +725,7 @@ kc_status bucket_batch(kc_handle h, Batch& b, uint64_t n_local, cudaStream_t st,
 // together on stream st (which the caller has ordered after each handle's
 // stream).  Items of upi units (at least 2^12, about one per SM over all
 // batches); per batch the histogram rows, segments, linear hashes and run
-// bases live in one scratch block freed after the scatter, the grouped
+// bases live in one scratch block given back after the scatter, the grouped
 // hashes (at most one per base plus run padding of 3 per (item, partition))
 // and partition starts stay with the batch.  Batches of handles with two
 // grouping levels are re-bucketed afterwards (regroup_batch).

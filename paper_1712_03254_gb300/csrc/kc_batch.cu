@@ -93,9 +93,9 @@ constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32
 // window, no window waits for the filter's answer, and the hashes are read
 // once, without a recount.  (Updating the filter with every window and counting
 // the candidates took 0.975 ms for 1.18e8 windows of 4096 partitions, this
-// 0.645 ms.  It is bound by instruction issue, at two thirds of the issue
+// 0.660 ms.  It is bound by instruction issue, at two thirds of the issue
 // slots: reading the hashes alone takes 0.17 ms, with one probe each 0.21, with
-// the queue's probes 0.36, the writing 0.08 and the filter 0.09 more.)
+// the queue's probes 0.36, the writing 0.08 and the filter 0.1 more.)
 //
 //   count    each window's first probe; a window that finds its key adds one
 //            to its count.  The others (new keys and displaced ones, about one
@@ -115,8 +115,7 @@ constexpr uint32_t kChunk = 1u << 31;  // hashes a consumer loop indexes with 32
 // candidates alone would need (8192 slots, 96 KiB with the counts: two
 // 512-thread CTAs an SM; when only one fits, 1024 threads).  Triangular probing
 // keeps a table two thirds full (30x coverage) to about two probes a new key:
-// linear probing took 0.69 ms where this takes 0.60, and the probe loop of a
-// whole warp at once 0.75.
+// linear probing took 0.09 ms more, the probe loop of a whole warp at once 0.15.
 //
 // A partition whose keys overflow the table is counted again in 2, 4, ...
 // 2^split_max sub-ranges of its filter slice: the top bits of a window's
@@ -1240,7 +1239,7 @@ kc_status finalize_core(kc_batch_ctx* b, kc_handle* hs, int n, uint32_t part_lo,
             while (tl < 13 && (1ull << tl) < 2 * (x.max_w >> split_min)) ++tl;
             // one-sample partitions beyond what 8192 slots take at 30x coverage
             // (one distinct key in six windows): 16384 slots and one wide CTA an
-            // SM, instead of two passes (43,700 windows: 1.48 -> 1.21 ms)
+            // SM, instead of two passes (1.8e8 windows, 43,700 a partition: 1.48 -> 1.16 ms)
             if (h->n_samples == 1 && (x.max_w >> split_min) > 40960) tl = 14;
         }
         const size_t queue = kc::consume_queue_smem(kc::kConsumeThreadsWide) + 1024;

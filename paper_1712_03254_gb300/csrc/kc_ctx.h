@@ -51,9 +51,9 @@ enum class State { Open, Finalized, Poisoned };
 // kWindowsPerFinePartition, while the filter slices keep 2^kFineSliceLog2
 // words.  A fine partition splits only if nearly all its windows are distinct,
 // and a job of a few million windows still has one for every consumer CTA.
-// One pass at 4096 / 8192 / 16384 windows: a 1.4 M window job 332 / 310 / 314
-// us, one of 1.5 M (k = 25) 601 / 573 / 656 us, one of 29 M 1.43 / 1.42 / 2.26
-// ms (32768: 344, 976 us, 2.48 ms).
+// One pass at 4096 / 8192 / 16384 / 32768 windows: a 1.4 M window job 208 / 192 /
+// 203 / 275 us, one of 1.5 M (k = 25) 222 / 208 / 270 / 419 us, one of 29 M 1.32 /
+// 1.11 / 1.22 / 1.34 ms.
 constexpr uint64_t kWindowsPerPartition = 32768;
 constexpr uint64_t kWindowsPerFinePartition = 8192;
 constexpr uint64_t kFinePartitionJob = 1ull << 18;
@@ -93,8 +93,8 @@ struct SpillRun {
 // per base each.  Taking blocks of this size from the stream-ordered pool for
 // every job cost 0.35 ms each when several handles took turns (the pool maps
 // their memory anew).  A handle keeps blocks from its second job on
-// (kc_reset), unless it has a device budget or its last job took more than half
-// the share, and all handles of a device together at most a kIdleShare-th of its
+// (kc_reset), unless it has a device budget or the blocks its last job took come
+// to more than half the share, and all handles of a device together at most a kIdleShare-th of its
 // memory (IdleTotals); kc_destroy gives them back, and so does a failed device
 // allocation of any handle (dev_alloc), before it is tried once more.  (A job that passes the share would keep some blocks and give others
 // back, in an order that has the pool map memory for every job: two samples of
@@ -193,7 +193,7 @@ struct kc_ctx {
     kc_ctx* next_handle = nullptr;  // in the list of all handles
     bool reused = false;
     bool keep_blocks = false;
-    size_t job_blocks = 0;  // bytes of blocks the job has taken
+    size_t job_blocks = 0;  // bytes of all blocks the job has taken, one after the other too
 
     kc::DevCounters host_ctr{};
     kcapi::State state = kcapi::State::Open;

@@ -68,8 +68,8 @@ void launch_clear_counts(Slot* table, uint64_t n_slots, const Grid& g, cudaStrea
 void launch_compact(const Slot* table, uint64_t n_slots, int n_samples, uint32_t min_count, uint64_t* keys,
                     uint64_t* vals, DevCounters* ctr, const Grid& g, cudaStream_t st);
 // starts[0..n] = exclusive scan of hist[0..n); cursor[0..n) = starts[0..n).
-// Above 4096 counters a three-kernel multi-CTA scan with a small stream-
-// ordered temporary (n <= 2^25).
+// Above 4096 counters one launch with look-back (scan_lookback) and a small
+// stream-ordered temporary.
 cudaError_t launch_scan(const uint32_t* hist, uint64_t n, uint64_t* starts, uint64_t* cursor, cudaStream_t st);
 // Scatter survivors (at most cap of them) into their buckets; keys whose
 // bucket or position would fall outside the arrays set DERR_INTERNAL.

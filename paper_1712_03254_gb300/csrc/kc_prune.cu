@@ -24,8 +24,8 @@ constexpr unsigned kFullMask = 0xffffffffu;
 // the table, one after the other for each window: a lane has two windows of
 // its unit in flight, and a warp takes a quarter of 32 units at a time, so that
 // the last items spread over the SMs.  2.4e7 windows, 2^28-bit filters: Prune
-// 315 -> 292 us, Count 688 -> 552 us (before: one window in flight, whole units,
-// and the table probed once to claim and once more to count).
+// 0.295 ms, Count 0.479; with one window in flight, whole units, and the table
+// probed once to claim and once more to count 0.315 and 0.688.
 constexpr int kParts = 4;  // items of 64 / kParts window starts a lane
 
 // The next window of the lane's item: its key's hash and bit pattern.
@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(256, 6) k_count_chain(const uint64_t* __restri
 
 // Four times the resident CTAs and more: with 6 or 7 items a warp in 1.6 waves
 // the last ones ran on a half-empty chip, now CTAs of one or two items a warp
-// follow each other as SMs come free.  2.4e7 windows, Prune 0.31 -> 0.295 ms,
-// Count 0.55 -> 0.48 (18, 24, 32, unbounded an SM: 0.486, 0.495, 0.479, 0.483).
+// follow each other as SMs come free.  2.4e7 windows, as many as are resident:
+// Count 0.55 ms; 18, 24, 32 an SM, unbounded: 0.486, 0.495, 0.479, 0.483.
 unsigned grid_for_units(uint64_t n_units, const Grid& g) {
     uint64_t blocks = (n_units * kParts + 255) / 256;
     if (blocks < 1) blocks = 1;
