@@ -96,17 +96,19 @@ def test_sort_of_a_genome_of_few_letters_in_proportion():
     assert skewed < 20 * base, (skewed, base)
 
 
-def test_one_key_making_up_a_third_of_the_reads():
-    """13 and 14 partition bits, whose streams such reads overflow, take little longer than
-    12 bits, which have none: the scatter of the streams is not made."""
+def test_one_key_making_up_much_of_the_reads():
+    """13 and 14 partition bits, whose streams such reads overflow, are grouped one level
+    after the other as 15 bits always are (by a narrower first level): what was tried before
+    that adds little, since the scatter of the streams is not made.  (Made, it took them to
+    1.23 and 1.25 times the time of 15 bits; now 0.68 and 0.87.)"""
     rng = np.random.default_rng(430)
     ascii = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, (200_000, 150))]
     ascii[:90_000] = ord("A")
     rng.shuffle(ascii)
     arrays = _device(synth.ReadSet(ascii.reshape(-1), np.arange(200_001, dtype=np.uint64) * np.uint64(150)))
     took = {}
-    for bits in (12, 13, 14):
+    for bits in (13, 14, 15):
         c = kc.KmerCounter(31, 1, 1 << 28, 4, 2, strategy="partitioned", part_bits=bits)
         took[bits] = _seconds(c, arrays)
         c.close()
-    assert took[13] < 1.5 * took[12] and took[14] < 1.5 * took[12], took
+    assert max(took[13], took[14]) < 1.05 * took[15], took
