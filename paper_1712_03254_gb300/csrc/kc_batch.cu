@@ -1670,6 +1670,7 @@ kc_status finalize_grouped(kc_batch_ctx* b, kc_handle h) {
                 if (s != KC_OK) break;
             }
         }
+        if (s != KC_OK) cudaStreamSynchronize(b->st);  // a failed group may have left fallback kernels that read the pieces
         for (Batch& pc : pieces)
             if (pc.deferred) {
                 leave_hashes(h, pc);

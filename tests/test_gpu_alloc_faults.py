@@ -362,3 +362,45 @@ def test_failed_calls_keep_no_memory(fail_alloc, place):
     assert torch.cuda.mem_get_info()[0] > before - (1 << 29)
     c.close()
     d.close()
+
+
+def test_kept_reads_whose_finalize_fails(oracle_mod, fail_alloc):
+    """A job whose reads were kept for want of room, each partition of which goes to a
+    global table: every allocation of its finalize fails in turn, and the finalize made
+    again after another handle's job gives the oracle's result."""
+    g = synth.genome(380, 60_000)
+    rs = synth.reads(381, g, 20_000, 90, 120, 0.005, 0.0005)
+    other = synth.reads(382, g, 30_000, 90, 120, 0.005, 0.0005)
+    want = _expect(oracle_mod.count(synth.Workload("job", [rs], 31, 1 << 20, 4, 2)))
+    want_other = _expect(oracle_mod.count(synth.Workload("other", [other], 31, 1 << 22, 4, 2)))
+    arrays, other_arrays = _device(rs), _device(other)
+    d = kc.KmerCounter(31, 1, 1 << 22, 4, 2, strategy="partitioned")
+    failed = 0
+    for n in range(0, 400, 7):
+        c = kc.KmerCounter(31, 1, 1 << 20, 4, 2, strategy="partitioned", part_bits=2, smem_table_log2=10, split_max=-1,
+                           device_budget=(1 << 17) + (8 << 20))
+        c.add_reads(0, *arrays)
+        assert c.stats()["deferred_batches"] == 1
+        _take_back_idle_blocks(fail_alloc)
+        fail_alloc(n, 1 << 40)
+        try:
+            c.finalize()
+            done = True
+        except kc.KcError as e:
+            assert e.name == "KC_ERR_OOM_DEVICE"
+            done = False
+        tried = fail_alloc(0, 0)
+        d.reset()
+        d.add_reads(0, *other_arrays)
+        d.finalize()
+        if not done:
+            failed += 1
+            c.finalize()
+        _same(c, want)
+        _same(d, want_other)
+        assert c.stats()["fallback_partitions"] > 0
+        c.close()
+        if tried <= n:
+            break
+    assert failed > 0
+    d.close()
