@@ -273,6 +273,9 @@ bool reclaim_idle(bool locked) {
     bool any = false;
     for (kc_ctx* h = g_handles; h; h = h->next_handle) {
         if (h->device != device || h->idle.empty()) continue;
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+            continue;  // a caller's own stream, in a capture of the caller's
         free_idle_locked(h);
         cudaStreamSynchronize(h->stream);
         any = true;
@@ -939,6 +942,7 @@ Grouping grouping_for(kc_handle h, uint64_t n_local) {
 // most of the reads has hundreds of them (36 M windows of a genome with 95 % A and
 // T: 483 ranges one after the other, a hundred launches each, took 159 ms).
 kc_status sort_ranges(std::vector<kc::SortRange>& ranges, cudaStream_t st, uint64_t* launches) {
+    if (ranges.empty()) return KC_OK;
     std::sort(ranges.begin(), ranges.end(), [](const kc::SortRange& x, const kc::SortRange& y) { return x.n < y.n; });
     kc::SortRange* list = nullptr;
     cudaError_t e = kc::dev_alloc(&list, ranges.size() * sizeof(kc::SortRange), st);

@@ -404,3 +404,46 @@ def test_kept_reads_whose_finalize_fails(oracle_mod, fail_alloc):
             break
     assert failed > 0
     d.close()
+
+
+def test_idle_blocks_of_a_stream_in_a_capture(fail_alloc):
+    """A handle on a caller's stream keeps blocks while the caller captures that stream: an
+    allocation that fails on another thread leaves the blocks and the capture alone."""
+    import threading
+
+    import torch
+
+    g = synth.genome(390, 60_000)
+    arrays = _device(synth.reads(391, g, 30_000, 90, 120, 0.005, 0.0005))
+    stream = torch.cuda.Stream()
+    c = kc.KmerCounter(31, 1, 1 << 22, 4, 2, strategy="partitioned", stream=stream.cuda_stream)
+    _take_back_idle_blocks(fail_alloc)
+    _keep_blocks(c, arrays)
+    kept = c.stats()["device_bytes"]
+    x = torch.zeros(64, device="cuda")
+    torch.cuda.synchronize()
+    seen = []
+
+    def other():
+        fail_alloc(0, 1)
+        try:
+            kc.KcBatch()
+        except kc.KcError as e:
+            seen.append(e.name)
+        fail_alloc(0, 0)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        x.add_(1)
+        t = threading.Thread(target=other)
+        t.start()
+        t.join()
+        x.add_(1)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert seen == ["KC_ERR_OOM_DEVICE"] and c.stats()["device_bytes"] == kept
+    assert float(x.sum()) == 128.0
+    c.add_reads(0, *arrays)
+    c.finalize()
+    assert c.result_size() > 0
+    c.close()
